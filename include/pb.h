@@ -133,8 +133,10 @@ typedef struct {
 } pb_params;
 
 /* Solver options.  precision PB_FP64: Jacobi-PCG entirely in FP64.
- * PB_MIXED: FP64 iterative refinement around an FP32 Jacobi-PCG (FP32
- * stencil, vectors and per-thread accumulation, FP64 global dots).
+ * PB_MIXED: FP64 iterative refinement around an FP32 PCG (FP32 stencil,
+ * vectors and per-thread accumulation, FP64 global dots), preconditioned on
+ * uniform grids of at least 9 nodes an axis by one multigrid V-cycle, else by
+ * the diagonal.
  * Stop when ||f - A phi||_2 <= rtol ||f||_2 (true residual, FP64).
  * max_iter caps the total inner iterations, max_outer the refinement
  * steps; inner_rtol (0 = default 1e-6) is the inner relative tolerance;
@@ -267,9 +269,9 @@ void pb_system_free(pb_system *s);
  * carries no FP32 rounding).  Results stay on the device inside s. */
 pb_status pb_coulomb_terms(pb_system *s, int32_t which, void *stream);
 
-/* pb_solve -- Jacobi-preconditioned CG for (G^T W G + C) phi = f (the
- * Krylov solve of Eq. matrixequation), zero initial guess, in the
- * precision of opts.  On PB_OK or PB_ERR_NOCONV the best phi is kept in s.
+/* pb_solve -- preconditioned CG (multigrid or Jacobi, see pb_solve_opts) for
+ * (G^T W G + C) phi = f (the Krylov solve of Eq. matrixequation), zero
+ * initial guess, in the precision of opts.  On PB_OK or PB_ERR_NOCONV the best phi is kept in s.
  * If phi_dev is not NULL the solution (all N nodes, boundary values
  * included, double) is also copied to that device buffer. */
 pb_status pb_solve(pb_system *s, const pb_solve_opts *opts, double *phi_dev, void *stream,
@@ -393,9 +395,8 @@ pb_status pb_set_tuning(pb_system *s, int32_t precision, int32_t variant, int32_
  * neighbours into each receiver's memory (cudaMemcpyPeerAsync); each
  * kernel round's partial dot products are added in rank order and the CG
  * update is written to every rank, so all ranks take the same decisions.
- * In this build every rank lives on the system's device.  ranks = 1 gives
- * pb_solve's result bit for bit (same z-chunk); more ranks change only the
- * order of the dot-product sums.  phi is gathered back into s (pb_energy
+ * In this build every rank lives on the system's device.  ranks = 1 is
+ * pb_solve itself; more ranks run the Jacobi-preconditioned PCG.  phi is gathered back into s (pb_energy
  * works as after pb_solve).  Errors: PB_ERR_ARG for a bad rank count or a
  * precision other than PB_MIXED, PB_ERR_UNIMPL for octree systems, and the
  * statuses of pb_solve. */

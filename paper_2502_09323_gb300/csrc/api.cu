@@ -302,6 +302,7 @@ void pb_system_free(pb_system *s) {
     oct_system_free(s, st);
     cudaStreamSynchronize(st);
     free_tma_state(s);
+    free_mg_state(s);
     if (s->h_st) cudaFreeHost(s->h_st);
     if (s->h_energy) cudaFreeHost(s->h_energy);
     delete s;

@@ -44,7 +44,7 @@ struct EngineSlot {
 // residual.  Arms the next inner solve in the slot's CG state, or ends the
 // solve (done = 1 keeps the PCG kernels off the slot).
 __global__ void k_ir_step(EngineSlot *slot, int first, long long ticket, double rtol,
-                          double inner_rtol, int max_iter, int max_outer) {
+                          double inner_rtol, int max_iter, int max_outer, int mg) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     CgState &st = slot->st;
     IrCtl &c = slot->ctl;
@@ -97,7 +97,8 @@ __global__ void k_ir_step(EngineSlot *slot, int first, long long ticket, double 
         if (itol > 0.5) itol = 0.5;
         const double rz = st.rz64, res64 = st.res64;
         CgState h{};
-        h.rho = rz;
+        h.mg = mg;
+        h.rho = mg ? 0.0 : rz;  // multigrid: the first cycle sets it
         h.rr0 = c.res2;
         h.rr = c.res2;
         h.rr_stop = itol * itol * c.res2;
@@ -140,8 +141,14 @@ struct Engine {
     cudaEvent_t ev_chunk[2] = {nullptr, nullptr}, ev_tab[2] = {nullptr, nullptr};
     bool tab_used[2] = {false, false};
     int tab_buf = 0;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    // one replay, by the number of multigrid levels above the bottom kernel
+    // that it runs (0: Jacobi-preconditioned systems only), captured when
+    // a table first needs it
+    cudaGraph_t graph[mg::LMAX] = {};
+    cudaGraphExec_t exec[mg::LMAX] = {};
+    int depth = 0;                                     // the current table's
+    mg::Entry *dmg = nullptr, *hmg = nullptr;          // staging: 2 x cap, pinned
+    mg::Head *dhead = nullptr, *hhead = nullptr;       // staging: 2, pinned
     dim3 grid;
 
     std::thread th;
@@ -197,7 +204,7 @@ bool engine_install(Engine *e, int q) {
     ENG_TRY(cudaMemsetAsync(sys->d32, 0, b32, e->cs), "correction reset");
     ENG_TRY(cudaMemsetAsync(sys->pa32, 0, b32, e->cs), "direction reset");
     k_ir_step<<<1, 32, 0, e->cs>>>(e->dslots + q, 1, hs.job.ticket, e->rtol, e->inner_rtol,
-                                   e->max_iter, e->max_outer);
+                                   e->max_iter, e->max_outer, sys->mg != nullptr);
     ENG_TRY(cudaGetLastError(), "refinement step launch");
     note_launch(2);
     return true;
@@ -229,10 +236,43 @@ bool engine_refine(Engine *e, int q, bool aborted) {
     ENG_TRY(cudaMemsetAsync(sys->d32, 0, b32, e->cs), "correction reset");
     ENG_TRY(cudaMemsetAsync(sys->pa32, 0, b32, e->cs), "direction reset");
     k_ir_step<<<1, 32, 0, e->cs>>>(e->dslots + q, 0, hs.job.ticket, e->rtol, e->inner_rtol,
-                                   e->max_iter, e->max_outer);
+                                   e->max_iter, e->max_outer, sys->mg != nullptr);
     ENG_TRY(cudaGetLastError(), "refinement step launch");
     note_launch(3);
     hs.expect_gen += 1;
+    return true;
+}
+
+// PCG iterations of one replay: few with multigrid (a solve takes about 15
+// a refinement step), more with Jacobi
+int engine_chunk(const Engine *e) { return e->depth > 0 ? 2 : e->chunk; }
+
+// capture one replay for tables of the current depth
+bool engine_capture(Engine *e) {
+    const int depth = e->depth;
+    if (e->exec[depth]) return true;
+    static const unsigned rd0 = mg_resident(k_mg_down<true, false>), rd1 = mg_resident(k_mg_down<false, false>),
+                          ru0 = mg_resident(k_mg_up<true, false>), ru1 = mg_resident(k_mg_up<false, false>);
+    const mg::Entry none{};
+    ENG_TRY(cudaStreamBeginCapture(e->cs, cudaStreamCaptureModeThreadLocal), "capture");
+    for (int c = 0; c < engine_chunk(e); ++c) {
+        for (int l = 0; l < depth; ++l)
+            if (l == 0)
+                k_mg_down<true, false><<<rd0, mg::NT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+            else
+                k_mg_down<false, false><<<rd1, mg::NT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+        if (depth > 0)
+            k_mg_bottom<false><<<e->cap, mg::BOT_T, 28 * mg::BOT_NODES, e->cs>>>(e->dmg, e->dhead, none);
+        for (int l = depth - 1; l >= 0; --l)
+            if (l == 0)
+                k_mg_up<true, false><<<ru0, mg::NT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+            else
+                k_mg_up<false, false><<<ru1, mg::NT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+        tma_launch<MODE_P>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
+        tma_launch<MODE_U>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
+    }
+    ENG_TRY(cudaStreamEndCapture(e->cs, &e->graph[depth]), "capture");
+    ENG_TRY(cudaGraphInstantiate(&e->exec[depth], e->graph[depth], 0), "graph instantiation");
     return true;
 }
 
@@ -242,7 +282,27 @@ bool engine_upload_table(Engine *e) {
     const int b = e->tab_buf;
     if (e->tab_used[b]) ENG_TRY(cudaEventSynchronize(e->ev_tab[b]), "table staging reuse");
     tma::SysEntry *h = e->htab + (size_t)b * e->cap;
-    int total = 0;
+    mg::Entry *hm = e->hmg + (size_t)b * e->cap;
+    mg::Head &head = e->hhead[b];
+    head = mg::Head{};
+    head.nsys = e->cap;
+    int total = 0, depth = 0;
+    for (int q = 0; q < e->cap; ++q) {
+        const HostSlot &hq = e->slots[q];
+        mg::Entry &me = hm[q];
+        if (hq.used && !hq.job.oct && hq.job.sys->mg)
+            me = ((const MgState *)hq.job.sys->mg)->e;
+        else
+            memset(&me, 0, sizeof(me));
+        me.st = &e->dslots[q].st;
+        depth = std::max(depth, me.nbot);
+        for (int l = 0; l < mg::LMAX; ++l) {
+            me.dbase[l] = head.dtotal[l];
+            me.ubase[l] = head.utotal[l];
+            head.dtotal[l] += mg::ditems(me, l);
+            head.utotal[l] += mg::uitems(me, l);
+        }
+    }
     for (int q = 0; q < e->cap; ++q) {
         tma::SysEntry &en = h[q];
         const HostSlot &hs = e->slots[q];
@@ -268,10 +328,15 @@ bool engine_upload_table(Engine *e) {
     ENG_TRY(cudaMemcpyAsync(e->queue + 2, hdr + 2, 2 * sizeof(unsigned int), cudaMemcpyHostToDevice,
                             e->cs),
             "table size upload");
+    ENG_TRY(cudaMemcpyAsync(e->dmg, hm, sizeof(mg::Entry) * e->cap, cudaMemcpyHostToDevice, e->cs),
+            "multigrid table upload");
+    ENG_TRY(cudaMemcpyAsync(e->dhead, &head, sizeof(mg::Head), cudaMemcpyHostToDevice, e->cs),
+            "multigrid table size upload");
     ENG_TRY(cudaEventRecord(e->ev_tab[b], e->cs), "table event");
     e->tab_used[b] = true;
     e->tab_buf ^= 1;
-    return true;
+    e->depth = depth;
+    return engine_capture(e);
 }
 
 // a slot's solve ended: report it and free the slot
@@ -291,7 +356,7 @@ void engine_complete(Engine *e, int q, const EngineSlot &m) {
     r.stats.kc = hs.job.oct ? 0 : hs.job.kc + 1000 + 10000 * hs.job.tw;
     r.stats.true_rel_res = m.ctl.fn2 > 0.0 ? sqrt(m.ctl.res2 / m.ctl.fn2) : 0.0;
     r.stats.dof = hs.job.dof;
-    r.stats.model_bytes = (long long)m.ctl.iters * r.stats.dof * (8 * 4 + 2) +
+    r.stats.model_bytes = (long long)m.ctl.iters * r.stats.dof * (8 * 4 + 2 + (sys->mg ? 24 : 0)) +
                           (long long)m.ctl.outer * g.N * 64;
     r.t_submit = hs.job.t_submit;
     r.t_admit = hs.t_admit;
@@ -306,13 +371,14 @@ void engine_complete(Engine *e, int q, const EngineSlot &m) {
 }
 
 bool engine_issue(Engine *e, int mb) {
-    ENG_TRY(cudaGraphLaunch(e->exec, e->cs), "replay");
-    note_launch(2 * e->chunk);
+    const int chunk = engine_chunk(e);
+    ENG_TRY(cudaGraphLaunch(e->exec[e->depth], e->cs), "replay");
+    note_launch(chunk * (2 + (e->depth > 0 ? 2 * e->depth + 1 : 0)));
     // octree systems: the same number of iterations with their brick kernels
     for (int q = 0; q < e->cap; ++q) {
         const HostSlot &hs = e->slots[q];
         if (!hs.used || !hs.job.oct) continue;
-        if (oct_engine_iterations(hs.job.sys, e->chunk, e->cs) != PB_OK) {
+        if (oct_engine_iterations(hs.job.sys, chunk, e->cs) != PB_OK) {
             engine_fail(e, "octree iterations", cudaGetLastError());
             return false;
         }
@@ -433,13 +499,17 @@ void engine_pump(Engine *e) {
 #undef ENG_TRY
 
 void engine_release(Engine *e) {
-    if (e->exec) cudaGraphExecDestroy(e->exec);
-    if (e->graph) cudaGraphDestroy(e->graph);
+    for (cudaGraphExec_t x : e->exec)
+        if (x) cudaGraphExecDestroy(x);
+    for (cudaGraph_t x : e->graph)
+        if (x) cudaGraphDestroy(x);
     if (e->cs) cudaStreamSynchronize(e->cs);
     for (cudaEvent_t ev : {e->ev_chunk[0], e->ev_chunk[1], e->ev_tab[0], e->ev_tab[1]})
         if (ev) cudaEventDestroy(ev);
     dfree(e->dslots, e->cs);
     dfree(e->dtab, e->cs);
+    dfree(e->dmg, e->cs);
+    dfree(e->dhead, e->cs);
     dfree(e->queue, e->cs);
     if (e->cs) {
         cudaStreamSynchronize(e->cs);
@@ -447,6 +517,8 @@ void engine_release(Engine *e) {
     }
     if (e->hmirror) cudaFreeHost(e->hmirror);
     if (e->htab) cudaFreeHost(e->htab);
+    if (e->hmg) cudaFreeHost(e->hmg);
+    if (e->hhead) cudaFreeHost(e->hhead);
     if (e->hhdr) cudaFreeHost(e->hhdr);
     delete e;
 }
@@ -479,29 +551,25 @@ pb_status engine_create(int device, int capacity, const pb_solve_opts *o, pb_eng
     e->dslots = (EngineSlot *)dalloc(sizeof(EngineSlot) * capacity, e->cs);
     e->dtab = (tma::SysEntry *)dalloc(sizeof(tma::SysEntry) * capacity, e->cs);
     e->queue = (unsigned int *)dalloc(4 * sizeof(unsigned int), e->cs);
-    if (!e->dslots || !e->dtab || !e->queue) return bail(PB_ERR_OOM, "device allocation");
+    e->dmg = (mg::Entry *)dalloc(sizeof(mg::Entry) * capacity, e->cs);
+    e->dhead = (mg::Head *)dalloc(sizeof(mg::Head), e->cs);
+    if (!e->dslots || !e->dtab || !e->queue || !e->dmg || !e->dhead) return bail(PB_ERR_OOM, "device allocation");
     if (cudaMallocHost((void **)&e->hmirror, 2 * sizeof(EngineSlot) * capacity) != cudaSuccess ||
         cudaMallocHost((void **)&e->htab, 2 * sizeof(tma::SysEntry) * capacity) != cudaSuccess ||
-        cudaMallocHost((void **)&e->hhdr, 8 * sizeof(unsigned int)) != cudaSuccess)
+        cudaMallocHost((void **)&e->hhdr, 8 * sizeof(unsigned int)) != cudaSuccess ||
+        cudaMallocHost((void **)&e->hmg, 2 * sizeof(mg::Entry) * capacity) != cudaSuccess ||
+        cudaMallocHost((void **)&e->hhead, 2 * sizeof(mg::Head)) != cudaSuccess)
         return bail(PB_ERR_OOM, "pinned host allocation");
     memset(e->hhdr, 0, 8 * sizeof(unsigned int));
     if (cudaMemsetAsync(e->dslots, 0, sizeof(EngineSlot) * capacity, e->cs) != cudaSuccess ||
         cudaMemsetAsync(e->dtab, 0, sizeof(tma::SysEntry) * capacity, e->cs) != cudaSuccess ||
-        cudaMemsetAsync(e->queue, 0, 4 * sizeof(unsigned int), e->cs) != cudaSuccess)
+        cudaMemsetAsync(e->queue, 0, 4 * sizeof(unsigned int), e->cs) != cudaSuccess ||
+        cudaMemsetAsync(e->dmg, 0, sizeof(mg::Entry) * capacity, e->cs) != cudaSuccess ||
+        cudaMemsetAsync(e->dhead, 0, sizeof(mg::Head), e->cs) != cudaSuccess)
         return bail(PB_ERR_CUDA, "initialisation");
-    if (tma_prepare<MODE_P>() != PB_OK || tma_prepare<MODE_U>() != PB_OK)
+    if (tma_prepare<MODE_P>() != PB_OK || tma_prepare<MODE_U>() != PB_OK || mg_prepare() != PB_OK)
         return bail(PB_ERR_CUDA, "kernel attributes");
     e->grid = tma_grid(PadGeo{}, 8);
-    // one replay: `chunk` PCG iterations of whatever the table holds
-    if (cudaStreamBeginCapture(e->cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
-        return bail(PB_ERR_CUDA, "capture");
-    for (int c = 0; c < e->chunk; ++c) {
-        tma_launch<MODE_P>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
-        tma_launch<MODE_U>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
-    }
-    if (cudaStreamEndCapture(e->cs, &e->graph) != cudaSuccess ||
-        cudaGraphInstantiate(&e->exec, e->graph, 0) != cudaSuccess)
-        return bail(PB_ERR_CUDA, "graph instantiation");
     if (cudaStreamSynchronize(e->cs) != cudaSuccess) return bail(PB_ERR_CUDA, "set-up");
     try {
         e->th = std::thread(engine_pump, e);
@@ -530,7 +598,7 @@ pb_status engine_submit(pb_engine *eh, pb_system *sys, cudaStream_t s, long long
         j.dof = sys->os->nunk;
     } else {
         if ((rc = ensure_solver_ws(sys, PB_MIXED, s)) != PB_OK) return rc;
-        if ((rc = build_tma_state(sys)) != PB_OK) return rc;
+        if ((rc = build_tma_state(sys, s)) != PB_OK) return rc;
         Tuning tune;
         if ((rc = autotune(sys, PB_MIXED, s, &tune)) != PB_OK) return rc;
         j.kc = tune.variant == 1 ? std::max(tune.kc, 4) : 8;

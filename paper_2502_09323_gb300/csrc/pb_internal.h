@@ -160,6 +160,9 @@ struct CgState {
     int split;       // 1: one slab of a split solve (the launch stores its totals in
                      // part0/part1; the CG update runs after the rank-ordered sum)
     double part0, part1;
+    int mg;          // 1: rho and beta come from the multigrid cycle (the update kernel
+                     // leaves them alone)
+    int pad;
 };
 
 struct EnergyAcc {
@@ -203,6 +206,7 @@ struct pb_system {
     int solved, have_surface, have_pairs;
     double fnorm2;
     void *tma;          // tensor maps of the FP32 stencil kernels (host object)
+    void *mg;           // multigrid hierarchy of the FP32 solver (host object; null: Jacobi)
     unsigned int *queue;  // work counters of the TMA stencil kernels (device)
     pbg::OctSys *os;    // octree systems: level-transition rows
 };
@@ -231,6 +235,7 @@ pb_status apply_op(pb_system *sys, int precision, const void *x, void *y, cudaSt
 pb_status ensure_solver_ws(pb_system *sys, int precision, cudaStream_t s);
 pb_status profile_kernels(pb_system *sys, int precision, int which, int reps, cudaStream_t s);
 void free_tma_state(pb_system *sys);
+void free_mg_state(pb_system *sys);
 pb_status set_tuning(pb_system *sys, int precision, int variant, int kc);
 pb_status set_wait_limit(long long polls);
 pb_status solve_batch(pb_system *const *systems, int n, const pb_solve_opts *o, cudaStream_t s,

@@ -1,9 +1,9 @@
 // Krylov solve of the condensed system A phi = f (Sec. 3.1, Eq.
-// matrixequation): Jacobi-preconditioned conjugate gradient with fused
-// stencil/dot/axpy kernels, in FP64, or in FP32 inside FP64 iterative
-// refinement.
+// matrixequation): preconditioned conjugate gradient with fused
+// stencil/dot/axpy kernels, in FP64 (Jacobi), or in FP32 (multigrid, mg.cuh;
+// Jacobi where a grid has no hierarchy) inside FP64 iterative refinement.
 //
-// Iteration (z = D^-1 r is stored instead of r; r = D z is formed on the fly):
+// Iteration with the Jacobi preconditioner (z = D^-1 r is stored instead of r; r = D z is formed on the fly):
 //   kernel P:  p <- z + beta p ;  q = A p ;  sigma = p.q      -> alpha = rho/sigma
 //   kernel U:  q = A p (recomputed) ; x += alpha p ; z -= alpha D^-1 q ;
 //              rho' = (Dz).z ; rr = |Dz|^2                    -> beta = rho'/rho
@@ -825,25 +825,34 @@ void tma_entry_geometry(tma::SysEntry &e, const PadGeo &g, int KC, int tw) {
     e.item_base = 0;
 }
 
-// the direction and update maps of a system's entry for tiles of width tw
+CoefC32 make_c32(const pb_system *sys);
+
+}  // namespace
+
+#include "mg.cuh"
+
+namespace {
+
+// the direction and update maps of a system's entry for tiles of width tw; the
+// direction kernel reads the multigrid cycle's result where there is one
 pb_status tma_sys_maps(pb_system *sys, tma::SysEntry &e, int tw) {
     const float *pbuf[2] = {sys->pa32, sys->pb32};
     pb_status rc = PB_OK;
     for (int c = 0; c < 2 && rc == PB_OK; ++c) {
-        rc = tma_maps(sys, MODE_P, sys->z32, pbuf[c], nullptr, nullptr, &e.P[c], tw);
+        rc = tma_maps(sys, MODE_P, sys->mg ? ((const MgState *)sys->mg)->v : sys->z32, pbuf[c], nullptr, nullptr,
+                      &e.P[c], tw);
         if (rc == PB_OK)
             rc = tma_maps(sys, MODE_U, pbuf[c ^ 1], nullptr, sys->d32, sys->z32, &e.U[c], tw);
     }
     return rc;
 }
 
-CoefC32 make_c32(const pb_system *sys);
-
-pb_status build_tma_state(pb_system *sys) {
+pb_status build_tma_state(pb_system *sys, cudaStream_t s) {
     if (sys->tma) return PB_OK;
+    const pb_status mrc = build_mg_state(sys, s);
+    if (mrc != PB_OK) return mrc;
     TmaState *t = new (std::nothrow) TmaState();
     if (!t) return PB_ERR_OOM;
-    cudaStream_t s = sys->stream;
     pb_status rc = PB_OK;
     tma::SysEntry &e = t->host;
     rc = tma_sys_maps(sys, e, t->tw);
@@ -1060,7 +1069,7 @@ pb_status residual(pb_system *sys, bool fp32_out, cudaStream_t s) {
 // copy of the state after every chunk, keeping two chunks in flight.
 template <typename T, class CP>
 pb_status run_pcg(pb_system *sys, const CP &cp, T *z, T *pa, T *pb, T *x, int KC, int variant,
-                  int tw, int chunk,
+                  int tw, bool mg, int chunk,
                   double deadline, cudaStream_t s, int *iters_out) {
     T *bufs[2] = {pa, pb};
     int cur = 0;  // index of p_old
@@ -1072,6 +1081,7 @@ pb_status run_pcg(pb_system *sys, const CP &cp, T *z, T *pa, T *pb, T *x, int KC
     auto issue = [&](int slot) -> pb_status {
         for (int c = 0; c < chunk; ++c) {
             if constexpr (std::is_same<T, float>::value) {
+                if (mg) note_launch(launch_vcycle(sys, s));
                 if (variant == 1)
                     launch_iter_tma(sys, cp, cur, KC, tw, s);
                 else
@@ -1135,10 +1145,11 @@ out:
 }
 
 pb_status init_state(pb_system *sys, double rho, double rr0, double rr_stop, int max_iter,
-                     cudaStream_t s, int profile = 0) {
+                     cudaStream_t s, int profile = 0, bool mg = false) {
     CgState h{};
     h.profile = profile;
-    h.rho = rho;
+    h.mg = mg;
+    h.rho = mg ? 0.0 : rho;  // the first cycle sets it
     h.rr0 = rr0;
     h.rr = rr0;
     h.rr_stop = rr_stop;
@@ -1295,8 +1306,9 @@ pb_status autotune(pb_system *sys, int precision, cudaStream_t s, Tuning *out) {
         // last tile that a wider candidate wrote and a narrower tile never
         // rewrites (the boundary column among them): clear them all.
         const size_t b32 = sizeof(float) * (size_t)g.Np;
-        for (float *v : {sys->z32, sys->pa32, sys->pb32, sys->d32})
-            PB_CUDA_TRY(cudaMemsetAsync(v, 0, b32, s));
+        for (float *v : {sys->z32, sys->pa32, sys->pb32, sys->d32,
+                         sys->mg ? ((MgState *)sys->mg)->v : nullptr})
+            if (v) PB_CUDA_TRY(cudaMemsetAsync(v, 0, b32, s));
     }
     float best_ms = 1e30f;
     for (size_t c = 0; c < cand.size(); ++c) {
@@ -1422,7 +1434,7 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
     const PadGeo &p = sys->pad;
     pb_status rc = ensure_solver_ws(sys, o->precision, s);
     if (rc != PB_OK) return rc;
-    if (o->precision == PB_MIXED && (rc = build_tma_state(sys)) != PB_OK) return rc;
+    if (o->precision == PB_MIXED && (rc = build_tma_state(sys, s)) != PB_OK) return rc;
     Tuning tune;
     if ((rc = autotune(sys, o->precision, s, &tune)) != PB_OK) return rc;
     int max_iter = o->max_iter > 0 ? o->max_iter : 100000;
@@ -1443,6 +1455,8 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
         res2 = fn2;
         outer = 1;
         CoefC32 cp = make_c32(sys);
+        // the multigrid preconditioner goes with the TMA-staged kernels
+        const bool mg = sys->mg && tune.variant == 1;
         int stagnant = 0;
         while (fn2 > 0.0 && res2 > rtol * rtol * fn2) {
             if (outer > max_outer || iters >= max_iter) {
@@ -1453,14 +1467,14 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
             double itol = std::max(inner_rtol, 0.5 * rtol / rel);
             if (itol > 0.5) itol = 0.5;
             double rz = sys->h_st->rz64;
-            if ((rc = init_state(sys, rz, res2, itol * itol * res2, max_iter - iters, s)) != PB_OK)
+            if ((rc = init_state(sys, rz, res2, itol * itol * res2, max_iter - iters, s, 0, mg)) != PB_OK)
                 return rc;
             size_t bytes32 = sizeof(float) * (size_t)p.Np;
             PB_CUDA_TRY(cudaMemsetAsync(sys->d32, 0, bytes32, s));
             PB_CUDA_TRY(cudaMemsetAsync(sys->pa32, 0, bytes32, s));
             int it = 0;
             rc = run_pcg<float, CoefC32>(sys, cp, sys->z32, sys->pa32, sys->pb32, sys->d32, tune.kc,
-                                         tune.variant, tune.tw, chunk, deadline, s, &it);
+                                         tune.variant, tune.tw, mg, mg ? 2 : chunk, deadline, s, &it);
             if (rc == PB_OK && sys->h_st[0].status == 3) {
                 // the correction of an aborted inner solve is incomplete: it
                 // is not promoted, phi keeps the last refined iterate
@@ -1513,7 +1527,7 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
             PB_CUDA_TRY(cudaMemsetAsync(sys->pa64, 0, bytes64, s));
             int it = 0;
             rc = run_pcg<double, CoefS64>(sys, cp, sys->z64, sys->pa64, sys->pb64, sys->x64, tune.kc,
-                                          0, tma::TWDEF, chunk, deadline, s, &it);
+                                          0, tma::TWDEF, false, chunk, deadline, s, &it);
             if (rc == PB_ERR_TIMEOUT) status = PB_ERR_TIMEOUT;
             else if (rc != PB_OK) return rc;
             if (rc == PB_OK) iters += it;
@@ -1540,7 +1554,9 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
         stats->dof = (long long)(g.nx - 2) * (g.ny - 2) * (g.nz - 2);
         // FP32: P reads z,p_old writes p; U reads p,x,z writes x,z (+2 code bytes);
         // FP64 plain: same vectors plus three weight arrays streamed twice.
+        // A multigrid cycle adds 15 B on the finest grid and about 9 on the coarse ones.
         long long per = o->precision == PB_MIXED ? (8 * 4 + 2) : (8 * 8 + 6 * 8 + 2);
+        if (o->precision == PB_MIXED && sys->mg && tune.variant == 1) per += 24;
         stats->model_bytes = (long long)iters * stats->dof * per + (long long)outer * g.N * 64;
     }
     return (pb_status)status;
@@ -1566,7 +1582,7 @@ pb_status profile_kernels(pb_system *sys, int precision, int which, int reps, cu
         return PB_ERR_STATE;
     }
     pb_status rc = PB_OK;
-    if (precision == PB_MIXED && (rc = build_tma_state(sys)) != PB_OK) return rc;
+    if (precision == PB_MIXED && (rc = build_tma_state(sys, s)) != PB_OK) return rc;
     Tuning tune;
     if ((rc = autotune(sys, precision, s, &tune)) != PB_OK) return rc;
     if ((rc = init_state(sys, 1.0, 1.0, -1.0, 1 << 30, s, 1)) != PB_OK) return rc;

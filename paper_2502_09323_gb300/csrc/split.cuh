@@ -24,9 +24,8 @@
 // and the last rank's high halo hold zeros (vectors) and the boundary values
 // (phi) and are never exchanged.
 //
-// One rank (R = 1) takes exactly the single solve's arithmetic: its result
-// is bit-identical to pb_solve's with the same z-chunk.  With R > 1 only the
-// order of the dot-product sums changes.
+// One rank (R = 1) is the single solve itself.  R > 1 ranks run the
+// Jacobi-preconditioned PCG on their slabs.
 
 namespace {
 
@@ -292,11 +291,13 @@ pb_status solve_split(pb_system *sys, int R, const pb_solve_opts *o, cudaStream_
         set_error("pb_solve_split: ranks must be between 1 and min(64, nz - 2)");
         return PB_ERR_ARG;
     }
+    // one rank is the single solve (and has its preconditioner)
+    if (R == 1) return solve(sys, o, s, stats);
     int dev = 0;
     PB_CUDA_TRY(cudaGetDevice(&dev));
     pb_status rc = ensure_solver_ws(sys, PB_MIXED, s);
     if (rc != PB_OK) return rc;
-    if ((rc = build_tma_state(sys)) != PB_OK) return rc;
+    if ((rc = build_tma_state(sys, s)) != PB_OK) return rc;
     Tuning tune;
     if ((rc = autotune(sys, PB_MIXED, s, &tune)) != PB_OK) return rc;
     const int KC = std::max(tune.kc, 4), TW = tune.tw;

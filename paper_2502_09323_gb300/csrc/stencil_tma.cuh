@@ -847,8 +847,10 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                     st->alpha = st->rho / t0;
                 }
             } else {
-                st->beta = t0 / st->rho;
-                st->rho = t0;
+                if (!st->mg) {  // else the multigrid cycle sets them
+                    st->beta = t0 / st->rho;
+                    st->rho = t0;
+                }
                 st->rr = t1;
                 st->iter += 1;
                 st->cur ^= 1;  // the new p_old is this iteration's p
