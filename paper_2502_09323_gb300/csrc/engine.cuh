@@ -251,23 +251,23 @@ int engine_chunk(const Engine *e) { return e->depth > 0 ? 2 : e->chunk; }
 bool engine_capture(Engine *e) {
     const int depth = e->depth;
     if (e->exec[depth]) return true;
-    static const unsigned rd0 = mg_resident(k_mg_down<true, false>), rd1 = mg_resident(k_mg_down<false, false>),
-                          ru0 = mg_resident(k_mg_up<true, false>), ru1 = mg_resident(k_mg_up<false, false>);
+    static const unsigned rd0 = mg_resident(k_mg_down<true, false>, mg::DNT), rd1 = mg_resident(k_mg_down<false, false>, mg::DNT),
+                          ru0 = mg_resident(k_mg_up<true, false>, mg::UNT), ru1 = mg_resident(k_mg_up<false, false>, mg::UNT);
     const mg::Entry none{};
     ENG_TRY(cudaStreamBeginCapture(e->cs, cudaStreamCaptureModeThreadLocal), "capture");
     for (int c = 0; c < engine_chunk(e); ++c) {
         for (int l = 0; l < depth; ++l)
             if (l == 0)
-                k_mg_down<true, false><<<rd0, mg::NT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                k_mg_down<true, false><<<rd0, mg::DNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
             else
-                k_mg_down<false, false><<<rd1, mg::NT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                k_mg_down<false, false><<<rd1, mg::DNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
         if (depth > 0)
-            k_mg_bottom<false><<<e->cap, mg::BOT_T, 28 * mg::BOT_NODES, e->cs>>>(e->dmg, e->dhead, none);
+            k_mg_bottom<false><<<e->cap, mg::BOT_T, mg::BOT_BYTES * mg::BOT_NODES, e->cs>>>(e->dmg, e->dhead, none);
         for (int l = depth - 1; l >= 0; --l)
             if (l == 0)
-                k_mg_up<true, false><<<ru0, mg::NT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                k_mg_up<true, false><<<ru0, mg::UNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
             else
-                k_mg_up<false, false><<<ru1, mg::NT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                k_mg_up<false, false><<<ru1, mg::UNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
         tma_launch<MODE_P>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
         tma_launch<MODE_U>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
     }
@@ -287,6 +287,11 @@ bool engine_upload_table(Engine *e) {
     head = mg::Head{};
     head.nsys = e->cap;
     int total = 0, depth = 0;
+    // tables that fill the GPU with the longest work items take those
+    long long nodes = 0;
+    for (const HostSlot &hq : e->slots)
+        if (hq.used && !hq.job.oct && hq.job.sys->mg) nodes += hq.job.sys->pad.Np;
+    const bool shared = nodes > 1024ll * 16 * 3 * num_sms();
     for (int q = 0; q < e->cap; ++q) {
         const HostSlot &hq = e->slots[q];
         mg::Entry &me = hm[q];
@@ -295,6 +300,7 @@ bool engine_upload_table(Engine *e) {
         else
             memset(&me, 0, sizeof(me));
         me.st = &e->dslots[q].st;
+        if (shared) mg_planes(me, true);
         depth = std::max(depth, me.nbot);
         for (int l = 0; l < mg::LMAX; ++l) {
             me.dbase[l] = head.dtotal[l];

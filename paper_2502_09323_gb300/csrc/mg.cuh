@@ -19,14 +19,18 @@
 //          s_coarse = D_c^-1 P^T r
 //   up:    v = w s + P z_coarse ; z = (1 - w) v + w (s + D^-1 sum_f W_f v_f)
 // Level 0 uses the compressed operator (code bytes and listed weights), the
-// coarse levels a float4 (W+x, W+y, W+z, diagonal) per node.  The levels
+// coarse levels stored weights and diagonals.  The levels
 // whose data fits one block's shared memory are solved by one block per
 // system in one launch (k_mg_bottom).  The up kernel of level 0 also sums
 // rho = r.z and takes the CG step beta = rho / rho_old.
 //
-// Measured (GB300, solves to 1e-12): 257^3 155.6 -> 20.5 ms (1,127 -> 30
-// iterations), 65^3 30.6 -> 3.8 ms, a batch of 24 systems of 97^3 to 161^3
-// 229 -> 71 ms.
+// Measured (GB300, solves to 1e-12): 257^3 155.6 -> 16.4 ms (1,127 -> 30
+// iterations), 65^3 30.1 -> 2.1 ms, a batch of 24 systems of 97^3 to 161^3
+// 229 -> 55 ms.  A first form of the kernels, a node a thread with all
+// neighbours in shared memory, took 176 us (down) and 152 us (up) on 257^3
+// and 22 us in the bottom kernel; units of four nodes with the planes in
+// registers take 102 and 139 us, most of it instruction issue and load
+// latency (16 % of DRAM bandwidth, 38 % of the warps resident).
 //
 // Bounds: down reads s and a code byte per fine node and writes an eighth of
 // a value; up reads s, an eighth of a value and a code byte and writes z.
@@ -36,17 +40,23 @@ namespace mg {
 
 constexpr int LMAX = 12;            // levels at most
 constexpr float OMEGA = 0.85f;      // Jacobi damping (0.8 to 0.9 take the same iterations)
-constexpr int NT = 256;
 constexpr int BOT_T = 1024;         // threads of the bottom kernel
-constexpr int BOT_NODES = 7300;     // nodes of all its levels (28 B each in shared memory)
+constexpr int BOT_BYTES = 34;       // shared memory of one of its nodes
+constexpr int BOT_NODES = 6600;     // nodes of all its levels
 constexpr int SWEEPS = 8;           // Jacobi sweeps on the coarsest level
-constexpr int FX = 64, FY = 16;     // fine nodes of a block's tile
-constexpr int CX = FX / 2, CY = FY / 2;
+// Tiles.  Down: 32 x 6 coarse nodes from node (1 + 32 bx, 1 + 6 by), whose
+// residuals are 13 rows of 17 units of 4 fine nodes; the first and the last
+// unit of a row need no neighbour outside it.  221 threads take a unit each,
+// 34 more the halo rows.  Up: 64 x 16 fine nodes from (64 bx, 1 + 16 by), 16
+// units a row, and a halo row on either side: 288 threads.
+constexpr int CX = 32, CY = 6, DU = 17, DR = 2 * CY + 1, DNT = 256;
+constexpr int FX = 64, FY = 16, UU = 16, UNT = 16 * (FY + 2);
+constexpr int RG = 4;               // planes of one partial of rho
 
 struct Lev {
-    int nx, ny, nz, sx, sxy;
+    int nx, ny, nz, sx, sxy;        // sx a multiple of 4 above the bottom kernel's levels, nx there
     float *s, *z;                   // D^-1 b, solution (level 0: the solver's z32 and v32)
-    float4 *cf;                     // W+x, W+y, W+z, diagonal (levels >= 1)
+    float *wx, *wy, *wz, *dg;       // weights of the +x, +y, +z edges, diagonal (levels >= 1)
 };
 
 // One system (device memory, or the kernel parameter of a one-system launch)
@@ -58,8 +68,11 @@ struct Entry {
     CgState *st;
     const uint8_t *code;
     CoefC32 cp;
-    float *partials;                // rho of each work item of the level-0 up kernel
+    float dg_in, dg_out;            // diagonals of the two pure media
+    float *partials;                // rho of every RG planes of each tile of level 0
     int nu0;                        // their number
+    void *blob;                     // of the bottom kernel (k_mg_pack)
+    int bot;                        // its nodes, rounded up to a multiple of 8
 };
 
 // launch totals of a table, read on the device
@@ -72,41 +85,94 @@ struct Head {
 __host__ __device__ inline int ditems(const Entry &e, int l) {
     if (l >= e.nbot) return 0;
     const Lev &c = e.lev[l + 1];
-    return ((c.nx - 1 + CX - 1) / CX) * ((c.ny - 1 + CY - 1) / CY) * ((c.nz - 2 + e.dk[l] - 1) / e.dk[l]);
+    return ((c.nx - 2 + CX - 1) / CX) * ((c.ny - 2 + CY - 1) / CY) * ((c.nz - 2 + e.dk[l] - 1) / e.dk[l]);
 }
 __host__ __device__ inline int uitems(const Entry &e, int l) {
     if (l >= e.nbot) return 0;
     const Lev &f = e.lev[l];
-    return ((f.nx - 1 + FX - 1) / FX) * ((f.ny - 1 + FY - 1) / FY) * ((f.nz - 2 + e.uk[l] - 1) / e.uk[l]);
+    return ((f.nx - 1 + FX - 1) / FX) * ((f.ny - 2 + FY - 1) / FY) * ((f.nz - 2 + e.uk[l] - 1) / e.uk[l]);
 }
 
-// sum over the six faces of W x_neighbour, and the diagonal
+__device__ __forceinline__ float4 f4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
+// Operator data of a unit (4 nodes of a row) in one plane.  Level 0: its code
+// bytes and those of the row below.  Coarse levels: the weights and the
+// diagonal.
 template <bool FINE>
-__device__ __forceinline__ float face_sum(const Entry &e, const Lev &L, int p, float xm, float xp, float ym,
-                                          float yp, float zm, float zp, float &d) {
-    if constexpr (FINE) {
-        const uint32_t c = e.code[p];
-        const uint32_t cx = e.code[p - 1], cy = e.code[p - L.sx], cz = e.code[p - L.sxy];
-        const float w = (c & 1) ? e.cp.w_in : e.cp.w_out;
-        const float kap = (c & 1) ? 0.f : e.cp.kap;
-        if (((c & 0xEu) | (cx & 2u) | (cy & 4u) | (cz & 8u)) == 0u) {
-            d = 6.f * w + kap;
-            return w * (((xm + xp) + (ym + yp)) + (zm + zp));
-        }
-        const float w0 = (cx & 2u) ? __ldg(e.cp.wx + p - 1) : w;
-        const float w1 = (c & 2u) ? __ldg(e.cp.wx + p) : w;
-        const float w2 = (cy & 4u) ? __ldg(e.cp.wy + p - L.sx) : w;
-        const float w3 = (c & 4u) ? __ldg(e.cp.wy + p) : w;
-        const float w4 = (cz & 8u) ? __ldg(e.cp.wz + p - L.sxy) : w;
-        const float w5 = (c & 8u) ? __ldg(e.cp.wz + p) : w;
-        d = (((((w0 + w1) + w2) + w3) + w4) + w5) + kap;
-        return ((w0 * xm + w1 * xp) + (w2 * ym + w3 * yp)) + (w4 * zm + w5 * zp);
-    } else {
-        const float4 q = __ldg(L.cf + p);
-        const float w0 = __ldg(&L.cf[p - 1].x), w2 = __ldg(&L.cf[p - L.sx].y), w4 = __ldg(&L.cf[p - L.sxy].z);
-        d = q.w;
-        return ((w0 * xm + q.x * xp) + (w2 * ym + q.y * yp)) + (w4 * zm + q.z * zp);
+struct Op;
+template <>
+struct Op<true> {
+    uint32_t c = 0, cy = 0, cl = 0;  // own, row j - 1, node i - 1
+    __device__ __forceinline__ void load(const Entry &e, const Lev &L, int p) {
+        c = *reinterpret_cast<const uint32_t *>(e.code + p);
+        cy = *reinterpret_cast<const uint32_t *>(e.code + p - L.sx);
+        cl = e.code[p - 1];
     }
+};
+template <>
+struct Op<false> {
+    float4 x = {}, y = {}, z = {}, ym = {}, d = {1.f, 1.f, 1.f, 1.f};
+    float xl = 0.f;
+    __device__ __forceinline__ void load(const Entry &, const Lev &L, int p) {
+        x = f4(L.wx + p);
+        y = f4(L.wy + p);
+        z = f4(L.wz + p);
+        ym = f4(L.wy + p - L.sx);
+        d = f4(L.dg + p);
+        xl = L.wx[p - 1];
+    }
+};
+
+// sum over the six faces of W times the neighbour, and the diagonal, of the
+// nodes of a unit; o: plane k, b: plane k - 1; l, r: neighbours in x
+__device__ __forceinline__ void face_sums(const Entry &e, const Lev &L, int p, const Op<true> &o, const Op<true> &b,
+                                          const float4 &x, float l, float r, const float4 &ym, const float4 &yp,
+                                          const float4 &zm, const float4 &zp, float (&sum)[4], float (&d)[4]) {
+    const float xx[6] = {l, x.x, x.y, x.z, x.w, r};
+    const float m[4] = {ym.x + yp.x, ym.y + yp.y, ym.z + yp.z, ym.w + yp.w};
+    const float n[4] = {zm.x + zp.x, zm.y + zp.y, zm.z + zp.z, zm.w + zp.w};
+    const uint32_t cx = (o.c << 8) | o.cl;
+    const uint32_t special = (o.c & 0x0E0E0E0Eu) | (cx & 0x02020202u) | (o.cy & 0x04040404u) | (b.c & 0x08080808u);
+    if (special == 0u) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool in = (o.c >> (8 * q)) & 1u;
+            const float w = in ? e.cp.w_in : e.cp.w_out;
+            d[q] = in ? e.dg_in : e.dg_out;
+            sum[q] = w * ((xx[q] + xx[q + 2]) + m[q] + n[q]);
+        }
+        return;
+    }
+    const float my[4] = {ym.x, ym.y, ym.z, ym.w}, py[4] = {yp.x, yp.y, yp.z, yp.w};
+    const float mz[4] = {zm.x, zm.y, zm.z, zm.w}, pz[4] = {zp.x, zp.y, zp.z, zp.w};
+    float wl = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t c = o.c >> (8 * q);
+        const float w = (c & 1u) ? e.cp.w_in : e.cp.w_out;
+        if (q == 0) wl = (o.cl & 2u) ? __ldg(e.cp.wx + p - 1) : w;
+        else wl = ((o.c >> (8 * q - 8)) & 2u) ? wl : w;
+        const float w1 = (c & 2u) ? __ldg(e.cp.wx + p + q) : w;
+        const float w2 = ((o.cy >> (8 * q)) & 4u) ? __ldg(e.cp.wy + p + q - L.sx) : w;
+        const float w3 = (c & 4u) ? __ldg(e.cp.wy + p + q) : w;
+        const float w4 = ((b.c >> (8 * q)) & 8u) ? __ldg(e.cp.wz + p + q - L.sxy) : w;
+        const float w5 = (c & 8u) ? __ldg(e.cp.wz + p + q) : w;
+        d[q] = (((((wl + w1) + w2) + w3) + w4) + w5) + ((c & 1u) ? 0.f : e.cp.kap);
+        sum[q] = ((wl * xx[q] + w1 * xx[q + 2]) + (w2 * my[q] + w3 * py[q])) + (w4 * mz[q] + w5 * pz[q]);
+        wl = w1;
+    }
+}
+__device__ __forceinline__ void face_sums(const Entry &, const Lev &, int, const Op<false> &o, const Op<false> &b,
+                                          const float4 &x, float l, float r, const float4 &ym, const float4 &yp,
+                                          const float4 &zm, const float4 &zp, float (&sum)[4], float (&d)[4]) {
+    sum[0] = ((o.xl * l + o.x.x * x.y) + (o.ym.x * ym.x + o.y.x * yp.x)) + (b.z.x * zm.x + o.z.x * zp.x);
+    sum[1] = ((o.x.x * x.x + o.x.y * x.z) + (o.ym.y * ym.y + o.y.y * yp.y)) + (b.z.y * zm.y + o.z.y * zp.y);
+    sum[2] = ((o.x.y * x.y + o.x.z * x.w) + (o.ym.z * ym.z + o.y.z * yp.z)) + (b.z.z * zm.z + o.z.z * zp.z);
+    sum[3] = ((o.x.z * x.z + o.x.w * r) + (o.ym.w * ym.w + o.y.w * yp.w)) + (b.z.w * zm.w + o.z.w * zp.w);
+    d[0] = o.d.x;
+    d[1] = o.d.y;
+    d[2] = o.d.z;
+    d[3] = o.d.w;
 }
 
 __device__ __forceinline__ bool interior(const Lev &L, int i, int j, int k) {
@@ -126,20 +192,23 @@ __device__ __forceinline__ int find_sys(const Entry *tab, int nsys, int it, int 
 
 }  // namespace mg
 
-// Residual after the pre-smoothing step and its restriction.  A block takes
-// CX x CY coarse nodes and marches over its coarse planes; the fine s of four
-// planes and the residual of two are in shared memory, so that one barrier
-// a fine plane suffices; a plane's loads are issued one plane ahead.
+// Residual after the pre-smoothing step and its restriction.  A block marches
+// over the coarse planes of its tile: a thread keeps its unit's s of three
+// planes in registers, rows are exchanged through shared memory (three planes
+// of s, two of the residual, so that one barrier a fine plane suffices), and a
+// plane's loads are issued one plane ahead.
 template <bool FINE, bool SINGLE>
-__global__ void __launch_bounds__(mg::NT, 5)
+__global__ void __launch_bounds__(mg::DNT, FINE ? 4 : 3)
 k_mg_down(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head, int l, int total,
           const __grid_constant__ mg::Entry e0) {
     using namespace mg;
-    constexpr int SW = FX + 4, SH = FY + 4, RW = FX + 1, RH = FY + 1;
-    constexpr int NLD = (SW / 2 * SH + NT - 1) / NT;
-    __shared__ float sp[4][SH][SW];
-    __shared__ float rb[2][RH][RW + 1];
+    __shared__ __align__(16) float sp[3][DR + 2][4 * DU];
+    __shared__ __align__(16) float rb[2][DR][4 * DU];
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    // unit u of row r of the tile's fine rows - 1 .. DR (rows - 1 and DR: halo)
+    const bool halo = tid >= DR * DU;
+    const int h = tid - DR * DU;
+    const int u = halo ? h % DU : tid % DU, r = halo ? (h < DU ? -1 : DR) : tid / DU;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int nsys = SINGLE ? 1 : head->nsys;
@@ -149,101 +218,96 @@ k_mg_down(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head, 
         if (*(volatile int *)&e.st->done) continue;
         const Lev L = e.lev[l], C = e.lev[l + 1];
         const int li = SINGLE ? it : it - e.dbase[l];
-        const int xt = (C.nx - 1 + CX - 1) / CX, yt = (C.ny - 1 + CY - 1) / CY;
+        const int xt = (C.nx - 2 + CX - 1) / CX, yt = (C.ny - 2 + CY - 1) / CY;
         const int col = li % (xt * yt), ch = li / (xt * yt);
-        const int i0 = (col % xt) * FX, j0 = (col / xt) * FY;
+        const int I0 = 1 + (col % xt) * CX, J0 = 1 + (col / xt) * CY;
         const int K0 = 1 + ch * e.dk[l], K1 = min(K0 + e.dk[l], C.nz - 1);
         const int ka = 2 * K0 - 1, kb = 2 * K1 - 1;  // fine planes ka .. kb of the residual
-        float2 ld[NLD];
+        const int ib = 2 * I0 - 2 + 4 * u, j = 2 * J0 - 1 + r;
+        const bool there = h < 2 * DU && ib < L.sx && j >= 0 && j < L.ny;
+        const bool row = there && !halo && j <= L.ny - 2;  // j >= 1
+        const int pj = j * L.sx + ib;
         auto load = [&](int k) {
-#pragma unroll
-            for (int q = 0; q < NLD; ++q) {
-                const int t = tid + q * NT, r = t / (SW / 2), c = t - r * (SW / 2);
-                const int i = i0 - 2 + 2 * c, j = j0 - 2 + r;
-                ld[q] = make_float2(0.f, 0.f);
-                if (t < SW / 2 * SH && i >= 0 && i < L.sx && j >= 0 && j < L.ny && k >= 0 && k < L.nz)
-                    ld[q] = *reinterpret_cast<const float2 *>(L.s + (k * L.sxy + j * L.sx + i));
-            }
+            return there && k < L.nz ? f4(L.s + (k * L.sxy + pj)) : make_float4(0.f, 0.f, 0.f, 0.f);
         };
-        auto store = [&](int k) {
-#pragma unroll
-            for (int q = 0; q < NLD; ++q) {
-                const int t = tid + q * NT, r = t / (SW / 2), c = t - r * (SW / 2);
-                if (t < SW / 2 * SH) *reinterpret_cast<float2 *>(&sp[k & 3][r][2 * c]) = ld[q];
-            }
-        };
+        float4 sm, sc, sn, s2;
+        Op<FINE> ob, oc, on;
+        sm = halo ? make_float4(0.f, 0.f, 0.f, 0.f) : load(ka - 1);
+        sc = load(ka);
+        sn = load(ka + 1);
+        if (row) {
+            ob.load(e, L, (ka - 1) * L.sxy + pj);
+            oc.load(e, L, ka * L.sxy + pj);
+        }
         __syncthreads();  // the previous item's last reads
-        load(ka - 1);
-        store(ka - 1);
-        load(ka);
-        store(ka);
-        load(ka + 1);
+        if (h < 2 * DU) *reinterpret_cast<float4 *>(&sp[ka % 3][r + 1][4 * u]) = sc;
         float acc = 0.f;
         for (int k = ka; k <= kb + 1; ++k) {
-            if (k <= kb) store(k + 1);
+            if (k < kb && h < 2 * DU) *reinterpret_cast<float4 *>(&sp[(k + 1) % 3][r + 1][4 * u]) = sn;
             __syncthreads();
-            if (k < kb) load(k + 2);
-            if (k <= kb) {
-                const float (*sm)[SW] = sp[(k - 1) & 3], (*sc)[SW] = sp[k & 3], (*sn)[SW] = sp[(k + 1) & 3];
-                const int pk = k * L.sxy;
-#pragma unroll
-                for (int q = 0; q < (RW * RH + NT - 1) / NT; ++q) {
-                    const int t = tid + q * NT, r = t / RW, c = t - r * RW;
-                    if (t < RW * RH) {
-                        const int i = i0 - 1 + c, j = j0 - 1 + r;
-                        float v = 0.f;
-                        if (interior(L, i, j, k)) {
-                            float d;
-                            const float s0 = sc[r + 1][c + 1];
-                            const float sum = face_sum<FINE>(e, L, pk + j * L.sx + i, sc[r + 1][c], sc[r + 1][c + 2],
-                                                             sc[r][c + 1], sc[r + 2][c + 1], sm[r + 1][c + 1],
-                                                             sn[r + 1][c + 1], d);
-                            v = (1.f - OMEGA) * d * s0 + OMEGA * sum;
-                        }
-                        rb[k & 1][r][c] = v;
-                    }
-                }
+            if (k < kb) {
+                s2 = load(k + 2);
+                if (row) on.load(e, L, (k + 1) * L.sxy + pj);
             }
-            if (k > ka) {  // restrict plane k - 1
-                const float (*b)[RW + 1] = rb[(k - 1) & 1];
+            if (k <= kb && !halo) {
+                float v[4] = {0.f, 0.f, 0.f, 0.f};
+                if (row && k <= L.nz - 2) {
+                    const float (*s)[4 * DU] = sp[k % 3];
+                    const float xl = u > 0 ? s[r + 1][4 * u - 1] : 0.f, xr = u < DU - 1 ? s[r + 1][4 * u + 4] : 0.f;
+                    float sum[4], d[4];
+                    face_sums(e, L, k * L.sxy + pj, oc, ob, sc, xl, xr, f4(&s[r][4 * u]), f4(&s[r + 2][4 * u]), sm, sn,
+                              sum, d);
+                    const float s4[4] = {sc.x, sc.y, sc.z, sc.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (ib + q >= 1 && ib + q <= L.nx - 2) v[q] = (1.f - OMEGA) * d[q] * s4[q] + OMEGA * sum[q];
+                }
+                *reinterpret_cast<float4 *>(&rb[k & 1][r][4 * u]) = make_float4(v[0], v[1], v[2], v[3]);
+            }
+            if (k > ka && ty < CY) {  // restrict plane k - 1
                 float t = 0.f;
 #pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    const float *row = &b[2 * ty + r][2 * tx];
-                    const float x = row[1] + 0.5f * (row[0] + row[2]);
-                    t += r == 1 ? x : 0.5f * x;
+                for (int b = 0; b < 3; ++b) {
+                    const float *x = &rb[(k - 1) & 1][2 * ty + b][2 * tx + 1];
+                    const float v = x[1] + 0.5f * (x[0] + x[2]);
+                    t += b == 1 ? v : 0.5f * v;
                 }
                 if ((k - 1) & 1) {
                     acc += 0.5f * t;
-                    const int K = (k - 2) >> 1, I = i0 / 2 + tx, J = j0 / 2 + ty;
-                    if (k - 1 > ka && interior(C, I, J, K)) {
+                    const int K = (k - 2) >> 1, I = I0 + tx, J = J0 + ty;
+                    if (k - 1 > ka && I <= C.nx - 2 && J <= C.ny - 2) {
                         const int pc = K * C.sxy + J * C.sx + I;
-                        C.s[pc] = __fdividef(acc, __ldg(&C.cf[pc].w));
+                        C.s[pc] = __fdividef(acc, __ldg(C.dg + pc));
                     }
                     acc = 0.5f * t;
                 } else {
                     acc += t;
                 }
             }
+            sm = sc;
+            sc = sn;
+            sn = s2;
+            ob = oc;
+            oc = on;
         }
     }
 }
 
 // Interpolated correction, post-smoothing step and (level 0) rho = r.z.  A
-// block takes FX x FY fine nodes and marches over its fine planes; v, s and
-// the coarse correction of four planes each are in shared memory.
+// block marches over the fine planes of its tile: a thread keeps its unit's v
+// of three planes and the coarse correction, interpolated in y, of two coarse
+// planes in registers; rows of v are exchanged through three planes of shared
+// memory (one barrier a plane).
 template <bool FINE, bool SINGLE>
-__global__ void __launch_bounds__(mg::NT, 4)
+__global__ void __launch_bounds__(mg::UNT, FINE ? 3 : 2)
 k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, int total,
         const __grid_constant__ mg::Entry e0) {
     using namespace mg;
-    constexpr int VW = FX + 2, VH = FY + 2, EW = CX + 2, EH = CY + 2;
-    constexpr int NV = (VW * VH + NT - 1) / NT, NE = (EW * EH + NT - 1) / NT;
-    __shared__ float vp[4][VH][VW];
-    __shared__ float ss[4][VH][VW];
-    __shared__ float ec[4][EH][EW];
-    __shared__ float sred[NT / 32];
+    constexpr int NT = UNT, VW = FX + 8;  // a row: col - 1 at [3], cols 0 .. 63 from [4], col 64 at [68]
+    __shared__ __align__(16) float vp[3][FY + 2][VW];
+    __shared__ float sred[2][NT / 32];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int u = tid & 15, r = tid >> 4;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int nsys = SINGLE ? 1 : head->nsys;
@@ -253,107 +317,132 @@ k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, i
         if (*(volatile int *)&e.st->done) continue;
         const Lev L = e.lev[l], C = e.lev[l + 1];
         const int li = SINGLE ? it : it - e.ubase[l];
-        const int xt = (L.nx - 1 + FX - 1) / FX, yt = (L.ny - 1 + FY - 1) / FY;
+        const int xt = (L.nx - 1 + FX - 1) / FX, yt = (L.ny - 2 + FY - 1) / FY;
         const int col = li % (xt * yt), ch = li / (xt * yt);
-        const int i0 = (col % xt) * FX, j0 = (col / xt) * FY;
+        const int i0 = (col % xt) * FX, ib = i0 + 4 * u, j = (col / xt) * FY + r;
         const int k0 = 1 + ch * e.uk[l], k1 = min(k0 + e.uk[l], L.nz - 1);
-        float lds[NV], lde[NE];
+        const bool row = ib <= L.nx - 2 && j >= 1 && j <= L.ny - 2;
+        const bool own = row && r >= 1 && r <= FY;
+        const int pj = j * L.sx + ib;
+        const bool left = u == 0 && i0 > 0 && row, right = u == UU - 1 && ib + 4 <= L.nx - 2 && row;
+        // s of a unit, and of the columns beside the tile
+        struct S {
+            float4 s;
+            float x;
+        };
         auto load_s = [&](int k) {
-#pragma unroll
-            for (int q = 0; q < NV; ++q) {
-                const int t = tid + q * NT, r = t / VW, c = t - r * VW;
-                const int i = i0 - 1 + c, j = j0 - 1 + r;
-                lds[q] = 0.f;
-                if (t < VW * VH && interior(L, i, j, k)) lds[q] = L.s[k * L.sxy + j * L.sx + i];
+            S t = {make_float4(0.f, 0.f, 0.f, 0.f), 0.f};
+            if (row && k >= 1 && k <= L.nz - 2) {
+                const float *p = L.s + (k * L.sxy + pj);
+                t.s = f4(p);
+                if (left) t.x = p[-1];
+                if (right) t.x = p[4];
             }
+            return t;
         };
+        // coarse correction at columns ib/2 .. ib/2 + 2 (and ib/2 - 1 beside
+        // the tile), interpolated to row j, of coarse plane K
+        struct E {
+            float x, y, z, l;
+        };
+        const int I = ib >> 1, pa = (j >> 1) * C.sx + I, pb = ((j + 1) >> 1) * C.sx + I;
+        const bool third = I + 2 < C.sx;
         auto load_e = [&](int K) {
-#pragma unroll
-            for (int q = 0; q < NE; ++q) {
-                const int t = tid + q * NT, r = t / EW, c = t - r * EW;
-                const int I = i0 / 2 - 1 + c, J = j0 / 2 - 1 + r;
-                lde[q] = 0.f;
-                if (t < EW * EH && interior(C, I, J, K)) lde[q] = C.z[K * C.sxy + J * C.sx + I];
+            E t = {0.f, 0.f, 0.f, 0.f};
+            if (row && K < C.nz) {
+                const float *a = C.z + (K * C.sxy + pa), *b = C.z + (K * C.sxy + pb);
+                t.x = 0.5f * (a[0] + b[0]);
+                t.y = 0.5f * (a[1] + b[1]);
+                if (third) t.z = 0.5f * (a[2] + b[2]);
+                if (left) t.l = 0.5f * (a[-1] + b[-1]);
             }
+            return t;
         };
-        auto store_e = [&](int K) {
-#pragma unroll
-            for (int q = 0; q < NE; ++q) {
-                const int t = tid + q * NT, r = t / EW, c = t - r * EW;
-                if (t < EW * EH) ec[K & 3][r][c] = lde[q];
+        // v = w s + P e of plane k, from the coarse planes k/2 and (k+1)/2;
+        // zero off the interior
+        auto make_v = [&](int k, const S &s, const E &a, const E &b) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row && k >= 1 && k <= L.nz - 2) {
+                const float x = 0.5f * (a.x + b.x), y = 0.5f * (a.y + b.y), z = 0.5f * (a.z + b.z);
+                if (ib >= 1) v.x = OMEGA * s.s.x + x;
+                if (ib + 1 <= L.nx - 2) v.y = OMEGA * s.s.y + 0.5f * (x + y);
+                if (ib + 2 <= L.nx - 2) v.z = OMEGA * s.s.z + y;
+                if (ib + 3 <= L.nx - 2) v.w = OMEGA * s.s.w + 0.5f * (y + z);
+                float *out = vp[k % 3][r];
+                if (left) out[3] = OMEGA * s.x + 0.5f * (0.5f * (a.l + b.l) + x);
+                if (right) out[4 + FX] = OMEGA * s.x + z;
             }
+            *reinterpret_cast<float4 *>(&vp[k % 3][r][4 + 4 * u]) = v;
+            return v;
         };
-        // v = w s + P e of plane k
-        auto make_v = [&](int k) {
-            const float (*ea)[EW] = ec[(k >> 1) & 3], (*eb)[EW] = ec[((k + 1) >> 1) & 3];
-#pragma unroll
-            for (int q = 0; q < NV; ++q) {
-                const int t = tid + q * NT, r = t / VW, c = t - r * VW;
-                if (t < VW * VH) {
-                    const int i = i0 - 1 + c, j = j0 - 1 + r;
-                    float v = 0.f;
-                    if (interior(L, i, j, k)) {
-                        // coarse columns and rows either side (the same one on a coarse line)
-                        const int a = (c + 1) >> 1, b = (c + 2) >> 1, m = (r + 1) >> 1, n = (r + 2) >> 1;
-                        const float x = (ea[m][a] + ea[m][b]) + (ea[n][a] + ea[n][b]);
-                        const float y = (eb[m][a] + eb[m][b]) + (eb[n][a] + eb[n][b]);
-                        v = OMEGA * lds[q] + 0.125f * (x + y);
-                    }
-                    vp[k & 3][r][c] = v;
-                    ss[k & 3][r][c] = lds[q];
-                }
-            }
-        };
-        __syncthreads();  // the previous item's last reads
-        for (int K = (k0 - 1) >> 1; K <= (k0 + 2) >> 1; ++K) {
-            load_e(K);
-            store_e(K);
+        S sa = load_s(k0 - 1), sc = load_s(k0), sn = load_s(k0 + 1);
+        E ea = load_e((k0 - 1) >> 1), eb = load_e(k0 >> 1), ec = load_e((k0 + 1) >> 1), en = load_e((k0 + 2) >> 1);
+        Op<FINE> ob, oc, on;
+        if (own) {
+            ob.load(e, L, (k0 - 1) * L.sxy + pj);
+            oc.load(e, L, k0 * L.sxy + pj);
         }
-        __syncthreads();
-        load_s(k0 - 1);
-        make_v(k0 - 1);
-        load_s(k0);
-        make_v(k0);
-        load_s(k0 + 1);
-        // coarse planes up to (k0 + 2) / 2 are here: those of v(k0 + 1)
+        __syncthreads();  // the previous item's last reads
+        if (u == 0 && !left)
+            for (int q = 0; q < 3; ++q) vp[q][r][3] = 0.f;
+        if (u == UU - 1 && !right)
+            for (int q = 0; q < 3; ++q) vp[q][r][4 + FX] = 0.f;
+        float4 vm = make_v(k0 - 1, sa, ea, eb);
+        float4 vc = make_v(k0, sc, eb, ec);
+        // coarse planes of v(k + 1): (k + 1) / 2 and (k + 2) / 2
+        ea = ec;
+        eb = en;
+        // rho: every RG planes of a tile have a partial of their own, so that
+        // the sum does not depend on the planes per work item (uk[0] is a
+        // multiple of RG).  The one that ends with plane k is written here,
+        // a barrier after the warps' sums.
+        auto flush = [&](int k) {
+            float t = 0.f;
+            for (int q = 0; q < NT / 32; ++q) t += sred[((k - 1) / RG) & 1][q];
+            e.partials[((k - 1) / RG) * xt * yt + col] = t;
+        };
         float rho = 0.f;
         for (int k = k0; k < k1; ++k) {
-            float s0[4];
-            make_v(k + 1);
-            // the coarse plane that v(k + 2) needs anew
-            const int Kn = (k + 3) >> 1;
-            const bool fresh = (k + 2) & 1;
-            if (fresh) load_e(Kn);
-            load_s(k + 2);
-            if (fresh) store_e(Kn);
+            const float4 vn = make_v(k + 1, sn, ea, eb);
             __syncthreads();
-            const float (*vm)[VW] = vp[(k - 1) & 3], (*vc)[VW] = vp[k & 3], (*vn)[VW] = vp[(k + 1) & 3];
-            const int pk = k * L.sxy;
+            if (FINE && tid == 0 && k > k0 && (k - 1) % RG == 0) flush(k - 1);
+            // issue the next plane's loads
+            S s2 = load_s(k + 2);
+            ec = eb;
+            if (!((k + 1) & 1)) ec = load_e((k + 3) >> 1);
+            if (own) {
+                if (k + 1 < k1) on.load(e, L, (k + 1) * L.sxy + pj);
+                const float (*v)[VW] = vp[k % 3];
+                float sum[4], d[4];
+                face_sums(e, L, k * L.sxy + pj, oc, ob, vc, v[r][3 + 4 * u], v[r][8 + 4 * u], f4(&v[r - 1][4 + 4 * u]),
+                          f4(&v[r + 1][4 + 4 * u]), vm, vn, sum, d);
+                const float v4[4] = {vc.x, vc.y, vc.z, vc.w}, s4[4] = {sc.s.x, sc.s.y, sc.s.z, sc.s.w};
+                float z[4];
 #pragma unroll
-            for (int q = 0; q < FX * FY / NT; ++q) {
-                const int t = tid + q * NT, r = 1 + t / FX, c = 1 + t % FX;
-                const int i = i0 - 1 + c, j = j0 - 1 + r;
-                s0[q] = ss[k & 3][r][c];
-                if (interior(L, i, j, k)) {
-                    const int p = pk + j * L.sx + i;
-                    float d;
-                    const float sum = face_sum<FINE>(e, L, p, vc[r][c - 1], vc[r][c + 1], vc[r - 1][c], vc[r + 1][c],
-                                                     vm[r][c], vn[r][c], d);
-                    const float z = (1.f - OMEGA) * vc[r][c] + OMEGA * (s0[q] + __fdividef(sum, d));
-                    L.z[p] = z;
-                    if (FINE) rho += d * s0[q] * z;
+                for (int q = 0; q < 4; ++q) {
+                    z[q] = (1.f - OMEGA) * v4[q] + OMEGA * (s4[q] + __fdividef(sum[q], d[q]));
+                    if (ib + q < 1 || ib + q > L.nx - 2) z[q] = 0.f;
+                    if (FINE) rho += d[q] * s4[q] * z[q];
                 }
+                *reinterpret_cast<float4 *>(L.z + (k * L.sxy + pj)) = make_float4(z[0], z[1], z[2], z[3]);
             }
+            if (FINE && (k % RG == 0 || k == k1 - 1)) {
+                rho = tma::warp_sum_f(rho);
+                if (lane == 0) sred[((k - 1) / RG) & 1][w] = rho;
+                rho = 0.f;
+            }
+            vm = vc;
+            vc = vn;
+            sc = sn;
+            sn = s2;
+            ea = ((k + 1) & 1) ? eb : ea;
+            eb = ec;
+            ob = oc;
+            oc = on;
         }
         if (FINE) {
-            rho = tma::warp_sum_f(rho);
-            if (lane == 0) sred[w] = rho;
             __syncthreads();
-            if (tid == 0) {
-                float t = 0.f;
-                for (int q = 0; q < NT / 32; ++q) t += sred[q];
-                e.partials[li] = t;
-            }
+            if (tid == 0) flush(k1 - 1);
         }
     }
     if (!FINE) return;
@@ -408,119 +497,163 @@ k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, i
     if (tid == 0) head->done = 0u;
 }
 
-// The levels nbot .. nlev - 1 of one system per block, in shared memory.
-// The same cycle as above; SWEEPS damped Jacobi steps on the last level.
+// What the bottom kernel keeps in shared memory besides its vectors, made with
+// the hierarchy: for every node of its levels, one after the other and
+// unpadded, the weights and the diagonal (arrays of T values); for every
+// interior node, its place in its level, its parent (the coarse node below it
+// and the three parities) and, on coarse levels, its fine node.
+__global__ void k_mg_pack(const __grid_constant__ mg::Entry e, int T) {
+    using namespace mg;
+    float *W = reinterpret_cast<float *>(e.blob);
+    uint16_t *list = reinterpret_cast<uint16_t *>(W + 4 * T), *up = list + T, *dn = up + T;
+    int off = 0;
+    for (int l = e.nbot; l < e.nlev; ++l) {
+        const Lev &L = e.lev[l];
+        const int n = L.nx * L.ny * L.nz, mx = L.nx - 2, my = L.ny - 2;
+        const int cx = L.nx / 2 + 1, cxy = cx * (L.ny / 2 + 1);
+        const int fx = l > e.nbot ? e.lev[l - 1].nx : 0, fxy = l > e.nbot ? fx * e.lev[l - 1].ny : 0;
+        for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+            W[off + p] = L.wx[p];
+            W[T + off + p] = L.wy[p];
+            W[2 * T + off + p] = L.wz[p];
+            W[3 * T + off + p] = L.dg[p];
+            const int i = p % L.nx, j = (p / L.nx) % L.ny, k = p / (L.nx * L.ny);
+            if (!interior(L, i, j, k)) continue;
+            const int t = off + ((k - 1) * my + j - 1) * mx + i - 1;
+            list[t] = (uint16_t)p;
+            up[t] = (uint16_t)((((k >> 1) * cxy + (j >> 1) * cx + (i >> 1)) << 3) | ((k & 1) << 2) | ((j & 1) << 1) |
+                               (i & 1));
+            dn[t] = (uint16_t)(2 * k * fxy + 2 * j * fx + 2 * i);
+        }
+        off += n;
+    }
+}
+
+// The levels nbot .. nlev - 1 of one system per block, in shared memory.  The
+// same cycle as above; SWEEPS damped Jacobi steps on the last level.  One SM
+// works here, and what it does serially counts: the coefficients and node lists come in
+// one asynchronous copy, before the previous kernel has ended (one-system
+// launches).
 template <bool SINGLE>
 __global__ void __launch_bounds__(mg::BOT_T, 1)
 k_mg_bottom(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head,
             const __grid_constant__ mg::Entry e0) {
     using namespace mg;
-    extern __shared__ __align__(16) float4 bsm[];
+    extern __shared__ __align__(16) float bsm[];
     const int tid = threadIdx.x;
-    if (!SINGLE) asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (!SINGLE && (int)blockIdx.x >= head->nsys) return;
-    const Entry &e = SINGLE ? e0 : tab[blockIdx.x];
-    const int lb = e.nbot, le = e.nlev;
-    if (le == 0) return;
-    // the coefficients do not depend on the previous kernel
-    int off = 0;
-    for (int l = lb; l < le; ++l) {
-        const Lev &L = e.lev[l];
-        const int n = L.sxy * L.nz;
-        for (int p = tid; p < n; p += BOT_T) bsm[off + p] = __ldg(L.cf + p);
-        off += n;
+    if (!SINGLE) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if ((int)blockIdx.x >= head->nsys) return;
     }
-    float *S = reinterpret_cast<float *>(bsm + off), *Z = S + off, *R = Z + off;
-    for (int p = tid; p < off; p += BOT_T) S[p] = Z[p] = R[p] = 0.f;
-    if (SINGLE) asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (*(volatile int *)&e.st->done) return;
+    const Entry &e = SINGLE ? e0 : tab[blockIdx.x];
+    const int lb = e.nbot, le = e.nlev, T = e.bot;
+    if (le == 0) return;
+    if (!SINGLE && *(volatile int *)&e.st->done) return;
+    const float *Wx = bsm, *Wy = Wx + T, *Wz = Wy + T, *D = Wz + T;
+    const uint16_t *list = reinterpret_cast<const uint16_t *>(D + T), *up = list + T, *dn = up + T;
+    float *S = bsm + 22 * T / 4, *Z = S + T, *R = Z + T;
+    // T is a multiple of 8, so the 22 T bytes are whole 16-byte pieces
+    for (int q = tid; q < 22 * T / 16; q += BOT_T)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tma::smem_u32(reinterpret_cast<char *>(bsm) + 16 * q)),
+                     "l"(reinterpret_cast<const char *>(e.blob) + 16 * q)
+                     : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int q = tid; q < 3 * T; q += BOT_T) S[q] = 0.f;
+    if (SINGLE) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+    const bool skip = SINGLE && *(volatile int *)&e.st->done;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (skip) return;
     __syncthreads();
     {
         const Lev &L = e.lev[lb];
-        const int n = L.sxy * L.nz;
+        const int n = L.nx * L.ny * L.nz;
+#pragma unroll 8
         for (int p = tid; p < n; p += BOT_T) S[p] = L.s[p];
     }
     __syncthreads();
-    // sum over the faces of node p of a level whose coefficients start at cf
-    auto faces = [&](const float4 *cf, const Lev &L, const float *x, int p) {
-        const float4 q = cf[p];
-        return ((cf[p - 1].x * x[p - 1] + q.x * x[p + 1]) + (cf[p - L.sx].y * x[p - L.sx] + q.y * x[p + L.sx])) +
-               (cf[p - L.sxy].z * x[p - L.sxy] + q.z * x[p + L.sxy]);
-    };
-    auto each = [&](const Lev &L, auto f) {  // interior nodes
-        const int mx = L.nx - 2, my = L.ny - 2, m = mx * my * (L.nz - 2);
-        for (int t = tid; t < m; t += BOT_T) {
-            const int r = t / mx, i = 1 + t - r * mx, k = 1 + r / my, j = 1 + r - (r / my) * my;
-            f(i, j, k, k * L.sxy + j * L.sx + i);
-        }
+    // sum over the faces of node p of the level whose nodes start at o
+    auto faces = [&](int o, int sx, int sxy, const float *x, int p) {
+        const float *a = Wx + o, *b = Wy + o, *c = Wz + o;
+        return ((a[p - 1] * x[p - 1] + a[p] * x[p + 1]) + (b[p - sx] * x[p - sx] + b[p] * x[p + sx])) +
+               (c[p - sxy] * x[p - sxy] + c[p] * x[p + sxy]);
     };
     int o = 0;
     for (int l = lb; l < le - 1; ++l) {
         const Lev &L = e.lev[l], &C = e.lev[l + 1];
-        const int oc = o + L.sxy * L.nz;
-        each(L, [&](int, int, int, int p) {
-            R[o + p] = (1.f - OMEGA) * bsm[o + p].w * S[o + p] + OMEGA * faces(bsm + o, L, S + o, p);
-        });
+        const int sx = L.nx, sxy = L.nx * L.ny, n = (L.nx - 2) * (L.ny - 2) * (L.nz - 2);
+        const int oc = o + sxy * L.nz, nc = (C.nx - 2) * (C.ny - 2) * (C.nz - 2);
+        for (int t = tid; t < n; t += BOT_T) {
+            const int p = list[o + t];
+            R[o + p] = (1.f - OMEGA) * D[o + p] * S[o + p] + OMEGA * faces(o, sx, sxy, S + o, p);
+        }
         __syncthreads();
-        each(C, [&](int I, int J, int K, int pc) {
+        for (int t = tid; t < nc; t += BOT_T) {
+            const int pc = list[oc + t];
+            const float *f = R + o + dn[oc + t];
             float acc = 0.f;
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
+            for (int c = -1; c <= 1; ++c)
 #pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    const float *x = R + o + (2 * K - 1 + c) * L.sxy + (2 * J - 1 + b) * L.sx + 2 * I;
-                    const float t = x[0] + 0.5f * (x[-1] + x[1]);
-                    acc += (b == 1 ? 1.f : 0.5f) * (c == 1 ? 1.f : 0.5f) * t;
+                for (int b = -1; b <= 1; ++b) {
+                    const float *x = f + c * sxy + b * sx;
+                    acc += (b ? 0.5f : 1.f) * (c ? 0.5f : 1.f) * (x[0] + 0.5f * (x[-1] + x[1]));
                 }
-            S[oc + pc] = __fdividef(acc, bsm[oc + pc].w);
-        });
+            S[oc + pc] = __fdividef(acc, D[oc + pc]);
+        }
         __syncthreads();
         o = oc;
     }
     {
         const Lev &L = e.lev[le - 1];
-        float *a = Z + o, *b = R + o;
-        each(L, [&](int, int, int, int p) { a[p] = OMEGA * S[o + p]; });
+        const int sx = L.nx, sxy = L.nx * L.ny, n = (L.nx - 2) * (L.ny - 2) * (L.nz - 2);
+        if (n == 1) {  // one unknown: its solution
+            if (tid == 0) Z[o + list[o]] = S[o + list[o]];
+        } else {
+            float *a = Z + o, *b = R + o;
+            for (int t = tid; t < n; t += BOT_T) a[list[o + t]] = OMEGA * S[o + list[o + t]];
+            __syncthreads();
+            for (int q = 1; q < SWEEPS; ++q) {
+                for (int t = tid; t < n; t += BOT_T) {
+                    const int p = list[o + t];
+                    b[p] = (1.f - OMEGA) * a[p] +
+                           OMEGA * (S[o + p] + __fdividef(faces(o, sx, sxy, a, p), D[o + p]));
+                }
+                __syncthreads();
+                float *t = a;
+                a = b;
+                b = t;
+            }
+            if (a != Z + o)
+                for (int t = tid; t < n; t += BOT_T) Z[o + list[o + t]] = a[list[o + t]];
+        }
         __syncthreads();
-        for (int q = 1; q < SWEEPS; ++q) {
-            each(L, [&](int, int, int, int p) {
-                b[p] = (1.f - OMEGA) * a[p] + OMEGA * (S[o + p] + __fdividef(faces(bsm + o, L, a, p), bsm[o + p].w));
-            });
-            __syncthreads();
-            float *t = a;
-            a = b;
-            b = t;
-        }
-        if (a != Z + o) {
-            each(L, [&](int, int, int, int p) { Z[o + p] = a[p]; });
-            __syncthreads();
-        }
     }
     for (int l = le - 2; l >= lb; --l) {
         const Lev &L = e.lev[l], &C = e.lev[l + 1];
-        const int oc = o;
-        o -= L.sxy * L.nz;
-        each(L, [&](int i, int j, int k, int p) {
-            float acc = 0.f;
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int b = 0; b < 2; ++b) {
-                    const float *x = Z + oc + ((k + c) >> 1) * C.sxy + ((j + b) >> 1) * C.sx;
-                    acc += x[i >> 1] + x[(i + 1) >> 1];
-                }
+        const int sx = L.nx, sxy = L.nx * L.ny, n = (L.nx - 2) * (L.ny - 2) * (L.nz - 2);
+        const int cx = C.nx, cxy = C.nx * C.ny, oc = o;
+        o -= sxy * L.nz;
+        for (int t = tid; t < n; t += BOT_T) {
+            const int p = list[o + t], c = up[o + t];
+            const float *x = Z + oc + (c >> 3);
+            const int di = c & 1, dj = (c & 2) ? cx : 0, dk = (c & 4) ? cxy : 0;
+            const float acc = ((x[0] + x[di]) + (x[dj] + x[dj + di])) + ((x[dk] + x[dk + di]) + (x[dk + dj] + x[dk + dj + di]));
             R[o + p] = OMEGA * S[o + p] + 0.125f * acc;
-        });
+        }
         __syncthreads();
-        each(L, [&](int, int, int, int p) {
-            Z[o + p] = (1.f - OMEGA) * R[o + p] +
-                       OMEGA * (S[o + p] + __fdividef(faces(bsm + o, L, R + o, p), bsm[o + p].w));
-        });
+        for (int t = tid; t < n; t += BOT_T) {
+            const int p = list[o + t];
+            const float z = (1.f - OMEGA) * R[o + p] +
+                            OMEGA * (S[o + p] + __fdividef(faces(o, sx, sxy, R + o, p), D[o + p]));
+            Z[o + p] = z;
+        }
         __syncthreads();
     }
     const Lev &L = e.lev[lb];
-    each(L, [&](int, int, int, int p) { L.z[p] = Z[p]; });
+    for (int p = tid; p < L.nx * L.ny * L.nz; p += BOT_T) L.z[p] = Z[p];
 }
 
 // Edge weights and ionic term (kept in z while the hierarchy is built) of a
@@ -538,8 +671,7 @@ __global__ void k_mg_coarsen(mg::Lev F, mg::Lev C, const double *__restrict__ Wx
             const double *W = d == 0 ? Wx : (d == 1 ? Wy : Wz);
             return (float)W[((long long)x[2] * F.ny + x[1]) * F.nx + x[0]];
         }
-        const float4 q = F.cf[x[2] * F.sxy + x[1] * F.sx + x[0]];
-        return d == 0 ? q.x : (d == 1 ? q.y : q.z);
+        return (d == 0 ? F.wx : (d == 1 ? F.wy : F.wz))[x[2] * F.sxy + x[1] * F.sx + x[0]];
     };
     float W[3];
     for (int d = 0; d < 3; ++d) {
@@ -574,7 +706,10 @@ __global__ void k_mg_coarsen(mg::Lev F, mg::Lev C, const double *__restrict__ Wx
         kap += (a ? 0.5f : 1.f) * (b ? 0.5f : 1.f) * (g ? 0.5f : 1.f) * k;
     }
     const int p = K * C.sxy + J * C.sx + I;
-    C.cf[p] = make_float4(W[0], W[1], W[2], 1.f);
+    C.wx[p] = W[0];
+    C.wy[p] = W[1];
+    C.wz[p] = W[2];
+    C.dg[p] = 1.f;
     C.z[p] = kap;
 }
 
@@ -584,8 +719,7 @@ __global__ void k_mg_diag(mg::Lev C) {
     const int I = t % C.nx, J = (t / C.nx) % C.ny, K = t / (C.nx * C.ny);
     if (!mg::interior(C, I, J, K)) return;
     const int p = K * C.sxy + J * C.sx + I;
-    const float4 q = C.cf[p];
-    C.cf[p].w = q.x + C.cf[p - 1].x + q.y + C.cf[p - C.sx].y + q.z + C.cf[p - C.sxy].z + C.z[p];
+    C.dg[p] = C.wx[p] + C.wx[p - 1] + C.wy[p] + C.wy[p - C.sx] + C.wz[p] + C.wz[p - C.sxy] + C.z[p];
 }
 
 // ------------------------------------------------------------------- host --
@@ -596,6 +730,33 @@ struct MgState {
     void *mem = nullptr;         // coarse levels
     float *partials = nullptr;
 };
+
+// Planes per work item.  A block marches over them after reading two more,
+// at about a microsecond a plane, and up to four (down) or three (up) blocks
+// share an SM: the count with the fewest rounds of blocks times planes.
+// shared: many systems fill the launch, and the longest items waste least.
+// Only the work is divided differently, the results are the same bits.
+void mg_planes(mg::Entry &e, bool shared) {
+    using namespace mg;
+    auto best = [&](long long cols, int n, int slots, int step, int most) {
+        int kc = most;
+        double cost = 1e30;
+        for (int c = step; c <= most && !shared; c += step) {
+            const double t = (double)cdiv(cols * cdiv(n, c), (long long)slots * num_sms()) * (c + 2.5);
+            if (t < cost) {
+                cost = t;
+                kc = c;
+            }
+        }
+        return kc;
+    };
+    for (int l = 0; l < e.nbot; ++l) {
+        const Lev &F = e.lev[l], &C = e.lev[l + 1];
+        // a coarse plane is two fine ones
+        e.dk[l] = best((long long)cdiv(C.nx - 2, CX) * cdiv(C.ny - 2, CY), 2 * (C.nz - 2), 4, 2, 16) / 2;
+        e.uk[l] = best((long long)cdiv(F.nx - 1, FX) * cdiv(F.ny - 2, FY), F.nz - 2, 3, l == 0 ? RG : 1, 16);
+    }
+}
 
 // The levels of a grid; false when the hierarchy does not reach the bottom
 // kernel's size (grids thinner than 9 nodes, or very long and thin ones):
@@ -621,23 +782,26 @@ bool mg_levels(const PadGeo &g, mg::Entry &e) {
     int b = e.nlev;
     while (b > 1) {
         const Lev &L = e.lev[b - 1];
-        if (nodes + (long long)L.sxy * L.nz > BOT_NODES) break;
-        nodes += (long long)L.sxy * L.nz;
+        const long long n = (long long)L.nx * L.ny * L.nz;
+        if (nodes + n > BOT_NODES) break;
+        nodes += n;
         --b;
     }
     if (b == e.nlev) return false;
     e.nbot = b;
-    // planes per work item: up to 8 coarse (16 fine) planes, fewer where that
-    // leaves less than about four items an SM
-    for (int l = 0; l < e.nbot; ++l) {
-        const Lev &F = e.lev[l], &C = e.lev[l + 1];
-        const long long cd = (long long)cdiv(C.nx - 1, CX) * cdiv(C.ny - 1, CY) * (C.nz - 2);
-        const long long cu = (long long)cdiv(F.nx - 1, FX) * cdiv(F.ny - 1, FY) * (F.nz - 2);
-        e.dk[l] = (int)std::max(1ll, std::min(8ll, cd / 608));
-        e.uk[l] = (int)std::max(1ll, std::min(16ll, cu / 608));
+    e.bot = (int)((nodes + 7) & ~7ll);
+    for (int l = b; l < e.nlev; ++l) {
+        e.lev[l].sx = e.lev[l].nx;
+        e.lev[l].sxy = e.lev[l].nx * e.lev[l].ny;
     }
+    const Lev &F = e.lev[0];
+    e.nu0 = cdiv(F.nx - 1, FX) * cdiv(F.ny - 2, FY) * cdiv(F.nz - 2, RG);
+    mg_planes(e, false);
     return true;
 }
+
+// floats of one array of a level (whole 16-byte pieces)
+size_t mg_lev_floats(const mg::Lev &L) { return ((size_t)L.sxy * L.nz + 3) & ~(size_t)3; }
 
 void free_mg_state(pb_system *sys) {
     MgState *m = (MgState *)sys->mg;
@@ -650,16 +814,12 @@ void free_mg_state(pb_system *sys) {
     sys->mg = nullptr;
 }
 
-size_t mg_bottom_bytes(const mg::Entry &e) {
-    size_t n = 0;
-    for (int l = e.nbot; l < e.nlev; ++l) n += (size_t)e.lev[l].sxy * e.lev[l].nz;
-    return 28 * n;
-}
+size_t mg_bottom_bytes(const mg::Entry &e) { return (size_t)mg::BOT_BYTES * e.bot; }
 
 pb_status mg_prepare() {
     static bool done = false;
     if (done) return PB_OK;
-    const int most = 28 * mg::BOT_NODES;
+    const int most = mg::BOT_BYTES * mg::BOT_NODES;
     PB_CUDA_TRY(cudaFuncSetAttribute(k_mg_bottom<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     PB_CUDA_TRY(cudaFuncSetAttribute(k_mg_bottom<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     done = true;
@@ -680,8 +840,9 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
     if (!m) return PB_ERR_OOM;
     sys->mg = m;
     size_t bytes = 0;
-    for (int l = 1; l < e.nlev; ++l) bytes += (size_t)e.lev[l].sxy * e.lev[l].nz * (sizeof(float4) + 8);
-    e.nu0 = uitems(e, 0);
+    for (int l = 1; l < e.nlev; ++l) bytes += mg_lev_floats(e.lev[l]) * 24;
+    const size_t blob = bytes;
+    bytes += 22 * (size_t)e.bot;
     m->head = (Head *)dalloc(sizeof(Head), s);
     m->v = (float *)dalloc(sizeof(float) * (size_t)sys->pad.Np, s);
     m->mem = dalloc(bytes, s);
@@ -698,15 +859,21 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
     char *at = (char *)m->mem;
     for (int l = 1; l < e.nlev; ++l) {
         Lev &L = e.lev[l];
-        const size_t n = (size_t)L.sxy * L.nz;
-        L.cf = (float4 *)at;
-        L.s = (float *)(at + n * sizeof(float4));
+        const size_t n = mg_lev_floats(L);
+        L.wx = (float *)at;  // n is a multiple of 4: every array is 16-byte aligned
+        L.wy = L.wx + n;
+        L.wz = L.wy + n;
+        L.dg = L.wz + n;
+        L.s = L.dg + n;
         L.z = L.s + n;
-        at += n * (sizeof(float4) + 8);
+        at += n * 24;
     }
+    e.blob = (char *)m->mem + blob;
     e.st = sys->st;
     e.code = sys->code;
     e.cp = make_c32(sys);
+    e.dg_in = 6.f * e.cp.w_in;
+    e.dg_out = 6.f * e.cp.w_out + e.cp.kap;
     e.partials = m->partials;
     for (int l = 1; l < e.nlev; ++l) {
         const Lev &F = e.lev[l - 1], &C = e.lev[l];
@@ -719,6 +886,8 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
         note_launch(1);
         PB_LAUNCH_CHECK();
     }
+    k_mg_pack<<<cdiv(e.bot, 256), 256, 0, s>>>(e, e.bot);
+    PB_LAUNCH_CHECK();
     for (int l = 1; l < e.nlev; ++l)  // z held the ionic terms
         PB_CUDA_TRY(cudaMemsetAsync(e.lev[l].z, 0, sizeof(float) * (size_t)e.lev[l].sxy * e.lev[l].nz, s));
     m->e = e;
@@ -726,9 +895,9 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
 }
 
 template <class K>
-unsigned mg_resident(K kernel) {
+unsigned mg_resident(K kernel, int nt) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, mg::NT, 0) != cudaSuccess || per_sm <= 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nt, 0) != cudaSuccess || per_sm <= 0) {
         cudaGetLastError();
         per_sm = 2;
     }
@@ -756,25 +925,25 @@ int launch_vcycle(const pb_system *sys, cudaStream_t s) {
     using namespace mg;
     const MgState *m = (const MgState *)sys->mg;
     const Entry &e = m->e;
-    static const unsigned rd0 = mg_resident(k_mg_down<true, true>), rd1 = mg_resident(k_mg_down<false, true>),
-                          ru0 = mg_resident(k_mg_up<true, true>), ru1 = mg_resident(k_mg_up<false, true>);
+    static const unsigned rd0 = mg_resident(k_mg_down<true, true>, DNT), rd1 = mg_resident(k_mg_down<false, true>, DNT),
+                          ru0 = mg_resident(k_mg_up<true, true>, UNT), ru1 = mg_resident(k_mg_up<false, true>, UNT);
     const Entry *none = nullptr;
     for (int l = 0; l < e.nbot; ++l) {
         const int n = ditems(e, l);
         if (l == 0)
-            mg_launch(k_mg_down<true, true>, std::min<unsigned>(n, rd0), NT, 0, s, true, none, (const Head *)m->head, l,
+            mg_launch(k_mg_down<true, true>, std::min<unsigned>(n, rd0), DNT, 0, s, true, none, (const Head *)m->head, l,
                       n, e);
         else
-            mg_launch(k_mg_down<false, true>, std::min<unsigned>(n, rd1), NT, 0, s, true, none, (const Head *)m->head,
+            mg_launch(k_mg_down<false, true>, std::min<unsigned>(n, rd1), DNT, 0, s, true, none, (const Head *)m->head,
                       l, n, e);
     }
     mg_launch(k_mg_bottom<true>, 1, BOT_T, mg_bottom_bytes(e), s, true, none, (const Head *)m->head, e);
     for (int l = e.nbot - 1; l >= 0; --l) {
         const int n = uitems(e, l);
         if (l == 0)
-            mg_launch(k_mg_up<true, true>, std::min<unsigned>(n, ru0), NT, 0, s, true, none, m->head, l, n, e);
+            mg_launch(k_mg_up<true, true>, std::min<unsigned>(n, ru0), UNT, 0, s, true, none, m->head, l, n, e);
         else
-            mg_launch(k_mg_up<false, true>, std::min<unsigned>(n, ru1), NT, 0, s, true, none, m->head, l, n, e);
+            mg_launch(k_mg_up<false, true>, std::min<unsigned>(n, ru1), UNT, 0, s, true, none, m->head, l, n, e);
     }
     return 2 * e.nbot + 1;
 }

@@ -814,6 +814,39 @@ int tma_items(const PadGeo &g, int KC, int tw) {
     return (int)(cdiv(g.nx - 1, tw) * cdiv(g.ny - 2, tma::tile_h(tw)) * cdiv(g.nz - 2, KC));
 }
 
+// A grid that cannot fill the GPU alone (fewer than four work items of 8
+// planes a resident block).
+bool tma_small(const PadGeo &g) {
+    const int n = std::min(tma_items(g, 8, 128), std::min(tma_items(g, 8, 64), tma_items(g, 8, 32)));
+    return n < 4 * (int)tma_grid(g, 8).x;
+}
+
+// Planes of one partial of the dot products: 4 on small grids, 8 on others,
+// or the whole z-chunk where it is no multiple of that.  The sums (and so the
+// solution's bits) depend on the group and the tile width, not on the z-chunk.
+int tma_group(const PadGeo &g, int KC) {
+    const int b = tma_small(g) ? 4 : 8;
+    return KC % b == 0 ? b : KC;
+}
+
+// z-chunk of a one-system launch of a system tuned to KC: on a small grid
+// shorter chunks with the same groups spread over more SMs, and fewer planes
+// follow one another (65^3: 36 -> 15 us a launch)
+int tma_alone_kc(const PadGeo &g, int KC, int tw) {
+    const int G = tma_group(g, KC);
+    if (!tma_small(g) || G != 4) return KC;
+    int best = KC;
+    double cost = 1e30;
+    for (int kc = 4; kc <= KC; kc += 4) {
+        const double t = (double)cdiv(tma_items(g, kc, tw), tma_grid(g, kc).x) * (kc + 2.5);
+        if (t < cost) {
+            cost = t;
+            best = kc;
+        }
+    }
+    return best;
+}
+
 // entry fields that depend on the z-chunk length and the tile width
 void tma_entry_geometry(tma::SysEntry &e, const PadGeo &g, int KC, int tw) {
     e.tw = tw;
@@ -823,6 +856,9 @@ void tma_entry_geometry(tma::SysEntry &e, const PadGeo &g, int KC, int tw) {
     e.nchunk = (int)cdiv(g.nz - 2, KC);
     e.nitems = e.xtiles * e.ytiles * e.nchunk;
     e.item_base = 0;
+    e.G = tma_group(g, KC);
+    e.nG = (int)cdiv(g.nz - 2, e.G);
+    e.npart = e.xtiles * e.ytiles * e.nG;
 }
 
 CoefC32 make_c32(const pb_system *sys);
@@ -1243,7 +1279,7 @@ pb_status autotune(pb_system *sys, int precision, cudaStream_t s, Tuning *out) {
     const int variant = precision == PB_MIXED ? 1 : 0;
     Tuning best;
     best.variant = variant;
-    const int kcs[] = {8, 6, 11, 16, 22, 32};  // first = default
+    const int kcs[] = {8, 16, 24, 32};  // first = default; multiples of a partial's planes
     // tile widths: those whose tiles cover the interior of a plane with the
     // fewest idle lanes (smallest padded area), widest first.  A small grid
     // timed alone cannot fill the GPU, so its timings would not show the idle
@@ -1269,7 +1305,7 @@ pb_status autotune(pb_system *sys, int precision, cudaStream_t s, Tuning *out) {
     // timed on about a quarter as many blocks as they have items and ranked
     // by block-time (time x blocks), the share of a full launch they take.
     const long long blocks = variant == 1 ? (long long)tma_grid(g, 8).x : 0;
-    const bool shared = variant == 1 && tma_items(g, kcs[0], tws[0]) < 4 * blocks;
+    const bool shared = variant == 1 && tma_small(g);
     std::vector<std::pair<int, int>> cand;  // (tile width, z-chunk)
     for (int tw : tws) {
         const long long floor_items =
@@ -1473,7 +1509,8 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
             PB_CUDA_TRY(cudaMemsetAsync(sys->d32, 0, bytes32, s));
             PB_CUDA_TRY(cudaMemsetAsync(sys->pa32, 0, bytes32, s));
             int it = 0;
-            rc = run_pcg<float, CoefC32>(sys, cp, sys->z32, sys->pa32, sys->pb32, sys->d32, tune.kc,
+            rc = run_pcg<float, CoefC32>(sys, cp, sys->z32, sys->pa32, sys->pb32, sys->d32,
+                                         tune.variant == 1 ? tma_alone_kc(p, tune.kc, tune.tw) : tune.kc,
                                          tune.variant, tune.tw, mg, mg ? 2 : chunk, deadline, s, &it);
             if (rc == PB_OK && sys->h_st[0].status == 3) {
                 // the correction of an aborted inner solve is incomplete: it

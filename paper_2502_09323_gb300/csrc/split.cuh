@@ -152,8 +152,8 @@ pb_status slab_build(const pb_system *sys, Slab &sl, int k0, int k1, int KC, int
     sl.npartials = (int)(2 * cdiv(cN, 256) + 64);
     sl.partials = (double *)dalloc(8 * (size_t)sl.npartials, s);
     sl.queue = (unsigned int *)dalloc(4 * sizeof(unsigned int), s);
-    const int nitems = tma_items(sl.pg, KC, tw);
-    sl.tpart = (float *)dalloc(sizeof(float) * 3 * (size_t)nitems, s);
+    tma_entry_geometry(sl.host, sl.pg, KC, tw);
+    sl.tpart = (float *)dalloc(sizeof(float) * 3 * (size_t)sl.host.npart, s);
     sl.dev = (tma::SysEntry *)dalloc(sizeof(tma::SysEntry), s);
     if (!sl.W[0] || !sl.W[1] || !sl.W[2] || !sl.w32[0] || !sl.w32[1] || !sl.w32[2] || !sl.diag ||
         !sl.rhs || !sl.phi || !sl.code || !sl.z || !sl.pbuf[0] || !sl.pbuf[1] || !sl.d || !sl.st ||
@@ -198,7 +198,6 @@ pb_status slab_build(const pb_system *sys, Slab &sl, int k0, int k1, int KC, int
     e.st = sl.st;
     e.partials = sl.tpart;
     e.cnt = nullptr;
-    tma_entry_geometry(e, sl.pg, KC, tw);
     PB_CUDA_TRY(cudaMemcpyAsync(sl.dev, &e, sizeof(e), cudaMemcpyHostToDevice, s));
     (void)dev;
     return PB_OK;

@@ -29,9 +29,9 @@
 // for the next plane, so the gathers overlap that wait (the update kernel
 // also prefetches the next plane's into L1).
 //
-// Dot products: each item's go to that item's own FP32 slot; the last block
-// of the launch sums every system's slots in an order fixed by its item
-// count (compensated FP32, FP64 for the total) and updates its CG state, so
+// Dot products: those of every G planes of a tile column go to an FP32 slot
+// of their own; the last block of the launch sums every system's slots in an
+// order fixed by their number (compensated FP32, FP64 for the total) and updates its CG state, so
 // every result is independent of scheduling and of the other systems.
 //
 // A one-system launch may overlap the previous kernel of its stream
@@ -135,10 +135,12 @@ struct SysEntry {  // aligned as CUtensorMap
     float *x, *z;       // solution increment, preconditioned residual
     float *y;           // apply output
     CgState *st;
-    float *partials;    // per item li: sigma at [li], rho and rr at
-                        // [nitems + 2 li] and [nitems + 2 li + 1]
+    float *partials;    // per tile column and group of G planes, slot i: sigma at
+                        // [i], rho and rr at [npart + 2 i] and [npart + 2 i + 1]
     unsigned int *cnt;  // items finished in the current launch
     int xtiles, ytiles, nchunk, KC, nitems, item_base;
+    int G, nG, npart;   // planes of a partial (KC is a multiple), partials of a
+                        // tile column, of the system
     int tw;             // tile width (128, 64 or 32) of the maps and items
 };
 
@@ -255,7 +257,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
     using L = SlotLayout<MODE, FIXW>;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int s_abort, s_nsys, s_total, s_skip;
-    __shared__ int s_desc[NSLOT][7];  // i0, j0, kfirst, len, system, local item, parity
+    __shared__ int s_desc[NSLOT][7];  // i0, j0, kfirst, len, system, first partial, parity
     // per-descriptor warp partials of the dot products, combined without a
     // barrier: the warp that completes a descriptor's count sums them
     __shared__ float s_part[NSLOT][ROWS][2];
@@ -345,8 +347,9 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                         if (cdone) continue;  // converged
                         cur = ccur;
                     }
-                    li = it - e->item_base;
-                    const int col = li / e->nchunk, c = li - col * e->nchunk;
+                    const int ci = it - e->item_base;
+                    const int col = ci / e->nchunk, c = ci - col * e->nchunk;
+                    li = col * e->nG + c * e->KC / e->G;
                     kfirst = 1 + c * e->KC;
                     len = min(e->KC, e->pg.nz - 2 - c * e->KC);
                     tw = FIXW ? FIXW : e->tw;
@@ -460,7 +463,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
             return *reinterpret_cast<const uint32_t *>(sl + L::code + rr * cw + 16 + xl * 4);
         };
 
-        int gt = 0, nseg = 0;
+        int gt = 0, nseg = 0, nfl = 0;  // planes, items, partials so far
         // per-system values, reloaded only when the system changes (they
         // cannot change during the launch: finalisation runs at its end)
         int ksys = -1;
@@ -514,7 +517,8 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
             const int *d = s_desc[nseg % NSLOT];
             const int len = d[3];
             if (len < 0) break;  // end of work
-            const int i0 = d[0], j0 = d[1], kfirst = d[2], sys = d[4], li = d[5], cur = d[6];
+            const int i0 = d[0], j0 = d[1], kfirst = d[2], sys = d[4], cur = d[6];
+            int li = d[5], left_in_group = 0;
             const SysEntry *e = SINGLE ? &e0 : tab + sys;
             if (!SINGLE && sys != ksys) {
                 g = e->pg;
@@ -759,42 +763,47 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                 }
                 cm = cc;
                 cc = cn;
+                // ---- dot products of this group of planes: the 8 row warps
+                // combine their partials in shared memory (the warp that
+                // completes the count sums them in row order) and that warp
+                // stores the group's partial.  The last block of the launch
+                // sums each system's partials in their order and updates its
+                // CG state.  No warp waits for another.  The groups, not the
+                // items, own the partials, so the sums do not depend on the
+                // z-chunk as long as it is a multiple of the group.
+                // (FP32 across the warp: the FP64 pipe of this part is narrow)
+                if (MODE == MODE_A) continue;
+                if (left_in_group == 0) left_in_group = e->G;
+                if (--left_in_group > 0 && t < len) continue;
+                left_in_group = 0;
+                const float b0 = warp_sum_f(acc0), b1 = MODE == MODE_U ? warp_sum_f(acc1) : 0.f;
+                acc0 = acc1 = 0.f;
+                const int ps = nfl++ % NSLOT;
+                if (lane == 0) {
+                    s_part[ps][w][0] = b0;
+                    s_part[ps][w][1] = b1;
+                    __threadfence_block();
+                    if (atomicAdd(&s_pcnt[ps], 1u) == (unsigned)ROWS - 1) {
+                        __threadfence_block();
+                        float t0 = 0.f, t1 = 0.f;
+                        for (int r = 0; r < ROWS; ++r) {
+                            t0 += *(volatile float *)&s_part[ps][r][0];
+                            t1 += *(volatile float *)&s_part[ps][r][1];
+                        }
+                        s_pcnt[ps] = 0u;
+                        if (MODE == MODE_P) {
+                            e->partials[li] = t0;
+                        } else {
+                            e->partials[e->npart + 2 * li] = t0;
+                            e->partials[e->npart + 2 * li + 1] = t1;
+                        }
+                    }
+                }
+                ++li;
             }
             if (!ok) break;
             release(gt0 + len + 1);  // the chunk's last plane (+z halo only)
             gt = gt0 + len + 2;
-            if (MODE == MODE_A) continue;
-
-            // ---- dot products of this item: the 8 row warps combine their
-            // partials in shared memory (the warp that completes the count
-            // sums them in row order) and that warp stores the item's partial.
-            // The last block of the launch sums each system's item partials
-            // in item order and updates its CG state.  No warp waits for
-            // another.
-            // (FP32 across the warp: the FP64 pipe of this part is narrow)
-            const float b0 = warp_sum_f(acc0), b1 = warp_sum_f(acc1);
-            const int ps = nseg % NSLOT;
-            if (lane == 0) {
-                s_part[ps][w][0] = b0;
-                s_part[ps][w][1] = b1;
-                __threadfence_block();
-                if (atomicAdd(&s_pcnt[ps], 1u) == (unsigned)ROWS - 1) {
-                    __threadfence_block();
-                    float t0 = 0.f, t1 = 0.f;
-                    for (int r = 0; r < ROWS; ++r) {
-                        t0 += *(volatile float *)&s_part[ps][r][0];
-                        t1 += *(volatile float *)&s_part[ps][r][1];
-                    }
-                    s_pcnt[ps] = 0u;
-                    const int nit = e->nitems;
-                    if (MODE == MODE_P) {
-                        e->partials[li] = t0;
-                    } else {
-                        e->partials[nit + 2 * li] = t0;
-                        e->partials[nit + 2 * li + 1] = t1;
-                    }
-                }
-            }
         }
     }
     // this thread's item partials are visible device-wide before the block
@@ -872,7 +881,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
         };
         // the warp's items summed; the totals are valid in lane 0
         auto item_sums = [&](const SysEntry *e, int first, int stride, double &t0, double &t1) {
-            const int nit = e->nitems;
+            const int nit = e->npart;
             float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
 #pragma unroll 4
             for (int i = first; i < nit; i += stride) {
@@ -891,7 +900,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
         // large systems: the whole block, one after the other
         for (int q = 0; q < nsys; ++q) {
             const SysEntry *e = tab + q;
-            const int nit = e->nitems;
+            const int nit = e->npart;
             if (nit <= BIGSYS || *(volatile int *)&e->st->done) continue;
             double t0, t1;
             item_sums(e, threadIdx.x, NTHREADS, t0, t1);
@@ -913,7 +922,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
         // small systems: one warp each
         for (int q = w; q < nsys; q += NTHREADS / 32) {
             const SysEntry *e = tab + q;
-            const int nit = e->nitems;
+            const int nit = e->npart;
             CgState *st = e->st;
             // systems that were done at launch (or stopped by an abort) have no partials
             if (nit == 0 || nit > BIGSYS || *(volatile int *)&st->done) continue;

@@ -33,7 +33,7 @@ CASES = [
     ((66, 16, 35), 4.0, 4.0, True),
     ((131, 31, 9), 2.0, 80.0, True),
     ((8, 20, 20), 2.0, 80.0, False),
-    ((9, 9, 9000), 2.0, 80.0, False),
+    ((9, 9, 4000), 2.0, 80.0, False),
 ]
 
 
