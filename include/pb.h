@@ -134,9 +134,10 @@ typedef struct {
 
 /* Solver options.  precision PB_FP64: Jacobi-PCG entirely in FP64.
  * PB_MIXED: FP64 iterative refinement around an FP32 PCG (FP32 stencil,
- * vectors and per-thread accumulation, FP64 global dots), preconditioned on
- * uniform grids of at least 9 nodes an axis by one multigrid V-cycle, else by
- * the diagonal.
+ * vectors and per-thread accumulation, FP64 global dots), preconditioned by
+ * one multigrid V-cycle on uniform grids of at least 9 nodes an axis, by a
+ * smoother and a lattice correction on octrees of one to three levels of
+ * refinement, else by the diagonal.
  * Stop when ||f - A phi||_2 <= rtol ||f||_2 (true residual, FP64).
  * max_iter caps the total inner iterations, max_outer the refinement
  * steps; inner_rtol (0 = default 1e-6) is the inner relative tolerance;

@@ -142,11 +142,12 @@ struct Engine {
     bool tab_used[2] = {false, false};
     int tab_buf = 0;
     // one replay, by the number of multigrid levels above the bottom kernel
-    // that it runs (0: Jacobi-preconditioned systems only), captured when
+    // that it runs, and whether it has any such system, captured when
     // a table first needs it
-    cudaGraph_t graph[mg::LMAX] = {};
-    cudaGraphExec_t exec[mg::LMAX] = {};
+    cudaGraph_t graph[mg::LMAX + 1] = {};
+    cudaGraphExec_t exec[mg::LMAX + 1] = {};
     int depth = 0;                                     // the current table's
+    bool mg = false;                                   // it has a preconditioned system
     mg::Entry *dmg = nullptr, *hmg = nullptr;          // staging: 2 x cap, pinned
     mg::Head *dhead = nullptr, *hhead = nullptr;       // staging: 2, pinned
     dim3 grid;
@@ -245,12 +246,12 @@ bool engine_refine(Engine *e, int q, bool aborted) {
 
 // PCG iterations of one replay: few with multigrid (a solve takes about 15
 // a refinement step), more with Jacobi
-int engine_chunk(const Engine *e) { return e->depth > 0 ? 2 : e->chunk; }
+int engine_chunk(const Engine *e) { return e->mg ? 2 : e->chunk; }
 
 // capture one replay for tables of the current depth
 bool engine_capture(Engine *e) {
-    const int depth = e->depth;
-    if (e->exec[depth]) return true;
+    const int depth = e->depth, g = e->mg ? depth : mg::LMAX;
+    if (e->exec[g]) return true;
     static const unsigned rd0 = mg_resident(k_mg_down<true, false>, mg::DNT), rd1 = mg_resident(k_mg_down<false, false>, mg::DNT),
                           ru0 = mg_resident(k_mg_up<true, false>, mg::UNT), ru1 = mg_resident(k_mg_up<false, false>, mg::UNT);
     const mg::Entry none{};
@@ -271,8 +272,8 @@ bool engine_capture(Engine *e) {
         tma_launch<MODE_P>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
         tma_launch<MODE_U>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
     }
-    ENG_TRY(cudaStreamEndCapture(e->cs, &e->graph[depth]), "capture");
-    ENG_TRY(cudaGraphInstantiate(&e->exec[depth], e->graph[depth], 0), "graph instantiation");
+    ENG_TRY(cudaStreamEndCapture(e->cs, &e->graph[g]), "capture");
+    ENG_TRY(cudaGraphInstantiate(&e->exec[g], e->graph[g], 0), "graph instantiation");
     return true;
 }
 
@@ -287,6 +288,7 @@ bool engine_upload_table(Engine *e) {
     head = mg::Head{};
     head.nsys = e->cap;
     int total = 0, depth = 0;
+    bool any = false;
     // tables that fill the GPU with the longest work items take those
     long long nodes = 0;
     for (const HostSlot &hq : e->slots)
@@ -302,6 +304,7 @@ bool engine_upload_table(Engine *e) {
         me.st = &e->dslots[q].st;
         if (shared) mg_planes(me, true);
         depth = std::max(depth, me.nbot);
+        any = any || (hq.used && hq.job.sys->mg);
         for (int l = 0; l < mg::LMAX; ++l) {
             me.dbase[l] = head.dtotal[l];
             me.ubase[l] = head.utotal[l];
@@ -342,6 +345,7 @@ bool engine_upload_table(Engine *e) {
     e->tab_used[b] = true;
     e->tab_buf ^= 1;
     e->depth = depth;
+    e->mg = any;
     return engine_capture(e);
 }
 
@@ -378,7 +382,7 @@ void engine_complete(Engine *e, int q, const EngineSlot &m) {
 
 bool engine_issue(Engine *e, int mb) {
     const int chunk = engine_chunk(e);
-    ENG_TRY(cudaGraphLaunch(e->exec[e->depth], e->cs), "replay");
+    ENG_TRY(cudaGraphLaunch(e->exec[e->mg ? e->depth : mg::LMAX], e->cs), "replay");
     note_launch(chunk * (2 + (e->depth > 0 ? 2 * e->depth + 1 : 0)));
     // octree systems: the same number of iterations with their brick kernels
     for (int q = 0; q < e->cap; ++q) {

@@ -709,7 +709,7 @@ __global__ void k_mg_coarsen(mg::Lev F, mg::Lev C, const double *__restrict__ Wx
     C.wx[p] = W[0];
     C.wy[p] = W[1];
     C.wz[p] = W[2];
-    C.dg[p] = 1.f;
+    if (C.dg) C.dg[p] = 1.f;
     C.z[p] = kap;
 }
 
@@ -728,6 +728,7 @@ struct MgState {
     mg::Head *head = nullptr;    // device, of one-system launches
     float *v = nullptr;          // preconditioned residual (padded, level 0)
     void *mem = nullptr;         // coarse levels
+    bool lattice = false;        // level 0 has stored coefficients too
     float *partials = nullptr;
 };
 
@@ -761,7 +762,7 @@ void mg_planes(mg::Entry &e, bool shared) {
 // The levels of a grid; false when the hierarchy does not reach the bottom
 // kernel's size (grids thinner than 9 nodes, or very long and thin ones):
 // those keep the Jacobi preconditioner.
-bool mg_levels(const PadGeo &g, mg::Entry &e) {
+bool mg_levels(const PadGeo &g, mg::Entry &e, bool lattice = false) {
     using namespace mg;
     if (std::min(g.nx, std::min(g.ny, g.nz)) < 9) return false;
     int n[3] = {g.nx, g.ny, g.nz}, nl = 0;
@@ -772,7 +773,7 @@ bool mg_levels(const PadGeo &g, mg::Entry &e) {
         L.nx = n[0];
         L.ny = n[1];
         L.nz = n[2];
-        L.sx = nl == 0 ? g.sx : ((n[0] + 3) & ~3);
+        L.sx = nl == 0 && !lattice ? g.sx : ((n[0] + 3) & ~3);
         L.sxy = L.sx * n[1];
         if (std::min(n[0], std::min(n[1], n[2])) < 5) break;
         for (int d = 0; d < 3; ++d) n[d] = n[d] / 2 + 1;
@@ -780,7 +781,7 @@ bool mg_levels(const PadGeo &g, mg::Entry &e) {
     e.nlev = nl + 1;
     long long nodes = 0;
     int b = e.nlev;
-    while (b > 1) {
+    while (b > (lattice ? 0 : 1)) {  // level 0 of a solver's grid is not the bottom kernel's
         const Lev &L = e.lev[b - 1];
         const long long n = (long long)L.nx * L.ny * L.nz;
         if (nodes + n > BOT_NODES) break;
@@ -793,6 +794,10 @@ bool mg_levels(const PadGeo &g, mg::Entry &e) {
     for (int l = b; l < e.nlev; ++l) {
         e.lev[l].sx = e.lev[l].nx;
         e.lev[l].sxy = e.lev[l].nx * e.lev[l].ny;
+    }
+    if (lattice) {
+        mg_planes(e, false);
+        return true;
     }
     const Lev &F = e.lev[0];
     e.nu0 = cdiv(F.nx - 1, FX) * cdiv(F.ny - 2, FY) * cdiv(F.nz - 2, RG);
@@ -826,6 +831,49 @@ pb_status mg_prepare() {
     return PB_OK;
 }
 
+// lays the arrays of levels first .. nlev - 1 and the bottom kernel's data out
+// in `base`; returns the bytes (base may be null)
+size_t mg_layout(mg::Entry &e, int first, char *base) {
+    size_t at = 0;
+    for (int l = first; l < e.nlev; ++l) {
+        mg::Lev &L = e.lev[l];
+        const size_t n = mg_lev_floats(L);
+        if (base) {
+            L.wx = (float *)(base + at);  // n is a multiple of 4: every array is 16-byte aligned
+            L.wy = L.wx + n;
+            L.wz = L.wy + n;
+            L.dg = L.wz + n;
+            L.s = L.dg + n;
+            L.z = L.s + n;
+        }
+        at += n * 24;
+    }
+    if (base) e.blob = base + at;
+    return at + 22 * (size_t)e.bot;
+}
+
+// coefficients of levels first .. nlev - 1 from the level above (level 1 of a
+// solver's grid from its FP64 operator; first == 0: level 0 is there already,
+// its ionic terms in z), and the bottom kernel's data
+pb_status mg_build_levels(const mg::Entry &e, int first, const pb_system *sys, cudaStream_t s) {
+    for (int l = first; l < e.nlev; ++l) {
+        const mg::Lev &C = e.lev[l];
+        const unsigned blocks = cdiv((long long)C.nx * C.ny * C.nz, 256);
+        if (l == 1 && first == 1)
+            k_mg_coarsen<true><<<blocks, 256, 0, s>>>(e.lev[0], C, sys->W[0], sys->W[1], sys->W[2], sys->code, e.cp.kap);
+        else if (l > 0)
+            k_mg_coarsen<false><<<blocks, 256, 0, s>>>(e.lev[l - 1], C, nullptr, nullptr, nullptr, nullptr, 0.f);
+        k_mg_diag<<<blocks, 256, 0, s>>>(C);
+        note_launch(1);
+        PB_LAUNCH_CHECK();
+    }
+    k_mg_pack<<<cdiv(e.bot, 256), 256, 0, s>>>(e, e.bot);
+    PB_LAUNCH_CHECK();
+    for (int l = first; l < e.nlev; ++l)  // z held the ionic terms
+        PB_CUDA_TRY(cudaMemsetAsync(e.lev[l].z, 0, sizeof(float) * (size_t)e.lev[l].sxy * e.lev[l].nz, s));
+    return PB_OK;
+}
+
 // hierarchy of a uniform system, built with its first mixed-precision solve
 // (coefficients and grids do not change after that); sys->mg stays null on
 // grids without one
@@ -839,10 +887,7 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
     MgState *m = new (std::nothrow) MgState();
     if (!m) return PB_ERR_OOM;
     sys->mg = m;
-    size_t bytes = 0;
-    for (int l = 1; l < e.nlev; ++l) bytes += mg_lev_floats(e.lev[l]) * 24;
-    const size_t blob = bytes;
-    bytes += 22 * (size_t)e.bot;
+    const size_t bytes = mg_layout(e, 1, nullptr);
     m->head = (Head *)dalloc(sizeof(Head), s);
     m->v = (float *)dalloc(sizeof(float) * (size_t)sys->pad.Np, s);
     m->mem = dalloc(bytes, s);
@@ -856,40 +901,14 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
     PB_CUDA_TRY(cudaMemsetAsync(m->mem, 0, bytes, s));
     e.lev[0].s = sys->z32;
     e.lev[0].z = m->v;
-    char *at = (char *)m->mem;
-    for (int l = 1; l < e.nlev; ++l) {
-        Lev &L = e.lev[l];
-        const size_t n = mg_lev_floats(L);
-        L.wx = (float *)at;  // n is a multiple of 4: every array is 16-byte aligned
-        L.wy = L.wx + n;
-        L.wz = L.wy + n;
-        L.dg = L.wz + n;
-        L.s = L.dg + n;
-        L.z = L.s + n;
-        at += n * 24;
-    }
-    e.blob = (char *)m->mem + blob;
+    mg_layout(e, 1, (char *)m->mem);
     e.st = sys->st;
     e.code = sys->code;
     e.cp = make_c32(sys);
     e.dg_in = 6.f * e.cp.w_in;
     e.dg_out = 6.f * e.cp.w_out + e.cp.kap;
     e.partials = m->partials;
-    for (int l = 1; l < e.nlev; ++l) {
-        const Lev &F = e.lev[l - 1], &C = e.lev[l];
-        const unsigned blocks = cdiv((long long)C.nx * C.ny * C.nz, 256);
-        if (l == 1)
-            k_mg_coarsen<true><<<blocks, 256, 0, s>>>(F, C, sys->W[0], sys->W[1], sys->W[2], sys->code, e.cp.kap);
-        else
-            k_mg_coarsen<false><<<blocks, 256, 0, s>>>(F, C, nullptr, nullptr, nullptr, nullptr, 0.f);
-        k_mg_diag<<<blocks, 256, 0, s>>>(C);
-        note_launch(1);
-        PB_LAUNCH_CHECK();
-    }
-    k_mg_pack<<<cdiv(e.bot, 256), 256, 0, s>>>(e, e.bot);
-    PB_LAUNCH_CHECK();
-    for (int l = 1; l < e.nlev; ++l)  // z held the ionic terms
-        PB_CUDA_TRY(cudaMemsetAsync(e.lev[l].z, 0, sizeof(float) * (size_t)e.lev[l].sxy * e.lev[l].nz, s));
+    if ((rc = mg_build_levels(e, 1, sys, s)) != PB_OK) return rc;
     m->e = e;
     return PB_OK;
 }
@@ -920,17 +939,20 @@ void mg_launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// one V-cycle of one system (z32 -> v); returns the number of launches
+// one V-cycle of one system (z32 -> v, or a lattice's s -> z); returns the
+// number of launches
 int launch_vcycle(const pb_system *sys, cudaStream_t s) {
     using namespace mg;
     const MgState *m = (const MgState *)sys->mg;
-    const Entry &e = m->e;
+    Entry e = m->e;
+    e.st = sys->st;  // the engine lends a system its slot's state
+    const bool fine = !m->lattice;
     static const unsigned rd0 = mg_resident(k_mg_down<true, true>, DNT), rd1 = mg_resident(k_mg_down<false, true>, DNT),
                           ru0 = mg_resident(k_mg_up<true, true>, UNT), ru1 = mg_resident(k_mg_up<false, true>, UNT);
     const Entry *none = nullptr;
     for (int l = 0; l < e.nbot; ++l) {
         const int n = ditems(e, l);
-        if (l == 0)
+        if (l == 0 && fine)
             mg_launch(k_mg_down<true, true>, std::min<unsigned>(n, rd0), DNT, 0, s, true, none, (const Head *)m->head, l,
                       n, e);
         else
@@ -940,10 +962,94 @@ int launch_vcycle(const pb_system *sys, cudaStream_t s) {
     mg_launch(k_mg_bottom<true>, 1, BOT_T, mg_bottom_bytes(e), s, true, none, (const Head *)m->head, e);
     for (int l = e.nbot - 1; l >= 0; --l) {
         const int n = uitems(e, l);
-        if (l == 0)
+        if (l == 0 && fine)
             mg_launch(k_mg_up<true, true>, std::min<unsigned>(n, ru0), UNT, 0, s, true, none, m->head, l, n, e);
         else
             mg_launch(k_mg_up<false, true>, std::min<unsigned>(n, ru1), UNT, 0, s, true, none, m->head, l, n, e);
     }
     return 2 * e.nbot + 1;
 }
+
+// The lattice of an octree's preconditioner: `up` coarsenings of the lattice
+// that fill() writes.
+pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cudaStream_t s) {
+    using namespace mg;
+    if (sys->mg) return PB_OK;
+    Entry e{};
+    PadGeo g{};
+    g.nx = g.ny = g.nz = n;
+    if (!mg_levels(g, e, true)) return PB_OK;
+    pb_status rc = mg_prepare();
+    if (rc != PB_OK) return rc;
+    MgState *m = new (std::nothrow) MgState();
+    if (!m) return PB_ERR_OOM;
+    sys->mg = m;
+    m->lattice = true;
+    const size_t bytes = mg_layout(e, 0, nullptr);
+    m->head = (Head *)dalloc(sizeof(Head), s);
+    m->mem = dalloc(bytes, s);
+    if (!m->head || !m->mem) {
+        free_mg_state(sys);
+        return PB_ERR_OOM;
+    }
+    PB_CUDA_TRY(cudaMemsetAsync(m->head, 0, sizeof(Head), s));
+    PB_CUDA_TRY(cudaMemsetAsync(m->mem, 0, bytes, s));
+    mg_layout(e, 0, (char *)m->mem);
+    e.st = sys->st;
+    // from the finest of the lattices down to level 0
+    Lev F{};
+    void *tmp = nullptr;
+    for (int q = up; q >= 0 && rc == PB_OK; --q) {
+        Lev C = e.lev[0];
+        void *mem = nullptr;
+        if (q > 0) {
+            C.nx = C.ny = C.nz = (n - 1) * (1 << q) + 1;
+            C.sx = (C.nx + 3) & ~3;
+            C.sxy = C.sx * C.ny;
+            const size_t c = mg_lev_floats(C);
+            mem = dalloc(16 * c, s);
+            if (!mem) {
+                rc = PB_ERR_OOM;
+                break;
+            }
+            C.wx = (float *)mem;
+            C.wy = C.wx + c;
+            C.wz = C.wy + c;
+            C.z = C.wz + c;
+            C.dg = nullptr;
+        }
+        if (q == up) {
+            rc = fill(sys, C.nx, C.sx, C.wx, C.wy, C.wz, C.z, s);
+        } else {
+            k_mg_coarsen<false><<<cdiv((long long)C.nx * C.ny * C.nz, 256), 256, 0, s>>>(F, C, nullptr, nullptr,
+                                                                                        nullptr, nullptr, 0.f);
+            note_launch(1);
+        }
+        dfree(tmp, s);
+        tmp = mem;
+        F = C;
+    }
+    dfree(tmp, s);
+    if (rc == PB_OK && cudaGetLastError() != cudaSuccess) rc = PB_ERR_CUDA;
+    if (rc == PB_OK) rc = mg_build_levels(e, 0, sys, s);
+    if (rc != PB_OK) {
+        free_mg_state(sys);
+        return rc;
+    }
+    m->e = e;
+    return PB_OK;
+}
+
+LatticeMg mg_lattice_view(const pb_system *sys) {
+    const mg::Lev &L = ((const MgState *)sys->mg)->e.lev[0];
+    LatticeMg v;
+    v.n = L.nx;
+    v.sx = L.sx;
+    v.sxy = L.sxy;
+    v.s = L.s;
+    v.z = L.z;
+    v.dg = L.dg;
+    return v;
+}
+
+int mg_lattice_cycle(const pb_system *sys, cudaStream_t s) { return launch_vcycle(sys, s); }

@@ -963,7 +963,11 @@ __global__ void k_oct_lift(OctDev t, BcDesc bd, const double *__restrict__ W0,
 // MODE_U: q = A p, x += alpha p, z -= alpha q / D, rho = sum D z^2,
 //         rr = sum (D z)^2 -> beta, stop test
 // MODE_A: y = A x
-enum { OM_P = 0, OM_U = 1, OM_A = 2 };
+// MODE_C: y = v + ca (v - prev) + cb (s - D^-1 A v), v = vs xin: a step of the
+//         preconditioner's smoother; MODE_L: its last one, with rho = sum D s y
+//         -> beta
+// MODE_R: y = D s - A xin
+enum { OM_P = 0, OM_U = 1, OM_A = 2, OM_C = 3, OM_L = 4, OM_R = 5 };
 
 template <typename T>
 struct OctArgs {
@@ -971,8 +975,10 @@ struct OctArgs {
     const T *z, *pold;   // P
     T *p;                // P out, U in
     T *x, *zz;           // U in/out
-    const T *xin;        // A in
-    T *y;                // A out
+    const T *xin;        // A, C, L, R in
+    T *y;                // A, C, L, R out
+    const T *sin, *prev; // C, L, R: s; C, L: x_k-1 / ps (may be null)
+    T vs, ps, ca, cb;    // C, L: scales of xin and prev, coefficients
     // compressed FP32 operator (pure rows)
     const uint8_t *code;
     const float *w32[3];
@@ -1119,9 +1125,23 @@ __device__ __forceinline__ void finalize_p(CgState *s, double t0) {
     }
 }
 
-__device__ __forceinline__ void finalize_u(CgState *s, double t0, double t1) {
-    s->beta = t0 / s->rho;
+// rho of the preconditioned residual (the first one of a solve has no
+// predecessor: beta = 0)
+__device__ __forceinline__ void finalize_l(CgState *s, double t0) {
+    if (!(t0 > 0.0) || !isfinite(t0)) {
+        s->done = 1;
+        s->status = 1;
+        return;
+    }
+    s->beta = s->rho > 0.0 ? t0 / s->rho : 0.0;
     s->rho = t0;
+}
+
+__device__ __forceinline__ void finalize_u(CgState *s, double t0, double t1) {
+    if (!s->mg) {  // else the preconditioner sets them
+        s->beta = t0 / s->rho;
+        s->rho = t0;
+    }
     s->rr = t1;
     s->iter += 1;
     if (s->profile) {
@@ -1205,6 +1225,8 @@ __global__ void __launch_bounds__(OB, MODE == OM_U ? 3 : 4) k_oct_pure(OctArgs<T
     auto value = [&](int n, uint8_t cd) -> T {
         if (MODE == OM_P) return A.z[n] + beta * A.pold[n];
         if (MODE == OM_U) return A.p[n];
+        if (MODE == OM_C || MODE == OM_L) return A.vs * A.xin[n];
+        if (MODE == OM_R) return A.xin[n];
         return (cd >> 4) == 1 || (cd >> 4) == 2 ? (T)0 : A.xin[n];  // boundary entries read as zero
     };
     float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
@@ -1264,7 +1286,8 @@ __global__ void __launch_bounds__(OB, MODE == OM_U ? 3 : 4) k_oct_pure(OctArgs<T
             kp = A.lc.kap32[level];
         }
         const int base = (b << 9) + c;
-        T v[8], xr[MODE == OM_U ? 8 : 1], zr[MODE == OM_U ? 8 : 1];
+        constexpr bool CL = MODE == OM_C || MODE == OM_L;
+        T v[8], xr[MODE == OM_U || CL ? 8 : 1], zr[MODE == OM_U || CL || MODE == OM_R ? 8 : 1];
         uint8_t cd[8];
         if constexpr (AW) {
 #pragma unroll
@@ -1285,6 +1308,8 @@ __global__ void __launch_bounds__(OB, MODE == OM_U ? 3 : 4) k_oct_pure(OctArgs<T
                 xr[k] = A.x[base + 64 * k];
                 zr[k] = A.zz[base + 64 * k];
             }
+            if constexpr (CL || MODE == OM_R) zr[k] = A.sin[base + 64 * k];
+            if constexpr (CL) xr[k] = A.prev ? A.ps * A.prev[base + 64 * k] : (T)0;
         }
         T hv[4];
         uint8_t hc[4];
@@ -1411,6 +1436,12 @@ __global__ void __launch_bounds__(OB, MODE == OM_U ? 3 : 4) k_oct_pure(OctArgs<T
                     d0 += dz * zn;
                     d1 += dz * dz;
                 }
+            } else if (CL) {
+                const T y = pa + A.ca * (pa - xr[k]) + A.cb * (zr[k] - qv / D);
+                A.y[a] = y;
+                if (MODE == OM_L) bs0 += D * zr[k] * y;
+            } else if (MODE == OM_R) {
+                A.y[a] = D * zr[k] - qv;
             } else {
                 A.y[a] = qv;
             }
@@ -1460,6 +1491,7 @@ __global__ void __launch_bounds__(OB, MODE == OM_U ? 3 : 4) k_oct_pure(OctArgs<T
                 T v;
                 if (MODE == OM_P) v = A.z[c] + beta * A.pold[c];
                 else if (MODE == OM_U) v = A.p[c];
+                else if (MODE == OM_C || MODE == OM_L) v = A.vs * A.xin[c];
                 else v = A.xin[c];
                 q += A.tr_val[e] * v;
             }
@@ -1482,16 +1514,29 @@ __global__ void __launch_bounds__(OB, MODE == OM_U ? 3 : 4) k_oct_pure(OctArgs<T
                     d0 += dz * zn;
                     d1 += dz * dz;
                 }
+            } else if (MODE == OM_C || MODE == OM_L) {
+                const T D = (T)A.tr_diag[r], pa = A.vs * A.xin[a], s = A.sin[a];
+                const T pr = A.prev ? A.ps * A.prev[a] : (T)0;
+                const T y = pa + A.ca * (pa - pr) + A.cb * (s - q / D);
+                A.y[a] = y;
+                if (MODE == OM_L) {
+                    if constexpr (sizeof(T) == 4) kahan(s0, c0, D * s * y);
+                    else d0 += D * s * y;
+                }
+            } else if (MODE == OM_R) {
+                A.y[a] = (T)A.tr_diag[r] * A.sin[a] - q;
             } else {
                 A.y[a] = q;
             }
         }
     }
-    if (MODE == OM_A) return;
+    if (MODE == OM_A || MODE == OM_C || MODE == OM_R) return;
     auto finish = [&](const double (&tot)[2]) {
         CgState *s = A.st;
         if (MODE == OM_P) {
             finalize_p(s, tot[0]);
+        } else if (MODE == OM_L) {
+            finalize_l(s, tot[0]);
         } else {
             finalize_u(s, tot[0], tot[1]);
         }
@@ -1511,6 +1556,8 @@ __global__ void __launch_bounds__(OB, MODE == OM_U ? 3 : 4) k_oct_pure(OctArgs<T
             finish(tot);
     }
 }
+
+#include "oct_mg.cuh"
 
 // FP64 true residual r = f - A x (x = phi on the unknowns), z = r / D in
 // the inner solver's precision; |r|^2 and r.z to the CG state
@@ -2152,7 +2199,7 @@ void oct_system_free(pb_system *sys, cudaStream_t s) {
     OctSys *os = sys->os;
     if (!os) return;
     void *ptrs[] = {os->tr_slot, os->tr_row, os->tr_ptr, os->tr_col, os->tr_val, os->tr_val32,
-                    os->tr_diag, os->tpart, os->partials, os->tcount};
+                    os->tr_diag, os->tpart, os->partials, os->tcount, os->mx[0], os->mx[1], os->mpart};
     for (void *p : ptrs) dfree(p, s);
     delete os;
     sys->os = nullptr;
@@ -2192,9 +2239,66 @@ OctArgs<T> oct_args(pb_system *sys) {
     return A;
 }
 
+// The preconditioner: s = D^-1 r in z32 -> z; the buffer that holds z
+const float *oct_precondition(pb_system *sys, OctArgs<float> A, const float *z32, cudaStream_t s) {
+    OctSys *os = sys->os;
+    const OctDev &t = sys->g->ot;
+    const OmgPoly P = omg_poly(t.Lmax);
+    const LatticeMg L = mg_lattice_view(sys);
+    A.sin = z32;
+    A.vs = A.ps = 1.f;
+    // smoothing from zero: x_1 = first s is read from s, scaled
+    A.xin = z32;
+    A.vs = P.first;
+    A.prev = nullptr;  // x_0 = 0
+    float *cur = os->mx[0], *other = os->mx[1];
+    for (int k = 1; k < P.degree; ++k) {
+        A.y = cur;
+        A.ca = P.step[k].a;
+        A.cb = P.step[k].b;
+        k_oct_pure<float, OM_C><<<pure_grid<float, OM_C>(), OB, 0, s>>>(A);
+        A.prev = A.xin;
+        A.ps = A.vs;
+        A.xin = cur;
+        A.vs = 1.f;
+        std::swap(cur, other);
+    }
+    // A.xin holds the smoothed iterate, cur is free
+    float *x = const_cast<float *>(A.xin);
+    A.y = cur;
+    k_oct_pure<float, OM_R><<<pure_grid<float, OM_R>(), OB, 0, s>>>(A);
+    const unsigned bb = (unsigned)std::min<long long>((t.nb + 3) / 4, 8ll * num_sms());
+    k_omg_partial<<<bb, OB, 0, s>>>(t, cur, os->mpart, A.st);
+    const long long m = L.n - 2;
+    k_omg_gather<<<cdiv(m * m * m, 256), 256, 0, s>>>(t, cur, os->mpart, L, A.st);
+    const int cycle = mg_lattice_cycle(sys, s);
+    k_omg_prolong<<<bb, OB, 0, s>>>(t, sys->code, L, x, A.st);
+    A.prev = nullptr;
+    A.vs = A.ps = 1.f;
+    for (int k = 0; k < P.degree; ++k) {
+        // x_k+1 may replace x_k-1: it is read at its own node only
+        float *out = k == 0 ? cur : const_cast<float *>(A.prev);
+        A.xin = x;
+        A.y = out;
+        A.ca = P.step[k].a;
+        A.cb = P.step[k].b;
+        if (k + 1 < P.degree)
+            k_oct_pure<float, OM_C><<<pure_grid<float, OM_C>(), OB, 0, s>>>(A);
+        else
+            k_oct_pure<float, OM_L><<<pure_grid<float, OM_L>(), OB, 0, s>>>(A);
+        A.prev = x;
+        x = out;
+    }
+    note_launch(2 * P.degree + 3 + cycle);
+    return x;
+}
+
 template <typename T>
 void oct_iteration(pb_system *sys, OctArgs<T> A, T *z, T *pold, T *p, T *x, cudaStream_t s) {
     A.z = z;
+    if constexpr (sizeof(T) == 4) {
+        if (sys->mg) A.z = oct_precondition(sys, A, z, s);
+    }
     A.pold = pold;
     A.p = p;
     A.x = x;
@@ -2202,6 +2306,36 @@ void oct_iteration(pb_system *sys, OctArgs<T> A, T *z, T *pold, T *p, T *x, cuda
     k_oct_pure<T, OM_P><<<pure_grid<T, OM_P>(), OB, 0, s>>>(A);
     k_oct_pure<T, OM_U><<<pure_grid<T, OM_U>(), OB, 0, s>>>(A);
     note_launch(2);
+}
+
+// Weights of the lattice at twice the finest spacing
+pb_status oct_lattice(const pb_system *sys, int n, int sx, float *wx, float *wy, float *wz, float *kap,
+                      cudaStream_t s) {
+    const OctDev &t = sys->g->ot;
+    const LevelConst lc = level_const(sys);
+    k_omg_lattice<<<cdiv((long long)n * n * n, 128), 128, 0, s>>>(t, sys->W[0], sys->W[1], sys->W[2], sys->g->inside,
+                                                                  lc.w_out[t.Lmax], lc.kap32[t.Lmax], n, sx, wx, wy,
+                                                                  wz, kap);
+    PB_LAUNCH_CHECK();
+    return PB_OK;
+}
+
+// the preconditioner's lattice and buffers (octrees of one to OMG_LMAX levels
+// of refinement; others keep Jacobi)
+pb_status oct_mg_make(pb_system *sys, cudaStream_t s) {
+    const OctDev &t = sys->g->ot;
+    OctSys *os = sys->os;
+    const long long nf = (long long)(t.NL / 2 + 1);  // nodes an axis at twice the finest spacing
+    if (sys->mg || t.Lmax < 1 || t.Lmax > OMG_LMAX || nf * nf * (nf + 3) > 0x7fffffffll) return PB_OK;
+    const size_t b32 = sizeof(float) * (size_t)t.N;
+    for (float *&q : os->mx) {
+        if (!q) q = (float *)dalloc(b32, s);
+        if (!q) return PB_ERR_OOM;
+        PB_CUDA_TRY(cudaMemsetAsync(q, 0, b32, s));
+    }
+    if (!os->mpart) os->mpart = (float *)dalloc(sizeof(float) * OMG_PART * (size_t)t.nb, s);
+    if (!os->mpart) return PB_ERR_OOM;
+    return mg_lattice_make(sys, t.NL / (1 << t.Lmax) + 1, t.Lmax - 1, oct_lattice, s);
 }
 
 pb_status oct_ensure_ws(pb_system *sys, int precision, cudaStream_t s) {
@@ -2212,7 +2346,8 @@ pb_status oct_ensure_ws(pb_system *sys, int precision, cudaStream_t s) {
         PB_CUDA_TRY(cudaMemsetAsync(sys->st, 0, sizeof(CgState), s));
         PB_CUDA_TRY(cudaMallocHost((void **)&sys->h_st, 4 * sizeof(CgState)));
         const int G = std::max(std::max(pure_grid<float, OM_P>(), pure_grid<float, OM_U>()),
-                               std::max(pure_grid<double, OM_P>(), pure_grid<double, OM_U>()));
+                               std::max(std::max(pure_grid<double, OM_P>(), pure_grid<double, OM_U>()),
+                                        pure_grid<float, OM_L>()));
         sys->npartials = 2 * (int)std::max<long long>(cdiv(N, OT), G) + 64;
         sys->partials = (double *)dalloc(sizeof(double) * sys->npartials, s);
         if (!sys->partials) return PB_ERR_OOM;
@@ -2240,10 +2375,11 @@ pb_status oct_ensure_ws(pb_system *sys, int precision, cudaStream_t s) {
 }
 
 pb_status oct_state(pb_system *sys, double rho, double rr0, double rr_stop, int max_iter,
-                    cudaStream_t s, int profile = 0) {
+                    cudaStream_t s, int profile = 0, bool mg = false) {
     CgState h{};
     h.profile = profile;
-    h.rho = rho;
+    h.mg = mg;
+    h.rho = mg ? 0.0 : rho;  // the first preconditioned residual sets it
     h.rr0 = rr0;
     h.rr = rr0;
     h.rr_stop = rr_stop;
@@ -2283,7 +2419,7 @@ pb_status oct_run(pb_system *sys, T *z, T *pa, T *pb, T *x, double deadline, cud
     OctArgs<T> A = oct_args<T>(sys);
     T *bufs[2] = {pa, pb};
     int cur = 0;
-    const int chunk = 16;
+    const int chunk = sizeof(T) == 4 && sys->mg ? 2 : 16;
     cudaEvent_t ev[2];
     PB_CUDA_TRY(cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming));
     PB_CUDA_TRY(cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming));
@@ -2345,6 +2481,7 @@ pb_status oct_solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_s
     const OctDev &t = sys->g->ot;
     const long long N = t.N;
     pb_status rc = oct_ensure_ws(sys, o->precision, s);
+    if (rc == PB_OK && o->precision == PB_MIXED) rc = oct_mg_make(sys, s);
     if (rc != PB_OK) return rc;
     const int max_iter = o->max_iter > 0 ? o->max_iter : 100000;
     const int max_outer = o->max_outer > 0 ? o->max_outer : 30;
@@ -2369,7 +2506,8 @@ pb_status oct_solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_s
             const double rel = sqrt(res2 / fn2);
             double itol = std::max(inner_rtol, 0.5 * rtol / rel);
             if (itol > 0.5) itol = 0.5;
-            if ((rc = oct_state(sys, sys->h_st->rz64, res2, itol * itol * res2, max_iter - iters, s)) != PB_OK)
+            if ((rc = oct_state(sys, sys->h_st->rz64, res2, itol * itol * res2, max_iter - iters, s, 0,
+                                sys->mg != nullptr)) != PB_OK)
                 return rc;
             PB_CUDA_TRY(cudaMemsetAsync(sys->d32, 0, sizeof(float) * N, s));
             PB_CUDA_TRY(cudaMemsetAsync(sys->pa32, 0, sizeof(float) * N, s));
@@ -2438,7 +2576,9 @@ pb_status oct_solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_s
         stats->seconds = wall_s() - t_start;
         const long long dof = sys->os->nunk;
         stats->dof = dof;
-        const long long per = o->precision == PB_MIXED ? (8 * 4 + 2) : (8 * 8 + 6 * 8 + 2);
+        // a preconditioned iteration adds 4 passes of 9 to 17 B, the restriction and the prolongation
+        long long per = o->precision == PB_MIXED ? (8 * 4 + 2) : (8 * 8 + 6 * 8 + 2);
+        if (o->precision == PB_MIXED && sys->mg) per += 64;
         stats->model_bytes = (long long)iters * dof * per + (long long)outer * N * 64;
     }
     return (pb_status)status;
@@ -2522,7 +2662,10 @@ pb_status oct_energy(pb_system *sys, cudaStream_t s, pb_energy_terms *out) {
 // system's CG state pointer is the engine slot's).
 namespace pbg {
 
-pb_status oct_engine_prepare(pb_system *sys, cudaStream_t s) { return oct_ensure_ws(sys, PB_MIXED, s); }
+pb_status oct_engine_prepare(pb_system *sys, cudaStream_t s) {
+    const pb_status rc = oct_ensure_ws(sys, PB_MIXED, s);
+    return rc == PB_OK ? oct_mg_make(sys, s) : rc;
+}
 
 pb_status oct_engine_residual(pb_system *sys, cudaStream_t s) { return oct_residual(sys, true, s); }
 

@@ -110,6 +110,8 @@ struct OctSys {
     double *partials;     // per-block partials of the transition kernels
     unsigned int *tcount; // last-block counter of the transition kernels
     int npart;
+    float *mx[2];         // preconditioner: iterates of the smoother
+    float *mpart;         // and the bricks' sums of the residual on the lattice
 };
 
 }  // namespace pbg
@@ -236,6 +238,18 @@ pb_status ensure_solver_ws(pb_system *sys, int precision, cudaStream_t s);
 pb_status profile_kernels(pb_system *sys, int precision, int which, int reps, cudaStream_t s);
 void free_tma_state(pb_system *sys);
 void free_mg_state(pb_system *sys);
+// Uniform lattice of n^3 nodes with stored coefficients, solved by one
+// multigrid V-cycle (s = D^-1 b in, z out); it becomes sys->mg.  `fill` writes
+// the weights and ionic terms of the lattice `up` times finer by a factor of two.
+struct LatticeMg {
+    int n, sx, sxy;
+    float *s, *z, *dg;
+};
+typedef pb_status (*lattice_fill)(const pb_system *sys, int n, int sx, float *wx, float *wy, float *wz, float *kap,
+                                  cudaStream_t s);
+pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cudaStream_t s);
+LatticeMg mg_lattice_view(const pb_system *sys);
+int mg_lattice_cycle(const pb_system *sys, cudaStream_t s);  // launches
 pb_status set_tuning(pb_system *sys, int precision, int variant, int kc);
 pb_status set_wait_limit(long long polls);
 pb_status solve_batch(pb_system *const *systems, int n, const pb_solve_opts *o, cudaStream_t s,

@@ -59,3 +59,29 @@ def test_solution_and_iterations(pb, orc, n, ein, eout, hierarchy):
     assert st2["iters_inner"] == st["iters_inner"] and np.array_equal(pb.pb_get_phi(s), phi)
     st3 = pb.pb_solve_split(s, 1, pb.SolveOpts(precision=pb.MIXED, rtol=1e-10))
     assert st3["iters_inner"] == st["iters_inner"] and np.array_equal(pb.pb_get_phi(s), phi)
+
+
+# h_bulk (one to four levels of refinement from 0.25 A), explicit coarse bricks (0: automatic),
+# lattice correction; the four-level tree keeps the Jacobi preconditioner
+OCTREES = [(0.5, 0, True), (1.0, 0, True), (1.0, 7, True), (2.0, 0, True), (2.0, 4, True), (4.0, 0, False)]
+
+
+@pytest.mark.parametrize("h_bulk,n0,lattice", OCTREES)
+def test_octree_solution_and_iterations(pb, h_bulk, n0, lattice):
+    atoms = pb_inputs.globular_molecule(25, seed=78)
+    o = tuple(atoms[:, :3].mean(0) - 4.0 * h_bulk * n0)
+    spec = pb.OctreeSpec(h_fine=0.25, h_bulk=h_bulk, refine_dist=6.0 if h_bulk > 2.0 else 3.0, n0=n0, origin=o)
+    s = pb.pb_assemble_coeffs(pb.pb_build_grid(spec, atoms), pb.Params(bc=pb.BC_DH))
+    # the plain FP64 solver (Jacobi, FP64 operator) on the same system
+    ref = pb.pb_solve(s, pb.SolveOpts(precision=pb.FP64, rtol=1e-12))
+    phi64 = pb.pb_get_phi(s)
+    st = pb.pb_solve(s, pb.SolveOpts(precision=pb.MIXED, rtol=1e-12))
+    phi = pb.pb_get_phi(s)
+    assert ref["status"] == 0 and st["status"] == 0 and st["true_rel_res"] <= 1e-12
+    # two solutions of relative residual 1e-12: their difference is at most the condition number
+    # (under 1e4 here) times that
+    assert np.linalg.norm(phi - phi64) <= 1e-8 * np.linalg.norm(phi64)
+    if lattice:
+        assert st["iters_inner"] <= 80  # 13 to 21 per 1e-6 in the CPU prototype
+    st2 = pb.pb_solve_batch([s], pb.SolveOpts(precision=pb.MIXED, rtol=1e-12))[0]
+    assert st2["iters_inner"] == st["iters_inner"] and np.array_equal(pb.pb_get_phi(s), phi)
