@@ -130,13 +130,13 @@ struct CoefS64 {
     __device__ __forceinline__ double kappa(uint8_t cs) const { return (cs & 1) ? 0.0 : kap; }
 };
 
-enum { MODE_P = 0, MODE_U = 1, MODE_A = 2 };
+enum { MODE_P = 0, MODE_U = 1 };
 
 template <typename T>
 struct KArgs {
-    const T *in;     // P: z ; U: p ; A: x
+    const T *in;     // P: z ; U: p
     const T *in2;    // P: p_old
-    T *out;          // P: p_new ; A: y
+    T *out;          // P: p_new
     T *xv;           // U: x (solution increment)
     T *zv;           // U: z
     const uint8_t *code;
@@ -211,7 +211,7 @@ struct CodeW<2> {
     static constexpr uint32_t rep(uint32_t b) { return b * 0x0101u; }
 };
 
-// One stencil kernel for the three uses (MODE_P / MODE_U / MODE_A).
+// One stencil kernel for both uses (MODE_P / MODE_U).
 // Each warp owns one grid row j (32*VEC consecutive x nodes, VEC per lane)
 // and marches along z over KC planes, carrying its row of planes k-1, k, k+1
 // in registers; the rows j-1 and j+1 of plane k are read from L1/L2 (the
@@ -228,11 +228,9 @@ k_stencil(KArgs<T> A, CP cp) {
     __shared__ double sred[NT / 32];
 
     T alpha = 0, beta = 0;
-    if (MODE != MODE_A) {
-        if (A.st->done) return;
-        if (MODE == MODE_P) beta = (T)A.st->beta;
-        if (MODE == MODE_U) alpha = (T)A.st->alpha;
-    }
+    if (A.st->done) return;
+    if (MODE == MODE_P) beta = (T)A.st->beta;
+    if (MODE == MODE_U) alpha = (T)A.st->alpha;
     const PadGeo g = A.pg;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i0 = blockIdx.x * TXP;
@@ -365,7 +363,6 @@ k_stencil(KArgs<T> A, CP cp) {
                                      (cym & CodeW<VEC>::rep(0x04u)) | (cm & CodeW<VEC>::rep(0x08u));
             fast = !__any_sync(0xffffffffu, special != 0u);
         }
-        T y[VEC];
 #pragma unroll
         for (int q = 0; q < VEC; ++q) {
             const int i = ib + q;
@@ -401,7 +398,6 @@ k_stencil(KArgs<T> A, CP cp) {
                 dinv = (T)1 / dg;
             }
             const bool interior = grp_ok && i >= 1 && i <= g.nx - 2;
-            y[q] = interior ? ap : (T)0;
             if (MODE == MODE_P) {
                 if (interior) acc0 += x0 * ap;
             } else if (MODE == MODE_U) {
@@ -421,7 +417,6 @@ k_stencil(KArgs<T> A, CP cp) {
                 vstore<T>(A.xv + base + ib, xv);
                 vstore<T>(A.zv + base + ib, zv);
             }
-            if (MODE == MODE_A) vstore<T>(A.out + base + ib, y);
         }
         // ---- rotate the pipeline
 #pragma unroll
@@ -447,7 +442,6 @@ k_stencil(KArgs<T> A, CP cp) {
         rn = (MODE == MODE_P) ? rn2a + beta * rn2b : rn2a;
         lcn = lcn2;
     }
-    if (MODE == MODE_A) return;
 
     const int nb = gridDim.x * gridDim.y * gridDim.z;
     double t0, t1;
@@ -596,24 +590,6 @@ __global__ void k_promote(double *__restrict__ phi, const TX *__restrict__ x, Gr
     long long i = a % g.nx, j = (a / g.nx) % g.ny, k = a / ((long long)g.nx * g.ny);
     bool interior = i > 0 && j > 0 && k > 0 && i < g.nx - 1 && j < g.ny - 1 && k < g.nz - 1;
     if (interior) phi[a] += (double)x[(k * g.ny + j) * pg.sx + i];
-}
-
-template <typename T>
-__global__ void k_canon_to_pad(const T *__restrict__ src, T *__restrict__ dst, GridGeo g, PadGeo pg) {
-    long long a = blockIdx.x * 256ll + threadIdx.x;
-    if (a >= g.N) return;
-    long long i = a % g.nx, j = (a / g.nx) % g.ny, k = a / ((long long)g.nx * g.ny);
-    bool interior = i > 0 && j > 0 && k > 0 && i < g.nx - 1 && j < g.ny - 1 && k < g.nz - 1;
-    dst[(k * g.ny + j) * pg.sx + i] = interior ? src[a] : (T)0;
-}
-
-template <typename T>
-__global__ void k_pad_to_canon(const T *__restrict__ src, T *__restrict__ dst, GridGeo g, PadGeo pg) {
-    long long a = blockIdx.x * 256ll + threadIdx.x;
-    if (a >= g.N) return;
-    long long i = a % g.nx, j = (a / g.nx) % g.ny, k = a / ((long long)g.nx * g.ny);
-    bool interior = i > 0 && j > 0 && k > 0 && i < g.nx - 1 && j < g.ny - 1 && k < g.nz - 1;
-    dst[a] = interior ? src[(k * g.ny + j) * pg.sx + i] : (T)0;
 }
 
 constexpr int TYC = 8;  // rows (warps) per stencil block
@@ -895,14 +871,12 @@ pb_status build_tma_state(pb_system *sys, cudaStream_t s) {
     e.tw = t->tw;
     if (rc == PB_OK) rc = tma_prepare<MODE_P>();
     if (rc == PB_OK) rc = tma_prepare<MODE_U>();
-    if (rc == PB_OK) rc = tma_prepare<MODE_A>();
     e.pg = sys->pad;
     e.cp = make_c32(sys);
     e.pbuf[0] = sys->pa32;
     e.pbuf[1] = sys->pb32;
     e.x = sys->d32;
     e.z = sys->z32;
-    e.y = nullptr;
     e.st = sys->st;
     t->max_items = std::max(tma_items(sys->pad, 4, 128),
                             std::max(tma_items(sys->pad, 4, 64), tma_items(sys->pad, 4, 32)));
@@ -1674,67 +1648,120 @@ pb_status profile_kernels(pb_system *sys, int precision, int which, int reps, cu
     return PB_OK;
 }
 
+namespace {
+
+// y = A x on the canonical layout (pb_apply): x and y are read and written once
+// and nothing else moves but the operator (FP32: code bytes and listed
+// weights; FP64: three weight arrays).  A thread takes PTS points of a plane,
+// 256 apart in the plane's flat order (rows of any length stay coalesced and
+// leave no idle lanes), and marches over KC planes with the values of three
+// planes in registers; x and y neighbours hit L1.  Each point's terms are
+// added in the order of the solver's kernels.  The former path copied x and y
+// to and from the padded layout around the TMA-staged kernel, with two
+// allocations, two clears and a host wait: 257^3 FP32 253 -> 96 us, 33^3 FP64
+// 32 -> 16 us (a Python call each).
+template <typename T, class CP, int PTS>
+__global__ void __launch_bounds__(256)
+k_apply(const T *__restrict__ x, T *__restrict__ y, const uint8_t *__restrict__ code, GridGeo g, int sx, CP cp,
+        int KC) {
+    const int nx = g.nx, ny = g.ny, nz = g.nz, plane = nx * ny;
+    const int k0 = blockIdx.y * KC, k1 = min(k0 + KC, nz);
+    int f[PTS], pc[PTS];
+    uint32_t edge[PTS];  // bit 0 interior column; 1..4 the -x, +x, -y, +y neighbour is interior
+    T xm[PTS], xc[PTS];
+    uint8_t cm[PTS], cc[PTS];
+#pragma unroll
+    for (int q = 0; q < PTS; ++q) {
+        f[q] = (blockIdx.x * PTS + q) * 256 + threadIdx.x;
+        const int j = f[q] / nx, i = f[q] - j * nx;
+        const bool in = f[q] < plane && i >= 1 && j >= 1 && i <= nx - 2 && j <= ny - 2;
+        edge[q] = in ? 1u | (i > 1) << 1 | (i < nx - 2) << 2 | (j > 1) << 3 | (j < ny - 2) << 4 : 0u;
+        pc[q] = j * sx + i;
+        xm[q] = in && k0 > 1 && k0 - 1 <= nz - 2 ? x[(long long)(k0 - 1) * plane + f[q]] : (T)0;
+        xc[q] = in && k0 >= 1 && k0 <= nz - 2 ? x[(long long)k0 * plane + f[q]] : (T)0;
+        cm[q] = in && k0 >= 1 ? code[(long long)(k0 - 1) * sx * ny + pc[q]] : 0;
+        cc[q] = in ? code[(long long)k0 * sx * ny + pc[q]] : 0;
+    }
+    for (int k = k0; k < k1; ++k) {
+        const bool inner = k >= 1 && k <= nz - 2;
+        T xn[PTS];
+        uint8_t cn[PTS];
+#pragma unroll
+        for (int q = 0; q < PTS; ++q) {
+            xn[q] = (edge[q] & 1) && k + 1 <= nz - 2 ? x[(long long)(k + 1) * plane + f[q]] : (T)0;
+            cn[q] = (edge[q] & 1) && k + 1 < nz ? code[(long long)(k + 1) * sx * ny + pc[q]] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < PTS; ++q) {
+            T out = 0;
+            const long long a = (long long)k * plane + f[q];
+            if (inner && (edge[q] & 1)) {
+                const uint32_t e = edge[q];
+                const T x0 = xc[q];
+                const T xl = (e & 2) ? x[a - 1] : (T)0, xr = (e & 4) ? x[a + 1] : (T)0;
+                const T yl = (e & 8) ? x[a - nx] : (T)0, yr = (e & 16) ? x[a + nx] : (T)0;
+                const int p = (int)((long long)k * sx * ny) + pc[q];
+                const uint8_t c0 = cc[q];
+                const T kp = cp.kappa(c0);
+                if constexpr (CP::kCompressed) {
+                    const uint8_t cl = code[p - 1], cy = code[p - sx];
+                    if (((c0 & 0x0E) | (cl & 2) | (cy & 4) | (cm[q] & 8)) == 0) {
+                        const T sum = ((x0 - xl) + (x0 - xr)) + ((x0 - yl) + (x0 - yr)) + ((x0 - xm[q]) + (x0 - xn[q]));
+                        out = cp.pure(c0) * sum + kp * x0;
+                    } else {
+                        out = kp * x0;
+                        out += cp.w(0, 0, 0, 0, p - 1, cl, c0) * (x0 - xl);
+                        out += cp.w(0, 0, 0, 0, p, c0, c0) * (x0 - xr);
+                        out += cp.w(1, 0, 0, 0, p - sx, cy, c0) * (x0 - yl);
+                        out += cp.w(1, 0, 0, 0, p, c0, c0) * (x0 - yr);
+                        out += cp.w(2, 0, 0, 0, p - sx * ny, cm[q], c0) * (x0 - xm[q]);
+                        out += cp.w(2, 0, 0, 0, p, c0, c0) * (x0 - xn[q]);
+                    }
+                } else {
+                    out = kp * x0;
+                    out += cp.W0[a - 1] * (x0 - xl);
+                    out += cp.W0[a] * (x0 - xr);
+                    out += cp.W1[a - nx] * (x0 - yl);
+                    out += cp.W1[a] * (x0 - yr);
+                    out += cp.W2[a - plane] * (x0 - xm[q]);
+                    out += cp.W2[a] * (x0 - xn[q]);
+                }
+            }
+            if (f[q] < plane) y[a] = out;
+            xm[q] = xc[q];
+            xc[q] = xn[q];
+            cm[q] = cc[q];
+            cc[q] = cn[q];
+        }
+    }
+}
+
+}  // namespace
+
 pb_status apply_op(pb_system *sys, int precision, const void *x, void *y, cudaStream_t s) {
     const GridGeo &g = sys->g->geo;
-    const PadGeo &p = sys->pad;
-    int KC = default_kc(p, precision);
-    size_t esz = precision == PB_MIXED ? 4 : 8;
-    void *xp = dalloc(esz * (size_t)p.Np, s), *yp = dalloc(esz * (size_t)p.Np, s);
-    if (!xp || !yp) return PB_ERR_OOM;
-    PB_CUDA_TRY(cudaMemsetAsync(xp, 0, esz * (size_t)p.Np, s));
-    PB_CUDA_TRY(cudaMemsetAsync(yp, 0, esz * (size_t)p.Np, s));
-    unsigned blocks = cdiv(g.N, 256);
-    if (precision == PB_MIXED) {
-        k_canon_to_pad<float><<<blocks, 256, 0, s>>>((const float *)x, (float *)xp, g, p);
-        if (ensure_queue(sys, s) != PB_OK) return PB_ERR_OOM;
-        // a one-entry table of its own (the solver's entry may be in use)
-        tma::SysEntry *e = new (std::nothrow) tma::SysEntry();
-        if (!e) return PB_ERR_OOM;
-        pb_status rc =
-            tma_maps(sys, MODE_A, (const float *)xp, nullptr, nullptr, nullptr, &e->A, tma::TWDEF);
-        if (rc == PB_OK) rc = tma_prepare<MODE_A>();
-        if (rc != PB_OK) {
-            delete e;
-            return rc;
-        }
-        e->pg = p;
-        e->cp = make_c32(sys);
-        e->y = (float *)yp;
-        tma_entry_geometry(*e, p, 8, tma::TWDEF);
-        tma::SysEntry *de = (tma::SysEntry *)dalloc(sizeof(tma::SysEntry), s);
-        if (!de) {
-            delete e;
-            return PB_ERR_OOM;
-        }
-        cudaError_t ce = cudaMemcpyAsync(de, e, sizeof(tma::SysEntry), cudaMemcpyHostToDevice, s);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-        const int nitems = e->nitems;
-        if (ce != cudaSuccess) {
-            delete e;
-            set_error("apply table upload: %s", cudaGetErrorString(ce));
-            return PB_ERR_CUDA;
-        }
-        tma_launch<MODE_A>(de, 1, nitems, sys->queue, tma_grid(p, 8), s, e);
-        delete e;
-        PB_LAUNCH_CHECK();
-        dfree(de, s);
-        k_pad_to_canon<float><<<blocks, 256, 0, s>>>((const float *)yp, (float *)y, g, p);
-    } else {
-        k_canon_to_pad<double><<<blocks, 256, 0, s>>>((const double *)x, (double *)xp, g, p);
-        KArgs<double> a{};
-        a.in = (const double *)xp;
-        a.out = (double *)yp;
-        a.code = sys->code;
-        a.pg = p;
-        a.KC = KC;
-        k_stencil<double, CoefS64, MODE_A, TYC, MinB<double>::v><<<stencil_grid<double>(p, KC), 32 * TYC, 0, s>>>(
-            a, make_s64(sys));
-        k_pad_to_canon<double><<<blocks, 256, 0, s>>>((const double *)yp, (double *)y, g, p);
+    // x and y may share memory: the kernel reads neighbours of what it writes
+    const size_t bytes = (precision == PB_MIXED ? 4 : 8) * (size_t)g.N;
+    void *copy = nullptr;
+    if ((const char *)x < (const char *)y + bytes && (const char *)y < (const char *)x + bytes) {
+        copy = dalloc(bytes, s);
+        if (!copy) return PB_ERR_OOM;
+        PB_CUDA_TRY(cudaMemcpyAsync(copy, x, bytes, cudaMemcpyDeviceToDevice, s));
+        x = copy;
     }
-    note_launch(2);
+    constexpr int PTS = 4;
+    const unsigned cols = cdiv((long long)g.nx * g.ny, 256 * PTS);
+    // up to 16 planes a block, fewer where that leaves less than eight blocks an SM
+    const int KC = (int)std::max(1ll, std::min(16ll, (long long)cols * g.nz / (8ll * num_sms())));
+    const dim3 grid(cols, cdiv(g.nz, KC));
+    if (precision == PB_MIXED)
+        k_apply<float, CoefC32, PTS><<<grid, 256, 0, s>>>((const float *)x, (float *)y, sys->code, g, sys->pad.sx,
+                                                          make_c32(sys), KC);
+    else
+        k_apply<double, CoefS64, PTS><<<grid, 256, 0, s>>>((const double *)x, (double *)y, sys->code, g, sys->pad.sx,
+                                                           make_s64(sys), KC);
     PB_LAUNCH_CHECK();
-    dfree(xp, s);
-    dfree(yp, s);
+    dfree(copy, s);
     return PB_OK;
 }
 

@@ -194,7 +194,6 @@ pb_status slab_build(const pb_system *sys, Slab &sl, int k0, int k1, int KC, int
     e.pbuf[1] = sl.pbuf[1];
     e.x = sl.d;
     e.z = sl.z;
-    e.y = nullptr;
     e.st = sl.st;
     e.partials = sl.tpart;
     e.cnt = nullptr;

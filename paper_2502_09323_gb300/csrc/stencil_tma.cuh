@@ -103,21 +103,13 @@ struct SlotLayout<1, FIXW> {
     static constexpr int stride = align128(code + code_region(FIXW));
     __device__ static unsigned tx(int tw) { return box_bytes(tw) + 2 * OWN_BYTES + code_bytes(tw); }
 };
-// apply: x box + codes
-template <int FIXW>
-struct SlotLayout<2, FIXW> {
-    static constexpr int a = 0, b = -1, x = -1, z = -1, code = align128(box_region(FIXW));
-    static constexpr int stride = align128(code + code_region(FIXW));
-    __device__ static unsigned tx(int tw) { return box_bytes(tw) + code_bytes(tw); }
-};
-
 template <int MODE, int FIXW>
 constexpr int smem_bytes() {
     return NSLOT * SlotLayout<MODE, FIXW>::stride + 2 * NSLOT * 8;
 }
 
 struct Maps {  // boxes of the system's tile width TW (TH = 1024 / TW)
-    CUtensorMap a;      // streamed vector, (TW + 8) x (TH + 2) box (P: z, U: p, A: x)
+    CUtensorMap a;      // streamed vector, (TW + 8) x (TH + 2) box (P: z, U: p)
     CUtensorMap b;      // P: p_old, same box
     CUtensorMap x;      // U: x, TW x TH box
     CUtensorMap z;      // U: z, TW x TH box
@@ -128,12 +120,10 @@ struct Maps {  // boxes of the system's tile width TW (TH = 1024 / TW)
 struct SysEntry {  // aligned as CUtensorMap
     Maps P[2];          // direction kernel, p_old = pa (parity 0) / pb (1)
     Maps U[2];          // update kernel, p = pb (parity 0) / pa (1)
-    Maps A;             // apply
     PadGeo pg;
     CoefC32 cp;
     float *pbuf[2];     // pa, pb
     float *x, *z;       // solution increment, preconditioned residual
-    float *y;           // apply output
     CgState *st;
     float *partials;    // per tile column and group of G planes, slot i: sigma at
                         // [i], rho and rr at [npart + 2 i] and [npart + 2 i + 1]
@@ -238,7 +228,7 @@ __device__ __forceinline__ void warp_nsum(float &s, float &c) {
 
 }  // namespace tma
 
-// MODE_P / MODE_U / MODE_A on the compressed FP32 operator, over every
+// MODE_P / MODE_U on the compressed FP32 operator, over every
 // system of tab (item_base ascending; total_items = sum of nitems).  With
 // nsys < 0 the table size and item total are read from queue[2] and
 // queue[3], so a captured launch follows a table that changes between
@@ -291,7 +281,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
     // gives up sets it, so blocks that start later may see it set while
     // earlier ones took items; every block is still counted at the exit.
     if (threadIdx.x == 0) {
-        s_skip = SINGLE && MODE != MODE_A && *(volatile int *)&e0.st->done;
+        s_skip = SINGLE && *(volatile int *)&e0.st->done;
         s_nsys = nsys < 0 ? (int)((volatile unsigned int *)queue)[2] : nsys;
         s_total = nsys < 0 ? (int)((volatile unsigned int *)queue)[3] : total_items;
     }
@@ -338,15 +328,13 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                         sys = lo;
                         e = tab + sys;
                     }
-                    if (MODE != MODE_A) {
-                        if (sys != csys) {
-                            cdone = *(volatile int *)&e->st->done;
-                            ccur = *(volatile int *)&e->st->cur;
-                            csys = sys;
-                        }
-                        if (cdone) continue;  // converged
-                        cur = ccur;
+                    if (sys != csys) {
+                        cdone = *(volatile int *)&e->st->done;
+                        ccur = *(volatile int *)&e->st->cur;
+                        csys = sys;
                     }
+                    if (cdone) continue;  // converged
+                    cur = ccur;
                     const int ci = it - e->item_base;
                     const int col = ci / e->nchunk, c = ci - col * e->nchunk;
                     li = col * e->nG + c * e->KC / e->G;
@@ -356,7 +344,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                     i0 = (col % e->xtiles) * tw;
                     j0 = 1 + (col / e->xtiles) * tile_h(tw);
                 }
-                const Maps *m = MODE == MODE_P ? &e->P[cur] : (MODE == MODE_U ? &e->U[cur] : &e->A);
+                const Maps *m = MODE == MODE_P ? &e->P[cur] : &e->U[cur];
                 const int nplanes = end ? 1 : len + 2;
                 bool stop = false;
                 for (int t = 0; t < nplanes; ++t, ++gt) {
@@ -470,7 +458,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
         PadGeo g{};
         CoefC32 cp{};
         float alpha = 0.f, dg_in = 0.f, dg_out = 0.f, dinv_in = 0.f, dinv_out = 0.f;
-        float *pb0 = nullptr, *pb1 = nullptr, *yg = nullptr, *xg = nullptr, *zg = nullptr;
+        float *pb0 = nullptr, *pb1 = nullptr, *xg = nullptr, *zg = nullptr;
         if constexpr (SINGLE) {
             g = e0.pg;
             cp = e0.cp;
@@ -482,7 +470,6 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
             dinv_out = 1.f / dg_out;
             pb0 = e0.pbuf[0];
             pb1 = e0.pbuf[1];
-            yg = e0.y;
             xg = e0.x;
             zg = e0.z;
             set_tile(e0.tw);
@@ -531,13 +518,12 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                 dinv_out = 1.f / dg_out;
                 pb0 = e->pbuf[0];
                 pb1 = e->pbuf[1];
-                yg = e->y;
                 xg = e->x;
                 zg = e->z;
                 set_tile(e->tw);
                 ksys = sys;
             }
-            float *const outp = MODE == MODE_P ? (cur ? pb0 : pb1) : (MODE == MODE_A ? yg : nullptr);
+            float *const outp = cur ? pb0 : pb1;  // direction kernel
             const int j = j0 + r - 1;
             const int ib = i0 + xl * 4;
             const bool active = j <= g.ny - 2;
@@ -642,7 +628,6 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                     wxm[2] = wxp[1];
                     wxm[3] = wxp[2];
                 }
-                float y[4];
                 if (fast) {
                     // packed: points (0,1) and (2,3) of this lane
 #pragma unroll
@@ -666,7 +651,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                             // x is zero on boundary nodes, padding and absent rows
                             const float2 c = __fmul2_rn(x, ap);
                             acc0 += c.x + c.y;
-                        } else if (MODE == MODE_U) {
+                        } else {
                             const float2 dinv = f2((ca & 1) ? dinv_in : dinv_out, (cb & 1) ? dinv_in : dinv_out);
                             const float2 dg = f2((ca & 1) ? dg_in : dg_out, (cb & 1) ? dg_in : dg_out);
                             const float2 xn = __ffma2_rn(f2(alpha, alpha), x, f2(xv[q0], xv[q0 + 1]));
@@ -682,9 +667,6 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                             xv[q0 + 1] = xn.y;
                             zv[q0] = zn.x;
                             zv[q0 + 1] = zn.y;
-                        } else {
-                            y[q0] = ia ? ap.x : 0.f;
-                            y[q0 + 1] = ib2 ? ap.y : 0.f;
                         }
                     }
                 } else {
@@ -715,7 +697,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                             const float2 c = __fmul2_rn(x, ap);
                             if (ia) acc0 += c.x;
                             if (ib2) acc0 += c.y;
-                        } else if (MODE == MODE_U) {
+                        } else {
                             const float2 dg = __fadd2_rn(
                                 __fadd2_rn(__fadd2_rn(__fadd2_rn(__fadd2_rn(__fadd2_rn(w0, w1), w2), w3), w4), w5),
                                 kp);
@@ -738,9 +720,6 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                                 acc0 += c0.y;
                                 acc1 += c1.y;
                             }
-                        } else {
-                            y[q0] = ia ? ap.x : 0.f;
-                            y[q0 + 1] = ib2 ? ap.y : 0.f;
                         }
                     }
                 }
@@ -753,8 +732,6 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                         *reinterpret_cast<float4 *>(xg + base + ib) = make_float4(xv[0], xv[1], xv[2], xv[3]);
                         *reinterpret_cast<float4 *>(zg + base + ib) = make_float4(zv[0], zv[1], zv[2], zv[3]);
                     }
-                    if (MODE == MODE_A)
-                        *reinterpret_cast<float4 *>(outp + base + ib) = make_float4(y[0], y[1], y[2], y[3]);
                 }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -772,7 +749,6 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                 // items, own the partials, so the sums do not depend on the
                 // z-chunk as long as it is a multiple of the group.
                 // (FP32 across the warp: the FP64 pipe of this part is narrow)
-                if (MODE == MODE_A) continue;
                 if (left_in_group == 0) left_in_group = e->G;
                 if (--left_in_group > 0 && t < len) continue;
                 left_in_group = 0;
@@ -811,7 +787,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
     __threadfence();
     __syncthreads();
     // a device-side wait gave up: stop every system of the table
-    if (s_abort && threadIdx.x == 0 && MODE != MODE_A) {
+    if (s_abort && threadIdx.x == 0) {
         for (int q = 0; q < nsys; ++q) {
             atomicExch(&tab[q].st->status, 3);
             atomicExch(&tab[q].st->done, 1);
@@ -827,109 +803,107 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
     __syncthreads();
     if (!s_lastblk) return;
     __threadfence();
-    if (MODE != MODE_A) {
-        // Each system's item partials are summed in an order fixed by its
-        // item count only: systems of more than BIGSYS items by the whole
-        // block (thread t takes items t, t+NTHREADS, ...), smaller ones by
-        // one warp each.  The sums are compensated FP32 up to the warps'
-        // totals (this block runs alone at the end of the launch, on the
-        // critical path, and FP64 is a narrow pipe of GB300) and FP64 after.
-        constexpr int BIGSYS = 512;
-        __shared__ double s_red[2][NTHREADS / 32];
-        auto finish = [&](CgState *st, double t0, double t1) {
-            if (st->split) {
-                // one slab of a split solve: its totals only
-                st->part0 = t0;
-                st->part1 = t1;
-                return;
-            }
-            if (MODE == MODE_P) {
-                st->sigma = t0;
-                if (st->status == 3) {
-                    st->done = 1;
-                } else if (st->profile) {
-                    st->alpha = isfinite(t0) && t0 != 0.0 ? st->rho / t0 : 0.0;
-                } else if (!(t0 > 0.0) || !isfinite(t0)) {
-                    st->done = 1;
-                    st->status = 1;
-                } else {
-                    st->alpha = st->rho / t0;
-                }
+    // Each system's item partials are summed in an order fixed by its
+    // item count only: systems of more than BIGSYS items by the whole
+    // block (thread t takes items t, t+NTHREADS, ...), smaller ones by
+    // one warp each.  The sums are compensated FP32 up to the warps'
+    // totals (this block runs alone at the end of the launch, on the
+    // critical path, and FP64 is a narrow pipe of GB300) and FP64 after.
+    constexpr int BIGSYS = 512;
+    __shared__ double s_red[2][NTHREADS / 32];
+    auto finish = [&](CgState *st, double t0, double t1) {
+        if (st->split) {
+            // one slab of a split solve: its totals only
+            st->part0 = t0;
+            st->part1 = t1;
+            return;
+        }
+        if (MODE == MODE_P) {
+            st->sigma = t0;
+            if (st->status == 3) {
+                st->done = 1;
+            } else if (st->profile) {
+                st->alpha = isfinite(t0) && t0 != 0.0 ? st->rho / t0 : 0.0;
+            } else if (!(t0 > 0.0) || !isfinite(t0)) {
+                st->done = 1;
+                st->status = 1;
             } else {
-                if (!st->mg) {  // else the multigrid cycle sets them
-                    st->beta = t0 / st->rho;
-                    st->rho = t0;
-                }
-                st->rr = t1;
-                st->iter += 1;
-                st->cur ^= 1;  // the new p_old is this iteration's p
-                if (st->status == 3) {
-                    st->done = 1;
-                } else if (st->profile) {
-                    // timing run: keep going
-                } else if (!isfinite(t1)) {
-                    st->done = 1;
-                    st->status = 1;
-                } else if (t1 <= st->rr_stop) {
-                    st->done = 1;
-                    st->status = 0;
-                } else if (st->iter >= st->max_iter) {
-                    st->done = 1;
-                    st->status = 2;
-                }
+                st->alpha = st->rho / t0;
             }
-        };
-        // the warp's items summed; the totals are valid in lane 0
-        auto item_sums = [&](const SysEntry *e, int first, int stride, double &t0, double &t1) {
-            const int nit = e->npart;
-            float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
+        } else {
+            if (!st->mg) {  // else the multigrid cycle sets them
+                st->beta = t0 / st->rho;
+                st->rho = t0;
+            }
+            st->rr = t1;
+            st->iter += 1;
+            st->cur ^= 1;  // the new p_old is this iteration's p
+            if (st->status == 3) {
+                st->done = 1;
+            } else if (st->profile) {
+                // timing run: keep going
+            } else if (!isfinite(t1)) {
+                st->done = 1;
+                st->status = 1;
+            } else if (t1 <= st->rr_stop) {
+                st->done = 1;
+                st->status = 0;
+            } else if (st->iter >= st->max_iter) {
+                st->done = 1;
+                st->status = 2;
+            }
+        }
+    };
+    // the warp's items summed; the totals are valid in lane 0
+    auto item_sums = [&](const SysEntry *e, int first, int stride, double &t0, double &t1) {
+        const int nit = e->npart;
+        float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
 #pragma unroll 4
-            for (int i = first; i < nit; i += stride) {
-                if (MODE == MODE_P) {
-                    nsum(s0, c0, __ldcg(e->partials + i));
-                } else {
-                    nsum(s0, c0, __ldcg(e->partials + nit + 2 * i));
-                    nsum(s1, c1, __ldcg(e->partials + nit + 2 * i + 1));
-                }
+        for (int i = first; i < nit; i += stride) {
+            if (MODE == MODE_P) {
+                nsum(s0, c0, __ldcg(e->partials + i));
+            } else {
+                nsum(s0, c0, __ldcg(e->partials + nit + 2 * i));
+                nsum(s1, c1, __ldcg(e->partials + nit + 2 * i + 1));
             }
-            warp_nsum(s0, c0);
-            if (MODE != MODE_P) warp_nsum(s1, c1);
-            t0 = (double)s0 + (double)c0;
-            t1 = (double)s1 + (double)c1;
-        };
-        // large systems: the whole block, one after the other
-        for (int q = 0; q < nsys; ++q) {
-            const SysEntry *e = tab + q;
-            const int nit = e->npart;
-            if (nit <= BIGSYS || *(volatile int *)&e->st->done) continue;
-            double t0, t1;
-            item_sums(e, threadIdx.x, NTHREADS, t0, t1);
-            if (lane == 0) {
-                s_red[0][w] = t0;
-                s_red[1][w] = t1;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double u0 = 0.0, u1 = 0.0;
-                for (int r = 0; r < NTHREADS / 32; ++r) {
-                    u0 += s_red[0][r];
-                    u1 += s_red[1][r];
-                }
-                finish(e->st, u0, u1);
-            }
-            __syncthreads();
         }
-        // small systems: one warp each
-        for (int q = w; q < nsys; q += NTHREADS / 32) {
-            const SysEntry *e = tab + q;
-            const int nit = e->npart;
-            CgState *st = e->st;
-            // systems that were done at launch (or stopped by an abort) have no partials
-            if (nit == 0 || nit > BIGSYS || *(volatile int *)&st->done) continue;
-            double t0, t1;
-            item_sums(e, lane, 32, t0, t1);
-            if (lane == 0) finish(st, t0, t1);
+        warp_nsum(s0, c0);
+        if (MODE != MODE_P) warp_nsum(s1, c1);
+        t0 = (double)s0 + (double)c0;
+        t1 = (double)s1 + (double)c1;
+    };
+    // large systems: the whole block, one after the other
+    for (int q = 0; q < nsys; ++q) {
+        const SysEntry *e = tab + q;
+        const int nit = e->npart;
+        if (nit <= BIGSYS || *(volatile int *)&e->st->done) continue;
+        double t0, t1;
+        item_sums(e, threadIdx.x, NTHREADS, t0, t1);
+        if (lane == 0) {
+            s_red[0][w] = t0;
+            s_red[1][w] = t1;
         }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double u0 = 0.0, u1 = 0.0;
+            for (int r = 0; r < NTHREADS / 32; ++r) {
+                u0 += s_red[0][r];
+                u1 += s_red[1][r];
+            }
+            finish(e->st, u0, u1);
+        }
+        __syncthreads();
+    }
+    // small systems: one warp each
+    for (int q = w; q < nsys; q += NTHREADS / 32) {
+        const SysEntry *e = tab + q;
+        const int nit = e->npart;
+        CgState *st = e->st;
+        // systems that were done at launch (or stopped by an abort) have no partials
+        if (nit == 0 || nit > BIGSYS || *(volatile int *)&st->done) continue;
+        double t0, t1;
+        item_sums(e, lane, 32, t0, t1);
+        if (lane == 0) finish(st, t0, t1);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
