@@ -132,7 +132,9 @@ typedef struct {
     int32_t bc;
 } pb_params;
 
-/* Solver options.  precision PB_FP64: Jacobi-PCG entirely in FP64.
+/* Solver options.  precision PB_FP64: PCG entirely in FP64 (preconditioned by
+ * an FP64 multigrid V-cycle where PB_MIXED has one on uniform grids, else by
+ * the diagonal).
  * PB_MIXED: FP64 iterative refinement around an FP32 PCG (FP32 stencil,
  * vectors and per-thread accumulation, FP64 global dots), preconditioned by
  * one multigrid V-cycle on uniform grids of at least 9 nodes an axis, by a

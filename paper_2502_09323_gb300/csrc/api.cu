@@ -303,6 +303,7 @@ void pb_system_free(pb_system *s) {
     cudaStreamSynchronize(st);
     free_tma_state(s);
     free_mg_state(s);
+    free_mg64_state(s);
     if (s->h_st) cudaFreeHost(s->h_st);
     if (s->h_energy) cudaFreeHost(s->h_energy);
     delete s;

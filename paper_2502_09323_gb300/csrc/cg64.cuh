@@ -1,11 +1,13 @@
-// Plain FP64 Jacobi-PCG kernels (included by solve.cu inside its anonymous
+// Plain FP64 PCG kernels (included by solve.cu inside its anonymous
 // namespace; needs CgState, PadGeo and last_block_total from there).
 //
-// The textbook preconditioned CG (Sec. 4) with the Jacobi preconditioner,
-// every vector and every operation in FP64, one solve at a time:
+// The textbook preconditioned CG (Sec. 4), every vector and every operation in
+// FP64, one solve at a time.  With the Jacobi preconditioner:
 //   kernel D:  p = z + beta p_old ;  q = A p ;  sigma = p.q       -> alpha = rho / sigma
 //   kernel U:  x += alpha p ;  r -= alpha q ;  z = D^-1 r ;
 //              rho' = r.z ;  rr = r.r                            -> beta = rho' / rho
+// With the multigrid preconditioner (FP64 too, mg.cuh) a cycle between U and D
+// turns z into the preconditioned residual and sets beta.
 // GB300's FP64 pipe (about 1/64 of the FP32 rate) binds before HBM does, so
 // the schedule keeps FP64 operations per unknown and iteration low: the
 // operator is applied once per iteration (q is stored), and the diagonal
@@ -238,8 +240,10 @@ __global__ void __launch_bounds__(cg64::UNT, 4) k_cg64_upd(cg64::UpdArgs A) {
     if (last_block_total<UNT, true>(A.st, A.partials, nb, rho, rr, sred, t0, t1)) {
         if (threadIdx.x == 0) {
             CgState *s = A.st;
-            s->beta = t0 / s->rho;
-            s->rho = t0;
+            if (!s->mg) {  // else the multigrid cycle sets them
+                s->beta = t0 / s->rho;
+                s->rho = t0;
+            }
             s->rr = t1;
             s->iter += 1;
             if (s->profile) {

@@ -263,7 +263,8 @@ bool engine_capture(Engine *e) {
             else
                 k_mg_down<false, false><<<rd1, mg::DNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
         if (depth > 0)
-            k_mg_bottom<false><<<e->cap, mg::BOT_T, mg::BOT_BYTES * mg::BOT_NODES, e->cs>>>(e->dmg, e->dhead, none);
+            k_mg_bottom<mg::Entry, false>
+                <<<e->cap, mg::BOT_T, mg::BOT_BYTES<float> * mg::BOT_NODES<float>, e->cs>>>(e->dmg, e->dhead, none);
         for (int l = depth - 1; l >= 0; --l)
             if (l == 0)
                 k_mg_up<true, false><<<ru0, mg::UNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);

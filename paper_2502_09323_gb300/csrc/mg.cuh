@@ -41,8 +41,14 @@ namespace mg {
 constexpr int LMAX = 12;            // levels at most
 constexpr float OMEGA = 0.85f;      // Jacobi damping (0.8 to 0.9 take the same iterations)
 constexpr int BOT_T = 1024;         // threads of the bottom kernel
-constexpr int BOT_BYTES = 34;       // shared memory of one of its nodes
-constexpr int BOT_NODES = 6600;     // nodes of all its levels
+// shared memory of a node of the bottom kernel: the blob's four coefficients
+// and three lists, and three vectors; nodes of all its levels at most
+template <typename T>
+constexpr int BLOB_BYTES = 4 * sizeof(T) + 6;
+template <typename T>
+constexpr int BOT_BYTES = 7 * sizeof(T) + 6;
+template <typename T>
+constexpr int BOT_NODES = sizeof(T) == 4 ? 6600 : 3600;
 constexpr int SWEEPS = 8;           // Jacobi sweeps on the coarsest level
 // Tiles.  Down: 32 x 6 coarse nodes from node (1 + 32 bx, 1 + 6 by), whose
 // residuals are 13 rows of 17 units of 4 fine nodes; the first and the last
@@ -53,14 +59,18 @@ constexpr int CX = 32, CY = 6, DU = 17, DR = 2 * CY + 1, DNT = 256;
 constexpr int FX = 64, FY = 16, UU = 16, UNT = 16 * (FY + 2);
 constexpr int RG = 4;               // planes of one partial of rho
 
-struct Lev {
-    int nx, ny, nz, sx, sxy;        // sx a multiple of 4 above the bottom kernel's levels, nx there
-    float *s, *z;                   // D^-1 b, solution (level 0: the solver's z32 and v32)
-    float *wx, *wy, *wz, *dg;       // weights of the +x, +y, +z edges, diagonal (levels >= 1)
+template <typename T>
+struct LevT {
+    int nx, ny, nz, sx, sxy;    // sx a multiple of 4 above the bottom kernel's levels, nx there
+    T *s, *z;                   // D^-1 b, solution (level 0: the solver's s and v)
+    T *wx, *wy, *wz, *dg;       // weights of the +x, +y, +z edges, diagonal (levels >= 1)
+    T *di, *r;                  // FP64 cycle: 1 / diagonal, work vector
 };
+using Lev = LevT<float>;
 
 // One system (device memory, or the kernel parameter of a one-system launch)
 struct Entry {
+    using T = float;
     Lev lev[LMAX];
     int nlev, nbot;                 // levels; first level of the bottom kernel
     int dbase[LMAX], ubase[LMAX];   // first work item of this system in a level's launches
@@ -92,6 +102,9 @@ __host__ __device__ inline int uitems(const Entry &e, int l) {
     const Lev &f = e.lev[l];
     return ((f.nx - 1 + FX - 1) / FX) * ((f.ny - 2 + FY - 1) / FY) * ((f.nz - 2 + e.uk[l] - 1) / e.uk[l]);
 }
+
+__device__ __forceinline__ float quotient(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ double quotient(double a, double b) { return a / b; }
 
 __device__ __forceinline__ float4 f4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
@@ -175,7 +188,8 @@ __device__ __forceinline__ void face_sums(const Entry &, const Lev &, int, const
     d[3] = o.d.w;
 }
 
-__device__ __forceinline__ bool interior(const Lev &L, int i, int j, int k) {
+template <typename T>
+__device__ __forceinline__ bool interior(const LevT<T> &L, int i, int j, int k) {
     return i >= 1 && j >= 1 && k >= 1 && i <= L.nx - 2 && j <= L.ny - 2 && k <= L.nz - 2;
 }
 
@@ -502,13 +516,15 @@ k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, i
 // unpadded, the weights and the diagonal (arrays of T values); for every
 // interior node, its place in its level, its parent (the coarse node below it
 // and the three parities) and, on coarse levels, its fine node.
-__global__ void k_mg_pack(const __grid_constant__ mg::Entry e, int T) {
+template <class E>
+__global__ void k_mg_pack(const __grid_constant__ E e, int T) {
     using namespace mg;
-    float *W = reinterpret_cast<float *>(e.blob);
+    using F = typename E::T;
+    F *W = reinterpret_cast<F *>(e.blob);
     uint16_t *list = reinterpret_cast<uint16_t *>(W + 4 * T), *up = list + T, *dn = up + T;
     int off = 0;
     for (int l = e.nbot; l < e.nlev; ++l) {
-        const Lev &L = e.lev[l];
+        const auto &L = e.lev[l];
         const int n = L.nx * L.ny * L.nz, mx = L.nx - 2, my = L.ny - 2;
         const int cx = L.nx / 2 + 1, cxy = cx * (L.ny / 2 + 1);
         const int fx = l > e.nbot ? e.lev[l - 1].nx : 0, fxy = l > e.nbot ? fx * e.lev[l - 1].ny : 0;
@@ -534,31 +550,33 @@ __global__ void k_mg_pack(const __grid_constant__ mg::Entry e, int T) {
 // works here, and what it does serially counts: the coefficients and node lists come in
 // one asynchronous copy, before the previous kernel has ended (one-system
 // launches).
-template <bool SINGLE>
+template <class E, bool SINGLE>
 __global__ void __launch_bounds__(mg::BOT_T, 1)
-k_mg_bottom(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head,
-            const __grid_constant__ mg::Entry e0) {
+k_mg_bottom(const E *__restrict__ tab, const mg::Head *__restrict__ head,
+            const __grid_constant__ E e0) {
     using namespace mg;
-    extern __shared__ __align__(16) float bsm[];
+    using F = typename E::T;
+    constexpr F OM = OMEGA;
+    extern __shared__ __align__(16) char bsm[];
     const int tid = threadIdx.x;
     if (!SINGLE) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         if ((int)blockIdx.x >= head->nsys) return;
     }
-    const Entry &e = SINGLE ? e0 : tab[blockIdx.x];
+    const E &e = SINGLE ? e0 : tab[blockIdx.x];
     const int lb = e.nbot, le = e.nlev, T = e.bot;
     if (le == 0) return;
     if (!SINGLE && *(volatile int *)&e.st->done) return;
-    const float *Wx = bsm, *Wy = Wx + T, *Wz = Wy + T, *D = Wz + T;
+    const F *Wx = reinterpret_cast<const F *>(bsm), *Wy = Wx + T, *Wz = Wy + T, *D = Wz + T;
     const uint16_t *list = reinterpret_cast<const uint16_t *>(D + T), *up = list + T, *dn = up + T;
-    float *S = bsm + 22 * T / 4, *Z = S + T, *R = Z + T;
-    // T is a multiple of 8, so the 22 T bytes are whole 16-byte pieces
-    for (int q = tid; q < 22 * T / 16; q += BOT_T)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tma::smem_u32(reinterpret_cast<char *>(bsm) + 16 * q)),
+    F *S = reinterpret_cast<F *>(bsm + BLOB_BYTES<F> * T), *Z = S + T, *R = Z + T;
+    // T is a multiple of 8, so the blob is whole 16-byte pieces
+    for (int q = tid; q < BLOB_BYTES<F> * T / 16; q += BOT_T)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tma::smem_u32(bsm + 16 * q)),
                      "l"(reinterpret_cast<const char *>(e.blob) + 16 * q)
                      : "memory");
     asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int q = tid; q < 3 * T; q += BOT_T) S[q] = 0.f;
+    for (int q = tid; q < 3 * T; q += BOT_T) S[q] = 0;
     if (SINGLE) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -568,61 +586,61 @@ k_mg_bottom(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head
     if (skip) return;
     __syncthreads();
     {
-        const Lev &L = e.lev[lb];
+        const auto &L = e.lev[lb];
         const int n = L.nx * L.ny * L.nz;
 #pragma unroll 8
         for (int p = tid; p < n; p += BOT_T) S[p] = L.s[p];
     }
     __syncthreads();
     // sum over the faces of node p of the level whose nodes start at o
-    auto faces = [&](int o, int sx, int sxy, const float *x, int p) {
-        const float *a = Wx + o, *b = Wy + o, *c = Wz + o;
+    auto faces = [&](int o, int sx, int sxy, const F *x, int p) {
+        const F *a = Wx + o, *b = Wy + o, *c = Wz + o;
         return ((a[p - 1] * x[p - 1] + a[p] * x[p + 1]) + (b[p - sx] * x[p - sx] + b[p] * x[p + sx])) +
                (c[p - sxy] * x[p - sxy] + c[p] * x[p + sxy]);
     };
     int o = 0;
     for (int l = lb; l < le - 1; ++l) {
-        const Lev &L = e.lev[l], &C = e.lev[l + 1];
+        const auto &L = e.lev[l], &C = e.lev[l + 1];
         const int sx = L.nx, sxy = L.nx * L.ny, n = (L.nx - 2) * (L.ny - 2) * (L.nz - 2);
         const int oc = o + sxy * L.nz, nc = (C.nx - 2) * (C.ny - 2) * (C.nz - 2);
         for (int t = tid; t < n; t += BOT_T) {
             const int p = list[o + t];
-            R[o + p] = (1.f - OMEGA) * D[o + p] * S[o + p] + OMEGA * faces(o, sx, sxy, S + o, p);
+            R[o + p] = ((F)1 - OM) * D[o + p] * S[o + p] + OM * faces(o, sx, sxy, S + o, p);
         }
         __syncthreads();
         for (int t = tid; t < nc; t += BOT_T) {
             const int pc = list[oc + t];
-            const float *f = R + o + dn[oc + t];
-            float acc = 0.f;
+            const F *f = R + o + dn[oc + t];
+            F acc = 0.f;
 #pragma unroll
             for (int c = -1; c <= 1; ++c)
 #pragma unroll
                 for (int b = -1; b <= 1; ++b) {
-                    const float *x = f + c * sxy + b * sx;
-                    acc += (b ? 0.5f : 1.f) * (c ? 0.5f : 1.f) * (x[0] + 0.5f * (x[-1] + x[1]));
+                    const F *x = f + c * sxy + b * sx;
+                    acc += (b ? (F)0.5 : (F)1) * (c ? (F)0.5 : (F)1) * (x[0] + (F)0.5 * (x[-1] + x[1]));
                 }
-            S[oc + pc] = __fdividef(acc, D[oc + pc]);
+            S[oc + pc] = quotient(acc, D[oc + pc]);
         }
         __syncthreads();
         o = oc;
     }
     {
-        const Lev &L = e.lev[le - 1];
+        const auto &L = e.lev[le - 1];
         const int sx = L.nx, sxy = L.nx * L.ny, n = (L.nx - 2) * (L.ny - 2) * (L.nz - 2);
         if (n == 1) {  // one unknown: its solution
             if (tid == 0) Z[o + list[o]] = S[o + list[o]];
         } else {
-            float *a = Z + o, *b = R + o;
-            for (int t = tid; t < n; t += BOT_T) a[list[o + t]] = OMEGA * S[o + list[o + t]];
+            F *a = Z + o, *b = R + o;
+            for (int t = tid; t < n; t += BOT_T) a[list[o + t]] = OM * S[o + list[o + t]];
             __syncthreads();
             for (int q = 1; q < SWEEPS; ++q) {
                 for (int t = tid; t < n; t += BOT_T) {
                     const int p = list[o + t];
-                    b[p] = (1.f - OMEGA) * a[p] +
-                           OMEGA * (S[o + p] + __fdividef(faces(o, sx, sxy, a, p), D[o + p]));
+                    b[p] = ((F)1 - OM) * a[p] +
+                           OM * (S[o + p] + quotient(faces(o, sx, sxy, a, p), D[o + p]));
                 }
                 __syncthreads();
-                float *t = a;
+                F *t = a;
                 a = b;
                 b = t;
             }
@@ -632,94 +650,199 @@ k_mg_bottom(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head
         __syncthreads();
     }
     for (int l = le - 2; l >= lb; --l) {
-        const Lev &L = e.lev[l], &C = e.lev[l + 1];
+        const auto &L = e.lev[l], &C = e.lev[l + 1];
         const int sx = L.nx, sxy = L.nx * L.ny, n = (L.nx - 2) * (L.ny - 2) * (L.nz - 2);
         const int cx = C.nx, cxy = C.nx * C.ny, oc = o;
         o -= sxy * L.nz;
         for (int t = tid; t < n; t += BOT_T) {
             const int p = list[o + t], c = up[o + t];
-            const float *x = Z + oc + (c >> 3);
+            const F *x = Z + oc + (c >> 3);
             const int di = c & 1, dj = (c & 2) ? cx : 0, dk = (c & 4) ? cxy : 0;
-            const float acc = ((x[0] + x[di]) + (x[dj] + x[dj + di])) + ((x[dk] + x[dk + di]) + (x[dk + dj] + x[dk + dj + di]));
-            R[o + p] = OMEGA * S[o + p] + 0.125f * acc;
+            const F acc = ((x[0] + x[di]) + (x[dj] + x[dj + di])) + ((x[dk] + x[dk + di]) + (x[dk + dj] + x[dk + dj + di]));
+            R[o + p] = OM * S[o + p] + (F)0.125 * acc;
         }
         __syncthreads();
         for (int t = tid; t < n; t += BOT_T) {
             const int p = list[o + t];
-            const float z = (1.f - OMEGA) * R[o + p] +
-                            OMEGA * (S[o + p] + __fdividef(faces(o, sx, sxy, R + o, p), D[o + p]));
+            const F z = ((F)1 - OM) * R[o + p] +
+                            OM * (S[o + p] + quotient(faces(o, sx, sxy, R + o, p), D[o + p]));
             Z[o + p] = z;
         }
         __syncthreads();
     }
-    const Lev &L = e.lev[lb];
+    const auto &L = e.lev[lb];
     for (int p = tid; p < L.nx * L.ny * L.nz; p += BOT_T) L.z[p] = Z[p];
 }
 
 // Edge weights and ionic term (kept in z while the hierarchy is built) of a
 // coarse level: from the FP64 weights and the code bytes of level 0, or
 // from a coarse level.
-template <bool FINE>
-__global__ void k_mg_coarsen(mg::Lev F, mg::Lev C, const double *__restrict__ Wx, const double *__restrict__ Wy,
-                             const double *__restrict__ Wz, const uint8_t *__restrict__ code, float kap0) {
+template <bool FINE, typename T>
+__global__ void k_mg_coarsen(mg::LevT<T> F, mg::LevT<T> C, const double *__restrict__ Wx, const double *__restrict__ Wy,
+                             const double *__restrict__ Wz, const uint8_t *__restrict__ code, T kap0) {
     const int t = blockIdx.x * 256 + threadIdx.x;
     if (t >= C.nx * C.ny * C.nz) return;
     const int I = t % C.nx, J = (t / C.nx) % C.ny, K = t / (C.nx * C.ny);
     const int n[3] = {F.nx, F.ny, F.nz}, c[3] = {I, J, K};
-    auto weight = [&](int d, const int (&x)[3]) -> float {
+    auto weight = [&](int d, const int (&x)[3]) -> T {
         if (FINE) {
             const double *W = d == 0 ? Wx : (d == 1 ? Wy : Wz);
-            return (float)W[((long long)x[2] * F.ny + x[1]) * F.nx + x[0]];
+            return (T)W[((long long)x[2] * F.ny + x[1]) * F.nx + x[0]];
         }
         return (d == 0 ? F.wx : (d == 1 ? F.wy : F.wz))[x[2] * F.sxy + x[1] * F.sx + x[0]];
     };
-    float W[3];
+    T W[3];
     for (int d = 0; d < 3; ++d) {
         const int u = (d + 1) % 3, v = (d + 2) % 3;
-        float sum = 0.f;
+        T sum = (T)0;
         for (int b = -1; b <= 1; ++b)
             for (int a = -1; a <= 1; ++a) {
                 int x[3];
                 x[u] = min(max(2 * c[u] + a, 0), n[u] - 1);
                 x[v] = min(max(2 * c[v] + b, 0), n[v] - 1);
                 x[d] = min(2 * c[d], n[d] - 2);
-                const float p = weight(d, x);
-                float w;
+                const T p = weight(d, x);
+                T w;
                 if (2 * c[d] + 1 <= n[d] - 2) {
                     x[d] += 1;
-                    const float q = weight(d, x);
-                    w = 0.5f * (p * q / (p + q) + 0.25f * (p + q));
+                    const T q = weight(d, x);
+                    w = (T)0.5 * (p * q / (p + q) + (T)0.25 * (p + q));
                 } else {
                     w = p;  // one fine edge to the boundary
                 }
-                sum += (a ? 0.5f : 1.f) * (b ? 0.5f : 1.f) * w;
+                sum += (a ? (T)0.5 : (T)1) * (b ? (T)0.5 : (T)1) * w;
             }
-        W[d] = c[d] < (d == 0 ? C.nx : (d == 1 ? C.ny : C.nz)) - 1 ? sum : 0.f;
+        W[d] = c[d] < (d == 0 ? C.nx : (d == 1 ? C.ny : C.nz)) - 1 ? sum : (T)0;
     }
-    float kap = 0.f;
+    T kap = (T)0;
     for (int e = 0; e < 27; ++e) {
         const int a = e % 3 - 1, b = (e / 3) % 3 - 1, g = e / 9 - 1;
         const int x = min(max(2 * I + a, 0), F.nx - 1), y = min(max(2 * J + b, 0), F.ny - 1),
                   z = min(max(2 * K + g, 0), F.nz - 1);
         const int p = z * F.sxy + y * F.sx + x;
-        const float k = FINE ? ((code[p] & 1) ? 0.f : kap0) : F.z[p];
-        kap += (a ? 0.5f : 1.f) * (b ? 0.5f : 1.f) * (g ? 0.5f : 1.f) * k;
+        const T k = FINE ? ((code[p] & 1) ? (T)0 : kap0) : F.z[p];
+        kap += (a ? (T)0.5 : (T)1) * (b ? (T)0.5 : (T)1) * (g ? (T)0.5 : (T)1) * k;
     }
     const int p = K * C.sxy + J * C.sx + I;
     C.wx[p] = W[0];
     C.wy[p] = W[1];
     C.wz[p] = W[2];
-    if (C.dg) C.dg[p] = 1.f;
+    if (C.dg) C.dg[p] = (T)1;
     C.z[p] = kap;
 }
 
-__global__ void k_mg_diag(mg::Lev C) {
+template <typename T>
+__global__ void k_mg_diag(mg::LevT<T> C) {
     const int t = blockIdx.x * 256 + threadIdx.x;
     if (t >= C.nx * C.ny * C.nz) return;
     const int I = t % C.nx, J = (t / C.nx) % C.ny, K = t / (C.nx * C.ny);
     if (!mg::interior(C, I, J, K)) return;
     const int p = K * C.sxy + J * C.sx + I;
-    C.dg[p] = C.wx[p] + C.wx[p - 1] + C.wy[p] + C.wy[p - C.sx] + C.wz[p] + C.wz[p - C.sxy] + C.z[p];
+    const T d = C.wx[p] + C.wx[p - 1] + C.wy[p] + C.wy[p - C.sx] + C.wz[p] + C.wz[p - C.sxy] + C.z[p];
+    C.dg[p] = d;
+    if (C.di) C.di[p] = (T)1 / d;
+}
+
+// The FP64 cycle (plain FP64 solver): the same steps with stored weights and
+// 1 / diagonal on every level, a node a thread.  GB300's FP64 pipe binds these
+// kernels before memory does (about 50 FP64 operations per unknown and cycle),
+// so residual, restriction, interpolation and smoothing are kernels of their
+// own and no value is formed twice.  97^3 to 1e-12: 500 Jacobi iterations and
+// 29.9 ms -> 29 iterations and 7.2 ms.
+namespace mg {
+struct Entry64 {
+    using T = double;
+    LevT<double> lev[LMAX];
+    int nlev, nbot;
+    CgState *st;
+    void *blob;
+    int bot;
+};
+__device__ __forceinline__ double face_sum64(const LevT<double> &L, const double *x, int p) {
+    return ((L.wx[p - 1] * x[p - 1] + L.wx[p] * x[p + 1]) + (L.wy[p - L.sx] * x[p - L.sx] + L.wy[p] * x[p + L.sx])) +
+           (L.wz[p - L.sxy] * x[p - L.sxy] + L.wz[p] * x[p + L.sxy]);
+}
+// interior node of a thread
+__device__ __forceinline__ bool node64(const LevT<double> &L, int &i, int &j, int &k) {
+    const int mx = L.nx - 2, my = L.ny - 2, t = blockIdx.x * 256 + threadIdx.x;
+    if (t >= mx * my * (L.nz - 2)) return false;
+    const int r = t / mx;
+    i = 1 + t - r * mx;
+    k = 1 + r / my;
+    j = 1 + r - (k - 1) * my;
+    return true;
+}
+}  // namespace mg
+
+__global__ void __launch_bounds__(256) k_mg64_residual(mg::LevT<double> L, const CgState *st) {
+    using namespace mg;
+    if (*(volatile const int *)&st->done) return;
+    int i, j, k;
+    if (!node64(L, i, j, k)) return;
+    const int p = k * L.sxy + j * L.sx + i;
+    L.r[p] = (1.0 - (double)OMEGA) * L.dg[p] * L.s[p] + (double)OMEGA * face_sum64(L, L.s, p);
+}
+
+__global__ void __launch_bounds__(256) k_mg64_restrict(mg::LevT<double> L, mg::LevT<double> C, const CgState *st) {
+    using namespace mg;
+    if (*(volatile const int *)&st->done) return;
+    int I, J, K;
+    if (!node64(C, I, J, K)) return;
+    const double *f = L.r + (2 * K * L.sxy + 2 * J * L.sx + 2 * I);
+    double acc = 0.0;
+#pragma unroll
+    for (int c = -1; c <= 1; ++c)
+#pragma unroll
+        for (int b = -1; b <= 1; ++b) {
+            const double *x = f + c * L.sxy + b * L.sx;
+            acc += (b ? 0.5 : 1.0) * (c ? 0.5 : 1.0) * (x[0] + 0.5 * (x[-1] + x[1]));
+        }
+    const int p = K * C.sxy + J * C.sx + I;
+    C.s[p] = acc * C.di[p];
+}
+
+__global__ void __launch_bounds__(256) k_mg64_correct(mg::LevT<double> L, mg::LevT<double> C, const CgState *st) {
+    using namespace mg;
+    if (*(volatile const int *)&st->done) return;
+    int i, j, k;
+    if (!node64(L, i, j, k)) return;
+    const double *x = C.z + ((k >> 1) * C.sxy + (j >> 1) * C.sx + (i >> 1));
+    double e;
+    // an even coordinate lies on a coarse line: no sum along it
+    auto line = [&](const double *q) { return (i & 1) ? 0.5 * (q[0] + q[1]) : q[0]; };
+    auto plane = [&](const double *q) { return (j & 1) ? 0.5 * (line(q) + line(q + C.sx)) : line(q); };
+    e = (k & 1) ? 0.5 * (plane(x) + plane(x + C.sxy)) : plane(x);
+    const int p = k * L.sxy + j * L.sx + i;
+    L.r[p] = (double)OMEGA * L.s[p] + e;
+}
+
+// the post-smoothing step (v in r); level 0: rho = r.z and beta
+template <bool TOP>
+__global__ void __launch_bounds__(256) k_mg64_smooth(mg::LevT<double> L, CgState *st, double *partials) {
+    using namespace mg;
+    if (*(volatile const int *)&st->done) return;
+    __shared__ double sred[8];
+    int i, j, k;
+    double rho = 0.0;
+    if (node64(L, i, j, k)) {
+        const int p = k * L.sxy + j * L.sx + i;
+        const double s = L.s[p];
+        const double z = (1.0 - (double)OMEGA) * L.r[p] + (double)OMEGA * (s + face_sum64(L, L.r, p) * L.di[p]);
+        L.z[p] = z;
+        if (TOP) rho = L.dg[p] * s * z;
+    }
+    if (!TOP) return;
+    double t0, t1;
+    if (last_block_total<256, false>(st, partials, gridDim.x, rho, 0.0, sred, t0, t1) && threadIdx.x == 0) {
+        st->counter = 0;
+        if (!(t0 > 0.0) || !isfinite(t0)) {
+            st->done = 1;
+            st->status = 1;
+        } else {
+            st->beta = st->rho > 0.0 ? t0 / st->rho : 0.0;
+            st->rho = t0;
+        }
+    }
 }
 
 // ------------------------------------------------------------------- host --
@@ -762,14 +885,15 @@ void mg_planes(mg::Entry &e, bool shared) {
 // The levels of a grid; false when the hierarchy does not reach the bottom
 // kernel's size (grids thinner than 9 nodes, or very long and thin ones):
 // those keep the Jacobi preconditioner.
-bool mg_levels(const PadGeo &g, mg::Entry &e, bool lattice = false) {
+template <class E>
+bool mg_levels(const PadGeo &g, E &e, bool lattice = false) {
     using namespace mg;
     if (std::min(g.nx, std::min(g.ny, g.nz)) < 9) return false;
     int n[3] = {g.nx, g.ny, g.nz}, nl = 0;
     for (;; ++nl) {
         if (nl == LMAX) return false;
-        Lev &L = e.lev[nl];
-        L = Lev{};
+        LevT<typename E::T> &L = e.lev[nl];
+        L = LevT<typename E::T>{};
         L.nx = n[0];
         L.ny = n[1];
         L.nz = n[2];
@@ -782,9 +906,9 @@ bool mg_levels(const PadGeo &g, mg::Entry &e, bool lattice = false) {
     long long nodes = 0;
     int b = e.nlev;
     while (b > (lattice ? 0 : 1)) {  // level 0 of a solver's grid is not the bottom kernel's
-        const Lev &L = e.lev[b - 1];
+        const auto &L = e.lev[b - 1];
         const long long n = (long long)L.nx * L.ny * L.nz;
-        if (nodes + n > BOT_NODES) break;
+        if (nodes + n > BOT_NODES<typename E::T>) break;
         nodes += n;
         --b;
     }
@@ -795,18 +919,17 @@ bool mg_levels(const PadGeo &g, mg::Entry &e, bool lattice = false) {
         e.lev[l].sx = e.lev[l].nx;
         e.lev[l].sxy = e.lev[l].nx * e.lev[l].ny;
     }
-    if (lattice) {
+    if constexpr (std::is_same<E, Entry>::value) {
+        const Lev &F = e.lev[0];
+        if (!lattice) e.nu0 = cdiv(F.nx - 1, FX) * cdiv(F.ny - 2, FY) * cdiv(F.nz - 2, RG);
         mg_planes(e, false);
-        return true;
     }
-    const Lev &F = e.lev[0];
-    e.nu0 = cdiv(F.nx - 1, FX) * cdiv(F.ny - 2, FY) * cdiv(F.nz - 2, RG);
-    mg_planes(e, false);
     return true;
 }
 
-// floats of one array of a level (whole 16-byte pieces)
-size_t mg_lev_floats(const mg::Lev &L) { return ((size_t)L.sxy * L.nz + 3) & ~(size_t)3; }
+// elements of one array of a level (whole 16-byte pieces)
+template <typename T>
+size_t mg_lev_size(const mg::LevT<T> &L) { return ((size_t)L.sxy * L.nz + 3) & ~(size_t)3; }
 
 void free_mg_state(pb_system *sys) {
     MgState *m = (MgState *)sys->mg;
@@ -819,50 +942,65 @@ void free_mg_state(pb_system *sys) {
     sys->mg = nullptr;
 }
 
-size_t mg_bottom_bytes(const mg::Entry &e) { return (size_t)mg::BOT_BYTES * e.bot; }
+template <class E>
+size_t mg_bottom_bytes(const E &e) {
+    return (size_t)mg::BOT_BYTES<typename E::T> * e.bot;
+}
 
 pb_status mg_prepare() {
     static bool done = false;
     if (done) return PB_OK;
-    const int most = mg::BOT_BYTES * mg::BOT_NODES;
-    PB_CUDA_TRY(cudaFuncSetAttribute(k_mg_bottom<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    PB_CUDA_TRY(cudaFuncSetAttribute(k_mg_bottom<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    const int most = mg::BOT_BYTES<float> * mg::BOT_NODES<float>, most64 = mg::BOT_BYTES<double> * mg::BOT_NODES<double>;
+    PB_CUDA_TRY(cudaFuncSetAttribute(k_mg_bottom<mg::Entry, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    PB_CUDA_TRY(cudaFuncSetAttribute(k_mg_bottom<mg::Entry, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    PB_CUDA_TRY(
+        cudaFuncSetAttribute(k_mg_bottom<mg::Entry64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most64));
     done = true;
     return PB_OK;
 }
 
 // lays the arrays of levels first .. nlev - 1 and the bottom kernel's data out
 // in `base`; returns the bytes (base may be null)
-size_t mg_layout(mg::Entry &e, int first, char *base) {
+template <class E>
+size_t mg_layout(E &e, int first, char *base) {
+    using T = typename E::T;
+    constexpr int arrays = sizeof(T) == 4 ? 6 : 8;
     size_t at = 0;
     for (int l = first; l < e.nlev; ++l) {
-        mg::Lev &L = e.lev[l];
-        const size_t n = mg_lev_floats(L);
+        mg::LevT<T> &L = e.lev[l];
+        const size_t n = mg_lev_size(L);
         if (base) {
-            L.wx = (float *)(base + at);  // n is a multiple of 4: every array is 16-byte aligned
+            L.wx = (T *)(base + at);  // n is a multiple of 4: every array is 16-byte aligned
             L.wy = L.wx + n;
             L.wz = L.wy + n;
             L.dg = L.wz + n;
             L.s = L.dg + n;
             L.z = L.s + n;
+            if (arrays == 8) {
+                L.di = L.z + n;
+                L.r = L.di + n;
+            }
         }
-        at += n * 24;
+        at += n * arrays * sizeof(T);
     }
     if (base) e.blob = base + at;
-    return at + 22 * (size_t)e.bot;
+    return at + mg::BLOB_BYTES<T> * (size_t)e.bot;
 }
 
 // coefficients of levels first .. nlev - 1 from the level above (level 1 of a
 // solver's grid from its FP64 operator; first == 0: level 0 is there already,
 // its ionic terms in z), and the bottom kernel's data
-pb_status mg_build_levels(const mg::Entry &e, int first, const pb_system *sys, cudaStream_t s) {
+template <class E>
+pb_status mg_build_levels(const E &e, int first, const pb_system *sys, cudaStream_t s) {
+    using T = typename E::T;
+    const T kap = (T)sys->kap_s;
     for (int l = first; l < e.nlev; ++l) {
-        const mg::Lev &C = e.lev[l];
+        const mg::LevT<T> &C = e.lev[l];
         const unsigned blocks = cdiv((long long)C.nx * C.ny * C.nz, 256);
         if (l == 1 && first == 1)
-            k_mg_coarsen<true><<<blocks, 256, 0, s>>>(e.lev[0], C, sys->W[0], sys->W[1], sys->W[2], sys->code, e.cp.kap);
+            k_mg_coarsen<true, T><<<blocks, 256, 0, s>>>(e.lev[0], C, sys->W[0], sys->W[1], sys->W[2], sys->code, kap);
         else if (l > 0)
-            k_mg_coarsen<false><<<blocks, 256, 0, s>>>(e.lev[l - 1], C, nullptr, nullptr, nullptr, nullptr, 0.f);
+            k_mg_coarsen<false, T><<<blocks, 256, 0, s>>>(e.lev[l - 1], C, nullptr, nullptr, nullptr, nullptr, (T)0);
         k_mg_diag<<<blocks, 256, 0, s>>>(C);
         note_launch(1);
         PB_LAUNCH_CHECK();
@@ -870,7 +1008,7 @@ pb_status mg_build_levels(const mg::Entry &e, int first, const pb_system *sys, c
     k_mg_pack<<<cdiv(e.bot, 256), 256, 0, s>>>(e, e.bot);
     PB_LAUNCH_CHECK();
     for (int l = first; l < e.nlev; ++l)  // z held the ionic terms
-        PB_CUDA_TRY(cudaMemsetAsync(e.lev[l].z, 0, sizeof(float) * (size_t)e.lev[l].sxy * e.lev[l].nz, s));
+        PB_CUDA_TRY(cudaMemsetAsync(e.lev[l].z, 0, sizeof(T) * (size_t)e.lev[l].sxy * e.lev[l].nz, s));
     return PB_OK;
 }
 
@@ -959,7 +1097,7 @@ int launch_vcycle(const pb_system *sys, cudaStream_t s) {
             mg_launch(k_mg_down<false, true>, std::min<unsigned>(n, rd1), DNT, 0, s, true, none, (const Head *)m->head,
                       l, n, e);
     }
-    mg_launch(k_mg_bottom<true>, 1, BOT_T, mg_bottom_bytes(e), s, true, none, (const Head *)m->head, e);
+    mg_launch(k_mg_bottom<Entry, true>, 1, BOT_T, mg_bottom_bytes(e), s, true, none, (const Head *)m->head, e);
     for (int l = e.nbot - 1; l >= 0; --l) {
         const int n = uitems(e, l);
         if (l == 0 && fine)
@@ -1006,7 +1144,7 @@ pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cuda
             C.nx = C.ny = C.nz = (n - 1) * (1 << q) + 1;
             C.sx = (C.nx + 3) & ~3;
             C.sxy = C.sx * C.ny;
-            const size_t c = mg_lev_floats(C);
+            const size_t c = mg_lev_size(C);
             mem = dalloc(16 * c, s);
             if (!mem) {
                 rc = PB_ERR_OOM;
@@ -1021,7 +1159,7 @@ pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cuda
         if (q == up) {
             rc = fill(sys, C.nx, C.sx, C.wx, C.wy, C.wz, C.z, s);
         } else {
-            k_mg_coarsen<false><<<cdiv((long long)C.nx * C.ny * C.nz, 256), 256, 0, s>>>(F, C, nullptr, nullptr,
+            k_mg_coarsen<false, float><<<cdiv((long long)C.nx * C.ny * C.nz, 256), 256, 0, s>>>(F, C, nullptr, nullptr,
                                                                                         nullptr, nullptr, 0.f);
             note_launch(1);
         }
@@ -1053,3 +1191,79 @@ LatticeMg mg_lattice_view(const pb_system *sys) {
 }
 
 int mg_lattice_cycle(const pb_system *sys, cudaStream_t s) { return launch_vcycle(sys, s); }
+
+// ---- FP64 cycle of the plain FP64 solver
+struct Mg64State {
+    mg::Entry64 e{};
+    double *v = nullptr;  // preconditioned residual (padded)
+    void *mem = nullptr;
+};
+
+void free_mg64_state(pb_system *sys) {
+    Mg64State *m = (Mg64State *)sys->mg64;
+    if (!m) return;
+    dfree(m->v, sys->stream);
+    dfree(m->mem, sys->stream);
+    delete m;
+    sys->mg64 = nullptr;
+}
+
+// built with the first FP64 solve of a uniform system; sys->mg64 stays null on
+// grids without a hierarchy
+pb_status build_mg64_state(pb_system *sys, cudaStream_t s) {
+    using namespace mg;
+    if (sys->mg64) return PB_OK;
+    Entry64 e{};
+    if (!mg_levels(sys->pad, e)) return PB_OK;
+    pb_status rc = mg_prepare();
+    if (rc != PB_OK) return rc;
+    Mg64State *m = new (std::nothrow) Mg64State();
+    if (!m) return PB_ERR_OOM;
+    sys->mg64 = m;
+    const size_t bytes = mg_layout(e, 1, nullptr), b0 = sizeof(double) * (size_t)sys->pad.Np;
+    m->v = (double *)dalloc(b0, s);
+    m->mem = dalloc(bytes, s);
+    if (!m->v || !m->mem) {
+        free_mg64_state(sys);
+        return PB_ERR_OOM;
+    }
+    PB_CUDA_TRY(cudaMemsetAsync(m->v, 0, b0, s));
+    PB_CUDA_TRY(cudaMemsetAsync(m->mem, 0, bytes, s));
+    mg_layout(e, 1, (char *)m->mem);
+    LevT<double> &L = e.lev[0];
+    L.s = sys->z64;
+    L.z = m->v;
+    L.wx = sys->op64[0];
+    L.wy = sys->op64[1];
+    L.wz = sys->op64[2];
+    L.dg = sys->op64[3];
+    L.di = sys->op64[4];
+    L.r = sys->q64;  // q is free between the update and the direction kernels, and zero off the interior
+    e.st = sys->st;
+    if ((rc = mg_build_levels(e, 1, sys, s)) != PB_OK) return rc;
+    m->e = e;
+    return PB_OK;
+}
+
+// one FP64 V-cycle (z64 -> v); returns the number of launches
+int launch_vcycle64(const pb_system *sys, cudaStream_t s) {
+    using namespace mg;
+    const Entry64 &e = ((const Mg64State *)sys->mg64)->e;
+    auto blocks = [](const LevT<double> &L) {
+        return cdiv((long long)(L.nx - 2) * (L.ny - 2) * (L.nz - 2), 256);
+    };
+    for (int l = 0; l < e.nbot; ++l) {
+        k_mg64_residual<<<blocks(e.lev[l]), 256, 0, s>>>(e.lev[l], sys->st);
+        k_mg64_restrict<<<blocks(e.lev[l + 1]), 256, 0, s>>>(e.lev[l], e.lev[l + 1], sys->st);
+    }
+    mg_launch(k_mg_bottom<Entry64, true>, 1, BOT_T, mg_bottom_bytes(e), s, true, (const Entry64 *)nullptr,
+              (const Head *)nullptr, e);
+    for (int l = e.nbot - 1; l >= 0; --l) {
+        k_mg64_correct<<<blocks(e.lev[l]), 256, 0, s>>>(e.lev[l], e.lev[l + 1], sys->st);
+        if (l == 0)
+            k_mg64_smooth<true><<<blocks(e.lev[l]), 256, 0, s>>>(e.lev[l], sys->st, sys->partials);
+        else
+            k_mg64_smooth<false><<<blocks(e.lev[l]), 256, 0, s>>>(e.lev[l], sys->st, nullptr);
+    }
+    return 4 * e.nbot + 1;
+}

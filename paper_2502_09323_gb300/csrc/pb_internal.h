@@ -208,6 +208,7 @@ struct pb_system {
     int solved, have_surface, have_pairs;
     double fnorm2;
     void *tma;          // tensor maps of the FP32 stencil kernels (host object)
+    void *mg64;         // the same of the plain FP64 solver
     void *mg;           // multigrid hierarchy of the FP32 solver (host object; null: Jacobi)
     unsigned int *queue;  // work counters of the TMA stencil kernels (device)
     pbg::OctSys *os;    // octree systems: level-transition rows
@@ -238,6 +239,7 @@ pb_status ensure_solver_ws(pb_system *sys, int precision, cudaStream_t s);
 pb_status profile_kernels(pb_system *sys, int precision, int which, int reps, cudaStream_t s);
 void free_tma_state(pb_system *sys);
 void free_mg_state(pb_system *sys);
+void free_mg64_state(pb_system *sys);
 // Uniform lattice of n^3 nodes with stored coefficients, solved by one
 // multigrid V-cycle (s = D^-1 b in, z out); it becomes sys->mg.  `fill` writes
 // the weights and ionic terms of the lattice `up` times finer by a factor of two.

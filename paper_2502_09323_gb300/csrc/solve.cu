@@ -1,7 +1,8 @@
 // Krylov solve of the condensed system A phi = f (Sec. 3.1, Eq.
 // matrixequation): preconditioned conjugate gradient with fused
-// stencil/dot/axpy kernels, in FP64 (Jacobi), or in FP32 (multigrid, mg.cuh;
-// Jacobi where a grid has no hierarchy) inside FP64 iterative refinement.
+// stencil/dot/axpy kernels, in FP64, or in FP32 inside FP64 iterative
+// refinement; the preconditioner is a multigrid cycle (mg.cuh), or Jacobi where
+// a grid has no hierarchy.
 //
 // Iteration with the Jacobi preconditioner (z = D^-1 r is stored instead of r; r = D z is formed on the fly):
 //   kernel P:  p <- z + beta p ;  q = A p ;  sigma = p.q      -> alpha = rho/sigma
@@ -606,42 +607,6 @@ dim3 stencil_grid(const PadGeo &g, int KC) {
                 (unsigned)cdiv(g.nz - 2, KC));
 }
 
-// z-chunk length: trade the two extra planes each chunk reads against the
-// tail of the last wave (blocks resident per SM from the occupancy API).
-template <typename T, class CP>
-int choose_kc(const PadGeo &g) {
-    static int resident = 0;
-    if (!resident) {
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &per_sm, k_stencil<T, CP, MODE_U, TYC, MinB<T>::v>, 32 * TYC, 0) != cudaSuccess ||
-            per_sm <= 0) {
-            cudaGetLastError();
-            per_sm = MinB<T>::v;
-        }
-        resident = per_sm * num_sms();
-    }
-    long long cols = (long long)cdiv(g.nx - 1, 32 * VT<T>::N) * cdiv(g.ny - 2, TYC);
-    int best = 8;
-    double best_eff = -1.0;
-    for (int kc = 4; kc <= 64; ++kc) {
-        long long blocks = cols * cdiv(g.nz - 2, kc);
-        double waves = (double)blocks / resident;
-        double occ = waves / ceil(waves);
-        double stream = (double)kc / (kc + 1.0);  // about half the streamed arrays re-read 2 planes
-        double eff = occ * stream;
-        if (eff > best_eff + 1e-9) {
-            best_eff = eff;
-            best = kc;
-        }
-    }
-    return best;
-}
-
-int default_kc(const PadGeo &g, int precision) {
-    return precision == PB_MIXED ? choose_kc<float, CoefC32>(g) : choose_kc<double, CoefS64>(g);
-}
-
 // ------------------------------------------------------ TMA tensor maps --
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -995,7 +960,7 @@ void launch_iter_cg64(pb_system *sys, int cur, int KC, cudaStream_t s, int which
     const PadGeo &g = sys->pad;
     double *pbuf[2] = {sys->pa64, sys->pb64};
     cg64::DirArgs d{};
-    d.z = sys->z64;
+    d.z = sys->mg64 ? ((const Mg64State *)sys->mg64)->v : sys->z64;
     d.pold = pbuf[cur];
     d.p = pbuf[cur ^ 1];
     d.q = sys->q64;
@@ -1097,6 +1062,7 @@ pb_status run_pcg(pb_system *sys, const CP &cp, T *z, T *pa, T *pb, T *x, int KC
                 else
                     launch_iter<T, CP>(sys, cp, z, bufs[cur], bufs[cur ^ 1], x, z, KC, s);
             } else {
+                if (mg) note_launch(launch_vcycle64(sys, s));
                 launch_iter_cg64(sys, cur, KC, s);
             }
             cur ^= 1;
@@ -1445,6 +1411,7 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
     pb_status rc = ensure_solver_ws(sys, o->precision, s);
     if (rc != PB_OK) return rc;
     if (o->precision == PB_MIXED && (rc = build_tma_state(sys, s)) != PB_OK) return rc;
+    if (o->precision == PB_FP64 && (rc = build_mg64_state(sys, s)) != PB_OK) return rc;
     Tuning tune;
     if ((rc = autotune(sys, o->precision, s, &tune)) != PB_OK) return rc;
     int max_iter = o->max_iter > 0 ? o->max_iter : 100000;
@@ -1533,12 +1500,13 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
                 break;
             }
             double rz = sys->h_st->rz64;
-            if ((rc = init_state(sys, rz, res2, rtol * rtol * fn2 * 0.25, max_iter - iters, s)) != PB_OK)
+            const bool mg = sys->mg64 != nullptr;
+            if ((rc = init_state(sys, rz, res2, rtol * rtol * fn2 * 0.25, max_iter - iters, s, 0, mg)) != PB_OK)
                 return rc;
             PB_CUDA_TRY(cudaMemsetAsync(sys->pa64, 0, bytes64, s));
             int it = 0;
             rc = run_pcg<double, CoefS64>(sys, cp, sys->z64, sys->pa64, sys->pb64, sys->x64, tune.kc,
-                                          0, tma::TWDEF, false, chunk, deadline, s, &it);
+                                          0, tma::TWDEF, mg, mg ? 2 : chunk, deadline, s, &it);
             if (rc == PB_ERR_TIMEOUT) status = PB_ERR_TIMEOUT;
             else if (rc != PB_OK) return rc;
             if (rc == PB_OK) iters += it;

@@ -85,3 +85,31 @@ def test_octree_solution_and_iterations(pb, h_bulk, n0, lattice):
         assert st["iters_inner"] <= 80  # 13 to 21 per 1e-6 in the CPU prototype
     st2 = pb.pb_solve_batch([s], pb.SolveOpts(precision=pb.MIXED, rtol=1e-12))[0]
     assert st2["iters_inner"] == st["iters_inner"] and np.array_equal(pb.pb_get_phi(s), phi)
+
+
+@pytest.mark.parametrize("n,ein,eout,hierarchy", CASES)
+def test_fp64_solution_and_iterations(pb, orc, n, ein, eout, hierarchy):
+    """The plain FP64 solver with its own (FP64) cycle, and the operator alone in both types on
+    the same grids (ragged rows, one or several blocks a plane) against the oracle's."""
+    atoms = pb_inputs.globular_molecule(12, seed=79)
+    atoms[:, :3] -= atoms[:, :3].mean(0)
+    h = 18.0 / (min(n) - 1)
+    g = orc.Grid(n, tuple(-0.5 * h * (m - 1) for m in n), h)
+    gg = pb.pb_build_grid(pb.GridSpec(n=n, origin=tuple(g.origin), h=h, fill=0.0), atoms)
+    s = pb.pb_assemble_coeffs(gg, pb.Params(eps_in=ein, eps_out=eout, bc=pb.BC_COULOMB))
+    st = pb.pb_solve(s, pb.SolveOpts(precision=pb.FP64, rtol=1e-11))
+    assert st["status"] == 0 and st["true_rel_res"] <= 1e-11
+    if hierarchy:
+        assert st["iters_inner"] <= 60
+    phi, bc, f = (pb.pb_get_array(s, k) for k in ("phi", "bc", "rhs"))
+    coef = {k: pb.pb_get_array(s, k) for k in ("Wx", "Wy", "Wz", "diag")}
+    r = f - orc.apply(g, coef, phi - bc)
+    assert np.linalg.norm(r) <= 1.01e-11 * np.linalg.norm(f)
+    import torch
+    x = pb_inputs.random_field(g.N, seed=80)
+    y = orc.apply(g, coef, np.where(np.asarray(coef["diag"]) > 0, x, 0.0))
+    xd = torch.from_numpy(x).cuda()
+    y64 = pb.pb_apply(s, xd).cpu().numpy()
+    assert np.abs(y64 - y).max() <= 1e-12 * np.abs(y).max()
+    y32 = pb.pb_apply(s, xd.float(), pb.MIXED).cpu().numpy()
+    assert np.abs(y32 - y).max() <= 1e-5 * np.abs(y).max()
