@@ -143,11 +143,12 @@ void pb_grid_free(pb_grid *g) {
     dfree(g->inside, s);
     dfree(g->cells.start, s);
     dfree(g->cells.atom, s);
+    dfree(g->cells.a64, s);
+    dfree(g->cells.a32, s);
     dfree(g->cid, s);
     dfree(g->calpha, s);
     dfree(g->crp, s);
     dfree(g->csign, s);
-    dfree(g->rowstart, s);
     dfree(g->mc_w, s);
     dfree(g->mc_n, s);
     dfree(g->d_info, s);

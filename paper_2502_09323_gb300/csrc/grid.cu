@@ -12,6 +12,7 @@
 // Sec. 2.3 / 3.4: the box is a cube of side fill * molecular extent (perfil).
 #include <math.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cub/block/block_reduce.cuh>
 #include <cub/block/block_scan.cuh>
@@ -248,6 +249,18 @@ __global__ void k_cell_sort(const int *__restrict__ start, int *__restrict__ lis
     }
 }
 
+// (x, y, z, R) of the atoms in cell order, in FP64 and, relative to the cell
+// list's corner, in FP32: a row of cells is one contiguous run, and a scan of
+// the 27 cells around a point is nine runs.
+__global__ void k_cell_atoms(const double *__restrict__ atoms, long long na, CellList cl) {
+    const long long q = blockIdx.x * 256ll + threadIdx.x;
+    if (q >= na) return;
+    const int i = cl.atom[q];
+    const double x = atoms[i], y = atoms[na + i], z = atoms[2 * na + i], r = atoms[3 * na + i];
+    cl.a64[q] = make_double4(x, y, z, r);
+    cl.a32[q] = make_float4((float)(x - cl.lo[0]), (float)(y - cl.lo[1]), (float)(z - cl.lo[2]), (float)r);
+}
+
 // ------------------------------------------------------- inside fraction --
 // Interval of the edge (x_a, x_a + h e_d) inside one ball, parameter t in
 // [0,1]: (u_d + t h)^2 = R^2 - |u_perp|^2 with u = x_a - c.  Split in the part
@@ -289,10 +302,15 @@ __device__ __forceinline__ bool edge_cut(double xad, double cd, double w, double
 // intervals are ordered by (t0, t1) and merged.  Returns false on overflow.
 // With COVER_EXIT the scan stops at the first ball whose interval is all of
 // [0, 1] (alpha = 1 exactly: the merged run then starts at 0 and ends at 1).
+// A ball that an FP32 test (with the cell list's margin) shows to miss the
+// edge contributes no interval and is passed over: about four of twenty
+// candidates reach the FP64 expressions.  An FP64 instruction holds GB300's
+// pipe for 16 cycles a warp however few lanes it serves, so each lane first walks to
+// its next candidate and the warp then evaluates all of them together
+// (257^3, 580,000 edges: with the FP64 part inside the walk 520 us, after it 220 us).
+// The intervals are sorted, so their order of arrival does not matter.
 template <bool COVER_EXIT>
-__device__ bool edge_alpha(const double *__restrict__ atoms, long long na, const CellList &cl,
-                           const int *__restrict__ cstart, const int *__restrict__ clist,
-                           const double xa[3], int d, double h, double &alpha) {
+__device__ bool edge_alpha(const CellList &cl, const double xa[3], int d, double h, double &alpha) {
     double t0s[MAX_EDGE_BALLS], t1s[MAX_EDGE_BALLS];
     int m = 0;
     int cc[3];
@@ -300,27 +318,44 @@ __device__ bool edge_alpha(const double *__restrict__ atoms, long long na, const
         double u = floor((xa[q] - cl.lo[q]) / cl.cs);
         cc[q] = (u < -4.0) ? -4 : ((u > (double)cl.dim[q] + 4.0) ? cl.dim[q] + 4 : (int)u);
     }
-    const int e = (d == 0) ? 1 : 0;
-    const int f = (d == 2) ? 1 : 2;
-    const double *Ce = atoms + (long long)e * na, *Cf = atoms + (long long)f * na;
-    const double *Cd = atoms + (long long)d * na, *R = atoms + 3 * na;
-    for (int cz = cc[2] - 1; cz <= cc[2] + 1; ++cz) {
-        if (cz < 0 || cz >= cl.dim[2]) continue;
-        for (int cy = cc[1] - 1; cy <= cc[1] + 1; ++cy) {
-            if (cy < 0 || cy >= cl.dim[1]) continue;
-            for (int cx = cc[0] - 1; cx <= cc[0] + 1; ++cx) {
-                if (cx < 0 || cx >= cl.dim[0]) continue;
-                int cid = (cz * cl.dim[1] + cy) * cl.dim[0] + cx;
-                for (int s = cstart[cid]; s < cstart[cid + 1]; ++s) {
-                    int at = clist[s];
-                    double w, t0, t1;
-                    if (!line_cut(xa, d, Ce[at], Cf[at], R[at], w)) continue;
-                    if (!edge_cut(xa[d], Cd[at], w, h, t0, t1)) continue;
-                    if (COVER_EXIT && !(t0 > 0.0) && !(t1 < 1.0)) {
-                        alpha = 1.0;
-                        return true;
-                    }
-                    if (m == MAX_EDGE_BALLS) return false;
+    const float x0 = (float)(xa[0] - cl.lo[0]), x1 = (float)(xa[1] - cl.lo[1]), x2 = (float)(xa[2] - cl.lo[2]);
+    const float mg = cl.margin, hm = (float)h + mg;
+    const int cx0 = cc[0] - 1 < 0 ? 0 : cc[0] - 1, cx1 = cc[0] + 1 >= cl.dim[0] ? cl.dim[0] - 1 : cc[0] + 1;
+    // the walk: nine rows of cells, each a run s .. s1 of the cell-ordered atoms
+    int row = cx0 > cx1 ? 9 : -1, s = 0, s1 = 0;
+    auto next = [&]() -> int {
+        for (;;) {
+            while (s >= s1) {
+                if (++row >= 9) return -1;
+                const int cy = cc[1] - 1 + row % 3, cz = cc[2] - 1 + row / 3;
+                if (cz < 0 || cz >= cl.dim[2] || cy < 0 || cy >= cl.dim[1]) continue;
+                const int c0 = (cz * cl.dim[1] + cy) * cl.dim[0];
+                s = cl.start[c0 + cx0];
+                s1 = cl.start[c0 + cx1 + 1];
+            }
+            const float4 b = cl.a32[s++];
+            const float v0 = b.x - x0, v1 = b.y - x1, v2 = b.z - x2, rm = b.w + mg;
+            const float vd = d == 0 ? v0 : (d == 1 ? v1 : v2);
+            const float ve = d == 0 ? v1 : v0, vf = d == 2 ? v1 : v2;
+            if (!(ve * ve + vf * vf > rm * rm || vd > rm + hm || vd < -rm)) return s - 1;
+        }
+    };
+    const unsigned lanes = __activemask();
+    bool over = false, covered = false;
+    for (;;) {
+        const int at = over || covered ? -1 : next();
+        __syncwarp(lanes);
+        if (!__any_sync(lanes, at >= 0)) break;
+        double w, t0, t1;
+        if (at >= 0) {
+            const double4 ball = cl.a64[at];
+            if (line_cut(xa, d, d == 0 ? ball.y : ball.x, d == 2 ? ball.y : ball.z, ball.w, w) &&
+                edge_cut(xa[d], d == 0 ? ball.x : (d == 1 ? ball.y : ball.z), w, h, t0, t1)) {
+                if (COVER_EXIT && !(t0 > 0.0) && !(t1 < 1.0)) {
+                    covered = true;
+                } else if (m == MAX_EDGE_BALLS) {
+                    over = true;
+                } else {
                     // insertion by (t0, t1)
                     int b = m - 1;
                     while (b >= 0 && (t0s[b] > t0 || (t0s[b] == t0 && t1s[b] > t1))) {
@@ -334,7 +369,13 @@ __device__ bool edge_alpha(const double *__restrict__ atoms, long long na, const
                 }
             }
         }
+        __syncwarp(lanes);
     }
+    if (covered) {
+        alpha = 1.0;
+        return true;
+    }
+    if (over) return false;
     if (m == 0) {
         alpha = 0.0;
         return true;
@@ -393,7 +434,8 @@ __global__ void k_edge_cand(const double *__restrict__ atoms, long long na, Grid
     const long long step[3] = {1, (long long)g.nx, (long long)g.nx * g.ny};
     for (long long at = blockIdx.x; at < na; at += gridDim.x) {
         const double c[3] = {X[at], Y[at], Z[at]};
-        const double r = R[at];
+        const double r = R[at], hinv = 1.0 / g.h;
+        const float r32 = (float)r;
         long long lo[3], hi[3], ext[3];
         for (int d = 0; d < 3; ++d) {
             lo[d] = clampll((long long)floor((c[d] - r - g.o[d]) / g.h) - 1, 0, nn[d] - 1);
@@ -425,12 +467,21 @@ __global__ void k_edge_cand(const double *__restrict__ atoms, long long na, Grid
             xa[d] = 0.0;
             xa[e] = node_coord(g, e, ie);
             xa[f] = node_coord(g, f, jf);
+            // a line that FP32 shows to miss the ball (distances here are at
+            // most a few radii, so FP32 is good to 1e-6 of them)
+            const float fe = (float)(xa[e] - c[e]), ff = (float)(xa[f] - c[f]);
+            if (fe * fe + ff * ff > 1.0001f * r32 * r32) continue;
             double w;
             if (!line_cut(xa, d, c[e], c[f], r, w)) continue;
             const long long base = (long long)d * g.N + ie * step[e] + jf * step[f];
+            // Edges more than a spacing below or above the ball have an empty
+            // interval (n0 >= h or n1 <= 0 by a whole spacing, far more than
+            // rounding): the scans start and end there.
+            const long long i_lo = max(ilo, (long long)floor((c[d] - w - g.o[d]) * hinv) - 1);
+            const long long i_hi = min(ihi, (long long)ceil((c[d] + w - g.o[d]) * hinv) + 1);
             long long iu = ihi + 1, id = ihi + 1;
             bool cov_iu = false;
-            for (long long i = ilo; i <= ihi; ++i) {
+            for (long long i = i_lo; i <= i_hi; ++i) {
                 double t0, t1;
                 if (!edge_cut(node_coord(g, d, i), c[d], w, g.h, t0, t1)) continue;
                 if (t0 > 0.0 || t1 < 1.0) flags[base + i * step[d]] = 2;
@@ -440,7 +491,7 @@ __global__ void k_edge_cand(const double *__restrict__ atoms, long long na, Grid
                     break;
                 }
             }
-            for (long long i = ihi; i > iu; --i) {
+            for (long long i = i_hi; i > iu; --i) {
                 double t0, t1;
                 if (!edge_cut(node_coord(g, d, i), c[d], w, g.h, t0, t1)) continue;
                 if (t0 > 0.0 || t1 < 1.0) flags[base + i * step[d]] = 2;
@@ -458,90 +509,122 @@ __global__ void k_edge_cand(const double *__restrict__ atoms, long long na, Grid
 }
 
 // flag[e] = 1 when edge e is listed: 0 < alpha < 1 or its end nodes differ in
-// `inside`.  One block per 4096 edges.  Edges whose end nodes differ are
-// listed; the others are listed only if they are candidates not covered by
-// one ball, and for those the block computes the inside fraction (union of
-// all balls' intervals): they are gathered in shared memory and shared out
-// over the block.
+// `inside`.  Edges whose end nodes differ are listed; the others are listed
+// only if they are candidates not covered by one ball, and for those the
+// inside fraction (union of all balls' intervals) decides.  This pass streams
+// the flags, 16 edges a thread, decides all but the last kind and appends those to a
+// list for k_edge_union (a thread each, whatever block they came from); an
+// edge that finds the list full keeps its 2.  The end nodes' bytes are
+// compared a word at a time.
+__device__ __forceinline__ uint4 load16(const uint8_t *p) {
+    // 16 bytes at any address from the aligned words around them
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)3);
+    const unsigned sh = 8u * (unsigned)(reinterpret_cast<uintptr_t>(p) & 3);
+    const uint32_t a = w[0], b = w[1], c = w[2], d = w[3], e = sh ? w[4] : 0u;
+    return make_uint4(__funnelshift_r(a, b, sh), __funnelshift_r(b, c, sh), __funnelshift_r(c, d, sh),
+                      __funnelshift_r(d, e, sh));
+}
+
 __global__ void __launch_bounds__(CHUNK_THREADS)
-k_edge_flags(const double *__restrict__ atoms, long long na, GridGeo g, CellList cl,
-             const int *__restrict__ cstart, const int *__restrict__ clist,
-             const uint8_t *__restrict__ inside, uint8_t *__restrict__ flags,
-             const uint8_t *__restrict__ cov, BuildInfo *info) {
-    __shared__ uint4 s_fl[CHUNK_THREADS];
-    __shared__ int s_list[CHUNK_BYTES];
-    __shared__ int s_list_n;
-    if (threadIdx.x == 0) s_list_n = 0;
-    __syncthreads();
-    const long long tile = (long long)blockIdx.x * CHUNK_BYTES;
-    uint4 v = reinterpret_cast<const uint4 *>(flags)[(long long)blockIdx.x * CHUNK_THREADS +
-                                                     threadIdx.x];
-    unsigned w[4] = {v.x, v.y, v.z, v.w};
+k_edge_flags(GridGeo g, const uint8_t *__restrict__ inside, uint8_t *__restrict__ flags,
+             const uint8_t *__restrict__ cov, long long *__restrict__ list, int cap, int *__restrict__ count) {
+    const long long t = (long long)blockIdx.x * CHUNK_THREADS + threadIdx.x;
+    const uint4 v = reinterpret_cast<const uint4 *>(flags)[t];
+    const unsigned w[4] = {v.x, v.y, v.z, v.w};
     uint4 cv = make_uint4(0u, 0u, 0u, 0u);
-    if (v.x | v.y | v.z | v.w)
-        cv = reinterpret_cast<const uint4 *>(cov)[(long long)blockIdx.x * CHUNK_THREADS +
-                                                 threadIdx.x];
+    if (v.x | v.y | v.z | v.w) cv = reinterpret_cast<const uint4 *>(cov)[t];
     const unsigned cw[4] = {cv.x, cv.y, cv.z, cv.w};
-    // first edge of this thread's 16, then stepped node by node
-    long long e0 = tile + 16ll * threadIdx.x;
-    int d = (int)(e0 / g.N);
-    long long a = e0 - (long long)d * g.N;
-    long long i = a % g.nx, row = a / g.nx;
-    long long j = row % g.ny, k = row / g.ny;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        unsigned out = 0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            unsigned u = (w[q] >> (8 * b)) & 0xffu;
-            unsigned fl = 0;
-            if (d < 3) {
-                long long id = d == 0 ? i : (d == 1 ? j : k);
-                long long nd = d == 0 ? g.nx : (d == 1 ? g.ny : g.nz);
-                long long st = d == 0 ? 1 : (d == 1 ? (long long)g.nx : (long long)g.nx * g.ny);
-                const bool differ = id < nd - 1 && inside[a] != inside[a + st];
-                const bool covered = ((cw[q] >> (8 * b)) & 0xffu) != 0u;
-                if (u == 2u && !differ && !covered) {
-                    int p = atomicAdd(&s_list_n, 1);
-                    s_list[p] = 16 * threadIdx.x + 4 * q + b;
-                } else if (differ) {
-                    fl = 1;
-                }
-            }
-            out |= fl << (8 * b);
-            ++a;
-            if (++i == g.nx) {
-                i = 0;
-                if (++j == g.ny) {
-                    j = 0;
-                    if (++k == g.nz) {
-                        k = 0;
-                        a = 0;
-                        ++d;
-                    }
-                }
-            }
+    // this thread's 16 edges: direction d, low nodes a .. a + 15
+    const long long e0 = 16 * t, plane = (long long)g.nx * g.ny;
+    const int d0 = (int)(e0 / g.N);
+    const long long a0 = e0 - (long long)d0 * g.N;
+    const long long row = a0 / g.nx;
+    const int i0 = (int)(a0 - row * g.nx);
+    unsigned df[4] = {0u, 0u, 0u, 0u};  // bytes 1 where the end nodes differ
+    const long long st0 = d0 == 0 ? 1 : (d0 == 1 ? (long long)g.nx : plane);
+    // one direction, at most two rows, and room to read whole words
+    if (d0 < 3 && g.nx >= 16 && a0 + st0 + 20 <= g.N) {
+        const uint4 p = load16(inside + a0), q = load16(inside + a0 + st0);
+        df[0] = p.x ^ q.x;
+        df[1] = p.y ^ q.y;
+        df[2] = p.z ^ q.z;
+        df[3] = p.w ^ q.w;
+        // edges that do not exist: from the last node of a row (d = 0), from
+        // a plane's last row (d = 1); the last plane (d = 2) is past the
+        // bound above.  first: nodes left in the row of a0.
+        const int first = g.nx - i0;
+        unsigned off = 0;  // bit b: edge b does not exist
+        if (d0 == 0 && first <= 16) off = 1u << (first - 1);
+        if (d0 == 1) {
+            const int j = (int)(row % g.ny);
+            if (j == g.ny - 1) off |= first >= 16 ? 0xffffu : (1u << first) - 1u;
+            if (j == g.ny - 2 && first < 16) off |= 0xffffu & ~((1u << first) - 1u);
         }
-        w[q] = out;
+#pragma unroll
+        for (int b = 0; b < 16; ++b)
+            if ((off >> b) & 1u) df[b >> 2] &= ~(0xffu << (8 * (b & 3)));
+    } else {
+        for (int b = 0; b < 16; ++b) {
+            const long long e = e0 + b;
+            const int d = (int)(e / g.N);
+            if (d > 2) break;
+            const long long a = e - (long long)d * g.N;
+            const long long r = a / g.nx, i = a - r * g.nx, j = r % g.ny, k = r / g.ny;
+            const bool ex = d == 0 ? i < g.nx - 1 : (d == 1 ? j < g.ny - 1 : k < g.nz - 1);
+            const long long st = d == 0 ? 1 : (d == 1 ? (long long)g.nx : plane);
+            if (ex && inside[a] != inside[a + st]) df[b >> 2] |= 1u << (8 * (b & 3));
+        }
     }
-    s_fl[threadIdx.x] = make_uint4(w[0], w[1], w[2], w[3]);
-    __syncthreads();
-    uint8_t *sb = reinterpret_cast<uint8_t *>(s_fl);
-    const int n = s_list_n;
-    for (int p = threadIdx.x; p < n; p += CHUNK_THREADS) {
-        const int off = s_list[p];
-        EdgeRef r = edge_ref(g, tile + off);
-        double xa[3] = {node_coord(g, 0, r.ijk[0]), node_coord(g, 1, r.ijk[1]),
-                        node_coord(g, 2, r.ijk[2])};
-        // an edge met by too many balls is listed, so that the record pass,
-        // which reports the overflow, meets it again
-        double al;
-        if (!edge_alpha<true>(atoms, na, cl, cstart, clist, xa, r.d, g.h, al)) al = 0.5;
-        sb[off] = (al > 0.0 && al < 1.0) ? 1 : 0;
+    // candidates (2) that neither differ nor are covered
+    unsigned todo = 0;
+#pragma unroll
+    for (int b = 0; b < 16; ++b) {
+        const unsigned sh = 8 * (b & 3), f = (w[b >> 2] >> sh) & 0xffu;
+        if (f == 2u && ((df[b >> 2] | cw[b >> 2]) >> sh & 0xffu) == 0u) todo |= 1u << b;
     }
-    __syncthreads();
-    reinterpret_cast<uint4 *>(flags)[(long long)blockIdx.x * CHUNK_THREADS + threadIdx.x] =
-        s_fl[threadIdx.x];
+    // one append a warp
+    const int lane = threadIdx.x & 31, n = __popc(todo);
+    int pos = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, pos, o);
+        if (lane >= o) pos += u;
+    }
+    int base = 0;
+    if (lane == 31 && pos) base = atomicAdd(count, pos);
+    base = __shfl_sync(0xffffffffu, base, 31);
+    pos += base - n;
+    while (todo) {
+        const int b = __ffs(todo) - 1;
+        todo &= todo - 1;
+        if (pos < cap) list[pos] = e0 + b;
+        else df[b >> 2] |= 2u << (8 * (b & 3));
+        ++pos;
+    }
+    reinterpret_cast<uint4 *>(flags)[t] = make_uint4(df[0], df[1], df[2], df[3]);
+}
+
+__device__ __forceinline__ uint8_t edge_listed(const GridGeo &g, const CellList &cl, long long e) {
+    const EdgeRef r = edge_ref(g, e);
+    const double xa[3] = {node_coord(g, 0, r.ijk[0]), node_coord(g, 1, r.ijk[1]), node_coord(g, 2, r.ijk[2])};
+    // an edge met by too many balls is listed, so that the record pass,
+    // which reports the overflow, meets it again
+    double al;
+    if (!edge_alpha<true>(cl, xa, r.d, g.h, al)) al = 0.5;
+    return (al > 0.0 && al < 1.0) ? 1 : 0;
+}
+
+// the listed ones among the appended edges; and, where the list was full, among
+// those still marked 2 (n_edge flags)
+__global__ void __launch_bounds__(128)
+k_edge_union(GridGeo g, CellList cl, const long long *__restrict__ list, int cap, const int *__restrict__ count,
+             uint8_t *__restrict__ flags, long long n_edge) {
+    const int n = *count;
+    const long long t0 = blockIdx.x * 128ll + threadIdx.x, step = gridDim.x * 128ll;
+    for (long long q = t0; q < min(n, cap); q += step) flags[list[q]] = edge_listed(g, cl, list[q]);
+    if (n <= cap) return;
+    for (long long e = t0; e < n_edge; e += step)
+        if (flags[e] == 2) flags[e] = edge_listed(g, cl, e);
 }
 
 // ------------------------------------------------- ordered compaction --
@@ -566,7 +649,7 @@ k_chunk_count(const uint4 *__restrict__ flags, int *__restrict__ counts) {
 
 __global__ void __launch_bounds__(CHUNK_THREADS)
 k_chunk_emit(const uint4 *__restrict__ flags, const int *__restrict__ offs,
-             long long *__restrict__ ids) {
+             long long *__restrict__ ids, uint16_t *__restrict__ emask, int *__restrict__ epos) {
     using BS = cub::BlockScan<int, CHUNK_THREADS>;
     __shared__ typename BS::TempStorage tmp;
     long long t = (long long)blockIdx.x * CHUNK_THREADS + threadIdx.x;
@@ -576,17 +659,21 @@ k_chunk_emit(const uint4 *__restrict__ flags, const int *__restrict__ offs,
     long long pos = offs[blockIdx.x] + ex;
     unsigned w[4] = {v.x, v.y, v.z, v.w};
     long long base = t * 16;
+    epos[t] = (int)pos;
+    unsigned mask = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int b = 0; b < 4; ++b)
-            if (((w[q] >> (8 * b)) & 0xffu) != 0u) ids[pos++] = base + 4 * q + b;
+            if (((w[q] >> (8 * b)) & 0xffu) != 0u) {
+                ids[pos++] = base + 4 * q + b;
+                mask |= 1u << (4 * q + b);
+            }
+    emask[t] = (uint16_t)mask;
 }
 
 // --------------------------------------------------- listed-edge records --
-__global__ void k_cross_fill(const double *__restrict__ atoms, long long na, GridGeo g,
-                             CellList cl, const int *__restrict__ cstart,
-                             const int *__restrict__ clist, const uint8_t *__restrict__ inside,
+__global__ void k_cross_fill(GridGeo g, CellList cl, const uint8_t *__restrict__ inside,
                              const long long *__restrict__ ids, long long ncross,
                              double *__restrict__ alpha_out, double *__restrict__ rp,
                              int8_t *__restrict__ sign, BuildInfo *info) {
@@ -596,7 +683,7 @@ __global__ void k_cross_fill(const double *__restrict__ atoms, long long na, Gri
     double xa[3] = {node_coord(g, 0, r.ijk[0]), node_coord(g, 1, r.ijk[1]),
                     node_coord(g, 2, r.ijk[2])};
     double al;
-    if (!edge_alpha<false>(atoms, na, cl, cstart, clist, xa, r.d, g.h, al)) {
+    if (!edge_alpha<false>(cl, xa, r.d, g.h, al)) {
         atomicOr(&info->err, ERRF_TOO_MANY_BALLS);
         al = 0.0;
     }
@@ -618,22 +705,9 @@ __global__ void k_cross_fill(const double *__restrict__ atoms, long long na, Gri
     rp[3 * s + 1] = p[1];
     rp[3 * s + 2] = p[2];
     sign[s] = (int8_t)sg;
-    if (sg != 0) atomicAdd(&info->nflux, 1ull);
-}
-
-// rowstart[r] = first listed edge with id >= r*nx, r = (d*nz + k)*ny + j
-__global__ void k_rowstart(const long long *__restrict__ ids, long long ncross, int nx,
-                           long long nrows, int *__restrict__ rowstart) {
-    long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (r > nrows) return;
-    long long key = r * nx;
-    long long lo = 0, hi = ncross;
-    while (lo < hi) {
-        long long mid = (lo + hi) >> 1;
-        if (ids[mid] < key) lo = mid + 1;
-        else hi = mid;
-    }
-    rowstart[r] = (int)lo;
+    // one atomic a warp
+    const unsigned act = __activemask(), fl = __ballot_sync(act, sg != 0);
+    if (fl && (threadIdx.x & 31) == __ffs(act) - 1) atomicAdd(&info->nflux, (unsigned long long)__popc(fl));
 }
 
 __global__ void k_count_inside(const uint8_t *__restrict__ inside, long long N, BuildInfo *info) {
@@ -744,6 +818,20 @@ pb_status grid_build(pb_grid *g, const pb_grid_spec *spec, cudaStream_t s) {
     PB_LAUNCH_CHECK();
     dfree(count, s);
     dfree(acell, s);
+    cl.a64 = (double4 *)dalloc(sizeof(double4) * (na + 1), s);
+    cl.a32 = (float4 *)dalloc(sizeof(float4) * (na + 1), s);
+    if (!cl.a64 || !cl.a32) return PB_ERR_OOM;
+    // The points tested in FP32 lie within the cell list's box widened by four
+    // cells; X its largest coordinate relative to lo.  Rounding a coordinate
+    // to FP32 costs 2^-24 X, so a difference, a radius or a distance formed
+    // from them is off by a few times that (and by 2^-22 of itself).
+    double ext = 0.0;
+    for (int d = 0; d < 3; ++d) ext = fmax(ext, (double)(cl.dim[d] + 8) * cl.cs);
+    cl.margin = (float)(1e-3 + 64.0 * ext * 5.9604644775390625e-8);
+    if (na > 0) {
+        k_cell_atoms<<<cdiv(na, 256), 256, 0, s>>>(g->atoms, na, cl);
+        PB_LAUNCH_CHECK();
+    }
 
     // ---- listed edges: flags -> ordered compaction -> records
     long long nedge = 3 * N;
@@ -760,10 +848,19 @@ pb_status grid_build(pb_grid *g, const pb_grid_spec *spec, cudaStream_t s) {
         k_edge_cand<<<atom_blocks, 128, 0, s>>>(g->atoms, na, geo, flags, cov);
         PB_LAUNCH_CHECK();
     }
-    k_edge_flags<<<(unsigned)nchunks, CHUNK_THREADS, 0, s>>>(g->atoms, na, geo, cl, cl.start,
-                                                              cl.atom, g->inside, flags, cov,
-                                                              g->d_info);
+    // candidates left for the union: an eighth of the nodes is far more than a
+    // molecular surface has
+    const int cap = (int)std::min<long long>(N / 8 + 1024, 1 << 30);
+    long long *elist = (long long *)dalloc(sizeof(long long) * (size_t)cap, s);
+    int *ecount = (int *)dalloc(sizeof(int), s);
+    if (!elist || !ecount) return PB_ERR_OOM;
+    PB_CUDA_TRY(cudaMemsetAsync(ecount, 0, sizeof(int), s));
+    k_edge_flags<<<(unsigned)nchunks, CHUNK_THREADS, 0, s>>>(geo, g->inside, flags, cov, elist, cap, ecount);
     PB_LAUNCH_CHECK();
+    k_edge_union<<<num_sms() * 8, 128, 0, s>>>(geo, cl, elist, cap, ecount, flags, nedge);
+    PB_LAUNCH_CHECK();
+    dfree(elist, s);
+    dfree(ecount, s);
     dfree(cov, s);
     k_chunk_count<<<(unsigned)nchunks, CHUNK_THREADS, 0, s>>>((const uint4 *)flags, ccount);
     PB_LAUNCH_CHECK();
@@ -783,20 +880,17 @@ pb_status grid_build(pb_grid *g, const pb_grid_spec *spec, cudaStream_t s) {
     g->calpha = (double *)dalloc(sizeof(double) * nc, s);
     g->crp = (double *)dalloc(sizeof(double) * 3 * nc, s);
     g->csign = (int8_t *)dalloc(nc, s);
-    long long nrows = 3ll * geo.ny * geo.nz;
-    g->rowstart = (int *)dalloc(sizeof(int) * (nrows + 1), s);
-    if (!g->cid || !g->calpha || !g->crp || !g->csign || !g->rowstart) return PB_ERR_OOM;
+    uint16_t *emask = (uint16_t *)dalloc(sizeof(uint16_t) * (size_t)(nflags / 16), s);
+    int *epos = (int *)dalloc(sizeof(int) * (size_t)(nflags / 16), s);
+    if (!g->cid || !g->calpha || !g->crp || !g->csign || !emask || !epos) return PB_ERR_OOM;
     if (total > 0) {
         k_chunk_emit<<<(unsigned)nchunks, CHUNK_THREADS, 0, s>>>((const uint4 *)flags, coffs,
-                                                                 g->cid);
+                                                                 g->cid, emask, epos);
         PB_LAUNCH_CHECK();
-        k_cross_fill<<<cdiv(total, 256), 256, 0, s>>>(g->atoms, na, geo, cl, cl.start, cl.atom,
-                                                      g->inside, g->cid, total, g->calpha,
-                                                      g->crp, g->csign, g->d_info);
+        k_cross_fill<<<cdiv(total, 128), 128, 0, s>>>(geo, cl, g->inside, g->cid, total, g->calpha, g->crp, g->csign,
+                                                      g->d_info);
         PB_LAUNCH_CHECK();
     }
-    k_rowstart<<<cdiv(nrows + 1, 256), 256, 0, s>>>(g->cid, total, geo.nx, nrows, g->rowstart);
-    PB_LAUNCH_CHECK();
     dfree(flags, s);
     dfree(ccount, s);
     dfree(coffs, s);
@@ -810,7 +904,10 @@ pb_status grid_build(pb_grid *g, const pb_grid_spec *spec, cudaStream_t s) {
     g->ninside = (long long)hinfo.ninside;
     // the surface re-triangulated through the crossing points (first
     // integral of Eq. energy_ion, Sec. 3.3.2): vertex weights and normals
-    return mc_surface(g, s);
+    const pb_status mrc = mc_surface(g, emask, epos, s);
+    dfree(emask, s);
+    dfree(epos, s);
+    return mrc;
 }
 
 }  // namespace pbg

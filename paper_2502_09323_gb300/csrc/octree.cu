@@ -1989,8 +1989,6 @@ pb_status oct_build(pb_grid *g, const pb_grid_spec *spec, cudaStream_t s) {
     }
     // the finest-lattice arrays are no longer needed
     dfree(g->inside, s);
-    dfree(g->rowstart, s);
-    g->rowstart = nullptr;
     g->inside = sin;
     g->ninside = (long long)hin;
     g->is_oct = 1;

@@ -60,6 +60,10 @@ struct CellList {
     int ncell;
     int *start;       // [ncell + 1]
     int *atom;        // [na] atom ids grouped by cell
+    double4 *a64;     // [na] (x, y, z, R) of those atoms
+    float4 *a32;      // [na] the same in FP32, relative to lo
+    float margin;     // what an FP32 distance between a point of the grid and an
+                      // atom may be off by, several times over (see grid.cu)
 };
 
 // Grid geometry passed by value to kernels.
@@ -129,7 +133,6 @@ struct pb_grid {
     double *calpha;       // [ncross]
     double *crp;          // [3*ncross] AoS
     int8_t *csign;        // [ncross]
-    int *rowstart;        // [3*ny*nz + 1] first list entry of each edge row
     pbg::BuildInfo *d_info;
     double center[3];     // shift used by the FP32 N-body kernels
     int is_oct;           // octree grid: geo is the flat slot layout (nx = N)
@@ -230,7 +233,8 @@ pb_status nbody_surface(pb_system *sys, cudaStream_t s);
 pb_status nbody_pairs(pb_system *sys, cudaStream_t s);
 
 // ------------------------------------------------------------ surface.cu --
-pb_status mc_surface(pb_grid *g, cudaStream_t s);
+// emask, epos: which of each 16 edges are listed, and the first one's place
+pb_status mc_surface(pb_grid *g, const uint16_t *emask, const int *epos, cudaStream_t s);
 
 // -------------------------------------------------------------- solve.cu --
 pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve_stats *st);
