@@ -18,25 +18,37 @@ namespace pbg {
 
 namespace {
 
-__device__ __forceinline__ bool is_bnd(const GridGeo &g, long long i, long long j, long long k) {
-    return i == 0 || j == 0 || k == 0 || i == g.nx - 1 || j == g.ny - 1 || k == g.nz - 1;
+// Row (j, k) of a thread's node and its first index; one warp takes a row at
+// a time, so that no node needs a division.
+struct Row {
+    int j, k;
+    long long a;  // canonical index of node (0, j, k)
+};
+__device__ __forceinline__ Row row_of(const GridGeo &g, long long r) {
+    Row w;
+    w.k = (int)(r / g.ny);
+    w.j = (int)(r - (long long)w.k * g.ny);
+    w.a = r * g.nx;
+    return w;
 }
+constexpr int ROWS = 8;  // rows (warps) of a block
 
 // Pure-medium weights for every existing edge; the code byte of the padded
 // FP32 layout starts as the solute bit.
-__global__ void k_coef_pure(const uint8_t *__restrict__ inside, GridGeo g, PadGeo p,
-                            double w_in, double w_out, double *__restrict__ Wx,
-                            double *__restrict__ Wy, double *__restrict__ Wz,
-                            uint8_t *__restrict__ code) {
-    long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (a >= g.N) return;
-    long long i = a % g.nx, j = (a / g.nx) % g.ny, k = a / ((long long)g.nx * g.ny);
-    int in = inside[a];
-    double w = in ? w_in : w_out;
-    Wx[a] = (i < g.nx - 1) ? w : 0.0;
-    Wy[a] = (j < g.ny - 1) ? w : 0.0;
-    Wz[a] = (k < g.nz - 1) ? w : 0.0;
-    code[(k * g.ny + j) * p.sx + i] = (uint8_t)in;
+__global__ void __launch_bounds__(32 * ROWS)
+k_coef_pure(const uint8_t *__restrict__ inside, GridGeo g, PadGeo p, double w_in, double w_out,
+            double *__restrict__ Wx, double *__restrict__ Wy, double *__restrict__ Wz, uint8_t *__restrict__ code) {
+    const long long r = blockIdx.x * (long long)ROWS + threadIdx.y;
+    if (r >= (long long)g.ny * g.nz) return;
+    const Row w = row_of(g, r);
+    for (int i = threadIdx.x; i < g.nx; i += 32) {
+        const int in = inside[w.a + i];
+        const double v = in ? w_in : w_out;
+        Wx[w.a + i] = (i < g.nx - 1) ? v : 0.0;
+        Wy[w.a + i] = (w.j < g.ny - 1) ? v : 0.0;
+        Wz[w.a + i] = (w.k < g.nz - 1) ? v : 0.0;
+        code[r * p.sx + i] = (uint8_t)in;
+    }
 }
 
 // Listed edges: WHA weight; FP32 copy for the compressed operator; flag bit
@@ -65,25 +77,38 @@ __global__ void k_coef_special(const long long *__restrict__ ids, const double *
 }
 
 // diag = ((((((Wx- + Wx+) + Wy-) + Wy+) + Wz-) + Wz+) + kappa), 0 on boundary.
-__global__ void k_diag(const double *__restrict__ Wx, const double *__restrict__ Wy,
-                       const double *__restrict__ Wz, const uint8_t *__restrict__ inside,
-                       GridGeo g, double kap_s, double *__restrict__ diag) {
-    long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (a >= g.N) return;
-    long long i = a % g.nx, j = (a / g.nx) % g.ny, k = a / ((long long)g.nx * g.ny);
-    if (is_bnd(g, i, j, k)) {
-        diag[a] = 0.0;
-        return;
+// An unlisted edge joins two nodes of one medium and has its pure weight, so a
+// node whose six edges are unlisted (its code bytes say so) has one of two
+// diagonals, formed by the same additions on the host: seven FP64 additions
+// a node had bound this kernel (257^3 228 us).
+__global__ void __launch_bounds__(32 * ROWS)
+k_diag(const double *__restrict__ Wx, const double *__restrict__ Wy, const double *__restrict__ Wz,
+       const uint8_t *__restrict__ code, GridGeo g, PadGeo p, double kap_s, double d_in, double d_out,
+       double *__restrict__ diag) {
+    const long long r = blockIdx.x * (long long)ROWS + threadIdx.y;
+    if (r >= (long long)g.ny * g.nz) return;
+    const Row w = row_of(g, r);
+    const bool rim = w.j == 0 || w.k == 0 || w.j == g.ny - 1 || w.k == g.nz - 1;
+    const long long sy = g.nx, sz = (long long)g.nx * g.ny;
+    for (int i = threadIdx.x; i < g.nx; i += 32) {
+        const long long a = w.a + i;
+        double s = 0.0;
+        if (!rim && i > 0 && i < g.nx - 1) {
+            const uint8_t *c = code + r * p.sx + i;
+            if (((c[0] & 0xE) | (c[-1] & 2) | (c[-p.sx] & 4) | (c[-p.sxy] & 8)) == 0) {
+                s = (c[0] & 1) ? d_in : d_out;
+            } else {
+                s = s + Wx[a - 1];
+                s = s + Wx[a];
+                s = s + Wy[a - sy];
+                s = s + Wy[a];
+                s = s + Wz[a - sz];
+                s = s + Wz[a];
+                s = s + ((c[0] & 1) ? 0.0 : kap_s);
+            }
+        }
+        diag[a] = s;
     }
-    long long sy = g.nx, sz = (long long)g.nx * g.ny;
-    double s = 0.0;
-    s = s + Wx[a - 1];
-    s = s + Wx[a];
-    s = s + Wy[a - sy];
-    s = s + Wy[a];
-    s = s + Wz[a - sz];
-    s = s + Wz[a];
-    diag[a] = s + (inside[a] ? 0.0 : kap_s);
 }
 
 __global__ void k_kappa(const uint8_t *__restrict__ inside, long long N, double kap_s,
@@ -132,77 +157,94 @@ __global__ void k_deposit(const double *__restrict__ atoms, long long na, GridGe
                          ti.c[2] + ((corner >> 2) & 1)};
     // position of the node, cell of the node in the atom cell list
     double xa[3];
+    float x32[3];
     int cc[3];
     for (int d = 0; d < 3; ++d) {
         xa[d] = g.o[d] + (double)node[d] * g.h;
+        x32[d] = (float)(xa[d] - cl.lo[d]);
         double u = floor((xa[d] - cl.lo[d]) / cl.cs);
         cc[d] = (u < -4.0) ? -4 : ((u > (double)cl.dim[d] + 4.0) ? cl.dim[d] + 4 : (int)u);
     }
-    // collect atoms whose cell has this node as a corner, in id order
+    // an atom whose cell has the node as a corner lies within h of it along
+    // every axis; FP32 (with the cell list's margin) passes the others over
+    const float reach = (float)(1.0001 * g.h) + cl.margin;
+    const int cx0 = max(cc[0] - 1, 0), cx1 = min(cc[0] + 1, cl.dim[0] - 1);
+    // atoms whose cell has this node as a corner, in id order, MAXC at a time
+    // (one round unless more than MAXC charges share the node)
     constexpr int MAXC = 32;
-    int ids[MAXC];
-    int m = 0;
-    for (int cz = cc[2] - 1; cz <= cc[2] + 1; ++cz) {
-        if (cz < 0 || cz >= cl.dim[2]) continue;
-        for (int cy = cc[1] - 1; cy <= cc[1] + 1; ++cy) {
-            if (cy < 0 || cy >= cl.dim[1]) continue;
-            for (int cx = cc[0] - 1; cx <= cc[0] + 1; ++cx) {
-                if (cx < 0 || cx >= cl.dim[0]) continue;
-                int cid = (cz * cl.dim[1] + cy) * cl.dim[0] + cx;
-                for (int s = cstart[cid]; s < cstart[cid + 1]; ++s) {
-                    int j = clist[s];
-                    Tri tj = (j == i) ? ti : tri_cell(g, X[j], Y[j], Z[j]);
+    int ids[MAXC], last = -1;
+    double acc = 0.0;
+    for (;;) {
+        int m = 0;
+        for (int cz = cc[2] - 1; cz <= cc[2] + 1; ++cz) {
+            if (cz < 0 || cz >= cl.dim[2] || cx0 > cx1) continue;
+            for (int cy = cc[1] - 1; cy <= cc[1] + 1; ++cy) {
+                if (cy < 0 || cy >= cl.dim[1]) continue;
+                const int c0 = (cz * cl.dim[1] + cy) * cl.dim[0];
+                for (int s = cstart[c0 + cx0], s1 = cstart[c0 + cx1 + 1]; s < s1; ++s) {
+                    const float4 b = cl.a32[s];
+                    if (fabsf(b.x - x32[0]) > reach || fabsf(b.y - x32[1]) > reach || fabsf(b.z - x32[2]) > reach)
+                        continue;
+                    const int j = clist[s];
+                    if (j <= last || (m == MAXC && j > ids[MAXC - 1])) continue;
+                    const Tri tj = (j == i) ? ti : tri_cell(g, X[j], Y[j], Z[j]);
                     bool corner_of = true;
                     for (int d = 0; d < 3; ++d) {
                         long long off = node[d] - tj.c[d];
                         if (off != 0 && off != 1) corner_of = false;
                     }
                     if (!corner_of) continue;
-                    if (m < MAXC) {
-                        int b = m - 1;
-                        while (b >= 0 && ids[b] > j) {
-                            ids[b + 1] = ids[b];
-                            --b;
-                        }
-                        ids[b + 1] = j;
-                        ++m;
+                    int q = m < MAXC ? m++ : MAXC - 1;  // a full list drops its largest id
+                    while (q > 0 && ids[q - 1] > j) {
+                        ids[q] = ids[q - 1];
+                        --q;
                     }
+                    ids[q] = j;
                 }
             }
         }
-    }
-    if (m == 0 || ids[0] != (int)i) return;  // another thread owns this node
-    double acc = 0.0;
-    for (int q = 0; q < m; ++q) {
-        int j = ids[q];
-        Tri tj = (j == i) ? ti : tri_cell(g, X[j], Y[j], Z[j]);
-        int dx = (int)(node[0] - tj.c[0]), dy = (int)(node[1] - tj.c[1]),
-            dz = (int)(node[2] - tj.c[2]);
-        double coef = coef0 * Q[j];
-        acc += coef * (tj.w[0][dx] * tj.w[1][dy] * tj.w[2][dz]);
+        if (last < 0 && (m == 0 || ids[0] != (int)i)) return;  // another thread owns this node
+        for (int q = 0; q < m; ++q) {
+            int j = ids[q];
+            Tri tj = (j == i) ? ti : tri_cell(g, X[j], Y[j], Z[j]);
+            int dx = (int)(node[0] - tj.c[0]), dy = (int)(node[1] - tj.c[1]),
+                dz = (int)(node[2] - tj.c[2]);
+            double coef = coef0 * Q[j];
+            acc += coef * (tj.w[0][dx] * tj.w[1][dy] * tj.w[2][dz]);
+        }
+        if (m < MAXC) break;
+        last = ids[MAXC - 1];
     }
     f[(node[2] * g.ny + node[1]) * g.nx + node[0]] = acc;
 }
 
 // f[a] += W_e phi_b for edges to Dirichlet nodes, in the order -x,+x,-y,+y,-z,+z.
-__global__ void k_lift(const double *__restrict__ Wx, const double *__restrict__ Wy,
-                       const double *__restrict__ Wz, const double *__restrict__ bc, GridGeo g,
-                       double *__restrict__ f) {
-    long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (a >= g.N) return;
-    long long i = a % g.nx, j = (a / g.nx) % g.ny, k = a / ((long long)g.nx * g.ny);
-    if (is_bnd(g, i, j, k)) return;
-    if (!(i == 1 || j == 1 || k == 1 || i == g.nx - 2 || j == g.ny - 2 || k == g.nz - 2)) return;
+// Only nodes next to the boundary have such edges: a warp takes a row, whole
+// rows in the outer layers and the two end nodes of the others.
+__global__ void __launch_bounds__(32 * ROWS)
+k_lift(const double *__restrict__ Wx, const double *__restrict__ Wy, const double *__restrict__ Wz,
+       const double *__restrict__ bc, GridGeo g, double *__restrict__ f) {
+    const long long r = blockIdx.x * (long long)ROWS + threadIdx.y;
+    if (r >= (long long)g.ny * g.nz) return;
+    const Row w = row_of(g, r);
+    const int j = w.j, k = w.k;
+    if (j == 0 || k == 0 || j == g.ny - 1 || k == g.nz - 1) return;
+    const bool layer = j == 1 || k == 1 || j == g.ny - 2 || k == g.nz - 2;
     const double *W[3] = {Wx, Wy, Wz};
-    long long st[3] = {1, g.nx, (long long)g.nx * g.ny};
-    long long c[3] = {i, j, k};
-    long long n[3] = {g.nx, g.ny, g.nz};
-    double v = f[a];
-    for (int d = 0; d < 3; ++d) {
-        if (c[d] - 1 == 0) v += W[d][a - st[d]] * bc[a - st[d]];
-        if (c[d] + 1 == n[d] - 1) v += W[d][a] * bc[a + st[d]];
+    const long long st[3] = {1, g.nx, (long long)g.nx * g.ny};
+    const int n[3] = {g.nx, g.ny, g.nz};
+    const int count = layer ? g.nx - 2 : (g.nx > 3 ? 2 : 1);
+    for (int q = threadIdx.x; q < count; q += 32) {
+        const int i = layer ? 1 + q : (q ? g.nx - 2 : 1);
+        const long long a = w.a + i;
+        const int c[3] = {i, j, k};
+        double v = f[a];
+        for (int d = 0; d < 3; ++d) {
+            if (c[d] - 1 == 0) v += W[d][a - st[d]] * bc[a - st[d]];
+            if (c[d] + 1 == n[d] - 1) v += W[d][a] * bc[a + st[d]];
+        }
+        f[a] = v;
     }
-    f[a] = v;
 }
 
 }  // namespace
@@ -232,8 +274,10 @@ pb_status assemble(pb_system *sys, cudaStream_t s) {
     PB_CUDA_TRY(cudaMemsetAsync(sys->code, 0, (size_t)((p.Np + 15) & ~15ll), s));
     PB_CUDA_TRY(cudaMemsetAsync(sys->bc, 0, sizeof(double) * N, s));
     const double eps_in = sys->p.eps_in, eps_out = sys->p.eps_out, h = geo.h;
-    k_coef_pure<<<cdiv(N, 256), 256, 0, s>>>(g->inside, geo, p, eps_in * h, eps_out * h, sys->W[0],
-                                             sys->W[1], sys->W[2], sys->code);
+    const dim3 rows(32, ROWS);
+    const unsigned rblocks = cdiv((long long)geo.ny * geo.nz, ROWS);
+    k_coef_pure<<<rblocks, rows, 0, s>>>(g->inside, geo, p, eps_in * h, eps_out * h, sys->W[0], sys->W[1], sys->W[2],
+                                         sys->code);
     PB_LAUNCH_CHECK();
     if (g->ncross > 0) {
         k_coef_special<<<cdiv(g->ncross, 256), 256, 0, s>>>(g->cid, g->calpha, g->ncross, geo, p,
@@ -242,8 +286,14 @@ pb_status assemble(pb_system *sys, cudaStream_t s) {
                                                             sys->w32[2], sys->code);
         PB_LAUNCH_CHECK();
     }
-    k_diag<<<cdiv(N, 256), 256, 0, s>>>(sys->W[0], sys->W[1], sys->W[2], g->inside, geo,
-                                        sys->kap_s, sys->diag);
+    // diagonals of a node with six pure edges, added as k_diag adds them
+    auto pure = [](double w, double kap) {
+        volatile double t = 0.0;
+        for (int q = 0; q < 6; ++q) t = t + w;
+        return (double)(t + kap);
+    };
+    k_diag<<<rblocks, rows, 0, s>>>(sys->W[0], sys->W[1], sys->W[2], sys->code, geo, p, sys->kap_s,
+                                    pure(eps_in * h, 0.0), pure(eps_out * h, sys->kap_s), sys->diag);
     PB_LAUNCH_CHECK();
     return PB_OK;
 }
@@ -259,9 +309,11 @@ pb_status deposit_rhs(pb_system *sys, cudaStream_t s) {
                                                        sys->rhs);
         PB_LAUNCH_CHECK();
     }
-    k_lift<<<cdiv(geo.N, 256), 256, 0, s>>>(sys->W[0], sys->W[1], sys->W[2], sys->bc, geo,
-                                           sys->rhs);
-    PB_LAUNCH_CHECK();
+    if (sys->p.bc != PB_BC_ZERO) {  // zero boundary values lift nothing
+        k_lift<<<cdiv((long long)geo.ny * geo.nz, ROWS), dim3(32, ROWS), 0, s>>>(sys->W[0], sys->W[1], sys->W[2],
+                                                                               sys->bc, geo, sys->rhs);
+        PB_LAUNCH_CHECK();
+    }
     return PB_OK;
 }
 
