@@ -146,6 +146,15 @@ __device__ __forceinline__ TgtLoad load_target(const TargetDesc &T, long long t)
     return r;
 }
 
+// 1/r of a pair from r^2; 0 for a point on itself.  The hardware instruction
+// alone: rsqrtf wraps it in a rescaling of subnormal arguments, that is of
+// distances below 1e-19 A, which are taken as 0 here (the same bits for all
+// others; surface sums of the 20,000-atom octree 84.7 -> 73.0 ms).
+__device__ __forceinline__ float rsqrt_pair(float r2) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(r2));
+    return r2 >= 1.17549435e-38f ? y : 0.f;
+}
 // Packed FP32 pair: lane .x works for the thread's first target, .y for its
 // second (one FP32x2 instruction does both).
 __device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
@@ -223,8 +232,7 @@ __device__ __forceinline__ void nb_tiles(float4 (*sp4)[4], const float4 *__restr
                                     sub2(tl[2], make_float2(p3.x, p3.y)));
                 }
                 const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-                const float2 ri = make_float2(r2.x > 0.f ? rsqrtf(r2.x) : 0.f,
-                                              r2.y > 0.f ? rsqrtf(r2.y) : 0.f);
+                const float2 ri = make_float2(rsqrt_pair(r2.x), rsqrt_pair(r2.y));
                 float2 v = __fmul2_rn(make_float2(p1.z, p1.w), ri);
                 if (SCREEN) {
                     v.x *= expf(-kscr * (r2.x * ri.x));
@@ -378,13 +386,60 @@ k_nbody(TargetDesc T, const float4 *__restrict__ shi, const float4 *__restrict__
     }
 }
 
+// 1/sqrt(a) in FP64 from the hardware's approximation y (PTX
+// rsqrt.approx.ftz.f64, good to about 2^-20): with e = 1 - a y^2,
+// 1/sqrt(a) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + O(e^3)), and e^3 is
+// below 2^-57, its term 5/16 of that.  Five FP64 operations; GB300 issues about two an SM
+// and clock, so their number is the cost of the FP64 sums below.  (Starting
+// from rsqrtf costs two conversions, which are FP64-rate too: 140 against 121
+// us for the pair sum of 2,000 atoms with the library's function.)  Zero and
+// subnormal arguments take the library's function.
+__device__ __forceinline__ double rsqrt_fp64(double a) {
+    if (__double2hiint(a) < 0x00100000) return rsqrt(a);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// exp(-u) for u >= 0 in FP64: -u = (n/64) ln 2 + f, |f| <= ln 2 / 128, the
+// Taylor polynomial of degree 5 of exp(f) (its remainder f^6/720 is below
+// 4e-17), and 2^(n/64) from the table of 64 values and an exponent.
+// ln 2 / 64 in two parts keeps f exact to rounding.  Ten FP64 operations.
+__device__ __forceinline__ double exp_neg_fp64(double u, const double *tab) {
+    constexpr double MAGIC = 6755399441055744.0;  // 1.5 * 2^52: rounds to an integer
+    constexpr double HI = 0x1.62e42fefa39efp-7, LO = 0x1.abc9e3b39803fp-62;
+    const double t = fma(u, -92.332482616893656, MAGIC);
+    const int n = __double2loint(t);
+    const double nd = t - MAGIC;
+    const double f = fma(nd, -LO, fma(nd, -HI, -u));
+    double p = 1.0 / 120.0;
+    p = fma(p, f, 1.0 / 24.0);
+    p = fma(p, f, 1.0 / 6.0);
+    p = fma(p, f, 0.5);
+    p = fma(p, f, 1.0);
+    p = fma(p, f, 1.0);
+    const double v = p * tab[n & 63];
+    const double r = __hiloint2double(__double2hiint(v) + (n >> 6) * 1048576, __double2loint(v));
+    return n < -64 * 1000 ? 0.0 : r;  // below 2^-1000
+}
+
 // Boundary values in FP64: they enter the linear system itself, so they are
-// summed exactly in double precision (atoms staged in shared memory).
-__global__ void __launch_bounds__(NB_THREADS)
+// summed in double precision (atoms staged in shared memory), in atom order.
+// FP64 issue binds: 24 operations a pair with screening (positions scaled by
+// k, so that the distance is the exponent), 13 without; the library's sqrt, exp
+// and division took about 70.  Blocks of 128 keep the
+// last wave full.  141 x 95 x 63 grid, 300 atoms, screened: 1,712 -> 780 us.
+constexpr int BT = 128;
+
+template <bool SCREEN>
+__global__ void __launch_bounds__(BT)
 k_boundary64(GridGeo g, const double *__restrict__ atoms, long long na, long long count, double k,
              double scale, double *__restrict__ bc) {
-    __shared__ double sx[NB_THREADS], sy[NB_THREADS], sz[NB_THREADS], sq[NB_THREADS];
-    long long t = blockIdx.x * (long long)NB_THREADS + threadIdx.x;
+    __shared__ double sx[BT], sy[BT], sz[BT], sq[BT], tab[64];
+    if (SCREEN && threadIdx.x < 64) tab[threadIdx.x] = exp2((double)threadIdx.x * 0.015625);
+    const double unit = SCREEN ? k : 1.0;  // 1 / length
+    long long t = blockIdx.x * (long long)BT + threadIdx.x;
     double p[3] = {0.0, 0.0, 0.0};
     long long i = 0, j = 0, kk = 0;
     if (t < count) {
@@ -392,26 +447,32 @@ k_boundary64(GridGeo g, const double *__restrict__ atoms, long long na, long lon
         p[0] = g.o[0] + (double)i * g.h;
         p[1] = g.o[1] + (double)j * g.h;
         p[2] = g.o[2] + (double)kk * g.h;
+        for (int q = 0; q < 3; ++q) p[q] *= unit;
     }
     double acc = 0.0;
-    for (long long base = 0; base < na; base += NB_THREADS) {
+    for (long long base = 0; base < na; base += BT) {
         long long si = base + threadIdx.x;
         __syncthreads();
         if (si < na) {
-            sx[threadIdx.x] = atoms[si];
-            sy[threadIdx.x] = atoms[na + si];
-            sz[threadIdx.x] = atoms[2 * na + si];
+            sx[threadIdx.x] = unit * atoms[si];
+            sy[threadIdx.x] = unit * atoms[na + si];
+            sz[threadIdx.x] = unit * atoms[2 * na + si];
             sq[threadIdx.x] = atoms[4 * na + si];
         }
         __syncthreads();
-        int m = (int)min((long long)NB_THREADS, na - base);
+        int m = (int)min((long long)BT, na - base);
+#pragma unroll 4
         for (int q = 0; q < m; ++q) {
-            double dx = p[0] - sx[q], dy = p[1] - sy[q], dz = p[2] - sz[q];
-            double r = sqrt((dx * dx + dy * dy) + dz * dz);
-            acc += (k > 0.0 ? sq[q] * exp(-k * r) : sq[q]) / r;
+            const double dx = p[0] - sx[q], dy = p[1] - sy[q], dz = p[2] - sz[q];
+            const double r2 = (dx * dx + dy * dy) + dz * dz;
+            const double y = rsqrt_fp64(r2);
+            if (SCREEN)
+                acc = fma(sq[q] * exp_neg_fp64(r2 * y, tab), y, acc);
+            else
+                acc = fma(sq[q], y, acc);
         }
     }
-    if (t < count) bc[(kk * g.ny + j) * g.nx + i] = scale * acc;
+    if (t < count) bc[(kk * g.ny + j) * g.nx + i] = scale * (unit * acc);
 }
 
 // Coulomb pair sum sum_{i<j} q_i q_j / r_ij in FP64 (the energy is a
@@ -419,7 +480,7 @@ k_boundary64(GridGeo g, const double *__restrict__ atoms, long long na, long lon
 // rounding).  Atoms in tiles of PT; block (a, b) of the nt x nt grid, a <= b,
 // takes the pairs i in tile a, j in tile b (j > i when a == b): thread t holds
 // atom i, tile b is staged in shared memory and taken in ascending order,
-// 1/r from the double-precision rsqrt.  The block's total goes to
+// 1/r from rsqrt_fp64.  The block's total goes to
 // part[b * nt + a] (zero for a > b); one block then adds the partials in
 // index order, so the sum is the same on every run.
 constexpr int PT = 128;
@@ -452,7 +513,7 @@ k_pairs64(const double *__restrict__ atoms, long long na, double *__restrict__ p
         for (int q = q0; q < m; ++q) {
             const double dx = px - sx[q], dy = py - sy[q], dz = pz - sz[q];
             const double r2 = (dx * dx + dy * dy) + dz * dz;
-            if (r2 > 0.0) acc += sq[q] * rsqrt(r2);
+            if (r2 > 0.0) acc = fma(sq[q], rsqrt_fp64(r2), acc);
         }
         mine = atoms[4 * na + i] * acc;
     }
@@ -511,8 +572,10 @@ pb_status nbody_boundary(pb_system *sys, cudaStream_t s) {
         2ll * geo.nx * geo.ny + (long long)(geo.nz - 2) * (2ll * geo.nx + 2ll * (geo.ny - 2));
     double scale = sys->lB / sys->p.eps_out;
     double k = sys->p.bc == PB_BC_DH ? sys->kD : 0.0;
-    k_boundary64<<<cdiv(count, NB_THREADS), NB_THREADS, 0, s>>>(geo, g->atoms, g->na, count, k,
-                                                                scale, sys->bc);
+    if (k > 0.0)
+        k_boundary64<true><<<cdiv(count, BT), BT, 0, s>>>(geo, g->atoms, g->na, count, k, scale, sys->bc);
+    else
+        k_boundary64<false><<<cdiv(count, BT), BT, 0, s>>>(geo, g->atoms, g->na, count, k, scale, sys->bc);
     PB_LAUNCH_CHECK();
     return PB_OK;
 }
