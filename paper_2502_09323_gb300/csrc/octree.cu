@@ -228,22 +228,25 @@ __global__ void __launch_bounds__(OT) k_oct_bbox(const double *__restrict__ atom
 // not near either).  Only an atom whose centre lies within reach = R_max +
 // dist of the box can pass the test, so the box scans the atom cell list
 // over the cells that meet the box grown by reach (one cell of margin on
-// each side); the flag is an OR over atoms, so the order does not matter.
+// each side); the flag is an OR over atoms, so the order does not matter.  A
+// warp takes a box, a lane a row of cells (one run of the cell-ordered atoms)
+// at a time; an FP32 test with the cell list's margin passes over atoms too
+// far to be near, and the warp stops at the first one that is.
 // On a de-refined domain the boxes of the levels coarser than h_tight that
 // meet the tight box [tlo, thi] are near too.
-__global__ void k_oct_near(const double *__restrict__ atoms, long long na, OctDev t, int level,
-                           double dist, double reach, CellList cl,
-                           const uint8_t *__restrict__ parent_near, uint8_t *__restrict__ near,
-                           bool tight, double3 tlo, double3 thi) {
+__global__ void __launch_bounds__(OT)
+k_oct_near(OctDev t, int level, double dist, double reach, CellList cl, const uint8_t *__restrict__ parent_near,
+           uint8_t *__restrict__ near, bool tight, double3 tlo, double3 thi) {
     const int nl = t.n0 << level;
     const long long nbox = (long long)nl * nl * nl;
-    const long long q = blockIdx.x * (long long)OT + threadIdx.x;
+    const long long q = (blockIdx.x * (long long)OT + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (q >= nbox) return;
     const int bx = (int)(q % nl), by = (int)((q / nl) % nl), bz = (int)(q / ((long long)nl * nl));
     if (level > 0) {
         const int pl = nl >> 1;
         if (!parent_near[((long long)(bz >> 1) * pl + (by >> 1)) * pl + (bx >> 1)]) {
-            near[q] = 0;
+            if (lane == 0) near[q] = 0;
             return;
         }
     }
@@ -256,10 +259,9 @@ __global__ void k_oct_near(const double *__restrict__ atoms, long long na, OctDe
     }
     if (tight && a[0] <= thi.x && b[0] >= tlo.x && a[1] <= thi.y && b[1] >= tlo.y &&
         a[2] <= thi.z && b[2] >= tlo.z) {
-        near[q] = 1;
+        if (lane == 0) near[q] = 1;
         return;
     }
-    const double *X = atoms, *Y = atoms + na, *Z = atoms + 2 * na, *R = atoms + 3 * na;
     int c0[3], c1[3];
     bool empty = false;
     for (int d = 0; d < 3; ++d) {
@@ -271,29 +273,44 @@ __global__ void k_oct_near(const double *__restrict__ atoms, long long na, OctDe
         c0[d] = empty ? 0 : (int)u0;
         c1[d] = empty ? -1 : (int)u1;
     }
-    uint8_t hit = 0;
-    for (int cz = c0[2]; cz <= c1[2] && !hit && !empty; ++cz)
-    for (int cy = c0[1]; cy <= c1[1] && !hit; ++cy)
-    for (int cx = c0[0]; cx <= c1[0] && !hit; ++cx) {
-    const int cid = (cz * cl.dim[1] + cy) * cl.dim[0] + cx;
-    for (int sidx = cl.start[cid]; sidx < cl.start[cid + 1] && !hit; ++sidx) {
-        const int i = cl.atom[sidx];
-        const double c[3] = {X[i], Y[i], Z[i]};
-        double tt[3], u[3];
-        for (int d = 0; d < 3; ++d) {
-            tt[d] = fmax(fmax(a[d] - c[d], 0.0), c[d] - b[d]);
-            u[d] = fmax(fabs(c[d] - a[d]), fabs(c[d] - b[d]));
+    // Boxes can lie far from the cell list: their FP32 coordinates carry the
+    // rounding of their own size.
+    float fa[3], fb[3], far = 0.f;
+    for (int d = 0; d < 3; ++d) {
+        fa[d] = (float)(a[d] - cl.lo[d]);
+        fb[d] = (float)(b[d] - cl.lo[d]);
+        far = fmaxf(far, fmaxf(fabsf(fa[d]), fabsf(fb[d])));
+    }
+    const float mg = cl.margin + 4e-6f * far, d32 = (float)dist;
+    const int ny = c1[1] - c0[1] + 1, rows = empty ? 0 : ny * (c1[2] - c0[2] + 1);
+    bool hit = false;
+    for (int r0 = 0; r0 < rows && !__any_sync(0xffffffffu, hit); r0 += 32) {
+        const int r = r0 + lane;
+        if (r >= rows) continue;
+        const int row = ((c0[2] + r / ny) * cl.dim[1] + c0[1] + r % ny) * cl.dim[0];
+        for (int s = cl.start[row + c0[0]], s1 = cl.start[row + c1[0] + 1]; s < s1 && !hit; ++s) {
+            const float4 f = cl.a32[s];
+            const float ex = fmaxf(fmaxf(fa[0] - f.x, 0.f), f.x - fb[0]), ey = fmaxf(fmaxf(fa[1] - f.y, 0.f), f.y - fb[1]),
+                        ez = fmaxf(fmaxf(fa[2] - f.z, 0.f), f.z - fb[2]), rm = f.w + d32 + mg;
+            if (ex * ex + ey * ey + ez * ez > 1.0001f * rm * rm) continue;
+            const double4 at = cl.a64[s];
+            const double c[3] = {at.x, at.y, at.z}, R = at.w;
+            double tt[3], u[3];
+            for (int d = 0; d < 3; ++d) {
+                tt[d] = fmax(fmax(a[d] - c[d], 0.0), c[d] - b[d]);
+                u[d] = fmax(fabs(c[d] - a[d]), fabs(c[d] - b[d]));
+            }
+            const double dmin2 = __dadd_rn(__dadd_rn(__dmul_rn(tt[0], tt[0]), __dmul_rn(tt[1], tt[1])),
+                                           __dmul_rn(tt[2], tt[2]));
+            const double dmax2 = __dadd_rn(__dadd_rn(__dmul_rn(u[0], u[0]), __dmul_rn(u[1], u[1])),
+                                           __dmul_rn(u[2], u[2]));
+            const double rin = __dmul_rn(R + dist, R + dist);
+            const double ro = R - dist;
+            if (dmin2 <= rin && (ro <= 0.0 || dmax2 >= __dmul_rn(ro, ro))) hit = true;
         }
-        const double dmin2 = __dadd_rn(__dadd_rn(__dmul_rn(tt[0], tt[0]), __dmul_rn(tt[1], tt[1])),
-                                       __dmul_rn(tt[2], tt[2]));
-        const double dmax2 = __dadd_rn(__dadd_rn(__dmul_rn(u[0], u[0]), __dmul_rn(u[1], u[1])),
-                                       __dmul_rn(u[2], u[2]));
-        const double rin = __dmul_rn(R[i] + dist, R[i] + dist);
-        const double ro = R[i] - dist;
-        if (dmin2 <= rin && (ro <= 0.0 || dmax2 >= __dmul_rn(ro, ro))) hit = 1;
     }
-    }
-    near[q] = hit;
+    hit = __any_sync(0xffffffffu, hit);
+    if (lane == 0) near[q] = hit;
 }
 
 struct LevelPtrs {
@@ -450,19 +467,34 @@ __device__ bool is_pure(const OctDev &t, const int P[3], int level) {
     return true;
 }
 
-// slot kinds and inside flags (from the finest-lattice classification)
-__global__ void k_oct_slots(OctDev t, const uint8_t *__restrict__ vin, GridGeo vg,
-                            uint8_t *__restrict__ inside, uint8_t *__restrict__ okind) {
-    const long long a = blockIdx.x * (long long)OT + threadIdx.x;
-    if (a >= t.N) return;
+// slot kinds and inside flags (from the finest-lattice classification).  In a
+// brick whose 26 neighbours (inside the domain) have its level every node is
+// pure or on the boundary: all leaves that touch the node or its six
+// neighbours are among them.  The other bricks test each node.
+__global__ void __launch_bounds__(OT)
+k_oct_slots(OctDev t, const uint8_t *__restrict__ vin, GridGeo vg, uint8_t *__restrict__ inside,
+            uint8_t *__restrict__ okind) {
+    const long long a = blockIdx.x * (long long)OT + threadIdx.x;  // half a brick a block
     int P[3], level;
     slot_pos(t, a, P, level);
+    bool same = true;
+    if (threadIdx.x < 27) {
+        const int4 L = t.blow[a >> 9];
+        const int S = spc(t.Lmax, L.w), q = threadIdx.x;
+        const int x = (L.x >> 3) + (q % 3 - 1) * S, y = (L.y >> 3) + (q / 3 % 3 - 1) * S, z = (L.z >> 3) + (q / 9 - 1) * S;
+        if (x >= 0 && y >= 0 && z >= 0 && x < t.nf && y < t.nf && z < t.nf) same = t.lev[cidx(t, x, y, z)] == L.w;
+    }
+    const bool uniform = __syncthreads_and(same);
     inside[a] = vin[((long long)P[2] * vg.ny + P[1]) * vg.nx + P[0]];
-    int k = pos_kind(t, P[0], P[1], P[2]);
     uint8_t kind;
-    if (k == 1) kind = 1;
-    else if (k == 2) kind = 2;
-    else kind = is_pure(t, P, level) ? 0 : 3;
+    if (uniform) {
+        kind = P[0] == 0 || P[1] == 0 || P[2] == 0 ? 1 : 0;  // an owned node has no coordinate NL
+    } else {
+        const int k = pos_kind(t, P[0], P[1], P[2]);
+        if (k == 1) kind = 1;
+        else if (k == 2) kind = 2;
+        else kind = is_pure(t, P, level) ? 0 : 3;
+    }
     okind[a] = kind;
 }
 
@@ -641,35 +673,43 @@ __device__ __forceinline__ void row_add(RowAcc &r, long long col, double v) {
     ++r.n;
 }
 
+// Kind (0 regular, 1 boundary, 2 hanging) and owning slot (-1 if none) of a
+// position: a node off the lattice of the leaf that contains it is hanging,
+// the others' kinds are in okind.
+struct PosInfo {
+    int kind;
+    long long slot;
+};
+__device__ __forceinline__ PosInfo pos_info(const OctDev &t, int px, int py, int pz) {
+    PosInfo p;
+    p.slot = owner_slot(t, px, py, pz);
+    if (px == 0 || py == 0 || pz == 0 || px == t.NL || py == t.NL || pz == t.NL) p.kind = 1;
+    else p.kind = p.slot < 0 || t.okind[p.slot] == 2 ? 2 : 0;
+    return p;
+}
+
 // contribution v * x~(Q): a regular node is a column, a boundary node moves
 // to the right-hand side, a hanging node spreads over its parents
-__device__ void row_add_pos(const OctDev &t, const BcDesc &bd, RowAcc &r, const int Q[3], double v) {
-    const int k = pos_kind(t, Q[0], Q[1], Q[2]);
-    if (k == 0) {
-        const long long c = owner_slot(t, Q[0], Q[1], Q[2]);
-        row_add(r, c, v);
-    } else if (k == 1) {
+__device__ void row_add_pos(const OctDev &t, const BcDesc &bd, RowAcc &r, const int Q[3], const PosInfo &p, double v) {
+    if (p.kind == 0) {
+        row_add(r, p.slot, v);
+    } else if (p.kind == 1) {
         r.lift -= v * bc_at(t, bd, Q);
     } else {
         int par[4][3];
         double w;
         const int np = hang_parents(t, Q, par, w);
         for (int q = 0; q < np; ++q) {
-            const int pk = pos_kind(t, par[q][0], par[q][1], par[q][2]);
-            if (pk == 0) {
-                row_add(r, owner_slot(t, par[q][0], par[q][1], par[q][2]), v * w);
-            } else if (pk == 1) {
+            const PosInfo pp = pos_info(t, par[q][0], par[q][1], par[q][2]);
+            if (pp.kind == 0) {
+                row_add(r, pp.slot, v * w);
+            } else if (pp.kind == 1) {
                 r.lift -= v * w * bc_at(t, bd, par[q]);
             } else {
                 r.err |= OERR_HANGING_PARENT;
             }
         }
     }
-}
-
-__device__ bool pos_inside(const OctDev &t, const uint8_t *inside, const int P[3]) {
-    const long long s = owner_slot(t, P[0], P[1], P[2]);
-    return s >= 0 && inside[s];
 }
 
 // row of A = P^T K P for the regular node at P (a level-transition row);
@@ -707,7 +747,7 @@ __device__ void transition_row(const OctDev &t, const BcDesc &bd, const uint8_t 
                     const int nz = (ox != 0) + (oy != 0) + (oz != 0);
                     if (nz == 0 || nz == 3) continue;
                     const int Q[3] = {P[0] + ox * half, P[1] + oy * half, P[2] + oz * half};
-                    if (pos_kind(t, Q[0], Q[1], Q[2]) != 2) continue;
+                    if (pos_info(t, Q[0], Q[1], Q[2]).kind != 2) continue;
                     int smin;
                     const int sq = touch_spacings(t, Q[0], Q[1], Q[2], smin);
                     if (sq != svals[q]) continue;
@@ -729,7 +769,8 @@ __device__ void transition_row(const OctDev &t, const BcDesc &bd, const uint8_t 
     for (int qa = 0; qa < na; ++qa) {
         const int *A = apos[qa];
         const double wa = aw[qa];
-        if (pos_inside(t, inside, A)) r.err |= OERR_SOLUTE_TRANSITION;
+        const PosInfo pa = pos_info(t, A[0], A[1], A[2]);
+        if (pa.slot >= 0 && inside[pa.slot]) r.err |= OERR_SOLUTE_TRANSITION;
         double kaa = 0.0;
         for (int o = 0; o < 8; ++o) {
             int c[3], sg[3];
@@ -744,13 +785,14 @@ __device__ void transition_row(const OctDev &t, const BcDesc &bd, const uint8_t 
             for (int d = 0; d < 3; ++d) {
                 int B[3] = {A[0], A[1], A[2]};
                 B[d] += sg[d] * s;
-                if (pos_inside(t, inside, B)) r.err |= OERR_SOLUTE_TRANSITION;
+                const PosInfo pb = pos_info(t, B[0], B[1], B[2]);
+                if (pb.slot >= 0 && inside[pb.slot]) r.err |= OERR_SOLUTE_TRANSITION;
                 kaa += we;
-                row_add_pos(t, bd, r, B, -wa * we);
+                row_add_pos(t, bd, r, B, pb, -wa * we);
             }
             kaa += lc.kap[l] * 0.125;
         }
-        row_add_pos(t, bd, r, A, wa * kaa);
+        row_add_pos(t, bd, r, A, pa, wa * kaa);
     }
     // columns in increasing order
     for (int q = 1; q < r.n; ++q) {
@@ -782,10 +824,16 @@ __global__ void k_oct_tr_rowmap(const int *__restrict__ tr_slot, long long ntr, 
     if (r < ntr) tr_row[tr_slot[r]] = (int)r;
 }
 
+// Entries of a row that the counting pass keeps (rows have 11 on average, 21
+// at most on the trees measured), row r's q-th at q * ntr + r; longer rows
+// are formed again when they are written out.
+constexpr int KEEP = 24;
+
 __global__ void __launch_bounds__(128)
 k_oct_tr_count(OctDev t, BcDesc bd, const uint8_t *__restrict__ inside, LevelConst lc,
                double eps_out, const int *__restrict__ tr_slot, long long ntr,
-               long long *__restrict__ nnz, unsigned *__restrict__ err) {
+               long long *__restrict__ nnz, unsigned *__restrict__ err, int *__restrict__ kcol,
+               double *__restrict__ kval) {
     const long long r = blockIdx.x * 128ll + threadIdx.x;
     if (r >= ntr) return;
     int P[3], level;
@@ -795,33 +843,50 @@ k_oct_tr_count(OctDev t, BcDesc bd, const uint8_t *__restrict__ inside, LevelCon
     zero.kind = PB_BC_ZERO;  // counting needs no boundary values
     transition_row(t, zero, inside, lc, eps_out, P, acc);
     nnz[r] = acc.n;
+    for (int q = 0; q < acc.n && q < KEEP; ++q) {
+        kcol[q * ntr + r] = acc.col[q];
+        kval[q * ntr + r] = acc.val[q];
+    }
     if (acc.err) atomicOr(err, acc.err);
 }
 
+// kcol, kval: the rows of the counting pass (null: none; they carry no lift)
 __global__ void __launch_bounds__(128)
 k_oct_tr_fill(OctDev t, BcDesc bd, const uint8_t *__restrict__ inside, LevelConst lc,
               double eps_out, const int *__restrict__ tr_slot, long long ntr,
               const long long *__restrict__ ptr, int *__restrict__ col, double *__restrict__ val,
               float *__restrict__ val32, double *__restrict__ tdiag, double *__restrict__ diag,
-              double *__restrict__ lift) {
+              double *__restrict__ lift, const int *__restrict__ kcol, const double *__restrict__ kval) {
     const long long r = blockIdx.x * 128ll + threadIdx.x;
     if (r >= ntr) return;
     const long long a = tr_slot[r];
-    int P[3], level;
-    slot_pos(t, a, P, level);
-    RowAcc acc;
-    transition_row(t, bd, inside, lc, eps_out, P, acc);
-    const long long p0 = ptr[r];
+    const long long p0 = ptr[r], n = ptr[r + 1] - p0;
     double dg = 0.0;
-    for (int q = 0; q < acc.n; ++q) {
-        col[p0 + q] = acc.col[q];
-        val[p0 + q] = acc.val[q];
-        val32[p0 + q] = (float)acc.val[q];
-        if (acc.col[q] == (int)a) dg = acc.val[q];
+    if (kcol && n <= KEEP && bd.kind == PB_BC_ZERO) {
+        for (int q = 0; q < (int)n; ++q) {
+            const int c = kcol[q * ntr + r];
+            const double v = kval[q * ntr + r];
+            col[p0 + q] = c;
+            val[p0 + q] = v;
+            val32[p0 + q] = (float)v;
+            if (c == (int)a) dg = v;
+        }
+        lift[r] = 0.0;
+    } else {
+        int P[3], level;
+        slot_pos(t, a, P, level);
+        RowAcc acc;
+        transition_row(t, bd, inside, lc, eps_out, P, acc);
+        for (int q = 0; q < acc.n; ++q) {
+            col[p0 + q] = acc.col[q];
+            val[p0 + q] = acc.val[q];
+            val32[p0 + q] = (float)acc.val[q];
+            if (acc.col[q] == (int)a) dg = acc.val[q];
+        }
+        lift[r] = acc.lift;
     }
     tdiag[r] = dg;
     diag[a] = dg;
-    lift[r] = acc.lift;
 }
 
 // ================================================================ rhs ===
@@ -1561,6 +1626,8 @@ __global__ void __launch_bounds__(OB, MODE == OM_U ? 3 : 4) k_oct_pure(OctArgs<T
 
 // FP64 true residual r = f - A x (x = phi on the unknowns), z = r / D in
 // the inner solver's precision; |r|^2 and r.z to the CG state
+// A thread takes every (grid size)-th slot (the blocks resident on the GPU), so
+// that a launch ends with few partial sums.
 template <typename TZ>
 __global__ void __launch_bounds__(OT)
 k_oct_residual(OctDev t, const double *__restrict__ phi, const double *__restrict__ f,
@@ -1569,33 +1636,33 @@ k_oct_residual(OctDev t, const double *__restrict__ phi, const double *__restric
                const int *__restrict__ tr_row, const long long *__restrict__ tr_ptr,
                const int *__restrict__ tr_col, const double *__restrict__ tr_val,
                TZ *__restrict__ zout, CgState *st, double *partials) {
-    const long long a = blockIdx.x * (long long)OT + threadIdx.x;
     double rr = 0.0, rz = 0.0;
-    if (a < t.N) {
+    for (long long a = blockIdx.x * (long long)OT + threadIdx.x; a < t.N; a += (long long)gridDim.x * OT) {
         const uint8_t kd = t.okind[a];
-        if (kd == 0 || kd == 3) {
-            double s;
-            if (kd == 0) {
-                const double *W[3] = {W0, W1, W2};
-                s = diag[a] * phi[a];
-                for (int d = 0; d < 3; ++d) {
-                    const long long m = nbr_slot(t, a, 2 * d), pn = nbr_slot(t, a, 2 * d + 1);
-                    if (m >= 0 && t.okind[m] != 1) s -= W[d][m] * phi[m];
-                    if (pn >= 0 && t.okind[pn] != 1) s -= W[d][a] * phi[pn];
-                }
-            } else {
-                const int r = tr_row[a];
-                s = 0.0;
-                for (long long e = tr_ptr[r]; e < tr_ptr[r + 1]; ++e) s += tr_val[e] * phi[tr_col[e]];
+        if (kd != 0 && kd != 3) continue;
+        const double dg = diag[a];
+        double s;
+        if (kd == 0) {
+            const double *W[3] = {W0, W1, W2};
+            s = dg * phi[a];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const long long m = nbr_slot(t, a, 2 * d), pn = nbr_slot(t, a, 2 * d + 1);
+                if (m >= 0 && t.okind[m] != 1) s -= W[d][m] * phi[m];
+                if (pn >= 0 && t.okind[pn] != 1) s -= W[d][a] * phi[pn];
             }
-            const double r = f[a] - s;
-            TZ z;
-            if (sizeof(TZ) == 4) z = (TZ)((float)r / (float)diag[a]);
-            else z = (TZ)(r / diag[a]);
-            zout[a] = z;
-            rr = r * r;
-            rz = r * (double)z;
+        } else {
+            const int r = tr_row[a];
+            s = 0.0;
+            for (long long e = tr_ptr[r]; e < tr_ptr[r + 1]; ++e) s += tr_val[e] * phi[tr_col[e]];
         }
+        const double r = f[a] - s;
+        TZ z;
+        if (sizeof(TZ) == 4) z = (TZ)((float)r / (float)dg);
+        else z = (TZ)(r / dg);
+        zout[a] = z;
+        rr += r * r;
+        rz += r * (double)z;
     }
     double mine[2] = {rr, rz}, tot[2];
     if (olast_total<OT, 2>(&st->counter, partials, mine, tot)) {
@@ -1835,10 +1902,9 @@ pb_status oct_build(pb_grid *g, const pb_grid_spec *spec, cudaStream_t s) {
         near[l] = (uint8_t *)dalloc(nl * nl * nl, s);
         split[l] = (uint8_t *)dalloc(nl * nl * nl, s);
         if (!near[l] || !split[l]) return PB_ERR_OOM;
-        k_oct_near<<<cdiv(nl * nl * nl, OT), OT, 0, s>>>(g->atoms, na, t, l, dist,
-                                                          hinfo.rmax + dist, g->cells,
-                                                          l > 0 ? near[l - 1] : nullptr, near[l],
-                                                          l < Lt, tlo, thi);
+        k_oct_near<<<cdiv(32 * nl * nl * nl, OT), OT, 0, s>>>(t, l, dist, hinfo.rmax + dist, g->cells,
+                                                              l > 0 ? near[l - 1] : nullptr, near[l], l < Lt, tlo,
+                                                              thi);
         PB_LAUNCH_CHECK();
         np.p[l] = near[l];
         sp.p[l] = split[l];
@@ -1910,7 +1976,7 @@ pb_status oct_build(pb_grid *g, const pb_grid_spec *spec, cudaStream_t s) {
     dfree(vals2, s);
     k_oct_nbr<<<cdiv(t.nb, OT), OT, 0, s>>>(t, t.bnbr);
     PB_LAUNCH_CHECK();
-    k_oct_slots<<<cdiv(t.N, OT), OT, 0, s>>>(t, g->inside, vg, sin, t.okind);
+    k_oct_slots<<<cdiv(t.N, OT), OT, 0, s>>>(t, g->inside, vg, sin, t.okind);  // N is a multiple of 512
     PB_LAUNCH_CHECK();
 
     // listed edges renumbered by slot, in increasing order
@@ -2017,7 +2083,7 @@ void oct_grid_free(pb_grid *g, cudaStream_t s) {
 }
 
 // ------------------------------------------------------- coefficients ---
-pb_status oct_boundary_rhs(pb_system *sys, cudaStream_t s) {
+static pb_status oct_boundary_rhs_rows(pb_system *sys, const int *kcol, const double *kval, cudaStream_t s) {
     pb_grid *g = sys->g;
     const OctDev &t = g->ot;
     OctSys *os = sys->os;
@@ -2034,7 +2100,7 @@ pb_status oct_boundary_rhs(pb_system *sys, cudaStream_t s) {
         k_oct_tr_fill<<<cdiv(os->ntr, 128), 128, 0, s>>>(t, bd, g->inside, lc, sys->p.eps_out,
                                                          os->tr_slot, os->ntr, os->tr_ptr, os->tr_col,
                                                          os->tr_val, os->tr_val32, os->tr_diag,
-                                                         sys->diag, tlift);
+                                                         sys->diag, tlift, kcol, kval);
         PB_LAUNCH_CHECK();
     }
     PB_CUDA_TRY(cudaMemsetAsync(sys->rhs, 0, sizeof(double) * N, s));
@@ -2060,6 +2126,8 @@ pb_status oct_boundary_rhs(pb_system *sys, cudaStream_t s) {
     }
     return PB_OK;
 }
+
+pb_status oct_boundary_rhs(pb_system *sys, cudaStream_t s) { return oct_boundary_rhs_rows(sys, nullptr, nullptr, s); }
 
 pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
     pb_grid *g = sys->g;
@@ -2132,6 +2200,8 @@ pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
     if (!err) return PB_ERR_OOM;
     PB_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(unsigned), s));
     long long nnz = 0;
+    int *kcol = nullptr;
+    double *kval = nullptr;
     if (ntr > 0) {
         // rows in increasing slot order
         size_t tb = 0;
@@ -2146,8 +2216,11 @@ pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
         long long *rn = (long long *)dalloc(sizeof(long long) * ntr, s);
         if (!rn) return PB_ERR_OOM;
         const BcDesc bd = bc_desc(sys);
+        kcol = (int *)dalloc(sizeof(int) * KEEP * ntr, s);
+        kval = (double *)dalloc(sizeof(double) * KEEP * ntr, s);
+        if (!kcol || !kval) return PB_ERR_OOM;
         k_oct_tr_count<<<cdiv(ntr, 128), 128, 0, s>>>(t, bd, g->inside, lc, sys->p.eps_out,
-                                                       os->tr_slot, ntr, rn, err);
+                                                       os->tr_slot, ntr, rn, err, kcol, kval);
         PB_LAUNCH_CHECK();
         tb = 0;
         PB_CUDA_TRY(cub::DeviceScan::InclusiveSum(nullptr, tb, rn, os->tr_ptr + 1, (int)ntr, s));
@@ -2167,6 +2240,8 @@ pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
     PB_CUDA_TRY(cudaStreamSynchronize(s));
     dfree(err, s);
     if (herr) {
+        dfree(kcol, s);
+        dfree(kval, s);
         set_error("octree: inconsistent level-transition row (flags %u)", herr);
         return PB_ERR_ARG;
     }
@@ -2190,7 +2265,10 @@ pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
     os->npart = 2 * (int)std::max<long long>(cdiv(ntr1, OT), 1) + 8;
     os->partials = (double *)dalloc(sizeof(double) * os->npart, s);
     if (!os->tr_col || !os->tr_val || !os->tr_val32 || !os->partials) return PB_ERR_OOM;
-    return oct_boundary_rhs(sys, s);
+    const pb_status brc = oct_boundary_rhs_rows(sys, kcol, kval, s);
+    dfree(kcol, s);
+    dfree(kval, s);
+    return brc;
 }
 
 void oct_system_free(pb_system *sys, cudaStream_t s) {
@@ -2398,12 +2476,13 @@ pb_status oct_sync(pb_system *sys, cudaStream_t s) {
 pb_status oct_residual(pb_system *sys, bool fp32_out, cudaStream_t s) {
     const OctDev &t = sys->g->ot;
     OctSys *os = sys->os;
+    const unsigned blocks = (unsigned)std::min<long long>(cdiv(t.N, OT), 8ll * num_sms());
     if (fp32_out)
-        k_oct_residual<float><<<cdiv(t.N, OT), OT, 0, s>>>(
+        k_oct_residual<float><<<blocks, OT, 0, s>>>(
             t, sys->phi, sys->rhs, sys->W[0], sys->W[1], sys->W[2], sys->diag, os->tr_row,
             os->tr_ptr, os->tr_col, os->tr_val, sys->z32, sys->st, sys->partials);
     else
-        k_oct_residual<double><<<cdiv(t.N, OT), OT, 0, s>>>(
+        k_oct_residual<double><<<blocks, OT, 0, s>>>(
             t, sys->phi, sys->rhs, sys->W[0], sys->W[1], sys->W[2], sys->diag, os->tr_row,
             os->tr_ptr, os->tr_col, os->tr_val, sys->z64, sys->st, sys->partials);
     PB_LAUNCH_CHECK();
