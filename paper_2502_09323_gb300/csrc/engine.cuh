@@ -252,24 +252,24 @@ int engine_chunk(const Engine *e) { return e->mg ? 2 : e->chunk; }
 bool engine_capture(Engine *e) {
     const int depth = e->depth, g = e->mg ? depth : mg::LMAX;
     if (e->exec[g]) return true;
-    static const unsigned rd0 = mg_resident(k_mg_down<true, false>, mg::DNT), rd1 = mg_resident(k_mg_down<false, false>, mg::DNT),
-                          ru0 = mg_resident(k_mg_up<true, false>, mg::UNT), ru1 = mg_resident(k_mg_up<false, false>, mg::UNT);
+    static const unsigned rd0 = mg_resident(k_mg_down0<false>, mg::D0NT), rd1 = mg_resident(k_mg_down<false>, mg::DNT),
+                          ru0 = mg_resident(k_mg_up0<false>, mg::U0NT), ru1 = mg_resident(k_mg_up<false>, mg::UNT);
     const mg::Entry none{};
     ENG_TRY(cudaStreamBeginCapture(e->cs, cudaStreamCaptureModeThreadLocal), "capture");
     for (int c = 0; c < engine_chunk(e); ++c) {
         for (int l = 0; l < depth; ++l)
             if (l == 0)
-                k_mg_down<true, false><<<rd0, mg::DNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                k_mg_down0<false><<<rd0, mg::D0NT, 0, e->cs>>>(e->dmg, e->dhead, 0, none);
             else
-                k_mg_down<false, false><<<rd1, mg::DNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                k_mg_down<false><<<rd1, mg::DNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
         if (depth > 0)
             k_mg_bottom<mg::Entry, false>
                 <<<e->cap, mg::BOT_T, mg::BOT_BYTES<float> * mg::BOT_NODES<float>, e->cs>>>(e->dmg, e->dhead, none);
         for (int l = depth - 1; l >= 0; --l)
             if (l == 0)
-                k_mg_up<true, false><<<ru0, mg::UNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                k_mg_up0<false><<<ru0, mg::U0NT, 0, e->cs>>>(e->dmg, e->dhead, 0, none);
             else
-                k_mg_up<false, false><<<ru1, mg::UNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                k_mg_up<false><<<ru1, mg::UNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
         tma_launch<MODE_P>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
         tma_launch<MODE_U>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
     }

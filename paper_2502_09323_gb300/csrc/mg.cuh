@@ -24,13 +24,9 @@
 // system in one launch (k_mg_bottom).  The up kernel of level 0 also sums
 // rho = r.z and takes the CG step beta = rho / rho_old.
 //
-// Measured (GB300, solves to 1e-12): 257^3 155.6 -> 16.4 ms (1,127 -> 30
+// Measured (GB300, solves to 1e-12): 257^3 155.6 -> 13.4 ms (1,127 -> 30
 // iterations), 65^3 30.1 -> 2.1 ms, a batch of 24 systems of 97^3 to 161^3
-// 229 -> 55 ms.  A first form of the kernels, a node a thread with all
-// neighbours in shared memory, took 176 us (down) and 152 us (up) on 257^3
-// and 22 us in the bottom kernel; units of four nodes with the planes in
-// registers take 102 and 139 us, most of it instruction issue and load
-// latency (16 % of DRAM bandwidth, 38 % of the warps resident).
+// 229 -> 51 ms.
 //
 // Bounds: down reads s and a code byte per fine node and writes an eighth of
 // a value; up reads s, an eighth of a value and a code byte and writes z.
@@ -50,7 +46,7 @@ constexpr int BOT_BYTES = 7 * sizeof(T) + 6;
 template <typename T>
 constexpr int BOT_NODES = sizeof(T) == 4 ? 6600 : 3600;
 constexpr int SWEEPS = 8;           // Jacobi sweeps on the coarsest level
-// Tiles.  Down: 32 x 6 coarse nodes from node (1 + 32 bx, 1 + 6 by), whose
+// Tiles of the coarse levels.  Down: 32 x 6 coarse nodes from node (1 + 32 bx, 1 + 6 by), whose
 // residuals are 13 rows of 17 units of 4 fine nodes; the first and the last
 // unit of a row need no neighbour outside it.  221 threads take a unit each,
 // 34 more the halo rows.  Up: 64 x 16 fine nodes from (64 bx, 1 + 16 by), 16
@@ -83,6 +79,7 @@ struct Entry {
     int nu0;                        // their number
     void *blob;                     // of the bottom kernel (k_mg_pack)
     int bot;                        // its nodes, rounded up to a multiple of 8
+    CUtensorMap sd, cd, su, cu;     // s and codes of level 0: boxes of k_mg_down0, of k_mg_up0
 };
 
 // launch totals of a table, read on the device
@@ -95,7 +92,8 @@ struct Head {
 __host__ __device__ inline int ditems(const Entry &e, int l) {
     if (l >= e.nbot) return 0;
     const Lev &c = e.lev[l + 1];
-    return ((c.nx - 2 + CX - 1) / CX) * ((c.ny - 2 + CY - 1) / CY) * ((c.nz - 2 + e.dk[l] - 1) / e.dk[l]);
+    const int cy = l == 0 && e.code ? 8 : CY;  // k_mg_down0's tile
+    return ((c.nx - 2 + CX - 1) / CX) * ((c.ny - 2 + cy - 1) / cy) * ((c.nz - 2 + e.dk[l] - 1) / e.dk[l]);
 }
 __host__ __device__ inline int uitems(const Entry &e, int l) {
     if (l >= e.nbot) return 0;
@@ -107,23 +105,15 @@ __device__ __forceinline__ float quotient(float a, float b) { return __fdividef(
 __device__ __forceinline__ double quotient(double a, double b) { return a / b; }
 
 __device__ __forceinline__ float4 f4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
 
 // Operator data of a unit (4 nodes of a row) in one plane.  Level 0: its code
-// bytes and those of the row below.  Coarse levels: the weights and the
-// diagonal.
-template <bool FINE>
-struct Op;
-template <>
-struct Op<true> {
-    uint32_t c = 0, cy = 0, cl = 0;  // own, row j - 1, node i - 1
-    __device__ __forceinline__ void load(const Entry &e, const Lev &L, int p) {
-        c = *reinterpret_cast<const uint32_t *>(e.code + p);
-        cy = *reinterpret_cast<const uint32_t *>(e.code + p - L.sx);
-        cl = e.code[p - 1];
-    }
+// bytes, those of the row below and of the node to the left.  Coarse levels:
+// the weights and the diagonal.
+struct Codes {
+    uint32_t c = 0, cy = 0, cl = 0;
 };
-template <>
-struct Op<false> {
+struct Weights {
     float4 x = {}, y = {}, z = {}, ym = {}, d = {1.f, 1.f, 1.f, 1.f};
     float xl = 0.f;
     __device__ __forceinline__ void load(const Entry &, const Lev &L, int p) {
@@ -137,45 +127,40 @@ struct Op<false> {
 };
 
 // sum over the six faces of W times the neighbour, and the diagonal, of the
-// nodes of a unit; o: plane k, b: plane k - 1; l, r: neighbours in x
-__device__ __forceinline__ void face_sums(const Entry &e, const Lev &L, int p, const Op<true> &o, const Op<true> &b,
-                                          const float4 &x, float l, float r, const float4 &ym, const float4 &yp,
-                                          const float4 &zm, const float4 &zp, float (&sum)[4], float (&d)[4]) {
+// nodes of a unit; l, r: neighbours in x.  Level 0, a unit with listed edges:
+// below holds its codes in plane k - 1.  The weights' arrays are dense, so the
+// whole unit's are loaded in six independent loads and the unlisted ones are
+// passed over: a load under a condition of its own for each face waited for
+// the one before it (about 10,000 cycles a plane for the slowest warp).
+__device__ __forceinline__ void listed_sums(const CoefC32 &cp, const Lev &L, int p, const Codes &o, uint32_t below,
+                                            const float4 &x, float l, float r, const float4 &ym, const float4 &yp,
+                                            const float4 &zm, const float4 &zp, float (&sum)[4], float (&d)[4]) {
+    const float4 g1 = ldg4(cp.wx + p), g2 = ldg4(cp.wy + p - L.sx), g3 = ldg4(cp.wy + p),
+                 g4 = ldg4(cp.wz + p - L.sxy), g5 = ldg4(cp.wz + p);
+    const float g0 = __ldg(cp.wx + p - 1);
     const float xx[6] = {l, x.x, x.y, x.z, x.w, r};
-    const float m[4] = {ym.x + yp.x, ym.y + yp.y, ym.z + yp.z, ym.w + yp.w};
-    const float n[4] = {zm.x + zp.x, zm.y + zp.y, zm.z + zp.z, zm.w + zp.w};
-    const uint32_t cx = (o.c << 8) | o.cl;
-    const uint32_t special = (o.c & 0x0E0E0E0Eu) | (cx & 0x02020202u) | (o.cy & 0x04040404u) | (b.c & 0x08080808u);
-    if (special == 0u) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const bool in = (o.c >> (8 * q)) & 1u;
-            const float w = in ? e.cp.w_in : e.cp.w_out;
-            d[q] = in ? e.dg_in : e.dg_out;
-            sum[q] = w * ((xx[q] + xx[q + 2]) + m[q] + n[q]);
-        }
-        return;
-    }
     const float my[4] = {ym.x, ym.y, ym.z, ym.w}, py[4] = {yp.x, yp.y, yp.z, yp.w};
     const float mz[4] = {zm.x, zm.y, zm.z, zm.w}, pz[4] = {zp.x, zp.y, zp.z, zp.w};
+    const float v1[4] = {g1.x, g1.y, g1.z, g1.w}, v2[4] = {g2.x, g2.y, g2.z, g2.w}, v3[4] = {g3.x, g3.y, g3.z, g3.w};
+    const float v4[4] = {g4.x, g4.y, g4.z, g4.w}, v5[4] = {g5.x, g5.y, g5.z, g5.w};
     float wl = 0.f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const uint32_t c = o.c >> (8 * q);
-        const float w = (c & 1u) ? e.cp.w_in : e.cp.w_out;
-        if (q == 0) wl = (o.cl & 2u) ? __ldg(e.cp.wx + p - 1) : w;
+        const float w = (c & 1u) ? cp.w_in : cp.w_out;
+        if (q == 0) wl = (o.cl & 2u) ? g0 : w;
         else wl = ((o.c >> (8 * q - 8)) & 2u) ? wl : w;
-        const float w1 = (c & 2u) ? __ldg(e.cp.wx + p + q) : w;
-        const float w2 = ((o.cy >> (8 * q)) & 4u) ? __ldg(e.cp.wy + p + q - L.sx) : w;
-        const float w3 = (c & 4u) ? __ldg(e.cp.wy + p + q) : w;
-        const float w4 = ((b.c >> (8 * q)) & 8u) ? __ldg(e.cp.wz + p + q - L.sxy) : w;
-        const float w5 = (c & 8u) ? __ldg(e.cp.wz + p + q) : w;
-        d[q] = (((((wl + w1) + w2) + w3) + w4) + w5) + ((c & 1u) ? 0.f : e.cp.kap);
+        const float w1 = (c & 2u) ? v1[q] : w;
+        const float w2 = ((o.cy >> (8 * q)) & 4u) ? v2[q] : w;
+        const float w3 = (c & 4u) ? v3[q] : w;
+        const float w4 = ((below >> (8 * q)) & 8u) ? v4[q] : w;
+        const float w5 = (c & 8u) ? v5[q] : w;
+        d[q] = (((((wl + w1) + w2) + w3) + w4) + w5) + ((c & 1u) ? 0.f : cp.kap);
         sum[q] = ((wl * xx[q] + w1 * xx[q + 2]) + (w2 * my[q] + w3 * py[q])) + (w4 * mz[q] + w5 * pz[q]);
         wl = w1;
     }
 }
-__device__ __forceinline__ void face_sums(const Entry &, const Lev &, int, const Op<false> &o, const Op<false> &b,
+__device__ __forceinline__ void face_sums(const Entry &, const Lev &, int, const Weights &o, const Weights &b,
                                           const float4 &x, float l, float r, const float4 &ym, const float4 &yp,
                                           const float4 &zm, const float4 &zp, float (&sum)[4], float (&d)[4]) {
     sum[0] = ((o.xl * l + o.x.x * x.y) + (o.ym.x * ym.x + o.y.x * yp.x)) + (b.z.x * zm.x + o.z.x * zp.x);
@@ -206,13 +191,14 @@ __device__ __forceinline__ int find_sys(const Entry *tab, int nsys, int it, int 
 
 }  // namespace mg
 
-// Residual after the pre-smoothing step and its restriction.  A block marches
+// Residual after the pre-smoothing step and its restriction, on coarse levels
+// (and a lattice's level 0).  A block marches
 // over the coarse planes of its tile: a thread keeps its unit's s of three
 // planes in registers, rows are exchanged through shared memory (three planes
 // of s, two of the residual, so that one barrier a fine plane suffices), and a
 // plane's loads are issued one plane ahead.
-template <bool FINE, bool SINGLE>
-__global__ void __launch_bounds__(mg::DNT, FINE ? 4 : 3)
+template <bool SINGLE>
+__global__ void __launch_bounds__(mg::DNT, 3)
 k_mg_down(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head, int l, int total,
           const __grid_constant__ mg::Entry e0) {
     using namespace mg;
@@ -245,7 +231,7 @@ k_mg_down(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head, 
             return there && k < L.nz ? f4(L.s + (k * L.sxy + pj)) : make_float4(0.f, 0.f, 0.f, 0.f);
         };
         float4 sm, sc, sn, s2;
-        Op<FINE> ob, oc, on;
+        Weights ob, oc, on;
         sm = halo ? make_float4(0.f, 0.f, 0.f, 0.f) : load(ka - 1);
         sc = load(ka);
         sn = load(ka + 1);
@@ -307,20 +293,19 @@ k_mg_down(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head, 
     }
 }
 
-// Interpolated correction, post-smoothing step and (level 0) rho = r.z.  A
+// Interpolated correction and post-smoothing step of a coarse level.  A
 // block marches over the fine planes of its tile: a thread keeps its unit's v
 // of three planes and the coarse correction, interpolated in y, of two coarse
 // planes in registers; rows of v are exchanged through three planes of shared
 // memory (one barrier a plane).
-template <bool FINE, bool SINGLE>
-__global__ void __launch_bounds__(mg::UNT, FINE ? 3 : 2)
-k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, int total,
+template <bool SINGLE>
+__global__ void __launch_bounds__(mg::UNT, 2)
+k_mg_up(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head, int l, int total,
         const __grid_constant__ mg::Entry e0) {
     using namespace mg;
-    constexpr int NT = UNT, VW = FX + 8;  // a row: col - 1 at [3], cols 0 .. 63 from [4], col 64 at [68]
+    constexpr int VW = FX + 8;  // a row: col - 1 at [3], cols 0 .. 63 from [4], col 64 at [68]
     __shared__ __align__(16) float vp[3][FY + 2][VW];
-    __shared__ float sred[2][NT / 32];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int tid = threadIdx.x;
     const int u = tid & 15, r = tid >> 4;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -391,7 +376,7 @@ k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, i
         };
         S sa = load_s(k0 - 1), sc = load_s(k0), sn = load_s(k0 + 1);
         E ea = load_e((k0 - 1) >> 1), eb = load_e(k0 >> 1), ec = load_e((k0 + 1) >> 1), en = load_e((k0 + 2) >> 1);
-        Op<FINE> ob, oc, on;
+        Weights ob, oc, on;
         if (own) {
             ob.load(e, L, (k0 - 1) * L.sxy + pj);
             oc.load(e, L, k0 * L.sxy + pj);
@@ -406,20 +391,9 @@ k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, i
         // coarse planes of v(k + 1): (k + 1) / 2 and (k + 2) / 2
         ea = ec;
         eb = en;
-        // rho: every RG planes of a tile have a partial of their own, so that
-        // the sum does not depend on the planes per work item (uk[0] is a
-        // multiple of RG).  The one that ends with plane k is written here,
-        // a barrier after the warps' sums.
-        auto flush = [&](int k) {
-            float t = 0.f;
-            for (int q = 0; q < NT / 32; ++q) t += sred[((k - 1) / RG) & 1][q];
-            e.partials[((k - 1) / RG) * xt * yt + col] = t;
-        };
-        float rho = 0.f;
         for (int k = k0; k < k1; ++k) {
             const float4 vn = make_v(k + 1, sn, ea, eb);
             __syncthreads();
-            if (FINE && tid == 0 && k > k0 && (k - 1) % RG == 0) flush(k - 1);
             // issue the next plane's loads
             S s2 = load_s(k + 2);
             ec = eb;
@@ -436,14 +410,8 @@ k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, i
                 for (int q = 0; q < 4; ++q) {
                     z[q] = (1.f - OMEGA) * v4[q] + OMEGA * (s4[q] + __fdividef(sum[q], d[q]));
                     if (ib + q < 1 || ib + q > L.nx - 2) z[q] = 0.f;
-                    if (FINE) rho += d[q] * s4[q] * z[q];
                 }
                 *reinterpret_cast<float4 *>(L.z + (k * L.sxy + pj)) = make_float4(z[0], z[1], z[2], z[3]);
-            }
-            if (FINE && (k % RG == 0 || k == k1 - 1)) {
-                rho = tma::warp_sum_f(rho);
-                if (lane == 0) sred[((k - 1) / RG) & 1][w] = rho;
-                rho = 0.f;
             }
             vm = vc;
             vc = vn;
@@ -454,12 +422,520 @@ k_mg_up(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int l, i
             ob = oc;
             oc = on;
         }
-        if (FINE) {
-            __syncthreads();
-            if (tid == 0) flush(k1 - 1);
+    }
+}
+
+// ---- level 0 of a solver's grid: two rows a thread
+// A thread takes a unit of four nodes in two neighbouring rows.  The planes of
+// s and codes come in by TMA, NS in shared memory and up to three ahead of
+// their use (the first thread issues them, out-of-range elements are zero);
+// arithmetic is in packed FP32 pairs; weights of unlisted units come from a
+// table by the units' four solute bits, those of listed ones from listed_sums.
+//
+// 257^3, down and up: one row a thread with loads into registers a plane
+// ahead 102 and 139 us; this form 70 and 88 us (the first 21 and 25 us at the
+// measured copy rate, all that is read and written counted).  What was in the
+// way, one after the other: a gather of its own for each listed face (below);
+// parameters read again after every asm statement (hence the local copies);
+// resident blocks that walked over their items, so that a block with the
+// molecule's surface in both of its items held up the launch (a one-system
+// launch now has a block an item); asynchronous copies of each thread's own,
+// 60 instructions a plane (TMA); the listed weights' latency (prefetched a
+// plane ahead).  Now bound by instruction issue (46 % of the issue slots) and
+// the barrier of each plane.
+namespace mg {
+constexpr int C0Y = 8, D0P = C0Y + 1, D0NT = 160;  // down: 32 x 8 coarse nodes, nine row pairs of 17 units
+constexpr int U0NT = 192;                          // up: eight row pairs, a warp of halo rows, a warp of halo columns
+constexpr int NS = 4;                              // planes of s and codes in shared memory
+constexpr int D0R = 2 * D0P + 1, D0W = 4 * DU;     // the down kernel's box of s
+constexpr int U0R = FY + 2, U0W = FX + 8;          // the up kernel's: columns from i0 - 4
+constexpr int C0W = FX + 32;                       // codes: columns from 16 to the left
+constexpr int up128(int b) { return (b + 127) & ~127; }
+// The ring of planes of one block.  Planes are counted over the whole launch;
+// every wait is bounded, and one that gives up is reported in the solver's
+// state (status 3) at the end of the launch.
+template <int R, int W, int RC>  // rows and columns of s, rows of codes
+struct Ring {
+    static constexpr int SB = up128(4 * R * W), CB = up128(RC * C0W);
+    struct Mem {
+        uint8_t s[NS][SB], c[NS][CB];
+    };
+    Mem &m;
+    uint32_t bar;        // NS mbarriers
+    int n = 0, put = 0;  // planes waited for, planes issued
+    bool bad = false;
+    __device__ __forceinline__ Ring(Mem &mem, uint64_t *bars) : m(mem), bar(tma::smem_u32(bars)) {
+        if (threadIdx.x == 0) {
+            for (int q = 0; q < NS; ++q) tma::mbar_init(bar + 8 * q, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
     }
-    if (!FINE) return;
+    __device__ __forceinline__ void issue(const CUtensorMap &sm, const CUtensorMap &cm, int x, int y, int k) {
+        if (threadIdx.x == 0) {
+            const int q = put & (NS - 1);
+            const uint32_t b = bar + 8 * q;
+            tma::mbar_expect_tx(b, 4 * R * W + RC * C0W);
+            tma::tma_load3(tma::smem_u32(m.s[q]), &sm, x - (W == U0W ? 4 : 0), y, k, b);
+            tma::tma_load3(tma::smem_u32(m.c[q]), &cm, x - 16, y, k, b);
+        }
+        ++put;
+    }
+    __device__ __forceinline__ void wait() {  // for the next plane
+        const uint32_t b = bar + 8 * (n & (NS - 1)), parity = (n / NS) & 1;
+        if (!tma::mbar_try(b, parity) && !tma::mbar_wait(b, parity, bad ? 0 : tma::TMA_WAIT_LIMIT)) bad = true;
+        ++n;
+    }
+    __device__ __forceinline__ const float (*s(int back) const)[W] {  // plane back before the last one waited for
+        return reinterpret_cast<const float (*)[W]>(m.s[(n - 1 - back) & (NS - 1)]);
+    }
+    __device__ __forceinline__ const uint8_t (*c(int back) const)[C0W] {
+        return reinterpret_cast<const uint8_t (*)[C0W]>(m.c[(n - 1 - back) & (NS - 1)]);
+    }
+    __device__ __forceinline__ void report(CgState *st) {
+        if (!bad) return;
+        st->status = 3;
+        st->done = 1;
+        if (threadIdx.x == 0)  // the block's own copies land before it leaves
+            for (int q = max(put - NS, 0); q < put; ++q)
+                tma::mbar_wait(bar + 8 * (q & (NS - 1)), (q / NS) & 1, tma::TMA_WAIT_LIMIT);
+    }
+};
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool there) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tma::smem_u32(dst)), "l"(src), "r"(there ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *dst, const void *src, bool there) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tma::smem_u32(dst)), "l"(src), "r"(there ? 4 : 0)
+                 : "memory");
+}
+struct Pair4 {  // four values as two packed pairs
+    float2 a, b;
+};
+__device__ __forceinline__ Pair4 p4(const float4 &v) { return {make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
+__device__ __forceinline__ float4 f4(const Pair4 &v) { return make_float4(v.a.x, v.a.y, v.b.x, v.b.y); }
+__device__ __forceinline__ Pair4 operator+(const Pair4 &x, const Pair4 &y) {
+    return {__fadd2_rn(x.a, y.a), __fadd2_rn(x.b, y.b)};
+}
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ Pair4 scale(float c, const Pair4 &x) {
+    return {__fmul2_rn(both(c), x.a), __fmul2_rn(both(c), x.b)};
+}
+__device__ __forceinline__ Pair4 fma4(float c, const Pair4 &x, const Pair4 &y) {  // c x + y
+    return {__ffma2_rn(both(c), x.a, y.a), __ffma2_rn(both(c), x.b, y.b)};
+}
+__device__ __forceinline__ Pair4 fma4(const Pair4 &c, const Pair4 &x, const Pair4 &y) {
+    return {__ffma2_rn(c.a, x.a, y.a), __ffma2_rn(c.b, x.b, y.b)};
+}
+__device__ __forceinline__ Pair4 mul4(const Pair4 &x, const Pair4 &y) {
+    return {__fmul2_rn(x.a, y.a), __fmul2_rn(x.b, y.b)};
+}
+// the six neighbours of a unit's nodes added up
+__device__ __forceinline__ Pair4 neighbours(const Pair4 &c, float l, float r, const Pair4 &ym, const Pair4 &yp,
+                                            const Pair4 &zm, const Pair4 &zp) {
+    const float2 mid = make_float2(c.a.y, c.b.x);
+    const Pair4 x = {__fadd2_rn(make_float2(l, c.a.x), mid), __fadd2_rn(mid, make_float2(c.b.y, r))};
+    return x + (ym + yp) + (zm + zp);
+}
+// byte offset into a table of 16 float4: the solute bits of four codes
+__device__ __forceinline__ uint32_t media(uint32_t c) { return ((c & 0x01010101u) * 0x01020408u) >> 20; }
+__device__ __forceinline__ Pair4 entry(const float4 *table, uint32_t at) {
+    return p4(*reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(table) + at));
+}
+// fills entry t of a table with one of two values by each bit of t
+__device__ __forceinline__ void fill_media(float4 *table, int t, float in, float out) {
+    table[t] = make_float4((t & 1) ? in : out, (t & 2) ? in : out, (t & 4) ? in : out, (t & 8) ? in : out);
+}
+__device__ __forceinline__ bool listed(const Codes &o, uint32_t below) {
+    const uint32_t cx = (o.c << 8) | o.cl;
+    return ((o.c & 0x0E0E0E0Eu) | (cx & 0x02020202u) | (o.cy & 0x04040404u) | (below & 0x08080808u)) != 0u;
+}
+__device__ __forceinline__ void listed_sums(const CoefC32 &cp, const Lev &L, int p, const Codes &o, uint32_t below,
+                                            const Pair4 &c, float l, float r, const Pair4 &ym, const Pair4 &yp,
+                                            const Pair4 &zm, const Pair4 &zp, Pair4 &sum, Pair4 &d) {
+    // the surface mostly goes on in the next plane
+    tma::prefetch_l1(cp.wx + p + L.sxy);
+    tma::prefetch_l1(cp.wy + p + L.sxy - L.sx);
+    tma::prefetch_l1(cp.wy + p + L.sxy);
+    tma::prefetch_l1(cp.wz + p + L.sxy);
+    float s4[4], d4[4];
+    listed_sums(cp, L, p, o, below, f4(c), l, r, f4(ym), f4(yp), f4(zm), f4(zp), s4, d4);
+    sum = {make_float2(s4[0], s4[1]), make_float2(s4[2], s4[3])};
+    d = {make_float2(d4[0], d4[1]), make_float2(d4[2], d4[3])};
+}
+}  // namespace mg
+
+// Residual and restriction of level 0.  Row pair p of a tile is rows 2 J - 1
+// and 2 J of its coarse row J; its share of the sums across y is formed in the
+// thread, half of the next pair's first row and the last column of the unit
+// to the left come through shared memory.  Planes are taken in pairs.
+template <bool SINGLE>
+__global__ void __launch_bounds__(mg::D0NT, 4)
+k_mg_down0(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head, int total,
+           const __grid_constant__ mg::Entry e0) {
+    using namespace mg;
+    using R = Ring<D0R, D0W, D0R>;
+    __shared__ __align__(128) R::Mem planes;
+    __shared__ __align__(16) float half[2][D0P][D0W];  // half the residual of each pair's first row
+    __shared__ float last[2][D0P][DU];                 // each unit's last column of a pair's share
+    __shared__ float4 tw[16], td[16];                  // omega w and (1 - omega) d
+    __shared__ uint64_t bars[NS];
+    const int tid = threadIdx.x;
+    const int pr = tid / DU, u = tid - pr * DU;  // pair and unit of a thread
+    const bool work = pr < D0P;
+    const int ra = work ? 2 * pr + 1 : 1, x = 4 * u;  // row of the box
+    R ring(planes, bars);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int nsys = SINGLE ? 1 : head->nsys;
+    if (!SINGLE) total = head->dtotal[0];
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        const Entry &e = SINGLE ? e0 : tab[find_sys(tab, nsys, it, &Entry::dbase, 0)];
+        // one answer for the block; and the previous item's last reads, the barriers' initialisation
+        if (__syncthreads_or(*(volatile int *)&e.st->done)) continue;
+        // local copies: the asm statements below would have e read again
+        const Lev L = e.lev[0], C = e.lev[1];
+        const CoefC32 cp = e.cp;
+        const int li = SINGLE ? it : it - e.dbase[0];
+        const int xt = (C.nx - 2 + CX - 1) / CX, yt = (C.ny - 2 + C0Y - 1) / C0Y;
+        const int col = li % (xt * yt), ch = li / (xt * yt);
+        const int I0 = 1 + (col % xt) * CX, J0 = 1 + (col / xt) * C0Y;
+        const int K0 = 1 + ch * e.dk[0], K1 = min(K0 + e.dk[0], C.nz - 1);
+        const int ka = 2 * K0 - 1, kb = 2 * K1 - 1;
+        const int i0 = 2 * I0 - 2, jb = 2 * J0 - 2, ib = i0 + x, ja = jb + ra;
+        const bool rowA = work && ib < L.sx && ja <= L.ny - 2, rowB = rowA && ja + 1 <= L.ny - 2 && pr < D0P - 1;
+        const int pj = ja * L.sx + ib;
+        const bool edge = ib < 1 || ib + 3 > L.nx - 2;
+        auto clip = [&](Pair4 &v) {  // nodes of the unit that are no unknowns
+            if (ib < 1 || ib > L.nx - 2) v.a.x = 0.f;
+            if (ib + 1 > L.nx - 2) v.a.y = 0.f;
+            if (ib + 2 > L.nx - 2) v.b.x = 0.f;
+            if (ib + 3 > L.nx - 2) v.b.y = 0.f;
+        };
+        const int I = I0 - 1 + 2 * u, J = J0 + pr;  // the thread's coarse nodes
+        const bool in0 = pr < C0Y && J <= C.ny - 2 && u > 0 && I <= C.nx - 2;
+        const bool in1 = pr < C0Y && J <= C.ny - 2 && u < DU - 1 && I + 1 <= C.nx - 2;
+        const int pcj = J * C.sx + I;
+        for (int k = ka - 1; k <= ka + 2; ++k)
+            if (k <= kb + 1) ring.issue(e.sd, e.cd, i0, jb, k);
+        if (tid < 16) fill_media(tw, tid, OMEGA * cp.w_in, OMEGA * cp.w_out);
+        else if (tid < 32) fill_media(td, tid - 16, (1.f - OMEGA) * e.dg_in, (1.f - OMEGA) * e.dg_out);
+        ring.wait();
+        ring.wait();
+        auto word = [&](const uint8_t (*c)[C0W], int r) { return *reinterpret_cast<const uint32_t *>(&c[r][16 + x]); };
+        uint32_t bA = word(ring.c(1), ra), bB = word(ring.c(1), ra + 1);  // codes of plane k - 1
+        Pair4 mA = p4(f4(&ring.s(1)[ra][x])), mB = p4(f4(&ring.s(1)[ra + 1][x]));
+        Pair4 cA = p4(f4(&ring.s(0)[ra][x])), cB = p4(f4(&ring.s(0)[ra + 1][x])), share = {};
+        float acc0 = 0.f, acc1 = 0.f, dc0 = 1.f, dc1 = 1.f;
+        // plane k, an odd one or not, and the restriction of the one before
+        auto step = [&](int k, auto odd, bool compute) {
+            constexpr bool ODD = decltype(odd)::value;
+            const bool done = !ODD && k - 1 > ka;  // completes coarse nodes
+            const int pc = ((k - (ODD ? 1 : 2)) >> 1) * C.sxy + pcj;
+            if (compute) ring.wait();  // plane k + 1
+            __syncthreads();
+            if (ODD && k > ka) {  // their diagonals, a plane ahead
+                if (in0) dc0 = __ldg(C.dg + pc);
+                if (in1) dc1 = __ldg(C.dg + pc + 1);
+            }
+            Pair4 next = {};
+            if (compute) {
+                if (k + 3 <= kb + 1) ring.issue(e.sd, e.cd, i0, jb, k + 3);  // over plane k - 1
+                const float (*s)[D0W] = ring.s(1), (*sn)[D0W] = ring.s(0);
+                const uint8_t (*cd)[C0W] = ring.c(1);
+                const Pair4 nA = p4(f4(&sn[ra][x])), nB = p4(f4(&sn[ra + 1][x]));
+                Pair4 rA = {}, rB = {};
+                const uint32_t nbA = word(cd, ra), nbB = word(cd, ra + 1);
+                if (rowA && k <= L.nz - 2) {
+                    const int p = k * L.sxy + pj;
+                    Codes o;
+                    auto residual = [&](int q, int r, const Pair4 &c, const Pair4 &ym, const Pair4 &yp,
+                                        const Pair4 &zm, const Pair4 &zp, uint32_t below) {
+                        // outside the box at both ends of a row: not used there
+                        const float l = s[r][x - 1], rt = s[r][x + 4];
+                        o.cl = cd[r][15 + x];
+                        if (!listed(o, below)) {
+                            const uint32_t m = media(o.c);
+                            return fma4(entry(tw, m), neighbours(c, l, rt, ym, yp, zm, zp), mul4(entry(td, m), c));
+                        }
+                        Pair4 sum, dg;
+                        listed_sums(cp, L, q, o, below, c, l, rt, ym, yp, zm, zp, sum, dg);
+                        return fma4(OMEGA, sum, mul4(scale(1.f - OMEGA, dg), c));
+                    };
+                    o.c = nbA;
+                    o.cy = word(cd, ra - 1);
+                    rA = residual(p, ra, cA, p4(f4(&s[ra - 1][x])), cB, mA, nA, bA);
+                    if (rowB) {
+                        o.c = nbB;
+                        o.cy = nbA;
+                        rB = residual(p + L.sx, ra + 1, cB, cA, p4(f4(&s[ra + 2][x])), mB, nB, bB);
+                    }
+                    if (edge) {
+                        clip(rA);
+                        clip(rB);
+                    }
+                }
+                const Pair4 h = scale(0.5f, rA);
+                next = h + rB;
+                if (work) {
+                    *reinterpret_cast<float4 *>(&half[ODD][pr][x]) = f4(h);
+                    last[ODD][pr][u] = next.b.y;
+                }
+                mA = cA;
+                mB = cB;
+                cA = nA;
+                cB = nB;
+                bA = nbA;
+                bB = nbB;
+            }
+            if (k > ka && pr < C0Y) {  // restrict plane k - 1
+                const float *h = half[!ODD][pr + 1] + x;
+                const Pair4 y = share + p4(f4(h));
+                const float left = u > 0 ? last[!ODD][pr][u - 1] + h[-1] : 0.f;
+                const float t0 = y.a.x + 0.5f * (left + y.a.y), t1 = y.b.x + 0.5f * (y.a.y + y.b.y);
+                if (ODD) {
+                    acc0 += t0;
+                    acc1 += t1;
+                } else {
+                    if (done && in0) C.s[pc] = __fdividef(acc0 + 0.5f * t0, dc0);
+                    if (done && in1) C.s[pc + 1] = __fdividef(acc1 + 0.5f * t1, dc1);
+                    acc0 = 0.5f * t0;
+                    acc1 = 0.5f * t1;
+                }
+            }
+            share = next;
+        };
+        for (int k = ka; k <= kb; k += 2) {
+            step(k, std::true_type{}, true);
+            step(k + 1, std::false_type{}, k + 1 <= kb);
+        }
+        ring.report(e.st);
+    }
+}
+
+// Correction, post-smoothing and rho of level 0.  Warps 0 to 3 own the tile's
+// eight row pairs (an odd row and the even one above), warp 4 the row on
+// either side, warp 5 the column on either side; all put v = omega s + P e in
+// shared memory, three planes deep.  Planes are taken in pairs, as a coarse
+// plane serves two of them; its tile comes in by asynchronous copies.
+template <bool SINGLE>
+__global__ void __launch_bounds__(mg::U0NT, 3)
+k_mg_up0(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int total,
+         const __grid_constant__ mg::Entry e0) {
+    using namespace mg;
+    using R = Ring<U0R, U0W, FY + 1>;
+    // a row: column i0 - 1 at [3], i0 .. i0 + 63 from [4], i0 + 64 at [68]
+    constexpr int NT = U0NT, VW = U0W, CZX = FX / 2 + 8, CZY = FY / 2 + 2, CZU = CZX / 4;
+    __shared__ __align__(16) float vp[3][FY + 2][VW];
+    __shared__ __align__(128) R::Mem planes;
+    __shared__ __align__(16) float cz[3][CZY][CZX];  // coarse planes: columns i0 / 2 - 4 .., rows (j0 - 1) / 2 ..
+    __shared__ float4 tq[16], td[16];                // omega w / d and d
+    __shared__ float sred[2][4];
+    __shared__ uint64_t bars[NS];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int u = lane & 15, hi = lane >> 4;
+    const bool own = w < 4, hrow = w == 4;
+    // row (0 .. FY + 1; own threads: their first) and column of vp and ss
+    const int r = own ? 1 + 4 * w + 2 * hi : (hrow ? (hi ? FY + 1 : 0) : 1 + u);
+    const int x = own || hrow ? 4 + 4 * u : (hi ? 4 + FX : 3);
+    R ring(planes, bars);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int nsys = SINGLE ? 1 : head->nsys;
+    if (!SINGLE) total = head->utotal[0];
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        const Entry &e = SINGLE ? e0 : tab[find_sys(tab, nsys, it, &Entry::ubase, 0)];
+        // one answer for the block; and the previous item's last reads, the barriers' initialisation
+        if (__syncthreads_or(*(volatile int *)&e.st->done)) continue;
+        const Lev L = e.lev[0], C = e.lev[1];
+        const CoefC32 cp = e.cp;
+        float *const partials = e.partials;
+        const bool padded = e.nbot > 1;
+        const int li = SINGLE ? it : it - e.ubase[0];
+        const int xt = (L.nx - 1 + FX - 1) / FX, yt = (L.ny - 2 + FY - 1) / FY;
+        const int col = li % (xt * yt), ch = li / (xt * yt);
+        const int i0 = (col % xt) * FX, j0 = 1 + (col / xt) * FY;
+        const int k0 = 1 + ch * e.uk[0], k1 = min(k0 + e.uk[0], L.nz - 1);  // k0 odd
+        const int j = j0 - 1 + r, ib = i0 - 4 + x;
+        const bool cols = ib >= 0 && ib <= L.nx - 2;
+        const bool rowA = cols && j >= 1 && j <= L.ny - 2, rowB = own && rowA && j + 1 <= L.ny - 2;
+        const int pj = j * L.sx + ib;
+        const bool edge = ib < 1 || ib + 3 > L.nx - 2;
+        auto clip = [&](Pair4 &v) {  // columns that are no unknowns
+            if (ib < 1) v.a.x = 0.f;
+            if (ib + 1 > L.nx - 2) v.a.y = 0.f;
+            if (ib + 2 > L.nx - 2) v.b.x = 0.f;
+            if (ib + 3 > L.nx - 2) v.b.y = 0.f;
+        };
+        // a coarse plane's tile into slot K % 3: a unit a thread
+        const int cu = tid % CZU, cv = tid / CZU;
+        const int Ic = i0 / 2 - 4 + 4 * cu, Jc = (j0 - 1) / 2 + cv;
+        const bool cin = cv < CZY && Ic >= 0 && Ic < C.sx && Jc < C.ny;
+        auto fetch_coarse = [&](int K) {
+            if (cv < CZY) {
+                const bool in = cin && K < C.nz;
+                const float *src = C.z + (in ? K * C.sxy + Jc * C.sx + Ic : 0);
+                float *dst = &cz[K % 3][cv][4 * cu];
+                if (padded) {
+                    cp_async16(dst, src, in);
+                } else {  // the bottom kernel's rows are not padded
+                    for (int q = 0; q < 4; ++q) {
+                        const bool t = in && Ic + q < C.nx;
+                        cp_async4(dst + q, t ? src + q : C.z, t);
+                    }
+                }
+            }
+        };
+        // coarse correction of plane K at the thread's nodes, interpolated in x
+        // and y: of its first row (or node), and of the row above
+        struct E2 {
+            Pair4 a, b;
+        };
+        const int ca = (j >> 1) - (j0 - 1) / 2, cb = ((j + 1) >> 1) - (j0 - 1) / 2, ci = (ib >> 1) - i0 / 2 + 4;
+        auto coarse = [&](int K) {
+            E2 t = {};
+            const float *a = &cz[K % 3][ca][ci], *b = &cz[K % 3][cb][ci];
+            if (own || hrow) {
+                const float2 b01 = *reinterpret_cast<const float2 *>(b), a01 = *reinterpret_cast<const float2 *>(a);
+                const float b2 = b[2], a2 = 0.5f * (a[2] + b2);
+                const float a0 = 0.5f * (a01.x + b01.x), a1 = 0.5f * (a01.y + b01.y);
+                t.a = {make_float2(a0, 0.5f * (a0 + a1)), make_float2(a1, 0.5f * (a1 + a2))};
+                t.b = {make_float2(b01.x, 0.5f * (b01.x + b01.y)), make_float2(b01.y, 0.5f * (b01.y + b2))};
+            } else {
+                const int o = ib & 1;  // an odd column lies between two coarse ones
+                t.a.a.x = 0.25f * ((a[0] + a[o]) + (b[0] + b[o]));
+            }
+            return t;
+        };
+        // v = omega s + P e of plane k, into vp[slot]
+        Pair4 vA, vB;  // the last one made (own rows)
+        auto make_v = [&](int k, int slot, const E2 &g) {  // of the last plane waited for
+            vA = vB = Pair4{};
+            const bool kin = k >= 1 && k <= L.nz - 2;
+            const float (*s)[VW] = ring.s(0);
+            if (own || hrow) {
+                if (rowA && kin) {
+                    vA = fma4(OMEGA, p4(f4(&s[r][x])), g.a);
+                    if (rowB) vB = fma4(OMEGA, p4(f4(&s[r + 1][x])), g.b);
+                    if (edge) {
+                        clip(vA);
+                        clip(vB);
+                    }
+                }
+                *reinterpret_cast<float4 *>(&vp[slot][r][x]) = f4(vA);
+                if (own) *reinterpret_cast<float4 *>(&vp[slot][r + 1][x]) = f4(vB);
+            } else {
+                vp[slot][r][x] = rowA && kin ? OMEGA * s[r][x] + g.a.a.x : 0.f;
+            }
+        };
+        auto mean = [](const E2 &p, const E2 &q) { return E2{scale(0.5f, p.a + q.a), scale(0.5f, p.b + q.b)}; };
+        for (int k = k0 - 1; k <= k0 + 2; ++k)
+            if (k <= k1) ring.issue(e.su, e.cu, i0, j0 - 1, k);
+        for (int K = (k0 - 1) >> 1; K <= (k0 + 3) >> 1; ++K) fetch_coarse(K);
+        if (tid < 16) fill_media(tq, tid, __fdividef(OMEGA * cp.w_in, e.dg_in), __fdividef(OMEGA * cp.w_out, e.dg_out));
+        else if (tid < 32) fill_media(td, tid - 16, e.dg_in, e.dg_out);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        E2 ec = coarse((k0 - 1) >> 1), en = coarse((k0 + 1) >> 1);
+        int slot = (k0 - 1) % 3;  // of plane k - 1
+        ring.wait();
+        make_v(k0 - 1, slot, ec);
+        Pair4 mA = vA, mB = vB;
+        ring.wait();
+        make_v(k0, slot == 2 ? 0 : slot + 1, mean(ec, en));
+        Pair4 cA = vA, cB = vB;
+        ec = en;  // coarse plane (k0 + 1) / 2
+        auto word = [&](const uint8_t (*c)[C0W], int q) { return *reinterpret_cast<const uint32_t *>(&c[q][12 + x]); };
+        uint32_t bA = 0, bB = 0;  // codes of plane k - 1
+        if (own) {
+            bA = word(ring.c(1), r);
+            bB = word(ring.c(1), r + 1);
+        }
+        // rho: every RG planes of a tile have a partial of their own, so that
+        // the sum does not depend on the planes per work item (uk[0] is a
+        // multiple of RG).  The one that ends with plane k is written here,
+        // a barrier after the warps' sums.
+        auto flush = [&](int k) {
+            const float *q = sred[((k - 1) / RG) & 1];
+            partials[((k - 1) / RG) * xt * yt + col] = ((q[0] + q[1]) + q[2]) + q[3];
+        };
+        Pair4 rho = {};
+        // one plane: v(k + 1) with the correction g, then z(k)
+        auto step = [&](int k, const E2 &g) {
+            const int sv = slot == 2 ? 0 : slot + 1, sn = sv == 2 ? 0 : sv + 1;
+            ring.wait();  // plane k + 1
+            make_v(k + 1, sn, g);
+            const Pair4 nA = vA, nB = vB;
+            __syncthreads();
+            if (k + 3 <= k1) ring.issue(e.su, e.cu, i0, j0 - 1, k + 3);  // over plane k - 1
+            if (tid == 0 && k > k0 && (k - 1) % RG == 0) flush(k - 1);
+            if (own) {
+                uint32_t nbA = 0, nbB = 0;
+                if (rowA) {
+                    const float (*v)[VW] = vp[sv];
+                    const float (*ss)[VW] = ring.s(1);
+                    const uint8_t (*cd)[C0W] = ring.c(1);
+                    nbA = word(cd, r);
+                    nbB = word(cd, r + 1);
+                    Codes o;
+                    auto relax = [&](int q, const Pair4 &s, const Pair4 &c, int rr, const Pair4 &ym, const Pair4 &yp,
+                                     const Pair4 &zm, const Pair4 &zp, uint32_t below) {
+                        const float l = v[rr][x - 1], rt = v[rr][x + 4];
+                        o.cl = cd[rr][11 + x];
+                        Pair4 z = fma4(1.f - OMEGA, c, scale(OMEGA, s)), d;
+                        if (!listed(o, below)) {
+                            const uint32_t m = media(o.c);
+                            d = entry(td, m);
+                            z = fma4(entry(tq, m), neighbours(c, l, rt, ym, yp, zm, zp), z);
+                        } else {
+                            Pair4 sum;
+                            listed_sums(cp, L, q, o, below, c, l, rt, ym, yp, zm, zp, sum, d);
+                            z = fma4(OMEGA,
+                                     Pair4{make_float2(__fdividef(sum.a.x, d.a.x), __fdividef(sum.a.y, d.a.y)),
+                                           make_float2(__fdividef(sum.b.x, d.b.x), __fdividef(sum.b.y, d.b.y))},
+                                     z);
+                        }
+                        if (edge) clip(z);
+                        rho = fma4(mul4(d, s), z, rho);
+                        *reinterpret_cast<float4 *>(L.z + q) = f4(z);
+                    };
+                    const int p = k * L.sxy + pj;
+                    o.c = nbA;
+                    o.cy = word(cd, r - 1);
+                    relax(p, p4(f4(&ss[r][x])), cA, r, p4(f4(&v[r - 1][x])), cB, mA, nA, bA);
+                    if (rowB) {
+                        o.c = nbB;
+                        o.cy = nbA;
+                        relax(p + L.sx, p4(f4(&ss[r + 1][x])), cB, r + 1, cA, p4(f4(&v[r + 2][x])), mB, nB, bB);
+                    }
+                }
+                if (k % RG == 0 || k == k1 - 1) {
+                    const float t = tma::warp_sum_f((rho.a.x + rho.a.y) + (rho.b.x + rho.b.y));
+                    if (lane == 0) sred[((k - 1) / RG) & 1][w] = t;
+                    rho = Pair4{};
+                }
+                mA = cA;
+                mB = cB;
+                cA = nA;
+                cB = nB;
+                bA = nbA;
+                bB = nbB;
+            }
+            slot = sv;
+        };
+        for (int k = k0; k < k1; k += 2) {
+            asm volatile("cp.async.wait_all;" ::: "memory");  // coarse plane (k + 3) / 2: behind the next barrier
+            step(k, ec);                                      // v(k + 1): an even plane, coarse plane (k + 1) / 2
+            if (k + 1 >= k1) break;
+            fetch_coarse((k + 5) >> 1);
+            en = coarse((k + 3) >> 1);
+            step(k + 1, mean(ec, en));
+            ec = en;
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        if (tid == 0) flush(k1 - 1);
+        ring.report(e.st);
+    }
     // the last block sums every system's items in item order and takes the
     // CG step: beta = rho / rho_old
     __shared__ int s_last;
@@ -865,7 +1341,8 @@ void mg_planes(mg::Entry &e, bool shared) {
     auto best = [&](long long cols, int n, int slots, int step, int most) {
         int kc = most;
         double cost = 1e30;
-        for (int c = step; c <= most && !shared; c += step) {
+        const int longest = shared ? 0 : most;
+        for (int c = step; c <= longest; c += step) {
             const double t = (double)cdiv(cols * cdiv(n, c), (long long)slots * num_sms()) * (c + 2.5);
             if (t < cost) {
                 cost = t;
@@ -877,7 +1354,8 @@ void mg_planes(mg::Entry &e, bool shared) {
     for (int l = 0; l < e.nbot; ++l) {
         const Lev &F = e.lev[l], &C = e.lev[l + 1];
         // a coarse plane is two fine ones
-        e.dk[l] = best((long long)cdiv(C.nx - 2, CX) * cdiv(C.ny - 2, CY), 2 * (C.nz - 2), 4, 2, 16) / 2;
+        e.dk[l] = best((long long)cdiv(C.nx - 2, CX) * cdiv(C.ny - 2, l == 0 && e.code ? C0Y : CY), 2 * (C.nz - 2),
+                       4, 2, 16) / 2;
         e.uk[l] = best((long long)cdiv(F.nx - 1, FX) * cdiv(F.ny - 2, FY), F.nz - 2, 3, l == 0 ? RG : 1, 16);
     }
 }
@@ -1019,6 +1497,7 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
     using namespace mg;
     if (sys->mg) return PB_OK;
     Entry e{};
+    e.code = sys->code;
     if (!mg_levels(sys->pad, e)) return PB_OK;
     pb_status rc = mg_prepare();
     if (rc != PB_OK) return rc;
@@ -1041,11 +1520,15 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
     e.lev[0].z = m->v;
     mg_layout(e, 1, (char *)m->mem);
     e.st = sys->st;
-    e.code = sys->code;
     e.cp = make_c32(sys);
     e.dg_in = 6.f * e.cp.w_in;
     e.dg_out = 6.f * e.cp.w_out + e.cp.kap;
     e.partials = m->partials;
+    if ((rc = make_map(&e.sd, sys->z32, false, sys->pad, D0W, D0R)) != PB_OK ||
+        (rc = make_map(&e.cd, sys->code, true, sys->pad, C0W, D0R)) != PB_OK ||
+        (rc = make_map(&e.su, sys->z32, false, sys->pad, U0W, U0R)) != PB_OK ||
+        (rc = make_map(&e.cu, sys->code, true, sys->pad, C0W, FY + 1)) != PB_OK)
+        return rc;
     if ((rc = mg_build_levels(e, 1, sys, s)) != PB_OK) return rc;
     m->e = e;
     return PB_OK;
@@ -1085,25 +1568,22 @@ int launch_vcycle(const pb_system *sys, cudaStream_t s) {
     Entry e = m->e;
     e.st = sys->st;  // the engine lends a system its slot's state
     const bool fine = !m->lattice;
-    static const unsigned rd0 = mg_resident(k_mg_down<true, true>, DNT), rd1 = mg_resident(k_mg_down<false, true>, DNT),
-                          ru0 = mg_resident(k_mg_up<true, true>, UNT), ru1 = mg_resident(k_mg_up<false, true>, UNT);
+    static const unsigned rd1 = mg_resident(k_mg_down<true>, DNT), ru1 = mg_resident(k_mg_up<true>, UNT);
     const Entry *none = nullptr;
     for (int l = 0; l < e.nbot; ++l) {
         const int n = ditems(e, l);
         if (l == 0 && fine)
-            mg_launch(k_mg_down<true, true>, std::min<unsigned>(n, rd0), DNT, 0, s, true, none, (const Head *)m->head, l,
-                      n, e);
+            mg_launch(k_mg_down0<true>, n, D0NT, 0, s, true, none, (const Head *)m->head, n, e);
         else
-            mg_launch(k_mg_down<false, true>, std::min<unsigned>(n, rd1), DNT, 0, s, true, none, (const Head *)m->head,
-                      l, n, e);
+            mg_launch(k_mg_down<true>, std::min<unsigned>(n, rd1), DNT, 0, s, true, none, (const Head *)m->head, l, n, e);
     }
     mg_launch(k_mg_bottom<Entry, true>, 1, BOT_T, mg_bottom_bytes(e), s, true, none, (const Head *)m->head, e);
     for (int l = e.nbot - 1; l >= 0; --l) {
         const int n = uitems(e, l);
         if (l == 0 && fine)
-            mg_launch(k_mg_up<true, true>, std::min<unsigned>(n, ru0), UNT, 0, s, true, none, m->head, l, n, e);
+            mg_launch(k_mg_up0<true>, n, U0NT, 0, s, true, none, m->head, n, e);
         else
-            mg_launch(k_mg_up<false, true>, std::min<unsigned>(n, ru1), UNT, 0, s, true, none, m->head, l, n, e);
+            mg_launch(k_mg_up<true>, std::min<unsigned>(n, ru1), UNT, 0, s, true, none, (const Head *)m->head, l, n, e);
     }
     return 2 * e.nbot + 1;
 }
