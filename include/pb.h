@@ -256,7 +256,8 @@ void pb_grid_free(pb_grid *g);
  * Sec. 3.2 WHA), the ionic diagonal C (Sec. 2.1 linearisation), boundary
  * values (Sec. 2.3) and the right-hand side (Eq. RVop + Dirichlet lift).
  * The Coulomb/DH boundary values are an N-body sum over the box faces run
- * by this call.  The system keeps a reference to g (g must outlive it). */
+ * by this call.  The system keeps a reference to g: a grid that is
+ * freed before its systems lives on until the last of them is freed. */
 pb_status pb_assemble_coeffs(pb_grid *g, const pb_params *params, void *stream,
                              pb_system **out);
 void pb_system_free(pb_system *s);

@@ -134,8 +134,9 @@ pb_status pb_set_allocator(pb_alloc_fn alloc, pb_free_fn release, void *ctx) {
     return PB_OK;
 }
 
+// the last reference (the caller's own, or a system's) frees the grid
 void pb_grid_free(pb_grid *g) {
-    if (!g) return;
+    if (!g || g->refs.fetch_sub(1) > 1) return;
     DeviceGuard dg(g->device);
     cudaStream_t s = g->stream;
     cudaStreamSynchronize(s);
@@ -292,7 +293,8 @@ pb_status pb_grid_info_get(const pb_grid *g, pb_grid_info *info) {
 
 void pb_system_free(pb_system *s) {
     if (!s) return;
-    DeviceGuard dg(s->g->device);
+    pb_grid *g = s->g;
+    DeviceGuard dg(g->device);
     cudaStream_t st = s->stream;
     cudaStreamSynchronize(st);
     void *ptrs[] = {s->W[0], s->W[1], s->W[2], s->diag, s->rhs, s->bc, s->phi, s->code, s->w32[0], s->w32[1], s->w32[2],
@@ -308,6 +310,7 @@ void pb_system_free(pb_system *s) {
     if (s->h_st) cudaFreeHost(s->h_st);
     if (s->h_energy) cudaFreeHost(s->h_energy);
     delete s;
+    pb_grid_free(g);
 }
 
 pb_status pb_assemble_coeffs(pb_grid *g, const pb_params *params, void *stream, pb_system **out) {
@@ -339,6 +342,7 @@ pb_status pb_assemble_coeffs(pb_grid *g, const pb_params *params, void *stream, 
     pb_system *sys = new (std::nothrow) pb_system();
     if (!sys) return PB_ERR_OOM;
     sys->g = g;
+    g->refs.fetch_add(1);
     sys->stream = s;
     sys->p = p;
     physical_units(p.temperature_K, p.ionic_strength_M, p.eps_out, &sys->lB, &sys->kD);

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 
 #include "../../include/pb.h"
@@ -122,6 +123,7 @@ struct OctSys {
 
 struct pb_grid {
     int device;
+    std::atomic<int> refs{1};  // the caller's reference and one of each system
     cudaStream_t stream;  // creation stream; memory is released on it
     pbg::GridGeo geo;
     long long na;
