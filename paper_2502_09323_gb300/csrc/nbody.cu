@@ -12,12 +12,16 @@
 // Kahan compensation in FP32, and the tile sum is added to an FP64
 // accumulator.  A thread's two targets share each
 // instruction through the packed FP32x2 arithmetic of sm_100-class GPUs.
-// It serves the surface terms Phi_p, Psi_p at the crossing points.
+// It serves the surface terms Phi_p, Psi_p at the crossing points; of large
+// sums it takes the near atoms only (nbody_far.cuh).
 //
 // FP64 kernels: the boundary values (they enter the linear system) and the
 // Coulomb energy sum_{i<j} q_i q_j / r_ij (a net value of large terms of
 // either sign), each summed in a fixed order.
 #include <cub/block/block_reduce.cuh>
+#include <cub/device/device_radix_sort.cuh>
+
+#include <algorithm>
 
 #include "pb_internal.h"
 
@@ -31,6 +35,11 @@ constexpr int NB_GRP = 16; // sources per plainly summed group
 // largest coordinate offset (A) of a block's targets from its first target
 // for the per-block origin form of the differences
 constexpr double NB_ORIGIN_EXT = 8.0;
+// At least so many pairs: local expansions for far atoms.  Sorting the targets
+// and the balls take about 0.2 ms: 129^3 with 2,000 atoms (2.8e8 pairs) 0.33 ms by
+// pairs and 0.39 by expansions, 257^3 with 1,000 (4.6e8) 0.47 and 0.35, an octree of
+// 1,000 atoms (3.2e8) 0.35 and 0.31.
+constexpr long long FAR_PAIRS = 300000000;
 
 struct SrcHi {
     float x, y, z, q;
@@ -65,6 +74,8 @@ struct TargetDesc {
     const long long *ids;
     const int8_t *sign;
     const double *nrm2; // optional second normal per target (PSI2): 3 per target
+    const int *order;   // optional: the targets in the order in which blocks take them
+    int pair_form;      // 1: differences always from FP32 pairs
     long long count;
 };
 
@@ -104,6 +115,11 @@ __device__ __forceinline__ void boundary_node(const GridGeo &g, long long b, lon
             j = 1 + q2 - (g.ny - 2);
         }
     }
+}
+
+// the target at place t of the blocks' order (T.count: none)
+__device__ __forceinline__ long long target_at(const TargetDesc &T, long long t) {
+    return T.order && t < T.count ? T.order[t] : t;
 }
 
 struct TgtLoad {
@@ -168,6 +184,8 @@ __device__ __forceinline__ void kahan_add2(float2 &s, float2 &c, float2 v) {
     s = t;
 }
 
+#include "nbody_far.cuh"
+
 // The source tiles of one block: per-pair work, group sums and tile sums as
 // described above, accumulated into acc_* (FP64).
 // ORIGIN: the block's targets lie within NB_ORIGIN_EXT of its first target
@@ -177,42 +195,39 @@ __device__ __forceinline__ void kahan_add2(float2 &s, float2 &c, float2 v) {
 // operation instead of three.  Near sources (at least one atom radius away
 // from a point of the molecular surface) then keep about 15 u of relative
 // accuracy in r, far ones about u.
-template <bool PSI, bool SCREEN, bool PSI2, int AXIS, bool ORIGIN>
-__device__ __forceinline__ void nb_tiles(float4 (*sp4)[4], const float4 *__restrict__ shi,
+// FAR: only the sources that are no far ones of `ball`, gathered in source
+// order into whole tiles.
+template <bool PSI, bool SCREEN, bool PSI2, int AXIS, bool ORIGIN, bool FAR>
+__device__ __forceinline__ void nb_tiles(float4 (*sp4)[4], const far::Ball &ball, const float4 *__restrict__ shi,
                                          const float4 *__restrict__ slo, long long ns, float kscr,
                                          const float (&oh)[3], const float (&ol)[3],
                                          const float2 (&th)[3], const float2 (&tl)[3],
                                          const float2 (&tn)[3], const float2 (&tn2)[3],
                                          double (&acc_phi)[NB_TPT], double (&acc_psi)[NB_TPT],
                                          double (&acc_psi2)[NB_TPT]) {
-    for (long long base = 0; base < ns; base += NB_THREADS) {
-        long long si = base + threadIdx.x;
-        __syncthreads();
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-        if (si < ns) {
-            a = shi[si];
-            b = slo[si];
-        }
+    auto stage = [&](int at, const float4 &a, const float4 &b) {
         if (ORIGIN) {
             const float rx = (a.x - oh[0]) + (b.x - ol[0]), ry = (a.y - oh[1]) + (b.y - ol[1]),
                         rz = (a.z - oh[2]) + (b.z - ol[2]);
-            sp4[threadIdx.x][0] = make_float4(rx, rx, ry, ry);
-            sp4[threadIdx.x][1] = make_float4(rz, rz, a.w, a.w);
+            sp4[at][0] = make_float4(rx, rx, ry, ry);
+            sp4[at][1] = make_float4(rz, rz, a.w, a.w);
         } else {
-            sp4[threadIdx.x][0] = make_float4(a.x, a.x, a.y, a.y);
-            sp4[threadIdx.x][1] = make_float4(a.z, a.z, a.w, a.w);
-            sp4[threadIdx.x][2] = make_float4(b.x, b.x, b.y, b.y);
-            sp4[threadIdx.x][3] = make_float4(b.z, b.z, 0.f, 0.f);
+            sp4[at][0] = make_float4(a.x, a.x, a.y, a.y);
+            sp4[at][1] = make_float4(a.z, a.z, a.w, a.w);
+            sp4[at][2] = make_float4(b.x, b.x, b.y, b.y);
+            sp4[at][3] = make_float4(b.z, b.z, 0.f, 0.f);
         }
-        __syncthreads();
-        int m = (int)min((long long)NB_THREADS, ns - base);
+    };
+    // the first m staged sources
+    auto pairs = [&](int m) {
         float2 sp = bc2(0.f), cp = bc2(0.f), sq = bc2(0.f), cq = bc2(0.f), s2 = bc2(0.f),
                c2 = bc2(0.f);
-        // groups of NB_GRP sources are summed plainly in FP32 (rounding error
-        // below (NB_GRP - 1) u of the group's absolute sum) and each group
+        // groups of GRP sources are summed plainly in FP32 (rounding error
+        // below (GRP - 1) u of the group's absolute sum) and each group
         // sum enters the tile sum with Kahan compensation
-        for (int q0 = 0; q0 < m; q0 += NB_GRP) {
-            const int q1 = min(q0 + NB_GRP, m);
+        constexpr int GRP = FAR ? NB_GRP / 2 : NB_GRP;
+        for (int q0 = 0; q0 < m; q0 += GRP) {
+            const int q1 = min(q0 + GRP, m);
             float2 gp = bc2(0.f), gq = bc2(0.f), g2 = bc2(0.f);
 #pragma unroll 4
             for (int q = q0; q < q1; ++q) {
@@ -274,6 +289,57 @@ __device__ __forceinline__ void nb_tiles(float4 (*sp4)[4], const float4 *__restr
             acc_psi2[0] += (double)s2.x - (double)c2.x;
             acc_psi2[1] += (double)s2.y - (double)c2.y;
         }
+    };
+    if constexpr (FAR) {
+        __shared__ int wcount[NB_THREADS / 32];
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        int have = 0;
+        for (long long base = 0; base < ns; base += NB_THREADS) {
+            const long long si = base + threadIdx.x;
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            bool near = false;
+            if (si < ns) {
+                a = shi[si];
+                b = slo[si];
+                float d[3], r2;
+                near = !far::offset(a, b, ball, d, r2);
+            }
+            const unsigned mask = __ballot_sync(0xffffffffu, near);
+            __syncthreads();  // the last reads of wcount and of the staged sources
+            if (lane == 0) wcount[w] = __popc(mask);
+            __syncthreads();
+            int at = have + __popc(mask & ((1u << lane) - 1u));
+#pragma unroll
+            for (int q = 0; q < NB_THREADS / 32; ++q) {
+                const int c = wcount[q];
+                if (q < w) at += c;
+                have += c;
+            }
+            if (near) stage(at, a, b);
+            if (have < NB_THREADS) continue;
+            __syncthreads();
+            pairs(NB_THREADS);
+            have -= NB_THREADS;
+            __syncthreads();
+            if ((int)threadIdx.x < have)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) sp4[threadIdx.x][q] = sp4[NB_THREADS + threadIdx.x][q];
+        }
+        __syncthreads();
+        pairs(have);
+    } else {
+        for (long long base = 0; base < ns; base += NB_THREADS) {
+            const long long si = base + threadIdx.x;
+            __syncthreads();
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            if (si < ns) {
+                a = shi[si];
+                b = slo[si];
+            }
+            stage(threadIdx.x, a, b);
+            __syncthreads();
+            pairs((int)min((long long)NB_THREADS, ns - base));
+        }
     }
 }
 
@@ -283,19 +349,25 @@ __device__ __forceinline__ void nb_tiles(float4 (*sp4)[4], const float4 *__restr
 // thread holds two targets in the two halves of FP32x2 registers; the
 // sources are staged in shared memory already duplicated into (v, v) pairs.
 static_assert(NB_TPT == 2, "two targets per thread, one per FP32x2 half");
-template <bool PSI, bool SCREEN, bool PSI2 = false>
+// FAR: far sources through the block's expansion (nbody_far.cuh).
+template <bool PSI, bool SCREEN, bool PSI2 = false, bool FAR = false>
 __global__ void __launch_bounds__(NB_THREADS)
-k_nbody(TargetDesc T, const float4 *__restrict__ shi, const float4 *__restrict__ slo,
+k_nbody(TargetDesc T, far::Args F, const float4 *__restrict__ shi, const float4 *__restrict__ slo,
         long long ns, float kscr, double scale, double *__restrict__ out_phi,
         double *__restrict__ out_psi, double *__restrict__ out_psi2 = nullptr) {
     // per source: (hx,hx,hy,hy) (hz,hz,q,q) (lx,lx,ly,ly) (lz,lz,0,0)
-    __shared__ float4 sp4[NB_THREADS][4];
-    long long t0 = ((long long)blockIdx.x * NB_THREADS * NB_TPT) + threadIdx.x;
+    __shared__ float4 sp4[FAR ? 2 * NB_THREADS : NB_THREADS][4];
+    const long long at0 = (F.block0 + (long long)blockIdx.x) * NB_THREADS * NB_TPT;
+    const long long tb = target_at(T, at0);
+    long long tt[NB_TPT];
+    far::Ball ball{};
+    if (FAR) ball = F.ball[F.block0 + blockIdx.x];
     TgtLoad tg[NB_TPT];
     double acc_phi[NB_TPT], acc_psi[NB_TPT], acc_psi2[NB_TPT];
 #pragma unroll
     for (int u = 0; u < NB_TPT; ++u) {
-        tg[u] = load_target(T, t0 + (long long)u * NB_THREADS);
+        tt[u] = target_at(T, at0 + threadIdx.x + (long long)u * NB_THREADS);
+        tg[u] = load_target(T, tt[u]);
         acc_phi[u] = 0.0;
         acc_psi[u] = 0.0;
         acc_psi2[u] = 0.0;
@@ -312,12 +384,11 @@ k_nbody(TargetDesc T, const float4 *__restrict__ shi, const float4 *__restrict__
     // crossing list is ordered by direction) takes the axis form of Psi
     int axis = -1;
     if (PSI && T.kind == TK_SURFACE) {
-        const long long tb = (long long)blockIdx.x * NB_THREADS * NB_TPT;
         const int dref = (int)(T.ids[tb] / T.g.N);
         bool same = true;
 #pragma unroll
         for (int u = 0; u < NB_TPT; ++u) {
-            const long long t = t0 + (long long)u * NB_THREADS;
+            const long long t = tt[u];
             if (t < T.count && (int)(T.ids[t] / T.g.N) != dref) same = false;
         }
         if (__syncthreads_and(same)) axis = dref;
@@ -327,14 +398,13 @@ k_nbody(TargetDesc T, const float4 *__restrict__ shi, const float4 *__restrict__
     bool origin = false;
     float oh[3] = {0.f, 0.f, 0.f}, ol[3] = {0.f, 0.f, 0.f};
     if (T.kind == TK_SURFACE) {
-        const long long tb = (long long)blockIdx.x * NB_THREADS * NB_TPT;
         double o[3], rel[NB_TPT][3];
-        bool near = true;
+        bool near = !T.pair_form;
 #pragma unroll
         for (int d = 0; d < 3; ++d) o[d] = T.rp[3 * tb + d];
 #pragma unroll
         for (int u = 0; u < NB_TPT; ++u) {
-            const long long t = t0 + (long long)u * NB_THREADS;
+            const long long t = tt[u];
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 rel[u][d] = t < T.count ? T.rp[3 * t + d] - o[d] : 0.0;
@@ -353,10 +423,10 @@ k_nbody(TargetDesc T, const float4 *__restrict__ shi, const float4 *__restrict__
         }
     }
 #define PB_NB_TILES(AX)                                                                          \
-    (origin ? nb_tiles<PSI, SCREEN, PSI2, AX, true>(sp4, shi, slo, ns, kscr, oh, ol, th, tl, tn, \
-                                                     tn2, acc_phi, acc_psi, acc_psi2)            \
-            : nb_tiles<PSI, SCREEN, PSI2, AX, false>(sp4, shi, slo, ns, kscr, oh, ol, th, tl, tn, \
-                                                      tn2, acc_phi, acc_psi, acc_psi2))
+    (origin ? nb_tiles<PSI, SCREEN, PSI2, AX, true, FAR>(sp4, ball, shi, slo, ns, kscr, oh, ol,  \
+                                                         th, tl, tn, tn2, acc_phi, acc_psi, acc_psi2) \
+            : nb_tiles<PSI, SCREEN, PSI2, AX, false, FAR>(sp4, ball, shi, slo, ns, kscr, oh, ol, \
+                                                          th, tl, tn, tn2, acc_phi, acc_psi, acc_psi2))
     switch (axis) {
         case 0: PB_NB_TILES(0); break;
         case 1: PB_NB_TILES(1); break;
@@ -364,6 +434,40 @@ k_nbody(TargetDesc T, const float4 *__restrict__ shi, const float4 *__restrict__
         default: PB_NB_TILES(-1);
     }
 #undef PB_NB_TILES
+    if constexpr (FAR) {
+        // Psi = -n . grad; the axis form takes the sign of n below
+        __syncthreads();  // the staged sources' last reads
+        far::Series &S = *reinterpret_cast<far::Series *>(sp4);
+        static_assert(sizeof(far::Series) + sizeof(double2) * far::NC <= sizeof(sp4), "the series fits the staging area");
+        far::make_series(F, reinterpret_cast<double2 *>(&S + 1), S);
+        __syncthreads();
+        double x[NB_TPT][3];
+#pragma unroll
+        for (int u = 0; u < NB_TPT; ++u) {
+            const long long t = tt[u];
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                x[u][d] = t < T.count ? ((T.rp[3 * t + d] - T.shift[d]) - (double)ball.c[d]) * ball.inv : 0.0;
+        }
+        float2 xx[3], v[4];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) xx[d] = make_float2((float)x[0][d], (float)x[1][d]);
+        far::evaluate(S, xx, v);
+#pragma unroll
+        for (int u = 0; u < NB_TPT; ++u) {
+            double g[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                g[d] = (S.top[1 + d] + (double)(u ? v[1 + d].y : v[1 + d].x)) * (ball.inv * ball.inv);
+            acc_phi[u] += (S.top[0] + (double)(u ? v[0].y : v[0].x)) * ball.inv;
+            const double ga = axis == 0 ? g[0] : (axis == 1 ? g[1] : g[2]);
+            acc_psi[u] -= axis >= 0 ? ga
+                                    : g[0] * (double)tg[u].n[0] + g[1] * (double)tg[u].n[1] + g[2] * (double)tg[u].n[2];
+            if (PSI2)
+                acc_psi2[u] -=
+                    g[0] * (double)tg[u].n2[0] + g[1] * (double)tg[u].n2[1] + g[2] * (double)tg[u].n2[2];
+        }
+    }
     if (PSI && axis >= 0) {
         // n = sign e_axis: the one nonzero component is the sign
 #pragma unroll
@@ -372,7 +476,7 @@ k_nbody(TargetDesc T, const float4 *__restrict__ shi, const float4 *__restrict__
     }
 #pragma unroll
     for (int u = 0; u < NB_TPT; ++u) {
-        long long t = t0 + (long long)u * NB_THREADS;
+        const long long t = tt[u];
         if (t >= T.count) continue;
         if (T.kind == TK_BOUNDARY) {
             long long i, j, k;
@@ -547,6 +651,78 @@ pb_status split_sources(pb_system *sys, cudaStream_t s, float4 **hi, float4 **lo
     return PB_OK;
 }
 
+// Bricks of 8^3 finest nodes in the order in which blocks take their targets:
+// rods of 2 x 2 bricks, a slice of four bricks at a time, up one rod and
+// down the next one beside it, so that neighbours in the order are neighbours
+// in space.
+struct RodOrder {
+    int nx, ny, nz;  // bricks along x, rods along y and z
+    __host__ __device__ long long keys() const { return (long long)nx * ny * nz; }
+    __device__ unsigned key(int bx, int by, int bz) const {
+        const int y = by >> 1, z = bz >> 1, rod = z * ny + ((z & 1) ? ny - 1 - y : y);
+        return (unsigned)rod * (unsigned)nx + (unsigned)((rod & 1) ? nx - 1 - bx : bx);
+    }
+};
+
+// sort keys of the crossing edges: the brick of their lower ends
+__global__ void k_target_keys(const long long *__restrict__ ids, long long n, GridGeo g, const int4 *__restrict__ blow,
+                              RodOrder rods, unsigned int *__restrict__ key, int *__restrict__ val) {
+    const long long t = blockIdx.x * 256ll + threadIdx.x;
+    if (t >= n) return;
+    long long a = ids[t];
+    while (a >= g.N) a -= g.N;
+    if (blow) {  // octree: a slot of a brick
+        const int4 low = blow[a >> 9];
+        key[t] = rods.key(low.x >> 3, low.y >> 3, low.z >> 3);
+    } else {
+        const long long r = a / g.nx, z = r / g.ny;
+        key[t] = rods.key((int)(a - r * g.nx) >> 3, (int)(r - z * g.ny) >> 3, (int)z >> 3);
+    }
+    val[t] = (int)t;
+}
+
+// The order in which blocks take the targets: by bricks, the three directions
+// together, so that a block's 512 lie close together (the crossing list goes
+// through the molecule three times, in node order on uniform grids; in an
+// octree's Morton order a few blocks at its jumps had most of the atoms near
+// them: 18.9 ms on 20,000 atoms).  A stable sort, so the order, and with it every bit of the
+// sums, is the same on every run.  Null beyond 2^31 targets or 2^32 keys.
+pb_status order_targets(pb_grid *g, int **order, cudaStream_t s) {
+    const long long n = g->ncross;
+    auto bricks = [&](long long nodes) { return (int)((nodes - 1) >> 3) + 1; };
+    const long long nx = g->is_oct ? g->ot.NL + 1 : g->geo.nx, ny = g->is_oct ? g->ot.NL + 1 : g->geo.ny,
+                    nz = g->is_oct ? g->ot.NL + 1 : g->geo.nz;
+    const RodOrder rods = {bricks(nx), (bricks(ny) + 1) / 2, (bricks(nz) + 1) / 2};
+    int bits = 1;
+    while ((rods.keys() - 1) >> bits) ++bits;
+    if (bits > 32 || n > 0x7fffffffll) return PB_OK;
+    unsigned *key = (unsigned *)dalloc(sizeof(unsigned) * n, s), *key2 = (unsigned *)dalloc(sizeof(unsigned) * n, s);
+    int *val = (int *)dalloc(sizeof(int) * n, s), *val2 = (int *)dalloc(sizeof(int) * n, s);
+    void *tmp = nullptr;
+    size_t bytes = 0;
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (key && key2 && val && val2) {
+        k_target_keys<<<cdiv(n, 256), 256, 0, s>>>(g->cid, n, g->geo, g->is_oct ? g->ot.blow : nullptr, rods, key,
+                                                      val);
+        e = cub::DeviceRadixSort::SortPairs(nullptr, bytes, key, key2, val, val2, (int)n, 0, bits, s);
+        if (e == cudaSuccess && !(tmp = dalloc(bytes, s))) e = cudaErrorMemoryAllocation;
+        if (e == cudaSuccess)
+            e = cub::DeviceRadixSort::SortPairs(tmp, bytes, key, key2, val, val2, (int)n, 0, bits, s);
+    }
+    dfree(tmp, s);
+    dfree(key, s);
+    dfree(key2, s);
+    dfree(val, s);
+    if (e != cudaSuccess) {
+        dfree(val2, s);
+        if (e == cudaErrorMemoryAllocation) return PB_ERR_OOM;
+        set_error("sorting the surface targets failed: %s", cudaGetErrorString(e));
+        return PB_ERR_CUDA;
+    }
+    *order = val2;
+    return PB_OK;
+}
+
 TargetDesc make_desc(pb_system *sys, int kind) {
     pb_grid *g = sys->g;
     TargetDesc T;
@@ -557,6 +733,8 @@ TargetDesc make_desc(pb_system *sys, int kind) {
     T.ids = g->cid;
     T.sign = g->csign;
     T.nrm2 = nullptr;
+    T.order = nullptr;
+    T.pair_form = 0;
     T.count = 0;
     return T;
 }
@@ -598,11 +776,45 @@ pb_status nbody_surface(pb_system *sys, cudaStream_t s) {
     if (!sys->PsiN) sys->PsiN = (double *)dalloc(sizeof(double) * nc, s);
     if (!sys->PsiN) return PB_ERR_OOM;
     T.nrm2 = g->mc_n;
-    k_nbody<true, false, true><<<cdiv(T.count, NB_THREADS * NB_TPT), NB_THREADS, 0, s>>>(
-        T, hi, lo, g->na, 0.f, 1.0, sys->Phi, sys->Psi, sys->PsiN);
-    PB_LAUNCH_CHECK();
+    int *order = nullptr;
+    if (g->na * g->ncross >= FAR_PAIRS && (st = order_targets(g, &order, s)) != PB_OK) return st;
+    T.order = order;
+    T.pair_form = order && !g->is_oct;
+    const int per = NB_THREADS * NB_TPT;
+    const unsigned blocks = cdiv(T.count, per);
+    far::Args F{};
+    if (!order) {
+        k_nbody<true, false, true>
+            <<<blocks, NB_THREADS, 0, s>>>(T, F, hi, lo, g->na, 0.f, 1.0, sys->Phi, sys->Psi, sys->PsiN);
+        PB_LAUNCH_CHECK();
+    } else {
+        // so many target blocks at a time that their partial sums stay within far::BYTES
+        F.chunks = (int)cdiv(g->na, far::CHUNK);
+        const size_t each = sizeof(float2) * far::NS * (size_t)F.chunks;
+        const unsigned parts = cdiv(blocks, std::max<long long>(far::BYTES / (long long)each, 1)), most = cdiv(blocks, parts);
+        far::Ball *ball = (far::Ball *)dalloc(sizeof(far::Ball) * blocks, s);
+        float2 *part = (float2 *)dalloc(each * most, s);
+        if (ball && part) {
+            F.ball = ball;
+            F.part = part;
+            k_far_ball<<<blocks, 256, 0, s>>>(g->crp, T.order, T.count, g->center[0], g->center[1], g->center[2], ball);
+            for (unsigned b = 0; b < blocks; b += most) {
+                const unsigned n = std::min(most, blocks - b);
+                F.block0 = b;
+                k_far_local<<<dim3(n, (unsigned)F.chunks), far::T, 0, s>>>(hi, lo, g->na, ball, b, part);
+                k_nbody<true, false, true, true>
+                    <<<n, NB_THREADS, 0, s>>>(T, F, hi, lo, g->na, 0.f, 1.0, sys->Phi, sys->Psi, sys->PsiN);
+            }
+        }
+        dfree(ball, s);
+        dfree(part, s);
+        if (!ball || !part) st = PB_ERR_OOM;
+    }
+    dfree(order, s);
     dfree(hi, s);
     dfree(lo, s);
+    if (st != PB_OK) return st;
+    PB_LAUNCH_CHECK();
     return PB_OK;
 }
 
