@@ -35,11 +35,11 @@ constexpr int NB_GRP = 16; // sources per plainly summed group
 // largest coordinate offset (A) of a block's targets from its first target
 // for the per-block origin form of the differences
 constexpr double NB_ORIGIN_EXT = 8.0;
-// At least so many pairs: local expansions for far atoms.  Sorting the targets
-// and the balls take about 0.2 ms: 129^3 with 2,000 atoms (2.8e8 pairs) 0.33 ms by
-// pairs and 0.39 by expansions, 257^3 with 1,000 (4.6e8) 0.47 and 0.35, an octree of
-// 1,000 atoms (3.2e8) 0.35 and 0.31.
-constexpr long long FAR_PAIRS = 300000000;
+// Octrees with at least so many pairs take local expansions for far atoms.
+// Sorting the targets and the balls take about 0.2 ms: pairs and expansions both
+// take 0.3 ms with 1,000 atoms (3.2e8 pairs), and 0.9 and 0.53 ms with 2,000 (1.2e9).
+// Uniform grids keep all pairs, whose sums are an output to the last bit.
+constexpr long long FAR_PAIRS = 400000000;
 
 struct SrcHi {
     float x, y, z, q;
@@ -75,7 +75,6 @@ struct TargetDesc {
     const int8_t *sign;
     const double *nrm2; // optional second normal per target (PSI2): 3 per target
     const int *order;   // optional: the targets in the order in which blocks take them
-    int pair_form;      // 1: differences always from FP32 pairs
     long long count;
 };
 
@@ -399,7 +398,7 @@ k_nbody(TargetDesc T, far::Args F, const float4 *__restrict__ shi, const float4 
     float oh[3] = {0.f, 0.f, 0.f}, ol[3] = {0.f, 0.f, 0.f};
     if (T.kind == TK_SURFACE) {
         double o[3], rel[NB_TPT][3];
-        bool near = !T.pair_form;
+        bool near = true;
 #pragma unroll
         for (int d = 0; d < 3; ++d) o[d] = T.rp[3 * tb + d];
 #pragma unroll
@@ -664,35 +663,29 @@ struct RodOrder {
     }
 };
 
-// sort keys of the crossing edges: the brick of their lower ends
-__global__ void k_target_keys(const long long *__restrict__ ids, long long n, GridGeo g, const int4 *__restrict__ blow,
-                              RodOrder rods, unsigned int *__restrict__ key, int *__restrict__ val) {
+// sort keys of an octree's crossing edges: the brick of their lower ends
+__global__ void
+k_target_keys(const long long *__restrict__ ids, long long n, long long slots, const int4 *__restrict__ blow, RodOrder rods,
+              unsigned int *__restrict__ key, int *__restrict__ val) {
     const long long t = blockIdx.x * 256ll + threadIdx.x;
     if (t >= n) return;
     long long a = ids[t];
-    while (a >= g.N) a -= g.N;
-    if (blow) {  // octree: a slot of a brick
-        const int4 low = blow[a >> 9];
-        key[t] = rods.key(low.x >> 3, low.y >> 3, low.z >> 3);
-    } else {
-        const long long r = a / g.nx, z = r / g.ny;
-        key[t] = rods.key((int)(a - r * g.nx) >> 3, (int)(r - z * g.ny) >> 3, (int)z >> 3);
-    }
+    while (a >= slots) a -= slots;
+    const int4 low = blow[a >> 9];
+    key[t] = rods.key(low.x >> 3, low.y >> 3, low.z >> 3);
     val[t] = (int)t;
 }
 
 // The order in which blocks take the targets: by bricks, the three directions
 // together, so that a block's 512 lie close together (the crossing list goes
-// through the molecule three times, in node order on uniform grids; in an
-// octree's Morton order a few blocks at its jumps had most of the atoms near
-// them: 18.9 ms on 20,000 atoms).  A stable sort, so the order, and with it every bit of the
-// sums, is the same on every run.  Null beyond 2^31 targets or 2^32 keys.
+// through the molecule three times; in the octree's Morton order a few blocks at
+// its jumps had most of the atoms near them: 18.9 ms on 20,000 atoms).  A stable
+// sort, so the order, and with it every bit of the sums, is the same on every
+// run.  Null beyond 2^31 targets or 2^32 keys.
 pb_status order_targets(pb_grid *g, int **order, cudaStream_t s) {
     const long long n = g->ncross;
-    auto bricks = [&](long long nodes) { return (int)((nodes - 1) >> 3) + 1; };
-    const long long nx = g->is_oct ? g->ot.NL + 1 : g->geo.nx, ny = g->is_oct ? g->ot.NL + 1 : g->geo.ny,
-                    nz = g->is_oct ? g->ot.NL + 1 : g->geo.nz;
-    const RodOrder rods = {bricks(nx), (bricks(ny) + 1) / 2, (bricks(nz) + 1) / 2};
+    const int side = g->ot.NL / 8 + 1, pairs = (side + 1) / 2;  // bricks an axis
+    const RodOrder rods = {side, pairs, pairs};
     int bits = 1;
     while ((rods.keys() - 1) >> bits) ++bits;
     if (bits > 32 || n > 0x7fffffffll) return PB_OK;
@@ -702,8 +695,7 @@ pb_status order_targets(pb_grid *g, int **order, cudaStream_t s) {
     size_t bytes = 0;
     cudaError_t e = cudaErrorMemoryAllocation;
     if (key && key2 && val && val2) {
-        k_target_keys<<<cdiv(n, 256), 256, 0, s>>>(g->cid, n, g->geo, g->is_oct ? g->ot.blow : nullptr, rods, key,
-                                                      val);
+        k_target_keys<<<cdiv(n, 256), 256, 0, s>>>(g->cid, n, g->geo.N, g->ot.blow, rods, key, val);
         e = cub::DeviceRadixSort::SortPairs(nullptr, bytes, key, key2, val, val2, (int)n, 0, bits, s);
         if (e == cudaSuccess && !(tmp = dalloc(bytes, s))) e = cudaErrorMemoryAllocation;
         if (e == cudaSuccess)
@@ -734,7 +726,6 @@ TargetDesc make_desc(pb_system *sys, int kind) {
     T.sign = g->csign;
     T.nrm2 = nullptr;
     T.order = nullptr;
-    T.pair_form = 0;
     T.count = 0;
     return T;
 }
@@ -777,9 +768,8 @@ pb_status nbody_surface(pb_system *sys, cudaStream_t s) {
     if (!sys->PsiN) return PB_ERR_OOM;
     T.nrm2 = g->mc_n;
     int *order = nullptr;
-    if (g->na * g->ncross >= FAR_PAIRS && (st = order_targets(g, &order, s)) != PB_OK) return st;
+    if (g->is_oct && g->na * g->ncross >= FAR_PAIRS && (st = order_targets(g, &order, s)) != PB_OK) return st;
     T.order = order;
-    T.pair_form = order && !g->is_oct;
     const int per = NB_THREADS * NB_TPT;
     const unsigned blocks = cdiv(T.count, per);
     far::Args F{};

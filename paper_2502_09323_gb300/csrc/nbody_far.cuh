@@ -20,8 +20,8 @@
 // rounding of the FP32 pair sum.  Atoms beyond 2 KAPPA a take degree PD.
 //
 // Measured (GB300, surface sums, all pairs -> this): octree of 20,000 atoms
-// 73.0 -> 8.7 ms (coefficients 4.5, near pairs and evaluation 3.9), 5,000 atoms
-// 5.8 -> 1.3 ms, 257^3 with 2,000 atoms 1.17 -> 0.52 ms.  Errors against 64 bits,
+// 73.0 -> 8.7 ms (coefficients 4.5, near pairs and evaluation 3.9), 2,000
+// atoms 0.9 -> 0.53 ms.  Errors against 64 bits,
 // 2-norm relative, of Phi 5.5e-8 -> 3.8e-8 and of Psi 1.83e-7 -> 1.69e-7 (20,000
 // atoms).  What gave it, one after the other: targets in list order, whose
 // blocks are wide, 20.6 ms; a power of two as unit and compensated sums of

@@ -8,9 +8,9 @@ import pb_inputs
 pytestmark = pytest.mark.gpu
 
 
-# a small molecule that takes the expansions, one source past a chunk, one whose
-# target blocks need two pairs of launches, and a ragged uniform grid
-@pytest.mark.parametrize("n, h, one_sign", [(1500, 0.25, False), (4097, 0.5, True), (13000, 0.25, False), (2000, 0.0, True)])
+# a small molecule that takes the expansions, one source past a chunk, and one whose
+# target blocks need two pairs of launches
+@pytest.mark.parametrize("n, h, one_sign", [(1500, 0.25, False), (4097, 0.5, True), (13000, 0.25, False)])
 def test_far_sums(n, h, one_sign):
     import torch
     if not torch.cuda.is_available():
@@ -19,17 +19,12 @@ def test_far_sums(n, h, one_sign):
     atoms = pb_inputs.globular_molecule(n, seed=31)
     if one_sign:
         atoms[:, 4] = np.abs(atoms[:, 4])
-    if h:
-        spec = pb.OctreeSpec(h_fine=h, h_bulk=1.0, refine_dist=3.0)
-    else:
-        lo, hi = (atoms[:, :3] - 2.5).min(0), (atoms[:, :3] + 2.5).max(0)
-        spec = pb.GridSpec(n=tuple(int(v) for v in (hi - lo) / 0.22), origin=tuple(float(v) for v in lo), h=0.22)
-    g = pb.pb_build_grid(spec, atoms)
+    g = pb.pb_build_grid(pb.OctreeSpec(h_fine=h, h_bulk=1.0, refine_dist=3.0), atoms)
     s = pb.pb_assemble_coeffs(g, pb.Params())
     pb.pb_coulomb_terms(s, pb.CT_SURFACE)
     arr = {k: pb.pb_get_array(s, k) for k in ("cross_sign", "cross_id", "cross_rp", "mc_normal", "phi_surf",
                                               "psi_surf", "psi_n")}
-    assert len(arr["cross_id"]) * n >= 300000000  # the library's threshold
+    assert len(arr["cross_id"]) * n >= 400000000  # the library's threshold
     flux = np.nonzero(arr["cross_sign"])[0]
     assert np.all(arr["phi_surf"][arr["cross_sign"] == 0] == 0.0)
     pick = np.concatenate([flux[:600], flux[-600:], np.random.default_rng(1).choice(flux, 20000)])
