@@ -298,6 +298,27 @@ __device__ __forceinline__ bool edge_cut(double xad, double cd, double w, double
     return true;
 }
 
+// What edge_cut says of an edge without its divisions: 0 for an empty interval, else
+// 1, with bit 1 for t0 > 0 and bit 2 for t1 < 1.  Division by h rounds to the
+// nearest: n0 / h > 0 for n0 > 0, and n1 / h < 1 for n1 < h (at most 1 - 2^-53,
+// which is a value of the type), both short of underflow, and
+// n1 / h > n0 / h where the two are more than rounding apart.  The others ask
+// edge_cut.
+__device__ __forceinline__ int edge_kind(double xad, double cd, double w, double h) {
+    const double ud = xad - cd;
+    const double n0 = -ud - w;
+    const double n1 = -ud + w;
+    if (n0 >= h || n1 <= 0.0) return 0;
+    const bool p0 = n0 > 0.0, p1 = n1 < h;
+    if (__double2hiint(n1) < 0x06000000 || (p0 && __double2hiint(n0) < 0x06000000) ||
+        (p0 && p1 && !(n1 - n0 > 1e-14 * n1))) {
+        double t0, t1;
+        if (!edge_cut(xad, cd, w, h, t0, t1)) return 0;
+        return 1 | (t0 > 0.0 ? 2 : 0) | (t1 < 1.0 ? 4 : 0);
+    }
+    return 1 | (p0 ? 2 : 0) | (p1 ? 4 : 0);
+}
+
 // Measure of the union of the intervals of all balls meeting the edge; the
 // intervals are ordered by (t0, t1) and merged.  Returns false on overflow.
 // With COVER_EXIT the scan stops at the first ball whose interval is all of
@@ -427,6 +448,10 @@ __device__ __forceinline__ EdgeRef edge_ref(const GridGeo &g, long long e) {
 // interval for this ball is all of [0, 1] get cov byte 1: on those the union
 // is [0, 1] whatever the other balls add, so alpha = 1 exactly.  (Several
 // balls may write the same byte, always with the same value.)
+//
+// FP64 issue binds (an instruction takes a warp 16 cycles): about 10 operations
+// an edge and four edges a line, against 26 (two divisions) and seven before:
+// 257^3 with 2,000 atoms 552 -> 310 us.
 __global__ void k_edge_cand(const double *__restrict__ atoms, long long na, GridGeo g,
                             uint8_t *__restrict__ flags, uint8_t *__restrict__ cov) {
     const double *X = atoms, *Y = atoms + na, *Z = atoms + 2 * na, *R = atoms + 3 * na;
@@ -436,13 +461,18 @@ __global__ void k_edge_cand(const double *__restrict__ atoms, long long na, Grid
         const double c[3] = {X[at], Y[at], Z[at]};
         const double r = R[at], hinv = 1.0 / g.h;
         const float r32 = (float)r;
-        long long lo[3], hi[3], ext[3];
+        long long lo[3], hi[3];
+        int ext[3];
+        // what rounding may move a crossing of a line by, in spacings, many times over
+        double slack[3];
         for (int d = 0; d < 3; ++d) {
             lo[d] = clampll((long long)floor((c[d] - r - g.o[d]) / g.h) - 1, 0, nn[d] - 1);
             hi[d] = clampll((long long)ceil((c[d] + r - g.o[d]) / g.h) + 1, 0, nn[d] - 1);
-            ext[d] = hi[d] - lo[d] + 1;
+            ext[d] = (int)(hi[d] - lo[d]) + 1;
+            slack[d] = 1e-6 + 1e-13 * hinv * (fabs(c[d]) + r + fabs(g.o[d]) + (double)nn[d] * g.h);
         }
-        const long long nl0 = ext[1] * ext[2], nl1 = ext[0] * ext[2], nl2 = ext[0] * ext[1];
+        const long long nl0 = (long long)ext[1] * ext[2], nl1 = (long long)ext[0] * ext[2],
+                        nl2 = (long long)ext[0] * ext[1];
         for (long long t = threadIdx.x; t < nl0 + nl1 + nl2; t += blockDim.x) {
             int d;
             long long q;
@@ -458,8 +488,9 @@ __global__ void k_edge_cand(const double *__restrict__ atoms, long long na, Grid
             }
             const int e = (d == 0) ? 1 : 0;
             const int f = (d == 2) ? 1 : 2;
-            const long long ie = lo[e] + q % ext[e];
-            const long long jf = lo[f] + q / ext[e];
+            const unsigned qf = q < 0x7fffffffll ? (unsigned)q / (unsigned)ext[e] : (unsigned)(q / ext[e]);
+            const long long ie = lo[e] + (q - (long long)qf * ext[e]);
+            const long long jf = lo[f] + qf;
             const long long ilo = lo[d];
             const long long ihi = hi[d] < (long long)nn[d] - 2 ? hi[d] : (long long)nn[d] - 2;
             if (ihi < ilo) continue;
@@ -474,28 +505,29 @@ __global__ void k_edge_cand(const double *__restrict__ atoms, long long na, Grid
             double w;
             if (!line_cut(xa, d, c[e], c[f], r, w)) continue;
             const long long base = (long long)d * g.N + ie * step[e] + jf * step[f];
-            // Edges more than a spacing below or above the ball have an empty
-            // interval (n0 >= h or n1 <= 0 by a whole spacing, far more than
-            // rounding): the scans start and end there.
-            const long long i_lo = max(ilo, (long long)floor((c[d] - w - g.o[d]) * hinv) - 1);
-            const long long i_hi = min(ihi, (long long)ceil((c[d] + w - g.o[d]) * hinv) + 1);
+            // Edges below or above the crossings of the ball's surface by
+            // more than rounding have an empty interval (n0 >= h or n1 <= 0):
+            // the scans start and end at the crossed ones.
+            const double mid = (c[d] - g.o[d]) * hinv, half = w * hinv;
+            const long long i_lo = max(ilo, (long long)floor(mid - half - slack[d]));
+            const long long i_hi = min(ihi, (long long)floor(mid + half + slack[d]));
             long long iu = ihi + 1, id = ihi + 1;
             bool cov_iu = false;
             for (long long i = i_lo; i <= i_hi; ++i) {
-                double t0, t1;
-                if (!edge_cut(node_coord(g, d, i), c[d], w, g.h, t0, t1)) continue;
-                if (t0 > 0.0 || t1 < 1.0) flags[base + i * step[d]] = 2;
-                if (!(t0 > 0.0)) {
+                const int kind = edge_kind(node_coord(g, d, i), c[d], w, g.h);
+                if (!kind) continue;
+                if (kind > 1) flags[base + i * step[d]] = 2;
+                if (!(kind & 2)) {
                     iu = i;
-                    cov_iu = !(t1 < 1.0);
+                    cov_iu = !(kind & 4);
                     break;
                 }
             }
             for (long long i = i_hi; i > iu; --i) {
-                double t0, t1;
-                if (!edge_cut(node_coord(g, d, i), c[d], w, g.h, t0, t1)) continue;
-                if (t0 > 0.0 || t1 < 1.0) flags[base + i * step[d]] = 2;
-                if (!(t1 < 1.0)) {
+                const int kind = edge_kind(node_coord(g, d, i), c[d], w, g.h);
+                if (!kind) continue;
+                if (kind > 1) flags[base + i * step[d]] = 2;
+                if (!(kind & 4)) {
                     id = i;
                     break;
                 }
