@@ -68,8 +68,10 @@ __device__ __forceinline__ double2 ld2(const double *a, int i) {
 __global__ void __launch_bounds__(cg64::NT, 2) k_cg64_dir(cg64::DirArgs A) {
     using namespace cg64;
     __shared__ double sred[NT / 32];
-    if (A.st->done) return;  // changes only at the end of a launch
-    const double beta = A.st->beta;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (*(volatile int *)&A.st->done) return;  // changes only at the end of a launch
+    const double beta = *(volatile double *)&A.st->beta;
     const PadGeo g = A.g;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i0 = blockIdx.x * TXP;
@@ -210,8 +212,10 @@ __global__ void __launch_bounds__(cg64::NT, 2) k_cg64_dir(cg64::DirArgs A) {
 __global__ void __launch_bounds__(cg64::UNT, 4) k_cg64_upd(cg64::UpdArgs A) {
     using namespace cg64;
     __shared__ double sred[UNT / 32];
-    if (A.st->done) return;
-    const double alpha = A.st->alpha;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (*(volatile int *)&A.st->done) return;
+    const double alpha = *(volatile double *)&A.st->alpha;
     double rho = 0.0, rr = 0.0;
     const long long n2 = A.count >> 1;
     const long long stride = (long long)gridDim.x * UNT;

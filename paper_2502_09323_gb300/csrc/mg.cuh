@@ -102,7 +102,15 @@ __host__ __device__ inline int uitems(const Entry &e, int l) {
 }
 
 __device__ __forceinline__ float quotient(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double quotient(double a, double b) { return a / b; }
+// FP64: the hardware's approximation y of 1/b (b a diagonal: positive and
+// normal), e = 1 - b y, 1/b = y / (1 - e) = y (1 + e + e^2 + O(e^3)); five FP64
+// operations
+__device__ __forceinline__ double quotient(double a, double b) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double e = fma(-b, y, 1.0);
+    return a * fma(y, fma(e, e, e), y);
+}
 
 __device__ __forceinline__ float4 f4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
@@ -1224,7 +1232,9 @@ __global__ void k_mg_diag(mg::LevT<T> C) {
 // kernels before memory does (about 50 FP64 operations per unknown and cycle),
 // so residual, restriction, interpolation and smoothing are kernels of their
 // own and no value is formed twice.  97^3 to 1e-12: 500 Jacobi iterations and
-// 29.9 ms -> 29 iterations and 7.2 ms.
+// 29.9 ms -> 29 iterations and 5.9 ms (7.3 ms with a node a thread in the top smoother, whose block sums
+// then cost as much as its stencil, with divisions in the bottom kernel and
+// without programmatic launches).
 namespace mg {
 struct Entry64 {
     using T = double;
@@ -1238,9 +1248,9 @@ __device__ __forceinline__ double face_sum64(const LevT<double> &L, const double
     return ((L.wx[p - 1] * x[p - 1] + L.wx[p] * x[p + 1]) + (L.wy[p - L.sx] * x[p - L.sx] + L.wy[p] * x[p + L.sx])) +
            (L.wz[p - L.sxy] * x[p - L.sxy] + L.wz[p] * x[p + L.sxy]);
 }
-// interior node of a thread
-__device__ __forceinline__ bool node64(const LevT<double> &L, int &i, int &j, int &k) {
-    const int mx = L.nx - 2, my = L.ny - 2, t = blockIdx.x * 256 + threadIdx.x;
+// interior node t
+__device__ __forceinline__ bool node64(const LevT<double> &L, int t, int &i, int &j, int &k) {
+    const int mx = L.nx - 2, my = L.ny - 2;
     if (t >= mx * my * (L.nz - 2)) return false;
     const int r = t / mx;
     i = 1 + t - r * mx;
@@ -1252,18 +1262,22 @@ __device__ __forceinline__ bool node64(const LevT<double> &L, int &i, int &j, in
 
 __global__ void __launch_bounds__(256) k_mg64_residual(mg::LevT<double> L, const CgState *st) {
     using namespace mg;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (*(volatile const int *)&st->done) return;
     int i, j, k;
-    if (!node64(L, i, j, k)) return;
+    if (!node64(L, blockIdx.x * 256 + threadIdx.x, i, j, k)) return;
     const int p = k * L.sxy + j * L.sx + i;
     L.r[p] = (1.0 - (double)OMEGA) * L.dg[p] * L.s[p] + (double)OMEGA * face_sum64(L, L.s, p);
 }
 
 __global__ void __launch_bounds__(256) k_mg64_restrict(mg::LevT<double> L, mg::LevT<double> C, const CgState *st) {
     using namespace mg;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (*(volatile const int *)&st->done) return;
     int I, J, K;
-    if (!node64(C, I, J, K)) return;
+    if (!node64(C, blockIdx.x * 256 + threadIdx.x, I, J, K)) return;
     const double *f = L.r + (2 * K * L.sxy + 2 * J * L.sx + 2 * I);
     double acc = 0.0;
 #pragma unroll
@@ -1279,35 +1293,44 @@ __global__ void __launch_bounds__(256) k_mg64_restrict(mg::LevT<double> L, mg::L
 
 __global__ void __launch_bounds__(256) k_mg64_correct(mg::LevT<double> L, mg::LevT<double> C, const CgState *st) {
     using namespace mg;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (*(volatile const int *)&st->done) return;
     int i, j, k;
-    if (!node64(L, i, j, k)) return;
+    if (!node64(L, blockIdx.x * 256 + threadIdx.x, i, j, k)) return;
+    // an even coordinate lies on a coarse line: no sum along it.  The values of
+    // the corners are added up and scaled once.
     const double *x = C.z + ((k >> 1) * C.sxy + (j >> 1) * C.sx + (i >> 1));
-    double e;
-    // an even coordinate lies on a coarse line: no sum along it
-    auto line = [&](const double *q) { return (i & 1) ? 0.5 * (q[0] + q[1]) : q[0]; };
-    auto plane = [&](const double *q) { return (j & 1) ? 0.5 * (line(q) + line(q + C.sx)) : line(q); };
-    e = (k & 1) ? 0.5 * (plane(x) + plane(x + C.sxy)) : plane(x);
+    const bool odd = i & 1;
+    auto line = [&](const double *q) { return odd ? q[0] + q[1] : q[0]; };
+    auto plane = [&](const double *q) { return (j & 1) ? line(q) + line(q + C.sx) : line(q); };
+    const double e = (k & 1) ? plane(x) + plane(x + C.sxy) : plane(x);
+    const double f = __hiloint2double(0x3FF00000 - (((i & 1) + (j & 1) + (k & 1)) << 20), 0);  // 2^-(odd coordinates)
     const int p = k * L.sxy + j * L.sx + i;
-    L.r[p] = (double)OMEGA * L.s[p] + e;
+    L.r[p] = fma(f, e, (double)OMEGA * L.s[p]);
 }
 
 // the post-smoothing step (v in r); level 0: rho = r.z and beta
 template <bool TOP>
 __global__ void __launch_bounds__(256) k_mg64_smooth(mg::LevT<double> L, CgState *st, double *partials) {
     using namespace mg;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (*(volatile const int *)&st->done) return;
     __shared__ double sred[8];
     int i, j, k;
     double rho = 0.0;
-    if (node64(L, i, j, k)) {
+    // level 0: several nodes a thread, as the block's sum takes six FP64
+    // operations a warp and value
+    for (int t = blockIdx.x * 256 + threadIdx.x; node64(L, t, i, j, k); t += gridDim.x * 256) {
         const int p = k * L.sxy + j * L.sx + i;
         const double s = L.s[p];
         const double z = (1.0 - (double)OMEGA) * L.r[p] + (double)OMEGA * (s + face_sum64(L, L.r, p) * L.di[p]);
         L.z[p] = z;
-        if (TOP) rho = L.dg[p] * s * z;
+        if (!TOP) return;
+        rho = fma(L.dg[p] * s, z, rho);
     }
-    if (!TOP) return;
+    if (!TOP) return;  // a thread without a node
     double t0, t1;
     if (last_block_total<256, false>(st, partials, gridDim.x, rho, 0.0, sred, t0, t1) && threadIdx.x == 0) {
         st->counter = 0;
@@ -1733,17 +1756,20 @@ int launch_vcycle64(const pb_system *sys, cudaStream_t s) {
         return cdiv((long long)(L.nx - 2) * (L.ny - 2) * (L.nz - 2), 256);
     };
     for (int l = 0; l < e.nbot; ++l) {
-        k_mg64_residual<<<blocks(e.lev[l]), 256, 0, s>>>(e.lev[l], sys->st);
-        k_mg64_restrict<<<blocks(e.lev[l + 1]), 256, 0, s>>>(e.lev[l], e.lev[l + 1], sys->st);
+        mg_launch(k_mg64_residual, blocks(e.lev[l]), 256, 0, s, true, e.lev[l], (const CgState *)sys->st);
+        mg_launch(k_mg64_restrict, blocks(e.lev[l + 1]), 256, 0, s, true, e.lev[l], e.lev[l + 1],
+                  (const CgState *)sys->st);
     }
     mg_launch(k_mg_bottom<Entry64, true>, 1, BOT_T, mg_bottom_bytes(e), s, true, (const Entry64 *)nullptr,
               (const Head *)nullptr, e);
+    static const unsigned top = mg_resident(k_mg64_smooth<true>, 256);
     for (int l = e.nbot - 1; l >= 0; --l) {
-        k_mg64_correct<<<blocks(e.lev[l]), 256, 0, s>>>(e.lev[l], e.lev[l + 1], sys->st);
+        mg_launch(k_mg64_correct, blocks(e.lev[l]), 256, 0, s, true, e.lev[l], e.lev[l + 1], (const CgState *)sys->st);
         if (l == 0)
-            k_mg64_smooth<true><<<blocks(e.lev[l]), 256, 0, s>>>(e.lev[l], sys->st, sys->partials);
+            mg_launch(k_mg64_smooth<true>, std::min(blocks(e.lev[l]), top), 256, 0, s, true, e.lev[l], sys->st,
+                      sys->partials);
         else
-            k_mg64_smooth<false><<<blocks(e.lev[l]), 256, 0, s>>>(e.lev[l], sys->st, nullptr);
+            mg_launch(k_mg64_smooth<false>, blocks(e.lev[l]), 256, 0, s, true, e.lev[l], sys->st, (double *)nullptr);
     }
     return 4 * e.nbot + 1;
 }

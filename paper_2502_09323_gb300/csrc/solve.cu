@@ -954,6 +954,22 @@ pb_status launch_iter(pb_system *sys, const CP &cp, const T *z, const T *pold, T
     return PB_OK;
 }
 
+// a launch that may set up while the stream's previous kernel drains (its
+// kernels begin with griddepcontrol.wait)
+template <class A>
+void cg64_launch(void (*kernel)(A), dim3 grid, unsigned threads, cudaStream_t s, const A &a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 // one plain FP64 PCG iteration (direction + update kernels); cur selects
 // which of pa/pb holds p_old; which: 0 direction only, 1 update only, 2 both
 void launch_iter_cg64(pb_system *sys, int cur, int KC, cudaStream_t s, int which = 2) {
@@ -974,7 +990,7 @@ void launch_iter_cg64(pb_system *sys, int cur, int KC, cudaStream_t s, int which
     d.KC = KC;
     const dim3 grid((unsigned)cdiv(g.nx - 1, cg64::TXP), (unsigned)cdiv(g.ny - 2, cg64::WARPS),
                     (unsigned)cdiv(g.nz - 2, KC));
-    if (which != 1) k_cg64_dir<<<grid, cg64::NT, 0, s>>>(d);
+    if (which != 1) cg64_launch(k_cg64_dir, grid, cg64::NT, s, d);
     if (which == 0) return;
     cg64::UpdArgs u{};
     u.x = sys->x64;
@@ -997,7 +1013,7 @@ void launch_iter_cg64(pb_system *sys, int cur, int KC, cudaStream_t s, int which
     // partials holds two slots per block
     const long long blocks = std::min<long long>(
         std::min<long long>(cdiv(u.count / 2, cg64::UNT), (long long)per_sm * num_sms()), sys->npartials / 2);
-    k_cg64_upd<<<(unsigned)blocks, cg64::UNT, 0, s>>>(u);
+    cg64_launch(k_cg64_upd, dim3((unsigned)blocks), cg64::UNT, s, u);
 }
 
 double now_s() {
