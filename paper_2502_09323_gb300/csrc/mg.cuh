@@ -1054,8 +1054,11 @@ k_mg_bottom(const E *__restrict__ tab, const mg::Head *__restrict__ head,
     const F *Wx = reinterpret_cast<const F *>(bsm), *Wy = Wx + T, *Wz = Wy + T, *D = Wz + T;
     const uint16_t *list = reinterpret_cast<const uint16_t *>(D + T), *up = list + T, *dn = up + T;
     F *S = reinterpret_cast<F *>(bsm + BLOB_BYTES<F> * T), *Z = S + T, *R = Z + T;
-    // T is a multiple of 8, so the blob is whole 16-byte pieces
-    for (int q = tid; q < BLOB_BYTES<F> * T / 16; q += BOT_T)
+    // T is a multiple of 8, so the blob is whole 16-byte pieces.  Not of a solve
+    // that has ended: the engine hands its system back while a replay that
+    // holds it may still be in flight, and its memory may be gone by then.
+    const bool ended = SINGLE && *(volatile int *)&e.st->done;
+    for (int q = ended ? INT_MAX : tid; q < BLOB_BYTES<F> * T / 16; q += BOT_T)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tma::smem_u32(bsm + 16 * q)),
                      "l"(reinterpret_cast<const char *>(e.blob) + 16 * q)
                      : "memory");
@@ -1065,7 +1068,7 @@ k_mg_bottom(const E *__restrict__ tab, const mg::Head *__restrict__ head,
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
-    const bool skip = SINGLE && *(volatile int *)&e.st->done;
+    const bool skip = ended || (SINGLE && *(volatile int *)&e.st->done);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (skip) return;
     __syncthreads();

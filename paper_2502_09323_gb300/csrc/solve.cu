@@ -22,6 +22,7 @@
 // medium, listed edges read their FP32 weight from the crossing list, found by
 // a binary search inside the edge's row.  The diagonal is rebuilt from the
 // six weights and the node's ionic term, so no coefficient array is streamed.
+#include <limits.h>
 #include <math.h>
 
 #include <cuda.h>
