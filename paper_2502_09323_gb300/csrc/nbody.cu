@@ -768,7 +768,11 @@ pb_status nbody_surface(pb_system *sys, cudaStream_t s) {
     if (!sys->PsiN) return PB_ERR_OOM;
     T.nrm2 = g->mc_n;
     int *order = nullptr;
-    if (g->is_oct && g->na * g->ncross >= FAR_PAIRS && (st = order_targets(g, &order, s)) != PB_OK) return st;
+    if (g->is_oct && g->na * g->ncross >= FAR_PAIRS && (st = order_targets(g, &order, s)) != PB_OK) {
+        dfree(hi, s);
+        dfree(lo, s);
+        return st;
+    }
     T.order = order;
     const int per = NB_THREADS * NB_TPT;
     const unsigned blocks = cdiv(T.count, per);
