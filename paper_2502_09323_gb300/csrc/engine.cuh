@@ -130,6 +130,13 @@ struct HostSlot {
     double t_admit = 0.0;
 };
 
+// Streams of the octree systems' iterations.  One system's iteration is about
+// 25 short kernels on grids that mostly leave the GPU idle; on a stream each,
+// between a fork and a join of the engine's own, those of several systems run
+// side by side (eight octrees of 400 to 3,800 atoms served at once: 157 ->
+// 127 ms, the same bits).
+constexpr int ENG_SIDE = 8;
+
 struct Engine {
     int device = 0, cap = 0, chunk = 8;
     double rtol = 1e-8, inner_rtol = 1e-6;
@@ -139,6 +146,8 @@ struct Engine {
     tma::SysEntry *dtab = nullptr, *htab = nullptr;    // staging: 2 x cap, pinned
     unsigned int *queue = nullptr, *hhdr = nullptr;    // hhdr: 2 x 4, pinned
     cudaEvent_t ev_chunk[2] = {nullptr, nullptr}, ev_tab[2] = {nullptr, nullptr};
+    cudaStream_t side[ENG_SIDE] = {};
+    cudaEvent_t ev_fork = nullptr, ev_join[ENG_SIDE] = {};
     bool tab_used[2] = {false, false};
     int tab_buf = 0;
     // one replay, by the number of multigrid levels above the bottom kernel
@@ -383,16 +392,38 @@ void engine_complete(Engine *e, int q, const EngineSlot &m) {
 
 bool engine_issue(Engine *e, int mb) {
     const int chunk = engine_chunk(e);
-    ENG_TRY(cudaGraphLaunch(e->exec[e->mg ? e->depth : mg::LMAX], e->cs), "replay");
-    note_launch(chunk * (2 + (e->depth > 0 ? 2 * e->depth + 1 : 0)));
     // octree systems: the same number of iterations with their brick kernels
+    int octs = 0, taken = 0;
+    for (const HostSlot &hs : e->slots) {
+        taken += hs.used;
+        octs += hs.used && hs.job.oct;
+    }
+    const int sides = octs > 1 ? std::min(octs, ENG_SIDE) : 0;
+    for (int k = 0; k < sides; ++k) {
+        if (!e->side[k]) {
+            ENG_TRY(cudaStreamCreateWithFlags(&e->side[k], cudaStreamNonBlocking), "octree stream");
+            ENG_TRY(cudaEventCreateWithFlags(&e->ev_join[k], cudaEventDisableTiming), "octree event");
+        }
+        if (!e->ev_fork) ENG_TRY(cudaEventCreateWithFlags(&e->ev_fork, cudaEventDisableTiming), "octree event");
+    }
+    if (sides > 0) ENG_TRY(cudaEventRecord(e->ev_fork, e->cs), "octree fork");
+    if (octs < taken) {
+        ENG_TRY(cudaGraphLaunch(e->exec[e->mg ? e->depth : mg::LMAX], e->cs), "replay");
+        note_launch(chunk * (2 + (e->depth > 0 ? 2 * e->depth + 1 : 0)));
+    }
+    for (int k = 0; k < sides; ++k) ENG_TRY(cudaStreamWaitEvent(e->side[k], e->ev_fork, 0), "octree fork");
+    int nth = 0;
     for (int q = 0; q < e->cap; ++q) {
         const HostSlot &hs = e->slots[q];
         if (!hs.used || !hs.job.oct) continue;
-        if (oct_engine_iterations(hs.job.sys, chunk, e->cs) != PB_OK) {
+        if (oct_engine_iterations(hs.job.sys, chunk, sides > 0 ? e->side[nth++ % sides] : e->cs) != PB_OK) {
             engine_fail(e, "octree iterations", cudaGetLastError());
             return false;
         }
+    }
+    for (int k = 0; k < sides; ++k) {
+        ENG_TRY(cudaEventRecord(e->ev_join[k], e->side[k]), "octree join");
+        ENG_TRY(cudaStreamWaitEvent(e->cs, e->ev_join[k], 0), "octree join");
     }
     ENG_TRY(cudaMemcpyAsync(e->hmirror + (size_t)mb * e->cap, e->dslots, sizeof(EngineSlot) * e->cap,
                             cudaMemcpyDeviceToHost, e->cs),
@@ -476,6 +507,8 @@ void engine_pump(Engine *e) {
         if (!engine_process(e, mb, &changed)) break;
     }
     cudaStreamSynchronize(e->cs);
+    for (cudaStream_t x : e->side)  // not joined after a failure
+        if (x) cudaStreamSynchronize(x);
     // hand back the systems still in the table, then fail what is left
     std::lock_guard<std::mutex> lk(e->mu);
     for (HostSlot &hs : e->slots) {
@@ -515,7 +548,11 @@ void engine_release(Engine *e) {
     for (cudaGraph_t x : e->graph)
         if (x) cudaGraphDestroy(x);
     if (e->cs) cudaStreamSynchronize(e->cs);
-    for (cudaEvent_t ev : {e->ev_chunk[0], e->ev_chunk[1], e->ev_tab[0], e->ev_tab[1]})
+    for (cudaStream_t x : e->side)
+        if (x) cudaStreamDestroy(x);
+    for (cudaEvent_t ev : {e->ev_chunk[0], e->ev_chunk[1], e->ev_tab[0], e->ev_tab[1], e->ev_fork})
+        if (ev) cudaEventDestroy(ev);
+    for (cudaEvent_t ev : e->ev_join)
         if (ev) cudaEventDestroy(ev);
     dfree(e->dslots, e->cs);
     dfree(e->dtab, e->cs);
