@@ -4,7 +4,7 @@
 One step = one pass of the whole hot path for one synthetic molecule:
 grid placement + classification + crossing edges (pb_build_grid), edge
 weights + right-hand side (pb_assemble_coeffs), surface and pair Coulomb sums
-(pb_coulomb_terms), mixed-precision Jacobi-PCG to a true FP64 residual of
+(pb_coulomb_terms), mixed-precision preconditioned CG to a true FP64 residual of
 1e-8 (pb_solve) and the energy terms (pb_energy).
 
 Default workload: 2,000-atom globular molecule (seed 2), uniform 257^3 grid
@@ -275,7 +275,7 @@ def run_batched(args, pb, pb_inputs, torch):
     """256 uneven molecules (atom counts log-uniform in [200, 3000], molecule
     i seeded 4000 + i), uniform grids of spacing 0.5 A, solved to 1e-8 by
     one graph-launched batch; beside them the same systems solved one at a
-    time by plain FP64 Jacobi-PCG."""
+    time by plain FP64 PCG."""
     from paper_2502_09323_gb300 import serving
     count = args.batch_count
     mols = pb_inputs.batch_molecules(count, 4000, 200, 3000)
@@ -778,7 +778,7 @@ def run_ours(args, wl):
     barrier()
     e2e_elapsed = max_over_ranks(ev2.elapsed_time(ev3) / 1e3)
 
-    # ---- plain FP64 Jacobi-PCG, same workload
+    # ---- plain FP64 PCG, same workload
     fp64 = None
     if not args.no_fp64:
         step(atoms_dev, pb.FP64)
