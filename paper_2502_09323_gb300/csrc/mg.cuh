@@ -24,7 +24,7 @@
 // system in one launch (k_mg_bottom).  The up kernel of level 0 also sums
 // rho = r.z and takes the CG step beta = rho / rho_old.
 //
-// Measured (GB300, solves to 1e-12): 257^3 155.6 -> 13.4 ms (1,127 -> 30
+// Measured (GB300, solves to 1e-12): 257^3 155.6 -> 12.9 ms (1,127 -> 30
 // iterations), 65^3 30.1 -> 2.1 ms, a batch of 24 systems of 97^3 to 161^3
 // 229 -> 51 ms.
 //
@@ -1358,8 +1358,11 @@ struct MgState {
 };
 
 // Planes per work item.  A block marches over them after reading two more,
-// at about a microsecond a plane, and up to four (down) or three (up) blocks
-// share an SM: the count with the fewest rounds of blocks times planes.
+// at about a microsecond a plane: the count with the fewest rounds of blocks
+// times planes, by the blocks that share an SM (level 0 of a solver's grid four
+// down and three up, stored levels three and two.  Counted as four and three
+// there too, the stored 129^3 level took a second round for some blocks: 257^3
+// 13.31 -> 12.93 ms, 150 x 97 x 118 3.82 -> 3.75 ms, others the same).
 // shared: many systems fill the launch, and the longest items waste least.
 // Only the work is divided differently, the results are the same bits.
 void mg_planes(mg::Entry &e, bool shared) {
@@ -1381,8 +1384,9 @@ void mg_planes(mg::Entry &e, bool shared) {
         const Lev &F = e.lev[l], &C = e.lev[l + 1];
         // a coarse plane is two fine ones
         e.dk[l] = best((long long)cdiv(C.nx - 2, CX) * cdiv(C.ny - 2, l == 0 && e.code ? C0Y : CY), 2 * (C.nz - 2),
-                       4, 2, 16) / 2;
-        e.uk[l] = best((long long)cdiv(F.nx - 1, FX) * cdiv(F.ny - 2, FY), F.nz - 2, 3, l == 0 ? RG : 1, 16);
+                       l == 0 && e.code ? 4 : 3, 2, 16) / 2;
+        e.uk[l] = best((long long)cdiv(F.nx - 1, FX) * cdiv(F.ny - 2, FY), F.nz - 2,
+                       l == 0 && e.code ? 3 : 2, l == 0 ? RG : 1, 16);
     }
 }
 
