@@ -23,6 +23,7 @@
 
 #include <algorithm>
 
+#include "fp64_math.cuh"
 #include "pb_internal.h"
 
 namespace pbg {
@@ -503,28 +504,6 @@ __device__ __forceinline__ double rsqrt_fp64(double a) {
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
     const double e = fma(-(a * y), y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
-// exp(-u) for u >= 0 in FP64: -u = (n/64) ln 2 + f, |f| <= ln 2 / 128, the
-// Taylor polynomial of degree 5 of exp(f) (its remainder f^6/720 is below
-// 4e-17), and 2^(n/64) from the table of 64 values and an exponent.
-// ln 2 / 64 in two parts keeps f exact to rounding.  Ten FP64 operations.
-__device__ __forceinline__ double exp_neg_fp64(double u, const double *tab) {
-    constexpr double MAGIC = 6755399441055744.0;  // 1.5 * 2^52: rounds to an integer
-    constexpr double HI = 0x1.62e42fefa39efp-7, LO = 0x1.abc9e3b39803fp-62;
-    const double t = fma(u, -92.332482616893656, MAGIC);
-    const int n = __double2loint(t);
-    const double nd = t - MAGIC;
-    const double f = fma(nd, -LO, fma(nd, -HI, -u));
-    double p = 1.0 / 120.0;
-    p = fma(p, f, 1.0 / 24.0);
-    p = fma(p, f, 1.0 / 6.0);
-    p = fma(p, f, 0.5);
-    p = fma(p, f, 1.0);
-    p = fma(p, f, 1.0);
-    const double v = p * tab[n & 63];
-    const double r = __hiloint2double(__double2hiint(v) + (n >> 6) * 1048576, __double2loint(v));
-    return n < -64 * 1000 ? 0.0 : r;  // below 2^-1000
 }
 
 // Boundary values in FP64: they enter the linear system itself, so they are
