@@ -4,6 +4,22 @@
 
 namespace pbg {
 
+// 1/sqrt(a), a >= 0, from the hardware's approximation y (rsqrt.approx.ftz.f64, whose
+// operand and result have 20 fraction bits) and one step of third order (A. S.
+// Householder, The Numerical Treatment of a Single Nonlinear Equation, 1970):
+// with e = 1 - a y^2, 1/sqrt(a) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + O(e^3)),
+// and e^3 is below 2^-54, its term 5/16 of that.  Five FP64 operations.
+// (Starting from rsqrtf costs two conversions, which are FP64-rate too: 140
+// against 121 us for the pair sum of 2,000 atoms with the library's function.)
+// Zero, subnormal arguments and infinity take the library's function.
+__device__ __forceinline__ double rsqrt_fp64(double a) {
+    if ((unsigned)__double2hiint(a) - 0x00100000u >= 0x7fe00000u) return rsqrt(a);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
 // exp(-u) for u >= 0, by argument reduction and a table (W. J. Cody and W.
 // Waite, Software Manual for the Elementary Functions, 1980; P. T. P. Tang,
 // ACM TOMS 15 (1989) 144): -u = (n/64) ln 2 + f, |f| <= ln 2 / 128, the Taylor

@@ -490,22 +490,6 @@ k_nbody(TargetDesc T, far::Args F, const float4 *__restrict__ shi, const float4 
     }
 }
 
-// 1/sqrt(a) in FP64 from the hardware's approximation y (PTX
-// rsqrt.approx.ftz.f64, good to about 2^-20): with e = 1 - a y^2,
-// 1/sqrt(a) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + O(e^3)), and e^3 is
-// below 2^-57, its term 5/16 of that.  Five FP64 operations; GB300 issues about two an SM
-// and clock, so their number is the cost of the FP64 sums below.  (Starting
-// from rsqrtf costs two conversions, which are FP64-rate too: 140 against 121
-// us for the pair sum of 2,000 atoms with the library's function.)  Zero and
-// subnormal arguments take the library's function.
-__device__ __forceinline__ double rsqrt_fp64(double a) {
-    if (__double2hiint(a) < 0x00100000) return rsqrt(a);
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double e = fma(-(a * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 // Boundary values in FP64: they enter the linear system itself, so they are
 // summed in double precision (atoms staged in shared memory), in atom order.
 // FP64 issue binds: 24 operations a pair with screening (positions scaled by

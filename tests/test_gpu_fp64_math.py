@@ -24,7 +24,7 @@ extern "C" int run(int which, const double *x, double *y, int n) {
     return (int)cudaDeviceSynchronize();
 }
 """
-FUNCTIONS = ["exp_neg_fp64(x[i], tab)"]
+FUNCTIONS = ["exp_neg_fp64(x[i], tab)", "rsqrt_fp64(x[i])"]
 
 
 @pytest.fixture(scope="module")
@@ -67,3 +67,18 @@ def test_exp_neg(call):
     big = np.concatenate([[708.0, 1e3, 2.3e7, np.inf, 1.7e308], 2.0 ** np.arange(10, 1024),
                           np.exp(rng.uniform(np.log(708.1), 700, 100000)), 2.33e7 * np.arange(1, 200)])
     assert np.all(call(0, big) == 0.0)
+
+
+def test_rsqrt(call):
+    rng = np.random.default_rng(2)
+    m = np.concatenate([1.0 + rng.random(300000), 1.0 + np.arange(1 << 20) * 2.0 ** -20, np.nextafter([1.0, 2.0], 3.0)])
+    a = np.concatenate([m, np.ldexp(m, rng.integers(-1022, 1023, len(m))), 2.0 ** np.arange(-1022, 1024),
+                        [np.finfo(float).max, np.finfo(float).tiny]])
+    exact = 1 / np.sqrt(a.astype(np.longdouble))
+    # in units of 2^-53: the last step 1, e (one rounding of a y, halved by the series) 0.5, the remainder
+    # 5/16 e^3, e up to 2^-18, 0.2
+    assert np.abs(call(1, a) / exact - 1).max() <= 1.75 * 2.0 ** -53
+    s = np.concatenate([[5e-324, np.nextafter(np.finfo(float).tiny, 0)], rng.integers(1, 1 << 52, 1000) * 5e-324])
+    # subnormal: CUDA's function, good to two units
+    assert np.abs(call(1, s) * np.sqrt(s.astype(np.longdouble)) - 1).max() <= 4 * 2.0 ** -53
+    assert call(1, np.array([0.0, np.inf])).tolist() == [np.inf, 0.0]
