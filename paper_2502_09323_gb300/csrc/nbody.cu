@@ -492,10 +492,12 @@ k_nbody(TargetDesc T, far::Args F, const float4 *__restrict__ shi, const float4 
 
 // Boundary values in FP64: they enter the linear system itself, so they are
 // summed in double precision (atoms staged in shared memory), in atom order.
-// FP64 issue binds: 24 operations a pair with screening (positions scaled by
-// k, so that the distance is the exponent), 13 without; the library's sqrt, exp
-// and division took about 70.  Blocks of 128 keep the
+// FP64 issue binds: 25 operations a pair with screening, 13 without; the
+// library's sqrt, exp and division took about 70.  Blocks of 128 keep the
 // last wave full.  141 x 95 x 63 grid, 300 atoms, screened: 1,712 -> 780 us.
+// Positions are subtracted before k scales the distance: scaled first (24
+// operations), their rounding is relative to the coordinates, and a molecule
+// 1,000 A from the origin got 7.6e-16 instead of 6e-17 of sum |q| exp(-k r) / r.
 constexpr int BT = 128;
 
 template <bool SCREEN>
@@ -504,7 +506,6 @@ k_boundary64(GridGeo g, const double *__restrict__ atoms, long long na, long lon
              double scale, double *__restrict__ bc) {
     __shared__ double sx[BT], sy[BT], sz[BT], sq[BT], tab[64];
     if (SCREEN && threadIdx.x < 64) tab[threadIdx.x] = exp2((double)threadIdx.x * 0.015625);
-    const double unit = SCREEN ? k : 1.0;  // 1 / length
     long long t = blockIdx.x * (long long)BT + threadIdx.x;
     double p[3] = {0.0, 0.0, 0.0};
     long long i = 0, j = 0, kk = 0;
@@ -513,16 +514,15 @@ k_boundary64(GridGeo g, const double *__restrict__ atoms, long long na, long lon
         p[0] = g.o[0] + (double)i * g.h;
         p[1] = g.o[1] + (double)j * g.h;
         p[2] = g.o[2] + (double)kk * g.h;
-        for (int q = 0; q < 3; ++q) p[q] *= unit;
     }
     double acc = 0.0;
     for (long long base = 0; base < na; base += BT) {
         long long si = base + threadIdx.x;
         __syncthreads();
         if (si < na) {
-            sx[threadIdx.x] = unit * atoms[si];
-            sy[threadIdx.x] = unit * atoms[na + si];
-            sz[threadIdx.x] = unit * atoms[2 * na + si];
+            sx[threadIdx.x] = atoms[si];
+            sy[threadIdx.x] = atoms[na + si];
+            sz[threadIdx.x] = atoms[2 * na + si];
             sq[threadIdx.x] = atoms[4 * na + si];
         }
         __syncthreads();
@@ -533,12 +533,12 @@ k_boundary64(GridGeo g, const double *__restrict__ atoms, long long na, long lon
             const double r2 = (dx * dx + dy * dy) + dz * dz;
             const double y = rsqrt_fp64(r2);
             if (SCREEN)
-                acc = fma(sq[q] * exp_neg_fp64(r2 * y, tab), y, acc);
+                acc = fma(sq[q] * exp_neg_fp64(k * (r2 * y), tab), y, acc);
             else
                 acc = fma(sq[q], y, acc);
         }
     }
-    if (t < count) bc[(kk * g.ny + j) * g.nx + i] = scale * (unit * acc);
+    if (t < count) bc[(kk * g.ny + j) * g.nx + i] = scale * acc;
 }
 
 // Coulomb pair sum sum_{i<j} q_i q_j / r_ij in FP64 (the energy is a
