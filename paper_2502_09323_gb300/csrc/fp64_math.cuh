@@ -4,6 +4,18 @@
 
 namespace pbg {
 
+// 1/b from the hardware's approximation y (rcp.approx.ftz.f64, whose operand and
+// result have 20 fraction bits) and one step of the hyperpower iteration of order
+// three (M. Altman, Pacific J. Math. 10 (1960) 1107): with e = 1 - b y,
+// 1/b = y / (1 - e) = y (1 + e + e^2 + O(e^3)), and e^3 is below 2^-55.
+// Four FP64 operations.  For b of 2^-1000 to 2^1000.
+__device__ __forceinline__ double rcp_fp64(double b) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double e = fma(-b, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
 // 1/sqrt(a), a >= 0, from the hardware's approximation y (rsqrt.approx.ftz.f64, whose
 // operand and result have 20 fraction bits) and one step of third order (A. S.
 // Householder, The Numerical Treatment of a Single Nonlinear Equation, 1970):

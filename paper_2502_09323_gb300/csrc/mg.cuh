@@ -102,15 +102,7 @@ __host__ __device__ inline int uitems(const Entry &e, int l) {
 }
 
 __device__ __forceinline__ float quotient(float a, float b) { return __fdividef(a, b); }
-// FP64: the hardware's approximation y of 1/b (b a diagonal: positive and
-// normal), e = 1 - b y, 1/b = y / (1 - e) = y (1 + e + e^2 + O(e^3)); five FP64
-// operations
-__device__ __forceinline__ double quotient(double a, double b) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    const double e = fma(-b, y, 1.0);
-    return a * fma(y, fma(e, e, e), y);
-}
+__device__ __forceinline__ double quotient(double a, double b) { return a * rcp_fp64(b); }  // b a diagonal
 
 __device__ __forceinline__ float4 f4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }

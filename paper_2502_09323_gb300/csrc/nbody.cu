@@ -162,10 +162,10 @@ __device__ __forceinline__ TgtLoad load_target(const TargetDesc &T, long long t)
     return r;
 }
 
-// 1/r of a pair from r^2; 0 for a point on itself.  The hardware instruction
-// alone: rsqrtf wraps it in a rescaling of subnormal arguments, that is of
-// distances below 1e-19 A, which are taken as 0 here (the same bits for all
-// others; surface sums of the 20,000-atom octree 84.7 -> 73.0 ms).
+// 1/r of a pair from r^2; 0 for a point on itself.  The hardware's approximate
+// root (documented relative error 2^-22.9) for normal arguments; subnormal
+// ones, distances below 1e-19 A, count as 0 (surface sums of the 20,000-atom
+// octree with rsqrtf, which also serves those: 84.7 -> 73.0 ms).
 __device__ __forceinline__ float rsqrt_pair(float r2) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(r2));

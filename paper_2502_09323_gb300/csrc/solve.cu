@@ -41,6 +41,7 @@
 #include <vector>
 #include <type_traits>
 
+#include "fp64_math.cuh"
 #include "pb_internal.h"
 
 namespace pbg {

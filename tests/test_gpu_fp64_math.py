@@ -24,7 +24,7 @@ extern "C" int run(int which, const double *x, double *y, int n) {
     return (int)cudaDeviceSynchronize();
 }
 """
-FUNCTIONS = ["exp_neg_fp64(x[i], tab)", "rsqrt_fp64(x[i])"]
+FUNCTIONS = ["exp_neg_fp64(x[i], tab)", "rsqrt_fp64(x[i])", "rcp_fp64(x[i])"]
 
 
 @pytest.fixture(scope="module")
@@ -82,3 +82,12 @@ def test_rsqrt(call):
     # subnormal: CUDA's function, good to two units
     assert np.abs(call(1, s) * np.sqrt(s.astype(np.longdouble)) - 1).max() <= 4 * 2.0 ** -53
     assert call(1, np.array([0.0, np.inf])).tolist() == [np.inf, 0.0]
+
+
+def test_rcp(call):
+    rng = np.random.default_rng(3)
+    m = np.concatenate([1.0 + rng.random(300000), 1.0 + np.arange(1 << 20) * 2.0 ** -20, np.nextafter([1.0, 2.0], 3.0)])
+    b = np.concatenate([m, np.ldexp(m, rng.integers(-1000, 1000, len(m))), 2.0 ** np.arange(-1000, 1001)])
+    exact = 1 / b.astype(np.longdouble)
+    # in units of 2^-53: the last step 1, e and e^2 2^-18 of that, the remainder e^3 (e up to 2^-18.5) 0.2
+    assert np.abs(call(2, b) / exact - 1).max() <= 1.25 * 2.0 ** -53
