@@ -1431,14 +1431,17 @@ bool mg_levels(const PadGeo &g, E &e, bool lattice = false) {
 template <typename T>
 size_t mg_lev_size(const mg::LevT<T> &L) { return ((size_t)L.sxy * L.nz + 3) & ~(size_t)3; }
 
-void free_mg_state(pb_system *sys) {
-    MgState *m = (MgState *)sys->mg;
+void mg_release(MgState *m, cudaStream_t s) {
     if (!m) return;
-    dfree(m->head, sys->stream);
-    dfree(m->v, sys->stream);
-    dfree(m->mem, sys->stream);
-    dfree(m->partials, sys->stream);
+    dfree(m->head, s);
+    dfree(m->v, s);
+    dfree(m->mem, s);
+    dfree(m->partials, s);
     delete m;
+}
+
+void free_mg_state(pb_system *sys) {
+    mg_release((MgState *)sys->mg, sys->stream);
     sys->mg = nullptr;
 }
 
@@ -1512,29 +1515,15 @@ pb_status mg_build_levels(const E &e, int first, const pb_system *sys, cudaStrea
     return PB_OK;
 }
 
-// hierarchy of a uniform system, built with its first mixed-precision solve
-// (coefficients and grids do not change after that); sys->mg stays null on
-// grids without one
-pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
+// the hierarchy of e's levels, in m
+pb_status mg_fill(const pb_system *sys, mg::Entry &e, MgState *m, cudaStream_t s) {
     using namespace mg;
-    if (sys->mg) return PB_OK;
-    Entry e{};
-    e.code = sys->code;
-    if (!mg_levels(sys->pad, e)) return PB_OK;
-    pb_status rc = mg_prepare();
-    if (rc != PB_OK) return rc;
-    MgState *m = new (std::nothrow) MgState();
-    if (!m) return PB_ERR_OOM;
-    sys->mg = m;
     const size_t bytes = mg_layout(e, 1, nullptr);
     m->head = (Head *)dalloc(sizeof(Head), s);
     m->v = (float *)dalloc(sizeof(float) * (size_t)sys->pad.Np, s);
     m->mem = dalloc(bytes, s);
     m->partials = (float *)dalloc(sizeof(float) * e.nu0, s);
-    if (!m->head || !m->v || !m->mem || !m->partials) {
-        free_mg_state(sys);
-        return PB_ERR_OOM;
-    }
+    if (!m->head || !m->v || !m->mem || !m->partials) return PB_ERR_OOM;
     PB_CUDA_TRY(cudaMemsetAsync(m->head, 0, sizeof(Head), s));
     PB_CUDA_TRY(cudaMemsetAsync(m->v, 0, sizeof(float) * (size_t)sys->pad.Np, s));
     PB_CUDA_TRY(cudaMemsetAsync(m->mem, 0, bytes, s));
@@ -1546,6 +1535,7 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
     e.dg_in = 6.f * e.cp.w_in;
     e.dg_out = 6.f * e.cp.w_out + e.cp.kap;
     e.partials = m->partials;
+    pb_status rc = PB_OK;
     if ((rc = make_map(&e.sd, sys->z32, false, sys->pad, D0W, D0R)) != PB_OK ||
         (rc = make_map(&e.cd, sys->code, true, sys->pad, C0W, D0R)) != PB_OK ||
         (rc = make_map(&e.su, sys->z32, false, sys->pad, U0W, U0R)) != PB_OK ||
@@ -1553,6 +1543,27 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
         return rc;
     if ((rc = mg_build_levels(e, 1, sys, s)) != PB_OK) return rc;
     m->e = e;
+    return PB_OK;
+}
+
+// hierarchy of a uniform system, built with its first mixed-precision solve
+// (coefficients and grids do not change after that); sys->mg is set once all
+// of it is there, and stays null on grids without one
+pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
+    using namespace mg;
+    if (sys->mg) return PB_OK;
+    Entry e{};
+    e.code = sys->code;
+    if (!mg_levels(sys->pad, e)) return PB_OK;
+    pb_status rc = mg_prepare();
+    if (rc != PB_OK) return rc;
+    MgState *m = new (std::nothrow) MgState();
+    if (!m) return PB_ERR_OOM;
+    if ((rc = mg_fill(sys, e, m, s)) != PB_OK) {
+        mg_release(m, s);
+        return rc;
+    }
+    sys->mg = m;
     return PB_OK;
 }
 
@@ -1610,33 +1621,21 @@ int launch_vcycle(const pb_system *sys, cudaStream_t s) {
     return 2 * e.nbot + 1;
 }
 
-// The lattice of an octree's preconditioner: `up` coarsenings of the lattice
-// that fill() writes.
-pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cudaStream_t s) {
+// the lattice's hierarchy, in m: `up` coarsenings of the lattice that fill() writes
+pb_status mg_lattice_fill(const pb_system *sys, mg::Entry &e, int up, lattice_fill fill, MgState *m, cudaStream_t s) {
     using namespace mg;
-    if (sys->mg) return PB_OK;
-    Entry e{};
-    PadGeo g{};
-    g.nx = g.ny = g.nz = n;
-    if (!mg_levels(g, e, true)) return PB_OK;
-    pb_status rc = mg_prepare();
-    if (rc != PB_OK) return rc;
-    MgState *m = new (std::nothrow) MgState();
-    if (!m) return PB_ERR_OOM;
-    sys->mg = m;
     m->lattice = true;
     const size_t bytes = mg_layout(e, 0, nullptr);
     m->head = (Head *)dalloc(sizeof(Head), s);
     m->mem = dalloc(bytes, s);
-    if (!m->head || !m->mem) {
-        free_mg_state(sys);
-        return PB_ERR_OOM;
-    }
+    if (!m->head || !m->mem) return PB_ERR_OOM;
     PB_CUDA_TRY(cudaMemsetAsync(m->head, 0, sizeof(Head), s));
     PB_CUDA_TRY(cudaMemsetAsync(m->mem, 0, bytes, s));
     mg_layout(e, 0, (char *)m->mem);
     e.st = sys->st;
     // from the finest of the lattices down to level 0
+    const int n = e.lev[0].nx;
+    pb_status rc = PB_OK;
     Lev F{};
     void *tmp = nullptr;
     for (int q = up; q >= 0 && rc == PB_OK; --q) {
@@ -1672,11 +1671,27 @@ pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cuda
     dfree(tmp, s);
     if (rc == PB_OK && cudaGetLastError() != cudaSuccess) rc = PB_ERR_CUDA;
     if (rc == PB_OK) rc = mg_build_levels(e, 0, sys, s);
-    if (rc != PB_OK) {
-        free_mg_state(sys);
+    m->e = e;
+    return rc;
+}
+
+// The lattice of an octree's preconditioner, of n nodes an axis
+pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cudaStream_t s) {
+    using namespace mg;
+    if (sys->mg) return PB_OK;
+    Entry e{};
+    PadGeo g{};
+    g.nx = g.ny = g.nz = n;
+    if (!mg_levels(g, e, true)) return PB_OK;
+    pb_status rc = mg_prepare();
+    if (rc != PB_OK) return rc;
+    MgState *m = new (std::nothrow) MgState();
+    if (!m) return PB_ERR_OOM;
+    if ((rc = mg_lattice_fill(sys, e, up, fill, m, s)) != PB_OK) {
+        mg_release(m, s);
         return rc;
     }
-    m->e = e;
+    sys->mg = m;
     return PB_OK;
 }
 
@@ -1701,34 +1716,24 @@ struct Mg64State {
     void *mem = nullptr;
 };
 
-void free_mg64_state(pb_system *sys) {
-    Mg64State *m = (Mg64State *)sys->mg64;
+void mg64_release(Mg64State *m, cudaStream_t s) {
     if (!m) return;
-    dfree(m->v, sys->stream);
-    dfree(m->mem, sys->stream);
+    dfree(m->v, s);
+    dfree(m->mem, s);
     delete m;
+}
+
+void free_mg64_state(pb_system *sys) {
+    mg64_release((Mg64State *)sys->mg64, sys->stream);
     sys->mg64 = nullptr;
 }
 
-// built with the first FP64 solve of a uniform system; sys->mg64 stays null on
-// grids without a hierarchy
-pb_status build_mg64_state(pb_system *sys, cudaStream_t s) {
+pb_status mg64_fill(const pb_system *sys, mg::Entry64 &e, Mg64State *m, cudaStream_t s) {
     using namespace mg;
-    if (sys->mg64) return PB_OK;
-    Entry64 e{};
-    if (!mg_levels(sys->pad, e)) return PB_OK;
-    pb_status rc = mg_prepare();
-    if (rc != PB_OK) return rc;
-    Mg64State *m = new (std::nothrow) Mg64State();
-    if (!m) return PB_ERR_OOM;
-    sys->mg64 = m;
     const size_t bytes = mg_layout(e, 1, nullptr), b0 = sizeof(double) * (size_t)sys->pad.Np;
     m->v = (double *)dalloc(b0, s);
     m->mem = dalloc(bytes, s);
-    if (!m->v || !m->mem) {
-        free_mg64_state(sys);
-        return PB_ERR_OOM;
-    }
+    if (!m->v || !m->mem) return PB_ERR_OOM;
     PB_CUDA_TRY(cudaMemsetAsync(m->v, 0, b0, s));
     PB_CUDA_TRY(cudaMemsetAsync(m->mem, 0, bytes, s));
     mg_layout(e, 1, (char *)m->mem);
@@ -1742,8 +1747,27 @@ pb_status build_mg64_state(pb_system *sys, cudaStream_t s) {
     L.di = sys->op64[4];
     L.r = sys->q64;  // q is free between the update and the direction kernels, and zero off the interior
     e.st = sys->st;
-    if ((rc = mg_build_levels(e, 1, sys, s)) != PB_OK) return rc;
+    const pb_status rc = mg_build_levels(e, 1, sys, s);
     m->e = e;
+    return rc;
+}
+
+// built with the first FP64 solve of a uniform system; sys->mg64 is set once
+// all of it is there, and stays null on grids without a hierarchy
+pb_status build_mg64_state(pb_system *sys, cudaStream_t s) {
+    using namespace mg;
+    if (sys->mg64) return PB_OK;
+    Entry64 e{};
+    if (!mg_levels(sys->pad, e)) return PB_OK;
+    pb_status rc = mg_prepare();
+    if (rc != PB_OK) return rc;
+    Mg64State *m = new (std::nothrow) Mg64State();
+    if (!m) return PB_ERR_OOM;
+    if ((rc = mg64_fill(sys, e, m, s)) != PB_OK) {
+        mg64_release(m, s);
+        return rc;
+    }
+    sys->mg64 = m;
     return PB_OK;
 }
 
