@@ -139,7 +139,8 @@ typedef struct {
  * vectors and per-thread accumulation, FP64 global dots), preconditioned by
  * one multigrid V-cycle on uniform grids of at least 9 nodes an axis, by a
  * smoother and a lattice correction on octrees of one to three levels of
- * refinement, else by the diagonal.
+ * refinement, else by the diagonal (so too where device memory has no room for
+ * the hierarchy).
  * Stop when ||f - A phi||_2 <= rtol ||f||_2 (true residual, FP64).
  * max_iter caps the total inner iterations, max_outer the refinement
  * steps; inner_rtol (0 = default 1e-6) is the inner relative tolerance;

@@ -636,6 +636,26 @@ pb_status engine_submit(pb_engine *eh, pb_system *sys, cudaStream_t s, long long
         set_error("the system lives on device %d, the engine on device %d", sys->g->device, e->device);
         return PB_ERR_ARG;
     }
+    // whether the engine has the system already (e->mu held): asked before the
+    // system is touched, as its preparation may add a hierarchy that memory had
+    // no room for when the running solve began
+    auto busy = [&] {
+        for (const HostSlot &hs : e->slots)
+            if (hs.used && hs.job.sys == sys) {
+                set_error("the system is already being solved by the engine");
+                return true;
+            }
+        for (const EngineJob &p : e->pending)
+            if (p.sys == sys) {
+                set_error("the system is already waiting in the engine");
+                return true;
+            }
+        return false;
+    };
+    {
+        std::lock_guard<std::mutex> lk(e->mu);
+        if (busy()) return PB_ERR_ARG;
+    }
     EngineJob j;
     j.sys = sys;
     pb_status rc = PB_OK;
@@ -671,18 +691,10 @@ pb_status engine_submit(pb_engine *eh, pb_system *sys, cudaStream_t s, long long
             set_error("%s", e->err != PB_OK ? e->errmsg : "engine is shutting down");
             return e->err != PB_OK ? e->err : PB_ERR_STATE;
         }
-        for (const HostSlot &hs : e->slots)
-            if (hs.used && hs.job.sys == sys) {
-                cudaEventDestroy(j.ready);
-                set_error("the system is already being solved by the engine");
-                return PB_ERR_ARG;
-            }
-        for (const EngineJob &p : e->pending)
-            if (p.sys == sys) {
-                cudaEventDestroy(j.ready);
-                set_error("the system is already waiting in the engine");
-                return PB_ERR_ARG;
-            }
+        if (busy()) {
+            cudaEventDestroy(j.ready);
+            return PB_ERR_ARG;
+        }
         j.ticket = e->next_ticket++;
         e->pending.push_back(j);
         *ticket = j.ticket;

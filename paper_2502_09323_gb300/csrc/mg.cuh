@@ -1546,6 +1546,14 @@ pb_status mg_fill(const pb_system *sys, mg::Entry &e, MgState *m, cudaStream_t s
     return PB_OK;
 }
 
+// A hierarchy that device memory has no room for is done without: Jacobi needs
+// none.  The next solve asks again.
+pb_status mg_optional(pb_status rc) {
+    if (rc != PB_ERR_OOM) return rc;
+    set_error("");
+    return PB_OK;
+}
+
 // hierarchy of a uniform system, built with its first mixed-precision solve
 // (coefficients and grids do not change after that); sys->mg is set once all
 // of it is there, and stays null on grids without one
@@ -1558,10 +1566,10 @@ pb_status build_mg_state(pb_system *sys, cudaStream_t s) {
     pb_status rc = mg_prepare();
     if (rc != PB_OK) return rc;
     MgState *m = new (std::nothrow) MgState();
-    if (!m) return PB_ERR_OOM;
+    if (!m) return PB_OK;
     if ((rc = mg_fill(sys, e, m, s)) != PB_OK) {
         mg_release(m, s);
-        return rc;
+        return mg_optional(rc);
     }
     sys->mg = m;
     return PB_OK;
@@ -1675,7 +1683,8 @@ pb_status mg_lattice_fill(const pb_system *sys, mg::Entry &e, int up, lattice_fi
     return rc;
 }
 
-// The lattice of an octree's preconditioner, of n nodes an axis
+// The lattice of an octree's preconditioner, of n nodes an axis; sys->mg stays
+// null where memory has no room for it
 pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cudaStream_t s) {
     using namespace mg;
     if (sys->mg) return PB_OK;
@@ -1686,10 +1695,10 @@ pb_status mg_lattice_make(pb_system *sys, int n, int up, lattice_fill fill, cuda
     pb_status rc = mg_prepare();
     if (rc != PB_OK) return rc;
     MgState *m = new (std::nothrow) MgState();
-    if (!m) return PB_ERR_OOM;
+    if (!m) return PB_OK;
     if ((rc = mg_lattice_fill(sys, e, up, fill, m, s)) != PB_OK) {
         mg_release(m, s);
-        return rc;
+        return mg_optional(rc);
     }
     sys->mg = m;
     return PB_OK;
@@ -1762,10 +1771,10 @@ pb_status build_mg64_state(pb_system *sys, cudaStream_t s) {
     pb_status rc = mg_prepare();
     if (rc != PB_OK) return rc;
     Mg64State *m = new (std::nothrow) Mg64State();
-    if (!m) return PB_ERR_OOM;
+    if (!m) return PB_OK;
     if ((rc = mg64_fill(sys, e, m, s)) != PB_OK) {
         mg64_release(m, s);
-        return rc;
+        return mg_optional(rc);
     }
     sys->mg64 = m;
     return PB_OK;

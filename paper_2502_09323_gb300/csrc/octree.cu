@@ -2397,21 +2397,34 @@ pb_status oct_lattice(const pb_system *sys, int n, int sx, float *wx, float *wy,
 }
 
 // the preconditioner's lattice and buffers (octrees of one to OMG_LMAX levels
-// of refinement; others keep Jacobi)
+// of refinement; others, and those that device memory has no room for them
+// beside, keep Jacobi)
 pb_status oct_mg_make(pb_system *sys, cudaStream_t s) {
     const OctDev &t = sys->g->ot;
     OctSys *os = sys->os;
     const long long nf = (long long)(t.NL / 2 + 1);  // nodes an axis at twice the finest spacing
     if (sys->mg || t.Lmax < 1 || t.Lmax > OMG_LMAX || nf * nf * (nf + 3) > 0x7fffffffll) return PB_OK;
     const size_t b32 = sizeof(float) * (size_t)t.N;
-    for (float *&q : os->mx) {
-        if (!q) q = (float *)dalloc(b32, s);
-        if (!q) return PB_ERR_OOM;
-        PB_CUDA_TRY(cudaMemsetAsync(q, 0, b32, s));
+    for (float *&q : os->mx) q = (float *)dalloc(b32, s);
+    os->mpart = (float *)dalloc(sizeof(float) * OMG_PART * (size_t)t.nb, s);
+    pb_status rc = PB_OK;
+    if (os->mx[0] && os->mx[1] && os->mpart) {
+        for (float *q : os->mx) {
+            const cudaError_t e = cudaMemsetAsync(q, 0, b32, s);
+            if (e == cudaSuccess) continue;
+            set_error("clearing the preconditioner's vectors: %s", cudaGetErrorString(e));
+            rc = PB_ERR_CUDA;
+        }
+        if (rc == PB_OK) rc = mg_lattice_make(sys, t.NL / (1 << t.Lmax) + 1, t.Lmax - 1, oct_lattice, s);
+    } else {
+        set_error("");
     }
-    if (!os->mpart) os->mpart = (float *)dalloc(sizeof(float) * OMG_PART * (size_t)t.nb, s);
-    if (!os->mpart) return PB_ERR_OOM;
-    return mg_lattice_make(sys, t.NL / (1 << t.Lmax) + 1, t.Lmax - 1, oct_lattice, s);
+    if (sys->mg) return PB_OK;
+    for (float **q : {&os->mx[0], &os->mx[1], &os->mpart}) {
+        dfree(*q, s);
+        *q = nullptr;
+    }
+    return rc;
 }
 
 pb_status oct_ensure_ws(pb_system *sys, int precision, cudaStream_t s) {

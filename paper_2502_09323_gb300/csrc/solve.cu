@@ -827,9 +827,19 @@ pb_status tma_sys_maps(pb_system *sys, tma::SysEntry &e, int tw) {
 }
 
 pb_status build_tma_state(pb_system *sys, cudaStream_t s) {
-    if (sys->tma) return PB_OK;
+    const bool had = sys->mg != nullptr;
     const pb_status mrc = build_mg_state(sys, s);
     if (mrc != PB_OK) return mrc;
+    if (sys->tma) {
+        // a hierarchy that an earlier solve did without: its result is what the
+        // direction kernel reads now
+        TmaState *t = (TmaState *)sys->tma;
+        if (had || !sys->mg) return PB_OK;
+        const pb_status rc = tma_sys_maps(sys, t->host, t->tw);
+        if (rc != PB_OK) free_mg_state(sys);
+        t->uploaded_kc = -1;
+        return rc;
+    }
     TmaState *t = new (std::nothrow) TmaState();
     if (!t) return PB_ERR_OOM;
     pb_status rc = PB_OK;

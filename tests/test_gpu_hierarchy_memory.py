@@ -1,5 +1,6 @@
-"""Multigrid hierarchies that cannot be built: nothing of a failed one stays on the system.
-Allocations are refused, or misplaced, by the allocator hooks."""
+"""Multigrid hierarchies that cannot be built: nothing of a failed one stays on the system, and
+one that memory has no room for is done without.  Allocations are refused, or misplaced, by the allocator hooks."""
+import numpy as np
 import pytest
 
 import pb_inputs
@@ -70,3 +71,50 @@ def test_failed_build_leaves_nothing(env):
         assert h.count(4 * n) == before + 4  # z, two directions and the correction
     s.free()
     assert h.count(4 * n) == 0
+
+
+def _octree(pb):
+    atoms = pb_inputs.globular_molecule(25, seed=52)
+    g = pb.pb_build_grid(pb.OctreeSpec(h_fine=0.25, h_bulk=1.0, refine_dist=3.0), atoms)
+    return pb.pb_assemble_coeffs(g, pb.Params()), g.N
+
+
+# system, precision, vectors of the solver itself, allocations of the preconditioner after them
+# (None: all), iterations that Jacobi exceeds and the preconditioned solver does not
+KINDS = {"uniform": (_uniform, 1, 4, 4, 60), "fp64": (_uniform, 0, 11, 2, 60), "octree": (_octree, 1, 4, None, 60)}
+
+
+@pytest.mark.parametrize("kind", list(KINDS))
+@pytest.mark.parametrize("batch", [False, True])
+def test_without_room_for_a_hierarchy(env, kind, batch):
+    pb, h = env
+    make, prec, vectors, after, few = KINDS[kind]
+    opts = pb.SolveOpts(precision=prec, rtol=1e-10)
+    esz = 4 if prec else 8
+
+    def solve(s):
+        return pb.pb_solve_batch([s], opts)[0] if batch else pb.pb_solve(s, opts)
+
+    s, n = make(pb)
+    h.reset()
+    ref = solve(s)
+    sizes, phi = list(h.sizes), pb.pb_get_phi(s)
+    assert ref["status"] == 0 and ref["iters_inner"] <= few
+    last = [at for at, b in enumerate(sizes) if b == esz * n][vectors - 1]
+    end = len(sizes) if after is None else last + 1 + after
+    assert end - last - 1 >= 2
+    for at in range(last + 1, end):
+        s, _ = make(pb)
+        h.reset(refuse=lambda q, _: q == at)
+        st = solve(s)
+        assert st["status"] == 0 and st["true_rel_res"] <= 1e-10 and st["iters_inner"] > few
+        # residuals of 1e-10 and a condition number under 1e3 on these grids
+        assert np.linalg.norm(pb.pb_get_phi(s) - phi) <= 1e-7 * np.linalg.norm(phi)
+        live = sum(b for _, b in h.live.values())
+        # with room again the same system takes the hierarchy
+        h.reset()
+        st = solve(s)
+        assert st["iters_inner"] == ref["iters_inner"] and np.array_equal(pb.pb_get_phi(s), phi)
+        # what was refused, and all that belongs to it, had been given back
+        assert sum(b for _, b in h.live.values()) - live >= sizes[at]
+        s.free()
