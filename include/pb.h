@@ -409,9 +409,10 @@ pb_status pb_solve_split(pb_system *s, int32_t ranks, const pb_solve_opts *opts,
                          pb_solve_stats *stats);
 
 /* pb_set_wait_limit -- failure-injection hook for tests: the number of polls
- * after which a ring-slot wait of the FP32 PCG kernels (one-system, batched
- * and served launches) gives up; polls < 0 restores the default (2^20).  With
- * 0 every slot wait gives up at once, so the next FP32 PCG launch stops, waits
+ * after which a ring-slot wait of the FP32 PCG kernels and of the multigrid
+ * cycle's kernels (one-system, batched and served launches) gives up; polls < 0
+ * restores the default (2^20).  With 0 every slot wait gives up at once, so the
+ * next launch of either (the cycle comes first) stops, waits
  * for its own copies in flight and marks every system of its launch with
  * device status 3: pb_solve and pb_solve_batch then return PB_ERR_TIMEOUT, and
  * a served system finishes with that status.  The drain of a block's own

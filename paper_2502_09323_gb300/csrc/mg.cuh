@@ -451,9 +451,13 @@ constexpr int D0R = 2 * D0P + 1, D0W = 4 * DU;     // the down kernel's box of s
 constexpr int U0R = FY + 2, U0W = FX + 8;          // the up kernel's: columns from i0 - 4
 constexpr int C0W = FX + 32;                       // codes: columns from 16 to the left
 constexpr int up128(int b) { return (b + 127) & ~127; }
-// The ring of planes of one block.  Planes are counted over the whole launch;
-// every wait is bounded, and one that gives up is reported in the solver's
-// state (status 3) at the end of the launch.
+// The ring of planes of one block.  Planes are counted over the whole launch.
+// Every wait is bounded by tma::g_slot_wait_limit, as in the stencil kernels.
+// After one that gives up, the thread polls each slot once; the first thread,
+// which issues the copies, first waits (with a limit of its own) for those in
+// flight, and issues no more: it did not see their slots filled.  The block
+// computes on with whatever its slots hold (no address depends on it) and says
+// so in the solver's state (status 3, whose correction is dropped).
 template <int R, int W, int RC>  // rows and columns of s, rows of codes
 struct Ring {
     static constexpr int SB = up128(4 * R * W), CB = up128(RC * C0W);
@@ -462,27 +466,37 @@ struct Ring {
     };
     Mem &m;
     uint32_t bar;        // NS mbarriers
-    int n = 0, put = 0;  // planes waited for, planes issued
-    bool bad = false;
-    __device__ __forceinline__ Ring(Mem &mem, uint64_t *bars) : m(mem), bar(tma::smem_u32(bars)) {
+    int n = 0;           // planes waited for
+    int who;             // the thread; another number for a first one that gave up
+    bool bad = false;    // a wait gave up
+    __device__ __forceinline__ Ring(Mem &mem, uint64_t *bars) : m(mem), bar(tma::smem_u32(bars)), who(threadIdx.x) {
         if (threadIdx.x == 0) {
             for (int q = 0; q < NS; ++q) tma::mbar_init(bar + 8 * q, 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
     }
-    __device__ __forceinline__ void issue(const CUtensorMap &sm, const CUtensorMap &cm, int x, int y, int k) {
-        if (threadIdx.x == 0) {
-            const int q = put & (NS - 1);
+    // plane k, the `at`-th after those waited for
+    __device__ __forceinline__ void issue(const CUtensorMap &sm, const CUtensorMap &cm, int x, int y, int k, int at) {
+        if (who == 0) {
+            const int q = (n + at) & (NS - 1);
             const uint32_t b = bar + 8 * q;
             tma::mbar_expect_tx(b, 4 * R * W + RC * C0W);
             tma::tma_load3(tma::smem_u32(m.s[q]), &sm, x - (W == U0W ? 4 : 0), y, k, b);
             tma::tma_load3(tma::smem_u32(m.c[q]), &cm, x - 16, y, k, b);
         }
-        ++put;
     }
-    __device__ __forceinline__ void wait() {  // for the next plane
+    // gives up; `flying` planes from the next one on may be in flight
+    __device__ __forceinline__ void give_up(int flying) {
+        bad = true;
+        if (who == 0)
+            for (int q = n; q < n + flying; ++q)
+                tma::mbar_wait(bar + 8 * (q & (NS - 1)), (q / NS) & 1, tma::TMA_WAIT_LIMIT);
+        who = -1;
+    }
+    // for the next plane; `after` it are in flight
+    __device__ __forceinline__ void wait(int after) {
         const uint32_t b = bar + 8 * (n & (NS - 1)), parity = (n / NS) & 1;
-        if (!tma::mbar_try(b, parity) && !tma::mbar_wait(b, parity, bad ? 0 : tma::TMA_WAIT_LIMIT)) bad = true;
+        if (!tma::mbar_try(b, parity) && !tma::mbar_wait(b, parity, bad ? 0 : tma::g_slot_wait_limit)) give_up(1 + after);
         ++n;
     }
     __device__ __forceinline__ const float (*s(int back) const)[W] {  // plane back before the last one waited for
@@ -491,13 +505,13 @@ struct Ring {
     __device__ __forceinline__ const uint8_t (*c(int back) const)[C0W] {
         return reinterpret_cast<const uint8_t (*)[C0W]>(m.c[(n - 1 - back) & (NS - 1)]);
     }
-    __device__ __forceinline__ void report(CgState *st) {
-        if (!bad) return;
+    __device__ __forceinline__ static void fail(CgState *st) {
+        if (st->done) return;
         st->status = 3;
         st->done = 1;
-        if (threadIdx.x == 0)  // the block's own copies land before it leaves
-            for (int q = max(put - NS, 0); q < put; ++q)
-                tma::mbar_wait(bar + 8 * (q & (NS - 1)), (q / NS) & 1, tma::TMA_WAIT_LIMIT);
+    }
+    __device__ __forceinline__ void report(CgState *st) {
+        if (bad) fail(st);
     }
 };
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool there) {
@@ -584,6 +598,9 @@ k_mg_down0(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head,
     const bool work = pr < D0P;
     const int ra = work ? 2 * pr + 1 : 1, x = 4 * u;  // row of the box
     R ring(planes, bars);
+    // a limit of no polls gives up before anything is issued: a wait looks at
+    // its slot once before it counts
+    const bool no_polls = tma::g_slot_wait_limit == 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int nsys = SINGLE ? 1 : head->nsys;
@@ -591,7 +608,10 @@ k_mg_down0(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head,
     for (int it = blockIdx.x; it < total; it += gridDim.x) {
         const Entry &e = SINGLE ? e0 : tab[find_sys(tab, nsys, it, &Entry::dbase, 0)];
         // one answer for the block; and the previous item's last reads, the barriers' initialisation
-        if (__syncthreads_or(*(volatile int *)&e.st->done)) continue;
+        if (__syncthreads_or(*(volatile int *)&e.st->done | (int)no_polls)) {
+            if (no_polls) ring.fail(e.st);
+            continue;
+        }
         // local copies: the asm statements below would have e read again
         const Lev L = e.lev[0], C = e.lev[1];
         const CoefC32 cp = e.cp;
@@ -615,12 +635,12 @@ k_mg_down0(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head,
         const bool in0 = pr < C0Y && J <= C.ny - 2 && u > 0 && I <= C.nx - 2;
         const bool in1 = pr < C0Y && J <= C.ny - 2 && u < DU - 1 && I + 1 <= C.nx - 2;
         const int pcj = J * C.sx + I;
-        for (int k = ka - 1; k <= ka + 2; ++k)
-            if (k <= kb + 1) ring.issue(e.sd, e.cd, i0, jb, k);
+        const int first = min(4, kb - ka + 3);  // planes to begin with
+        for (int q = 0; q < first; ++q) ring.issue(e.sd, e.cd, i0, jb, ka - 1 + q, q);
         if (tid < 16) fill_media(tw, tid, OMEGA * cp.w_in, OMEGA * cp.w_out);
         else if (tid < 32) fill_media(td, tid - 16, (1.f - OMEGA) * e.dg_in, (1.f - OMEGA) * e.dg_out);
-        ring.wait();
-        ring.wait();
+        ring.wait(first - 1);
+        ring.wait(first - 2);
         auto word = [&](const uint8_t (*c)[C0W], int r) { return *reinterpret_cast<const uint32_t *>(&c[r][16 + x]); };
         uint32_t bA = word(ring.c(1), ra), bB = word(ring.c(1), ra + 1);  // codes of plane k - 1
         Pair4 mA = p4(f4(&ring.s(1)[ra][x])), mB = p4(f4(&ring.s(1)[ra + 1][x]));
@@ -631,7 +651,7 @@ k_mg_down0(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head,
             constexpr bool ODD = decltype(odd)::value;
             const bool done = !ODD && k - 1 > ka;  // completes coarse nodes
             const int pc = ((k - (ODD ? 1 : 2)) >> 1) * C.sxy + pcj;
-            if (compute) ring.wait();  // plane k + 1
+            if (compute) ring.wait(k + 2 <= kb + 1);  // plane k + 1
             __syncthreads();
             if (ODD && k > ka) {  // their diagonals, a plane ahead
                 if (in0) dc0 = __ldg(C.dg + pc);
@@ -639,7 +659,7 @@ k_mg_down0(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head,
             }
             Pair4 next = {};
             if (compute) {
-                if (k + 3 <= kb + 1) ring.issue(e.sd, e.cd, i0, jb, k + 3);  // over plane k - 1
+                if (k + 3 <= kb + 1) ring.issue(e.sd, e.cd, i0, jb, k + 3, 1);  // over plane k - 1
                 const float (*s)[D0W] = ring.s(1), (*sn)[D0W] = ring.s(0);
                 const uint8_t (*cd)[C0W] = ring.c(1);
                 const Pair4 nA = p4(f4(&sn[ra][x])), nB = p4(f4(&sn[ra + 1][x]));
@@ -738,6 +758,9 @@ k_mg_up0(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int tot
     const int r = own ? 1 + 4 * w + 2 * hi : (hrow ? (hi ? FY + 1 : 0) : 1 + u);
     const int x = own || hrow ? 4 + 4 * u : (hi ? 4 + FX : 3);
     R ring(planes, bars);
+    // a limit of no polls gives up before anything is issued: a wait looks at
+    // its slot once before it counts
+    const bool no_polls = tma::g_slot_wait_limit == 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int nsys = SINGLE ? 1 : head->nsys;
@@ -745,7 +768,10 @@ k_mg_up0(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int tot
     for (int it = blockIdx.x; it < total; it += gridDim.x) {
         const Entry &e = SINGLE ? e0 : tab[find_sys(tab, nsys, it, &Entry::ubase, 0)];
         // one answer for the block; and the previous item's last reads, the barriers' initialisation
-        if (__syncthreads_or(*(volatile int *)&e.st->done)) continue;
+        if (__syncthreads_or(*(volatile int *)&e.st->done | (int)no_polls)) {
+            if (no_polls) ring.fail(e.st);
+            continue;
+        }
         const Lev L = e.lev[0], C = e.lev[1];
         const CoefC32 cp = e.cp;
         float *const partials = e.partials;
@@ -828,8 +854,8 @@ k_mg_up0(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int tot
             }
         };
         auto mean = [](const E2 &p, const E2 &q) { return E2{scale(0.5f, p.a + q.a), scale(0.5f, p.b + q.b)}; };
-        for (int k = k0 - 1; k <= k0 + 2; ++k)
-            if (k <= k1) ring.issue(e.su, e.cu, i0, j0 - 1, k);
+        const int first = min(4, k1 - k0 + 2);  // planes to begin with
+        for (int q = 0; q < first; ++q) ring.issue(e.su, e.cu, i0, j0 - 1, k0 - 1 + q, q);
         for (int K = (k0 - 1) >> 1; K <= (k0 + 3) >> 1; ++K) fetch_coarse(K);
         if (tid < 16) fill_media(tq, tid, __fdividef(OMEGA * cp.w_in, e.dg_in), __fdividef(OMEGA * cp.w_out, e.dg_out));
         else if (tid < 32) fill_media(td, tid - 16, e.dg_in, e.dg_out);
@@ -837,10 +863,10 @@ k_mg_up0(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int tot
         __syncthreads();
         E2 ec = coarse((k0 - 1) >> 1), en = coarse((k0 + 1) >> 1);
         int slot = (k0 - 1) % 3;  // of plane k - 1
-        ring.wait();
+        ring.wait(first - 1);
         make_v(k0 - 1, slot, ec);
         Pair4 mA = vA, mB = vB;
-        ring.wait();
+        ring.wait(first - 2);
         make_v(k0, slot == 2 ? 0 : slot + 1, mean(ec, en));
         Pair4 cA = vA, cB = vB;
         ec = en;  // coarse plane (k0 + 1) / 2
@@ -862,11 +888,11 @@ k_mg_up0(const mg::Entry *__restrict__ tab, mg::Head *__restrict__ head, int tot
         // one plane: v(k + 1) with the correction g, then z(k)
         auto step = [&](int k, const E2 &g) {
             const int sv = slot == 2 ? 0 : slot + 1, sn = sv == 2 ? 0 : sv + 1;
-            ring.wait();  // plane k + 1
+            ring.wait(k + 2 <= k1);  // plane k + 1
             make_v(k + 1, sn, g);
             const Pair4 nA = vA, nB = vB;
             __syncthreads();
-            if (k + 3 <= k1) ring.issue(e.su, e.cu, i0, j0 - 1, k + 3);  // over plane k - 1
+            if (k + 3 <= k1) ring.issue(e.su, e.cu, i0, j0 - 1, k + 3, 1);  // over plane k - 1
             if (tid == 0 && k > k0 && (k - 1) % RG == 0) flush(k - 1);
             if (own) {
                 uint32_t nbA = 0, nbB = 0;
