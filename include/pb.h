@@ -400,9 +400,11 @@ pb_status pb_set_tuning(pb_system *s, int32_t precision, int32_t variant, int32_
  * neighbours into each receiver's memory (cudaMemcpyPeerAsync); each
  * kernel round's partial dot products are added in rank order and the CG
  * update is written to every rank, so all ranks take the same decisions.
- * In this build every rank lives on the system's device.  ranks = 1 is
- * pb_solve itself; more ranks run the Jacobi-preconditioned PCG.  phi is gathered back into s (pb_energy
- * works as after pb_solve).  Errors: PB_ERR_ARG for a bad rank count or a
+ * In this build every rank lives on the system's device.  ranks = 1 gives
+ * pb_solve's result bit for bit; more ranks run the Jacobi-preconditioned PCG
+ * (no hierarchy is built for them), and their number changes only the order of
+ * the dot-product sums.  phi is gathered back into s (pb_energy works as after
+ * pb_solve).  Errors: PB_ERR_ARG for a bad rank count or a
  * precision other than PB_MIXED, PB_ERR_UNIMPL for octree systems, and the
  * statuses of pb_solve. */
 pb_status pb_solve_split(pb_system *s, int32_t ranks, const pb_solve_opts *opts, void *stream,

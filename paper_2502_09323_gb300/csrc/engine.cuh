@@ -666,7 +666,7 @@ pb_status engine_submit(pb_engine *eh, pb_system *sys, cudaStream_t s, long long
         j.dof = sys->os->nunk;
     } else {
         if ((rc = ensure_solver_ws(sys, PB_MIXED, s)) != PB_OK) return rc;
-        if ((rc = build_tma_state(sys, s)) != PB_OK) return rc;
+        if ((rc = build_tma_state(sys, true, s)) != PB_OK) return rc;
         Tuning tune;
         if ((rc = autotune(sys, PB_MIXED, s, &tune)) != PB_OK) return rc;
         j.kc = tune.variant == 1 ? std::max(tune.kc, 4) : 8;

@@ -826,12 +826,13 @@ pb_status tma_sys_maps(pb_system *sys, tma::SysEntry &e, int tw) {
     return rc;
 }
 
-pb_status build_tma_state(pb_system *sys, cudaStream_t s) {
+// hierarchy: build that too, where the grid has one
+pb_status build_tma_state(pb_system *sys, bool hierarchy, cudaStream_t s) {
     const bool had = sys->mg != nullptr;
-    const pb_status mrc = build_mg_state(sys, s);
+    const pb_status mrc = hierarchy ? build_mg_state(sys, s) : PB_OK;
     if (mrc != PB_OK) return mrc;
     if (sys->tma) {
-        // a hierarchy that an earlier solve did without: its result is what the
+        // a hierarchy that earlier calls did without: its result is what the
         // direction kernel reads now
         TmaState *t = (TmaState *)sys->tma;
         if (had || !sys->mg) return PB_OK;
@@ -1438,7 +1439,7 @@ pb_status solve(pb_system *sys, const pb_solve_opts *o, cudaStream_t s, pb_solve
     const PadGeo &p = sys->pad;
     pb_status rc = ensure_solver_ws(sys, o->precision, s);
     if (rc != PB_OK) return rc;
-    if (o->precision == PB_MIXED && (rc = build_tma_state(sys, s)) != PB_OK) return rc;
+    if (o->precision == PB_MIXED && (rc = build_tma_state(sys, true, s)) != PB_OK) return rc;
     if (o->precision == PB_FP64 && (rc = build_mg64_state(sys, s)) != PB_OK) return rc;
     Tuning tune;
     if ((rc = autotune(sys, o->precision, s, &tune)) != PB_OK) return rc;
@@ -1589,7 +1590,7 @@ pb_status profile_kernels(pb_system *sys, int precision, int which, int reps, cu
         return PB_ERR_STATE;
     }
     pb_status rc = PB_OK;
-    if (precision == PB_MIXED && (rc = build_tma_state(sys, s)) != PB_OK) return rc;
+    if (precision == PB_MIXED && (rc = build_tma_state(sys, false, s)) != PB_OK) return rc;
     Tuning tune;
     if ((rc = autotune(sys, precision, s, &tune)) != PB_OK) return rc;
     if ((rc = init_state(sys, 1.0, 1.0, -1.0, 1 << 30, s, 1)) != PB_OK) return rc;

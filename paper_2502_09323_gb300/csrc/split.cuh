@@ -24,8 +24,9 @@
 // and the last rank's high halo hold zeros (vectors) and the boundary values
 // (phi) and are never exchanged.
 //
-// One rank (R = 1) is the single solve itself.  R > 1 ranks run the
-// Jacobi-preconditioned PCG on their slabs.
+// The ranks run the Jacobi-preconditioned PCG on their slabs.  One rank (R = 1)
+// gives the single solve's bits: a system with a multigrid hierarchy is solved
+// by it, and one without (Jacobi there too) on a slab, with the same z-groups.
 
 namespace {
 
@@ -289,13 +290,13 @@ pb_status solve_split(pb_system *sys, int R, const pb_solve_opts *o, cudaStream_
         set_error("pb_solve_split: ranks must be between 1 and min(64, nz - 2)");
         return PB_ERR_ARG;
     }
-    // one rank is the single solve (and has its preconditioner)
-    if (R == 1) return solve(sys, o, s, stats);
     int dev = 0;
     PB_CUDA_TRY(cudaGetDevice(&dev));
     pb_status rc = ensure_solver_ws(sys, PB_MIXED, s);
     if (rc != PB_OK) return rc;
-    if ((rc = build_tma_state(sys, s)) != PB_OK) return rc;
+    if ((rc = build_tma_state(sys, R == 1, s)) != PB_OK) return rc;
+    // one rank of a system with a hierarchy is the single solve
+    if (R == 1 && sys->mg) return solve(sys, o, s, stats);
     Tuning tune;
     if ((rc = autotune(sys, PB_MIXED, s, &tune)) != PB_OK) return rc;
     const int KC = std::max(tune.kc, 4), TW = tune.tw;
