@@ -1476,15 +1476,14 @@ size_t mg_bottom_bytes(const E &e) {
     return (size_t)mg::BOT_BYTES<typename E::T> * e.bot;
 }
 
+// attributes of the bottom kernels on the current device (set again with every
+// hierarchy and engine: nothing is remembered across threads and devices)
 pb_status mg_prepare() {
-    static bool done = false;
-    if (done) return PB_OK;
     const int most = mg::BOT_BYTES<float> * mg::BOT_NODES<float>, most64 = mg::BOT_BYTES<double> * mg::BOT_NODES<double>;
     PB_CUDA_TRY(cudaFuncSetAttribute(k_mg_bottom<mg::Entry, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     PB_CUDA_TRY(cudaFuncSetAttribute(k_mg_bottom<mg::Entry, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     PB_CUDA_TRY(
         cudaFuncSetAttribute(k_mg_bottom<mg::Entry64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most64));
-    done = true;
     return PB_OK;
 }
 
