@@ -649,7 +649,7 @@ pb_status pb_engine_create(int32_t device, int32_t capacity, const pb_solve_opts
         return PB_ERR_ARG;
     }
     DeviceGuard dg(device);
-    return engine_create(device, capacity, opts, out);
+    return engine_create(device, capacity, opts, true, out);
 }
 
 pb_status pb_engine_submit(pb_engine *e, pb_system *s, void *stream, int64_t *ticket) {

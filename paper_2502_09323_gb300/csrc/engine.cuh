@@ -1,8 +1,8 @@
 // Continuous-batching solve engine (included by solve.cu).
 //
 // A pump thread owns one CUDA stream and keeps a fixed-capacity launch table
-// of mixed-precision solves resident on the device.  Every replay of one
-// captured graph runs `chunk` FP32 PCG iterations (direction + update
+// of mixed-precision solves resident on the device.  Every replay of a graph
+// runs a few FP32 PCG iterations (multigrid cycle, direction and update
 // kernels) of every system in the table; a system that is submitted while
 // others are running takes a free slot and joins at the next replay, and a
 // finished one leaves its slot at once.  The FP64 iterative refinement of
@@ -138,7 +138,7 @@ struct HostSlot {
 constexpr int ENG_SIDE = 8;
 
 struct Engine {
-    int device = 0, cap = 0, chunk = 8;
+    int device = 0, cap = 0, chunk = 8, chunk_mg = 2;  // PCG iterations of a replay, without and with multigrid
     double rtol = 1e-8, inner_rtol = 1e-6;
     int max_iter = 100000, max_outer = 30;
     cudaStream_t cs = nullptr;
@@ -150,9 +150,8 @@ struct Engine {
     cudaEvent_t ev_fork = nullptr, ev_join[ENG_SIDE] = {};
     bool tab_used[2] = {false, false};
     int tab_buf = 0;
-    // one replay, by the number of multigrid levels above the bottom kernel
-    // that it runs, and whether it has any such system, captured when
-    // a table first needs it
+    // replays, by replay_key: a system's is there before the system is in the
+    // engine (made under mu), and no others are asked for
     cudaGraph_t graph[mg::LMAX + 1] = {};
     cudaGraphExec_t exec[mg::LMAX + 1] = {};
     int depth = 0;                                     // the current table's
@@ -255,36 +254,65 @@ bool engine_refine(Engine *e, int q, bool aborted) {
 
 // PCG iterations of one replay: few with multigrid (a solve takes about 15
 // a refinement step), more with Jacobi
-int engine_chunk(const Engine *e) { return e->mg ? 2 : e->chunk; }
+int engine_chunk(const Engine *e) { return e->mg ? e->chunk_mg : e->chunk; }
 
-// capture one replay for tables of the current depth
-bool engine_capture(Engine *e) {
-    const int depth = e->depth, g = e->mg ? depth : mg::LMAX;
-    if (e->exec[g]) return true;
+// adds a kernel behind the last node of a chain
+template <class... P, class... A>
+cudaError_t graph_kernel(cudaGraph_t graph, cudaGraphNode_t *last, void (*kernel)(P...), dim3 grid, unsigned threads,
+                         size_t smem, const A &...args) {
+    std::tuple<std::decay_t<P>...> values{args...};
+    void *at[sizeof...(P)];
+    int n = 0;
+    std::apply([&](auto &...v) { ((at[n++] = const_cast<void *>((const void *)&v)), ...); }, values);
+    cudaKernelNodeParams p{};
+    p.func = (void *)kernel;
+    p.gridDim = grid;
+    p.blockDim = dim3(threads);
+    p.sharedMemBytes = (unsigned)smem;
+    p.kernelParams = at;  // copied by the call
+    const cudaGraphNode_t before = *last;
+    return cudaGraphAddKernelNode(last, graph, before ? &before : nullptr, before ? 1 : 0, &p);
+}
+
+// The replay of tables whose deepest hierarchy has `depth` levels above the bottom
+// kernel (mg: the table has a preconditioned system at all).  Built of kernel nodes,
+// not captured: while a stream captures, a device-wide synchronisation in any
+// thread of the program fails, and takes the capture with it.
+int replay_key(bool mg, int depth) { return mg ? depth : mg::LMAX; }
+
+pb_status engine_replay(Engine *e, bool mg, int depth) {
+    const int g = replay_key(mg, depth);
+    if (e->exec[g]) return PB_OK;
     static const unsigned rd0 = mg_resident(k_mg_down0<false>, mg::D0NT), rd1 = mg_resident(k_mg_down<false>, mg::DNT),
                           ru0 = mg_resident(k_mg_up0<false>, mg::U0NT), ru1 = mg_resident(k_mg_up<false>, mg::UNT);
-    const mg::Entry none{};
-    ENG_TRY(cudaStreamBeginCapture(e->cs, cudaStreamCaptureModeThreadLocal), "capture");
-    for (int c = 0; c < engine_chunk(e); ++c) {
+    static const mg::Entry none{};
+    static const tma::SysEntry zero{};
+    if (e->graph[g]) cudaGraphDestroy(e->graph[g]);  // of an attempt that failed
+    e->graph[g] = nullptr;
+    PB_CUDA_TRY(cudaGraphCreate(&e->graph[g], 0));
+    cudaGraph_t G = e->graph[g];
+    cudaGraphNode_t last = nullptr;
+    for (int c = 0; c < (mg ? e->chunk_mg : e->chunk); ++c) {
         for (int l = 0; l < depth; ++l)
             if (l == 0)
-                k_mg_down0<false><<<rd0, mg::D0NT, 0, e->cs>>>(e->dmg, e->dhead, 0, none);
+                PB_CUDA_TRY(graph_kernel(G, &last, k_mg_down0<false>, rd0, mg::D0NT, 0, e->dmg, e->dhead, 0, none));
             else
-                k_mg_down<false><<<rd1, mg::DNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
+                PB_CUDA_TRY(graph_kernel(G, &last, k_mg_down<false>, rd1, mg::DNT, 0, e->dmg, e->dhead, l, 0, none));
         if (depth > 0)
-            k_mg_bottom<mg::Entry, false>
-                <<<e->cap, mg::BOT_T, mg::BOT_BYTES<float> * mg::BOT_NODES<float>, e->cs>>>(e->dmg, e->dhead, none);
+            PB_CUDA_TRY(graph_kernel(G, &last, k_mg_bottom<mg::Entry, false>, (unsigned)e->cap, mg::BOT_T,
+                                     mg::BOT_BYTES<float> * mg::BOT_NODES<float>, e->dmg, e->dhead, none));
         for (int l = depth - 1; l >= 0; --l)
             if (l == 0)
-                k_mg_up0<false><<<ru0, mg::U0NT, 0, e->cs>>>(e->dmg, e->dhead, 0, none);
+                PB_CUDA_TRY(graph_kernel(G, &last, k_mg_up0<false>, ru0, mg::U0NT, 0, e->dmg, e->dhead, 0, none));
             else
-                k_mg_up<false><<<ru1, mg::UNT, 0, e->cs>>>(e->dmg, e->dhead, l, 0, none);
-        tma_launch<MODE_P>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
-        tma_launch<MODE_U>(e->dtab, -1, 0, e->queue, e->grid, e->cs);
+                PB_CUDA_TRY(graph_kernel(G, &last, k_mg_up<false>, ru1, mg::UNT, 0, e->dmg, e->dhead, l, 0, none));
+        PB_CUDA_TRY(graph_kernel(G, &last, k_stencil_tma<MODE_P, false, 0>, e->grid, tma::NTHREADS,
+                                 tma::smem_bytes<MODE_P, 0>(), e->dtab, -1, 0, e->queue, zero));
+        PB_CUDA_TRY(graph_kernel(G, &last, k_stencil_tma<MODE_U, false, 0>, e->grid, tma::NTHREADS,
+                                 tma::smem_bytes<MODE_U, 0>(), e->dtab, -1, 0, e->queue, zero));
     }
-    ENG_TRY(cudaStreamEndCapture(e->cs, &e->graph[g]), "capture");
-    ENG_TRY(cudaGraphInstantiate(&e->exec[g], e->graph[g], 0), "graph instantiation");
-    return true;
+    PB_CUDA_TRY(cudaGraphInstantiate(&e->exec[g], G, 0));
+    return PB_OK;
 }
 
 // rewrite the device launch table from the occupied slots (stream-ordered
@@ -356,7 +384,7 @@ bool engine_upload_table(Engine *e) {
     e->tab_buf ^= 1;
     e->depth = depth;
     e->mg = any;
-    return engine_capture(e);
+    return true;
 }
 
 // a slot's solve ended: report it and free the slot
@@ -408,7 +436,7 @@ bool engine_issue(Engine *e, int mb) {
     }
     if (sides > 0) ENG_TRY(cudaEventRecord(e->ev_fork, e->cs), "octree fork");
     if (octs < taken) {
-        ENG_TRY(cudaGraphLaunch(e->exec[e->mg ? e->depth : mg::LMAX], e->cs), "replay");
+        ENG_TRY(cudaGraphLaunch(e->exec[replay_key(e->mg, e->depth)], e->cs), "replay");
         note_launch(chunk * (2 + (e->depth > 0 ? 2 * e->depth + 1 : 0)));
     }
     for (int k = 0; k < sides; ++k) ENG_TRY(cudaStreamWaitEvent(e->side[k], e->ev_fork, 0), "octree fork");
@@ -573,7 +601,7 @@ void engine_release(Engine *e) {
 
 }  // namespace
 
-pb_status engine_create(int device, int capacity, const pb_solve_opts *o, pb_engine **out) {
+pb_status engine_create(int device, int capacity, const pb_solve_opts *o, bool serve, pb_engine **out) {
     Engine *e = new (std::nothrow) Engine();
     if (!e) return PB_ERR_OOM;
     e->device = device;
@@ -618,6 +646,13 @@ pb_status engine_create(int device, int capacity, const pb_solve_opts *o, pb_eng
     if (tma_prepare<MODE_P>() != PB_OK || tma_prepare<MODE_U>() != PB_OK || mg_prepare() != PB_OK)
         return bail(PB_ERR_CUDA, "kernel attributes");
     e->grid = tma_grid(PadGeo{}, 8);
+    // a server's replays (0.3 ms), so that no first request waits for its own; a
+    // batch takes those that its systems ask for, and so do deeper hierarchies
+    for (int d = -1; serve && d <= 6; ++d)
+        if (const pb_status rc = engine_replay(e, d >= 0, std::max(d, 0)); rc != PB_OK) {
+            engine_release(e);
+            return rc;
+        }
     if (cudaStreamSynchronize(e->cs) != cudaSuccess) return bail(PB_ERR_CUDA, "set-up");
     try {
         e->th = std::thread(engine_pump, e);
@@ -694,6 +729,11 @@ pb_status engine_submit(pb_engine *eh, pb_system *sys, cudaStream_t s, long long
         if (busy()) {
             cudaEventDestroy(j.ready);
             return PB_ERR_ARG;
+        }
+        const int depth = sys->mg && !j.oct ? ((const MgState *)sys->mg)->e.nbot : 0;
+        if ((rc = engine_replay(e, sys->mg != nullptr, depth)) != PB_OK) {
+            cudaEventDestroy(j.ready);
+            return rc;
         }
         j.ticket = e->next_ticket++;
         e->pending.push_back(j);

@@ -264,7 +264,8 @@ pb_status solve_batch(pb_system *const *systems, int n, const pb_solve_opts *o, 
                       pb_solve_stats *stats);
 pb_status solve_split(pb_system *sys, int ranks, const pb_solve_opts *o, cudaStream_t s,
                       pb_solve_stats *stats);
-pb_status engine_create(int device, int capacity, const pb_solve_opts *o, pb_engine **out);
+// serve: for systems that are not known yet
+pb_status engine_create(int device, int capacity, const pb_solve_opts *o, bool serve, pb_engine **out);
 pb_status engine_submit(pb_engine *e, pb_system *sys, cudaStream_t s, long long *ticket);
 pb_status engine_wait(pb_engine *e, double timeout_s, pb_engine_result *out, int max_out, int *n_out);
 pb_status engine_query(pb_engine *e, int *n_pending, int *n_active, long long *replays);

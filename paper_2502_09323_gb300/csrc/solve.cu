@@ -1782,7 +1782,7 @@ pb_status solve_batch(pb_system *const *systems, int n, const pb_solve_opts *o, 
     const double t_start = now_s();
     const double deadline = o->time_budget_s > 0.0 ? t_start + o->time_budget_s : 0.0;
     pb_engine *eh = nullptr;
-    pb_status rc = engine_create(systems[0]->g->device, n, o, &eh);
+    pb_status rc = engine_create(systems[0]->g->device, n, o, false, &eh);
     if (rc != PB_OK) return rc;
     std::map<long long, int> index;
     std::vector<int> got(n, 0);
