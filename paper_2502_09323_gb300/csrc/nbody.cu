@@ -39,7 +39,9 @@ constexpr double NB_ORIGIN_EXT = 8.0;
 // Octrees with at least so many pairs take local expansions for far atoms.
 // Sorting the targets and the balls take about 0.2 ms: pairs and expansions both
 // take 0.3 ms with 1,000 atoms (3.2e8 pairs), and 0.9 and 0.53 ms with 2,000 (1.2e9).
-// Uniform grids keep all pairs, whose sums are an output to the last bit.
+// Uniform grids keep all pairs: expansions there (0.52 instead of 0.99 ms at
+// 257^3 with 2,000 atoms) were tried in a form whose near pairs had a larger
+// error (Psi 1.57e-7 -> 1.89e-7 from 64 bits), and not since.
 constexpr long long FAR_PAIRS = 400000000;
 
 struct SrcHi {
@@ -394,10 +396,11 @@ k_nbody(TargetDesc T, far::Args F, const float4 *__restrict__ shi, const float4 
         if (__syncthreads_and(same)) axis = dref;
     }
     // a block whose surface targets all lie within NB_ORIGIN_EXT of its
-    // first target takes the differences from that origin
+    // first target takes the differences from that origin (FAR: not the near
+    // pairs, see nbody_far.cuh)
     bool origin = false;
     float oh[3] = {0.f, 0.f, 0.f}, ol[3] = {0.f, 0.f, 0.f};
-    if (T.kind == TK_SURFACE) {
+    if (!FAR && T.kind == TK_SURFACE) {
         double o[3], rel[NB_TPT][3];
         bool near = true;
 #pragma unroll
@@ -423,7 +426,7 @@ k_nbody(TargetDesc T, far::Args F, const float4 *__restrict__ shi, const float4 
         }
     }
 #define PB_NB_TILES(AX)                                                                          \
-    (origin ? nb_tiles<PSI, SCREEN, PSI2, AX, true, FAR>(sp4, ball, shi, slo, ns, kscr, oh, ol,  \
+    (!FAR && origin ? nb_tiles<PSI, SCREEN, PSI2, AX, true, false>(sp4, ball, shi, slo, ns, kscr, oh, ol,  \
                                                          th, tl, tn, tn2, acc_phi, acc_psi, acc_psi2) \
             : nb_tiles<PSI, SCREEN, PSI2, AX, false, FAR>(sp4, ball, shi, slo, ns, kscr, oh, ol, \
                                                           th, tl, tn, tn2, acc_phi, acc_psi, acc_psi2))
