@@ -462,7 +462,8 @@ k_nbody(TargetDesc T, far::Args F, const float4 *__restrict__ shi, const float4 
 #pragma unroll
             for (int d = 0; d < 3; ++d)
                 g[d] = (S.top[1 + d] + (double)(u ? v[1 + d].y : v[1 + d].x)) * (ball.inv * ball.inv);
-            acc_phi[u] += (S.top[0] + (double)(u ? v[0].y : v[0].x)) * ball.inv;
+            acc_phi[u] += fma(S.top[3], x[u][2], fma(S.top[2], x[u][1], fma(S.top[1], x[u][0], S.top[0]))) * ball.inv +
+                          (double)(u ? v[0].y : v[0].x) * ball.inv;
             const double ga = axis == 0 ? g[0] : (axis == 1 ? g[1] : g[2]);
             acc_psi[u] -= axis >= 0 ? ga
                                     : g[0] * (double)tg[u].n[0] + g[1] * (double)tg[u].n[1] + g[2] * (double)tg[u].n[2];

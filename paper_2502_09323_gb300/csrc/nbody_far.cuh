@@ -25,7 +25,7 @@
 // Measured (GB300, surface sums, all pairs -> this): octree of 20,000 atoms
 // 73.0 -> 8.7 ms (coefficients 4.5, near pairs and evaluation 3.9), 2,000
 // atoms 0.9 -> 0.53 ms.  Errors against 64 bits,
-// 2-norm relative, of Phi 1.26e-7 -> 8.3e-8 and of Psi 1.84e-7 -> 1.53e-7 (20,000
+// 2-norm relative, of Phi 1.26e-7 -> 8.1e-8 and of Psi 1.84e-7 -> 1.53e-7 (20,000
 // atoms).  What gave it, one after the other: targets in list order, whose
 // blocks are wide, 20.6 ms; a power of two as unit and compensated sums of
 // degrees 0 and 1, no slower and more exact than all pairs; rods of bricks as
@@ -287,7 +287,8 @@ namespace far {
 // The block's expansion in shared memory: for every (l, m) the coefficients of
 // the potential and of its three derivatives, each value twice (a thread's two
 // targets share an instruction), 2 for m > 0 included; those of R_00, which
-// are the largest, apart in FP64.
+// are the largest, apart in FP64 (the gradient's are the potential's linear
+// term too: with charges of one sign that is a tenth of the potential).
 struct Series {
     float4 c[NC][4];  // potential, d/dx, d/dy, d/dz: (re, re, im, im)
     double top[4];
@@ -334,7 +335,8 @@ __device__ __forceinline__ void make_series(const Args &A, double2 *L, Series &S
         }
     }
 }
-// potential and gradient (without the terms of R_00) at two targets, in the ball's unit
+// potential (without its terms of degrees 0 and 1, top[0] + top[1..3] . x) and
+// gradient (without those of degree 0, top[1..3]) at two targets, in the ball's unit
 __device__ __forceinline__ void evaluate(const Series &S, const float2 (&x)[3], float2 (&out)[4]) {
     const float2 one = make_float2(1.f, 1.f), r2 = __ffma2_rn(x[2], x[2], __ffma2_rn(x[1], x[1], __fmul2_rn(x[0], x[0])));
     const float2 nr2 = make_float2(-r2.x, -r2.y), ny = make_float2(-x[1].x, -x[1].y);
@@ -364,7 +366,7 @@ __device__ __forceinline__ void evaluate(const Series &S, const float2 (&x)[3], 
             }
             if (l == 0) continue;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = l == 1 ? 1 : 0; q < 4; ++q) {
                 const float4 v = S.c[at(l, m)][q];
                 out[q] = __ffma2_rn(make_float2(v.x, v.y), ar, __ffma2_rn(make_float2(v.z, v.w), ai, out[q]));
             }
