@@ -17,10 +17,11 @@
 // all pairs had no such blocks (9,000 atoms at 0.5 A: Psi 2.02e-7 from 64
 // bits against 1.69e-7; split 1.55e-7, in the same time).
 //
-// P = 12 and KAPPA = 3 leave a truncation error of at most 3e-8 of
-// sum |q| / r^2 in the gradient and 2e-10 of sum |q| / r in the potential
-// (20,000 atoms in a 45 A ball, a = 3 and 5 A, against 64 bits), below the
-// rounding of the FP32 pair sum.  Atoms beyond 2 KAPPA a take degree PD.
+// P = 12 and KAPPA = 3 leave a truncation error below one FP32 rounding of
+// sum |q| / r^2 in the gradient (at most 4.2e-8 in blocks at the surface of
+// 20,000 atoms in a 45 A ball, a = 3 and 5 A, against 64 bits; P = 11: 9.5e-8)
+// and 2.8e-10 of sum |q| / r in the potential, below the rounding of the FP32
+// pair sum.  Atoms beyond 2 KAPPA a take degree PD.
 //
 // Measured (GB300, surface sums, all pairs -> this): octree of 20,000 atoms
 // 73.0 -> 8.7 ms (coefficients 4.5, near pairs and evaluation 3.9), 2,000
