@@ -2429,37 +2429,23 @@ pb_status oct_mg_make(pb_system *sys, cudaStream_t s) {
 
 pb_status oct_ensure_ws(pb_system *sys, int precision, cudaStream_t s) {
     const long long N = sys->g->ot.N;
-    if (!sys->st) {
-        sys->st = (CgState *)dalloc(sizeof(CgState), s);
-        if (!sys->st) return PB_ERR_OOM;
-        PB_CUDA_TRY(cudaMemsetAsync(sys->st, 0, sizeof(CgState), s));
-        PB_CUDA_TRY(cudaMallocHost((void **)&sys->h_st, 4 * sizeof(CgState)));
+    pb_status rc = PB_OK;
+    if ((rc = keep(sys->st, sizeof(CgState), s)) != PB_OK) return rc;
+    if (!sys->h_st) PB_CUDA_TRY(cudaMallocHost((void **)&sys->h_st, 4 * sizeof(CgState)));
+    if (!sys->partials) {
         const int G = std::max(std::max(pure_grid<float, OM_P>(), pure_grid<float, OM_U>()),
                                std::max(std::max(pure_grid<double, OM_P>(), pure_grid<double, OM_U>()),
                                         pure_grid<float, OM_L>()));
         sys->npartials = 2 * (int)std::max<long long>(cdiv(N, OT), G) + 64;
-        sys->partials = (double *)dalloc(sizeof(double) * sys->npartials, s);
-        if (!sys->partials) return PB_ERR_OOM;
     }
+    if ((rc = keep(sys->partials, sizeof(double) * sys->npartials, s, false)) != PB_OK) return rc;
     const size_t b32 = sizeof(float) * (size_t)N, b64 = sizeof(double) * (size_t)N;
-    if (precision == PB_MIXED && !sys->z32) {
-        sys->z32 = (float *)dalloc(b32, s);
-        sys->pa32 = (float *)dalloc(b32, s);
-        sys->pb32 = (float *)dalloc(b32, s);
-        sys->d32 = (float *)dalloc(b32, s);
-        if (!sys->z32 || !sys->pa32 || !sys->pb32 || !sys->d32) return PB_ERR_OOM;
-        for (float *q : {sys->z32, sys->pa32, sys->pb32, sys->d32})
-            PB_CUDA_TRY(cudaMemsetAsync(q, 0, b32, s));
-    }
-    if (precision == PB_FP64 && !sys->z64) {
-        sys->z64 = (double *)dalloc(b64, s);
-        sys->pa64 = (double *)dalloc(b64, s);
-        sys->pb64 = (double *)dalloc(b64, s);
-        sys->x64 = (double *)dalloc(b64, s);
-        if (!sys->z64 || !sys->pa64 || !sys->pb64 || !sys->x64) return PB_ERR_OOM;
-        for (double *q : {sys->z64, sys->pa64, sys->pb64, sys->x64})
-            PB_CUDA_TRY(cudaMemsetAsync(q, 0, b64, s));
-    }
+    if (precision == PB_MIXED)
+        for (float **q : {&sys->z32, &sys->pa32, &sys->pb32, &sys->d32})
+            if ((rc = keep(*q, b32, s)) != PB_OK) return rc;
+    if (precision == PB_FP64)
+        for (double **q : {&sys->z64, &sys->pa64, &sys->pb64, &sys->x64})
+            if ((rc = keep(*q, b64, s)) != PB_OK) return rc;
     return PB_OK;
 }
 

@@ -34,6 +34,22 @@ void note_launch(long long n);
 void *dalloc(size_t bytes, cudaStream_t s);   // nullptr on failure
 void dfree(void *p, cudaStream_t s);
 
+// Memory that a system keeps between calls: allocated (and cleared) where it is
+// not there yet, so that a call after one that ran out of memory goes on where
+// that one stopped.
+template <typename T>
+pb_status keep(T *&p, size_t bytes, cudaStream_t s, bool clear = true) {
+    if (p) return PB_OK;
+    p = (T *)dalloc(bytes, s);
+    if (!p) return PB_ERR_OOM;
+    const cudaError_t e = clear ? cudaMemsetAsync(p, 0, bytes, s) : cudaSuccess;
+    if (e == cudaSuccess) return PB_OK;
+    dfree(p, s);
+    p = nullptr;
+    set_error("clearing a workspace failed: %s", cudaGetErrorString(e));
+    return PB_ERR_CUDA;
+}
+
 // Device-side error flags written by kernels (bit mask).
 enum : uint32_t {
     ERRF_ATOM_VALUE = 1u,      // NaN/Inf coordinate or non-positive radius

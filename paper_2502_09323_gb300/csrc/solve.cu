@@ -1376,54 +1376,31 @@ pb_status ensure_queue(pb_system *sys, cudaStream_t s) {
 
 pb_status ensure_solver_ws(pb_system *sys, int precision, cudaStream_t s) {
     const PadGeo &p = sys->pad;
-    pb_status rc0 = PB_OK;
-    if (!sys->st) {
-        sys->st = (CgState *)dalloc(sizeof(CgState), s);
-        if (!sys->st) return PB_ERR_OOM;
-        PB_CUDA_TRY(cudaMemsetAsync(sys->st, 0, sizeof(CgState), s));
-        PB_CUDA_TRY(cudaMallocHost((void **)&sys->h_st, 4 * sizeof(CgState)));
+    pb_status rc = PB_OK;
+    if ((rc = keep(sys->st, sizeof(CgState), s)) != PB_OK) return rc;
+    if (!sys->h_st) PB_CUDA_TRY(cudaMallocHost((void **)&sys->h_st, 4 * sizeof(CgState)));
+    if (!sys->partials) {
         dim3 g32 = stencil_grid<float>(p, 4), g64 = stencil_grid<double>(p, 4);
         long long nb = std::max<long long>((long long)g32.x * g32.y * g32.z,
                                            (long long)g64.x * g64.y * g64.z);
         nb = std::max<long long>(nb, cdiv(p.N, 256));
         sys->npartials = (int)(2 * nb + 64);
-        sys->partials = (double *)dalloc(sizeof(double) * sys->npartials, s);
-        if (!sys->partials) return PB_ERR_OOM;
-        if ((rc0 = ensure_queue(sys, s)) != PB_OK) return rc0;
     }
-    size_t bytes32 = sizeof(float) * (size_t)p.Np, bytes64 = sizeof(double) * (size_t)p.Np;
-    if (precision == PB_MIXED && !sys->z32) {
-        sys->z32 = (float *)dalloc(bytes32, s);
-        sys->pa32 = (float *)dalloc(bytes32, s);
-        sys->pb32 = (float *)dalloc(bytes32, s);
-        sys->d32 = (float *)dalloc(bytes32, s);
-        if (!sys->z32 || !sys->pa32 || !sys->pb32 || !sys->d32) return PB_ERR_OOM;
-        PB_CUDA_TRY(cudaMemsetAsync(sys->z32, 0, bytes32, s));
-        PB_CUDA_TRY(cudaMemsetAsync(sys->pa32, 0, bytes32, s));
-        PB_CUDA_TRY(cudaMemsetAsync(sys->pb32, 0, bytes32, s));
-        PB_CUDA_TRY(cudaMemsetAsync(sys->d32, 0, bytes32, s));
-    }
-    if (precision == PB_FP64 && !sys->z64) {
-        sys->z64 = (double *)dalloc(bytes64, s);
-        sys->pa64 = (double *)dalloc(bytes64, s);
-        sys->pb64 = (double *)dalloc(bytes64, s);
-        sys->x64 = (double *)dalloc(bytes64, s);
-        if (!sys->z64 || !sys->pa64 || !sys->pb64 || !sys->x64) return PB_ERR_OOM;
-        PB_CUDA_TRY(cudaMemsetAsync(sys->z64, 0, bytes64, s));
-        PB_CUDA_TRY(cudaMemsetAsync(sys->pa64, 0, bytes64, s));
-        PB_CUDA_TRY(cudaMemsetAsync(sys->pb64, 0, bytes64, s));
-        PB_CUDA_TRY(cudaMemsetAsync(sys->x64, 0, bytes64, s));
-    }
-    if (precision == PB_FP64 && !sys->r64 && !sys->g->is_oct) {
+    if ((rc = keep(sys->partials, sizeof(double) * sys->npartials, s, false)) != PB_OK) return rc;
+    if ((rc = ensure_queue(sys, s)) != PB_OK) return rc;
+    const size_t bytes32 = sizeof(float) * (size_t)p.Np, bytes64 = sizeof(double) * (size_t)p.Np;
+    if (precision == PB_MIXED)
+        for (float **q : {&sys->z32, &sys->pa32, &sys->pb32, &sys->d32})
+            if ((rc = keep(*q, bytes32, s)) != PB_OK) return rc;
+    if (precision == PB_FP64)
+        for (double **q : {&sys->z64, &sys->pa64, &sys->pb64, &sys->x64})
+            if ((rc = keep(*q, bytes64, s)) != PB_OK) return rc;
+    if (precision == PB_FP64 && !sys->op64[4]) {
         // the plain solver keeps r and q, and a padded copy of the operator
-        sys->r64 = (double *)dalloc(bytes64, s);
-        sys->q64 = (double *)dalloc(bytes64, s);
-        for (int a = 0; a < 5; ++a) sys->op64[a] = (double *)dalloc(bytes64, s);
-        if (!sys->r64 || !sys->q64 || !sys->op64[0] || !sys->op64[1] || !sys->op64[2] ||
-            !sys->op64[3] || !sys->op64[4])
-            return PB_ERR_OOM;
-        PB_CUDA_TRY(cudaMemsetAsync(sys->r64, 0, bytes64, s));
-        PB_CUDA_TRY(cudaMemsetAsync(sys->q64, 0, bytes64, s));
+        for (double **q : {&sys->r64, &sys->q64})
+            if ((rc = keep(*q, bytes64, s)) != PB_OK) return rc;
+        for (double *&q : sys->op64)
+            if ((rc = keep(q, bytes64, s, false)) != PB_OK) return rc;
         k_cg64_operator<<<cdiv(p.Np, 256), 256, 0, s>>>(sys->W[0], sys->W[1], sys->W[2], sys->diag,
                                                          sys->g->geo, p, sys->op64[0], sys->op64[1],
                                                          sys->op64[2], sys->op64[3], sys->op64[4]);

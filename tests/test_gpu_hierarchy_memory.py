@@ -118,3 +118,25 @@ def test_without_room_for_a_hierarchy(env, kind, batch):
         # what was refused, and all that belongs to it, had been given back
         assert sum(b for _, b in h.live.values()) - live >= sizes[at]
         s.free()
+
+
+@pytest.mark.parametrize("kind", list(KINDS))
+def test_solve_after_one_that_ran_out_of_memory(env, kind):
+    """Every allocation of a first solve that it cannot do without, refused in turn: the solve
+    reports it, and the next one of the same system goes on from what is there."""
+    pb, h = env
+    make, prec, vectors, _, _ = KINDS[kind]
+    opts = pb.SolveOpts(precision=prec, rtol=1e-10)
+    s, n = make(pb)
+    h.reset()
+    ref = pb.pb_solve(s, opts)
+    sizes, phi = list(h.sizes), pb.pb_get_phi(s)
+    last = [at for at, b in enumerate(sizes) if b == (4 if prec else 8) * n][vectors - 1]
+    for at in range(last + 1):
+        s, _ = make(pb)
+        h.reset(refuse=lambda q, _: q == at)
+        assert pb.pb_solve(s, opts, check=False)["rc"] == -2
+        h.reset()
+        st = pb.pb_solve(s, opts)
+        assert st["iters_inner"] == ref["iters_inner"] and np.array_equal(pb.pb_get_phi(s), phi)
+        s.free()
