@@ -734,46 +734,47 @@ pb_status nbody_surface(pb_system *sys, cudaStream_t s) {
     if (!sys->PsiN) sys->PsiN = (double *)dalloc(sizeof(double) * nc, s);
     if (!sys->PsiN) return PB_ERR_OOM;
     T.nrm2 = g->mc_n;
-    int *order = nullptr;
-    if (g->is_oct && g->na * g->ncross >= FAR_PAIRS && (st = order_targets(g, &order, s)) != PB_OK) {
-        dfree(hi, s);
-        dfree(lo, s);
-        return st;
-    }
-    T.order = order;
     const int per = NB_THREADS * NB_TPT;
     const unsigned blocks = cdiv(T.count, per);
     far::Args F{};
-    if (!order) {
+    F.chunks = (int)cdiv(g->na, far::CHUNK);
+    // so many target blocks at a time that their partial sums stay within far::BYTES
+    const size_t each = sizeof(float2) * far::NS * (size_t)F.chunks;
+    const unsigned parts = cdiv(blocks, std::max<long long>(far::BYTES / (long long)std::max<size_t>(each, 1), 1)), most = cdiv(blocks, parts);
+    int *order = nullptr;
+    far::Ball *ball = nullptr;
+    float2 *part = nullptr;
+    if (g->is_oct && g->na * g->ncross >= FAR_PAIRS && F.chunks <= 65535) {  // chunks: the grid's y
+        st = order_targets(g, &order, s);
+        if (order) {
+            ball = (far::Ball *)dalloc(sizeof(far::Ball) * blocks, s);
+            part = (float2 *)dalloc(each * most, s);
+            if (!ball || !part) st = PB_ERR_OOM;
+        }
+        if (st == PB_ERR_OOM) {  // all pairs need no scratch
+            dfree(order, s);
+            order = nullptr;
+            set_error("");
+            st = PB_OK;
+        }
+    }
+    if (order) {
+        T.order = order;
+        F.ball = ball;
+        F.part = part;
+        k_far_ball<<<blocks, 256, 0, s>>>(g->crp, T.order, T.count, g->center[0], g->center[1], g->center[2], ball);
+        for (unsigned b = 0; b < blocks; b += most) {
+            const unsigned n = std::min(most, blocks - b);
+            F.block0 = b;
+            k_far_local<<<dim3(n, (unsigned)F.chunks), far::T, 0, s>>>(hi, lo, g->na, ball, b, part);
+            k_nbody<true, false, true, true>
+                <<<n, NB_THREADS, 0, s>>>(T, F, hi, lo, g->na, 0.f, 1.0, sys->Phi, sys->Psi, sys->PsiN);
+        }
+    } else if (st == PB_OK) {
         k_nbody<true, false, true>
             <<<blocks, NB_THREADS, 0, s>>>(T, F, hi, lo, g->na, 0.f, 1.0, sys->Phi, sys->Psi, sys->PsiN);
-        PB_LAUNCH_CHECK();
-    } else {
-        // so many target blocks at a time that their partial sums stay within far::BYTES
-        F.chunks = (int)cdiv(g->na, far::CHUNK);
-        const size_t each = sizeof(float2) * far::NS * (size_t)F.chunks;
-        const unsigned parts = cdiv(blocks, std::max<long long>(far::BYTES / (long long)each, 1)), most = cdiv(blocks, parts);
-        far::Ball *ball = (far::Ball *)dalloc(sizeof(far::Ball) * blocks, s);
-        float2 *part = (float2 *)dalloc(each * most, s);
-        if (ball && part) {
-            F.ball = ball;
-            F.part = part;
-            k_far_ball<<<blocks, 256, 0, s>>>(g->crp, T.order, T.count, g->center[0], g->center[1], g->center[2], ball);
-            for (unsigned b = 0; b < blocks; b += most) {
-                const unsigned n = std::min(most, blocks - b);
-                F.block0 = b;
-                k_far_local<<<dim3(n, (unsigned)F.chunks), far::T, 0, s>>>(hi, lo, g->na, ball, b, part);
-                k_nbody<true, false, true, true>
-                    <<<n, NB_THREADS, 0, s>>>(T, F, hi, lo, g->na, 0.f, 1.0, sys->Phi, sys->Psi, sys->PsiN);
-            }
-        }
-        dfree(ball, s);
-        dfree(part, s);
-        if (!ball || !part) st = PB_ERR_OOM;
     }
-    dfree(order, s);
-    dfree(hi, s);
-    dfree(lo, s);
+    for (void *q : {(void *)order, (void *)ball, (void *)part, (void *)hi, (void *)lo}) dfree(q, s);
     if (st != PB_OK) return st;
     PB_LAUNCH_CHECK();
     return PB_OK;
