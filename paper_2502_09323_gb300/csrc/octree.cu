@@ -826,7 +826,8 @@ __global__ void k_oct_tr_rowmap(const int *__restrict__ tr_slot, long long ntr, 
 
 // Entries of a row that the counting pass keeps (rows have 11 on average, 21
 // at most on the trees measured), row r's q-th at q * ntr + r; longer rows
-// are formed again when they are written out.
+// are formed again when they are written out, and so are all where memory has
+// no room for the kept ones.
 constexpr int KEEP = 24;
 
 __global__ void __launch_bounds__(128)
@@ -843,7 +844,7 @@ k_oct_tr_count(OctDev t, BcDesc bd, const uint8_t *__restrict__ inside, LevelCon
     zero.kind = PB_BC_ZERO;  // counting needs no boundary values
     transition_row(t, zero, inside, lc, eps_out, P, acc);
     nnz[r] = acc.n;
-    for (int q = 0; q < acc.n && q < KEEP; ++q) {
+    for (int q = 0; kcol && q < acc.n && q < KEEP; ++q) {
         kcol[q * ntr + r] = acc.col[q];
         kval[q * ntr + r] = acc.val[q];
     }
@@ -2202,6 +2203,16 @@ pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
     long long nnz = 0;
     int *kcol = nullptr;
     double *kval = nullptr;
+    auto drop_kept = [&] {
+        dfree(kcol, s);
+        dfree(kval, s);
+        kcol = nullptr;
+        kval = nullptr;
+    };
+    struct AtEnd {
+        decltype(drop_kept) &drop;
+        ~AtEnd() { drop(); }
+    } at_end{drop_kept};
     if (ntr > 0) {
         // rows in increasing slot order
         size_t tb = 0;
@@ -2218,7 +2229,10 @@ pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
         const BcDesc bd = bc_desc(sys);
         kcol = (int *)dalloc(sizeof(int) * KEEP * ntr, s);
         kval = (double *)dalloc(sizeof(double) * KEEP * ntr, s);
-        if (!kcol || !kval) return PB_ERR_OOM;
+        if (!kcol || !kval) {  // no room: the rows are formed again when they are written out
+            drop_kept();
+            set_error("");
+        }
         k_oct_tr_count<<<cdiv(ntr, 128), 128, 0, s>>>(t, bd, g->inside, lc, sys->p.eps_out,
                                                        os->tr_slot, ntr, rn, err, kcol, kval);
         PB_LAUNCH_CHECK();
@@ -2240,8 +2254,6 @@ pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
     PB_CUDA_TRY(cudaStreamSynchronize(s));
     dfree(err, s);
     if (herr) {
-        dfree(kcol, s);
-        dfree(kval, s);
         set_error("octree: inconsistent level-transition row (flags %u)", herr);
         return PB_ERR_ARG;
     }
@@ -2259,16 +2271,20 @@ pb_status oct_assemble(pb_system *sys, cudaStream_t s) {
         os->nunk = (long long)h0 + ntr;
     }
     const long long nnz1 = nnz > 0 ? nnz : 1;
-    os->tr_col = (int *)dalloc(sizeof(int) * nnz1, s);
-    os->tr_val = (double *)dalloc(sizeof(double) * nnz1, s);
-    os->tr_val32 = (float *)dalloc(sizeof(float) * nnz1, s);
     os->npart = 2 * (int)std::max<long long>(cdiv(ntr1, OT), 1) + 8;
-    os->partials = (double *)dalloc(sizeof(double) * os->npart, s);
-    if (!os->tr_col || !os->tr_val || !os->tr_val32 || !os->partials) return PB_ERR_OOM;
-    const pb_status brc = oct_boundary_rhs_rows(sys, kcol, kval, s);
-    dfree(kcol, s);
-    dfree(kval, s);
-    return brc;
+    auto rows = [&] {
+        const bool ok = keep(os->tr_col, sizeof(int) * nnz1, s, false) == PB_OK &&
+                        keep(os->tr_val, sizeof(double) * nnz1, s, false) == PB_OK &&
+                        keep(os->tr_val32, sizeof(float) * nnz1, s, false) == PB_OK;
+        return ok && keep(os->partials, sizeof(double) * os->npart, s, false) == PB_OK;
+    };
+    if (!rows()) {
+        if (!kcol) return PB_ERR_OOM;
+        drop_kept();  // their room may do
+        if (!rows()) return PB_ERR_OOM;
+        set_error("");
+    }
+    return oct_boundary_rhs_rows(sys, kcol, kval, s);
 }
 
 void oct_system_free(pb_system *sys, cudaStream_t s) {

@@ -33,3 +33,37 @@ def test_surface_sums_without_room_for_expansions(env):  # noqa: F811
             assert np.linalg.norm(a - b) <= 1e-6 * np.linalg.norm(a)
             assert at is None or not np.array_equal(a, b)
         s.free()
+
+
+def test_transition_rows_without_room_for_kept_ones(env):  # noqa: F811
+    """The rows that the counting pass of an octree's assembly keeps: refused, they are formed again,
+    to the same bits; and they make room for the system's own arrays."""
+    pb, h = env
+    atoms = pb_inputs.globular_molecule(25, seed=54)
+    g = pb.pb_build_grid(pb.OctreeSpec(h_fine=0.25, h_bulk=1.0, refine_dist=3.0), atoms)
+    names = ("rhs", "diag")
+    opts = pb.SolveOpts(precision=pb.FP64, rtol=1e-12)
+
+    def assemble():
+        s = pb.pb_assemble_coeffs(g, pb.Params(bc=pb.BC_ZERO))
+        assert pb.pb_last_error() == ""
+        out = [pb.pb_get_array(s, k) for k in names]
+        pb.pb_solve(s, opts)
+        return s, out + [pb.pb_get_phi(s)]
+
+    h.reset()
+    s, ref = assemble()
+    sizes = list(h.sizes)
+    kept = [q for q in range(len(sizes) - 1) if sizes[q] % 96 == 0 and sizes[q] and sizes[q + 1] == 2 * sizes[q]]
+    assert len(kept) == 1
+    k = kept[0]
+    rows = sizes[k] // 96
+    values = next(q for q in range(k + 2, len(sizes)) if sizes[q + 1] == 2 * sizes[q] and sizes[q] > 4 * rows)
+    s.free()
+    before = len(h.live)
+    for at in (k, k + 1, values, values + 1):
+        h.reset(refuse=lambda q, _: q == at)
+        s, got = assemble()
+        assert all(np.array_equal(a, b) for a, b in zip(ref, got))
+        s.free()
+        assert len(h.live) == before
