@@ -882,10 +882,14 @@ pb_status grid_build(pb_grid *g, const pb_grid_spec *spec, cudaStream_t s) {
     }
     // candidates left for the union: an eighth of the nodes is far more than a
     // molecular surface has
-    const int cap = (int)std::min<long long>(N / 8 + 1024, 1 << 30);
+    int cap = (int)std::min<long long>(N / 8 + 1024, 1 << 30);
     long long *elist = (long long *)dalloc(sizeof(long long) * (size_t)cap, s);
+    if (!elist) {  // no room: all of them are found among the flags
+        cap = 0;
+        set_error("");
+    }
     int *ecount = (int *)dalloc(sizeof(int), s);
-    if (!elist || !ecount) return PB_ERR_OOM;
+    if (!ecount) return PB_ERR_OOM;
     PB_CUDA_TRY(cudaMemsetAsync(ecount, 0, sizeof(int), s));
     k_edge_flags<<<(unsigned)nchunks, CHUNK_THREADS, 0, s>>>(geo, g->inside, flags, cov, elist, cap, ecount);
     PB_LAUNCH_CHECK();

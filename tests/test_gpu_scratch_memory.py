@@ -67,3 +67,22 @@ def test_transition_rows_without_room_for_kept_ones(env):  # noqa: F811
         assert all(np.array_equal(a, b) for a, b in zip(ref, got))
         s.free()
         assert len(h.live) == before
+
+
+@pytest.mark.parametrize("n", [(49, 49, 49), (16, 37, 70)])
+def test_grid_without_room_for_the_candidate_list(env, n):  # noqa: F811
+    pb, h = env
+    atoms = pb_inputs.globular_molecule(40, seed=55)
+    atoms[:, :3] -= atoms[:, :3].mean(0)
+    step = 20.0 / (min(n) - 1)
+    spec = pb.GridSpec(n=n, origin=tuple(-0.5 * step * (m - 1) for m in n), h=step, fill=0.0)
+    names = ("cross_id", "cross_alpha", "cross_rp", "cross_sign", "mc_weight", "mc_normal")
+    h.reset()
+    g = pb.pb_build_grid(spec, atoms)
+    ref = [pb.pb_get_array(g, k) for k in names]
+    size = 8 * (n[0] * n[1] * n[2] // 8 + 1024)
+    assert h.sizes.count(size) == 1
+    h.reset(refuse=lambda q, sizes: sizes[q] == size)
+    g = pb.pb_build_grid(spec, atoms)
+    assert pb.pb_last_error() == "" and h.sizes.count(size) == 1
+    assert all(np.array_equal(a, pb.pb_get_array(g, k)) for a, k in zip(ref, names))
