@@ -1211,7 +1211,7 @@ __global__ void k_mg_coarsen(mg::LevT<T> F, mg::LevT<T> C, const double *__restr
                 if (2 * c[d] + 1 <= n[d] - 2) {
                     x[d] += 1;
                     const T q = weight(d, x);
-                    w = (T)0.5 * (p * q / (p + q) + (T)0.25 * (p + q));
+                    w = (T)0.5 * (p * (q / (p + q)) + (T)0.25 * (p + q));  // p q may leave the range of the type
                 } else {
                     w = p;  // one fine edge to the boundary
                 }

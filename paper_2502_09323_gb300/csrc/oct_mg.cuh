@@ -238,7 +238,7 @@ k_omg_lattice(OctDev t, const double *__restrict__ W0, const double *__restrict_
                 x[d] += 1;
                 m = slot(x[0], x[1], x[2]);
                 const float g = m >= 0 ? (float)W[d][m] : w_out;
-                sum += (b ? 0.5f : 1.f) * (c ? 0.5f : 1.f) * 0.5f * (f * g / (f + g) + 0.25f * (f + g));
+                sum += (b ? 0.5f : 1.f) * (c ? 0.5f : 1.f) * 0.5f * (f * (g / (f + g)) + 0.25f * (f + g));
             }
         out[d] = ex[d] ? sum : 0.f;
     }
