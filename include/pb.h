@@ -307,7 +307,7 @@ pb_status pb_apply(pb_system *s, int32_t precision, const void *x, void *y, void
  * sizes, uniform or octree) together: the CG solve of Eq. matrixequation
  * (Sec. 4) with FP32 inner iterations and FP64 iterative refinement.  PB_MIXED:
  * every system holds a slot of one launch table of persistent TMA-staged PCG
- * kernels, replayed as one captured CUDA graph; each system's refinement step
+ * kernels, replayed as a CUDA graph; each system's refinement step
  * is decided on the device as soon as its own inner solve ends (the
  * continuous-batching engine below, with capacity n).  PB_FP64: plain PCG,
  * one system after the other.  stats has n entries (each system's status;

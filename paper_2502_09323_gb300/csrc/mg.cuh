@@ -24,9 +24,9 @@
 // system in one launch (k_mg_bottom).  The up kernel of level 0 also sums
 // rho = r.z and takes the CG step beta = rho / rho_old.
 //
-// Measured (GB300, solves to 1e-12): 257^3 155.6 -> 12.9 ms (1,127 -> 30
-// iterations), 65^3 30.1 -> 2.1 ms, a batch of 24 systems of 97^3 to 161^3
-// 229 -> 51 ms.
+// Measured (GB300, solves to 1e-12): 257^3 155.6 -> 13.1 ms (1,127 -> 30
+// iterations; 33 to 36 are launched, as the host looks every other one), 65^3
+// 30.1 -> 2.1 ms, a batch of 24 systems of 97^3 to 161^3 229 -> 51 ms.
 //
 // Bounds: down reads s and a code byte per fine node and writes an eighth of
 // a value; up reads s, an eighth of a value and a code byte and writes z.
@@ -433,16 +433,17 @@ k_mg_up(const mg::Entry *__restrict__ tab, const mg::Head *__restrict__ head, in
 // table by the units' four solute bits, those of listed ones from listed_sums.
 //
 // 257^3, down and up: one row a thread with loads into registers a plane
-// ahead 102 and 139 us; this form 70 and 88 us (the first 21 and 25 us at the
-// measured copy rate, all that is read and written counted).  What was in the
-// way, one after the other: a gather of its own for each listed face (below);
+// ahead 102 and 139 us; this form 70 and 88 us by the same timing, 61 and 73 us
+// among the other kernels of a solve (21 and 25 us at the measured copy rate,
+// all that is read and written counted).  What was in the way, one after the other: a gather of its own for each listed face (below);
 // parameters read again after every asm statement (hence the local copies);
 // resident blocks that walked over their items, so that a block with the
 // molecule's surface in both of its items held up the launch (a one-system
 // launch now has a block an item); asynchronous copies of each thread's own,
 // 60 instructions a plane (TMA); the listed weights' latency (prefetched a
-// plane ahead).  Now bound by instruction issue (46 % of the issue slots) and
-// the barrier of each plane.
+// plane ahead).  Counters now (257^3): instructions issue in 44 and 47 % of
+// the cycles, the DRAM moves at 25 % of its rate; the listed weights' loads
+// (down) and the barrier of each plane (up) are what warps wait for most.
 namespace mg {
 constexpr int C0Y = 8, D0P = C0Y + 1, D0NT = 160;  // down: 32 x 8 coarse nodes, nine row pairs of 17 units
 constexpr int U0NT = 192;                          // up: eight row pairs, a warp of halo rows, a warp of halo columns

@@ -498,7 +498,7 @@ k_nbody(TargetDesc T, far::Args F, const float4 *__restrict__ shi, const float4 
 // summed in double precision (atoms staged in shared memory), in atom order.
 // FP64 issue binds: 25 operations a pair with screening, 13 without; the
 // library's sqrt, exp and division took about 70.  Blocks of 128 keep the
-// last wave full.  141 x 95 x 63 grid, 300 atoms, screened: 1,712 -> 780 us.
+// last wave full.  141 x 95 x 63 grid, 300 atoms, screened: 1,712 -> 813 us.
 // Positions are subtracted before k scales the distance: scaled first (24
 // operations), their rounding is relative to the coordinates, and a molecule
 // 1,000 A from the origin got 7.6e-16 instead of 6e-17 of sum |q| exp(-k r) / r.

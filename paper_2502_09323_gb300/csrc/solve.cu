@@ -19,9 +19,9 @@
 //
 // FP32 operator: per node one code byte (bit 0 solute, bits 1..3 "the +x/+y/+z
 // edge is listed"); unlisted edges have the pure weight eps h of the node's
-// medium, listed edges read their FP32 weight from the crossing list, found by
-// a binary search inside the edge's row.  The diagonal is rebuilt from the
-// six weights and the node's ionic term, so no coefficient array is streamed.
+// medium, listed edges read theirs from an FP32 array of the grid's shape.  The
+// diagonal is rebuilt from the six weights and the node's ionic term, so no
+// coefficient array is streamed.
 #include <limits.h>
 #include <math.h>
 
@@ -1632,8 +1632,8 @@ namespace {
 // planes in registers; x and y neighbours hit L1.  Each point's terms are
 // added in the order of the solver's kernels.  The former path copied x and y
 // to and from the padded layout around the TMA-staged kernel, with two
-// allocations, two clears and a host wait: 257^3 FP32 253 -> 96 us, 33^3 FP64
-// 32 -> 16 us (a Python call each).
+// allocations, two clears and a host wait: 257^3 FP32 253 -> 95 us, 33^3 FP64
+// 29 -> 15 us (a Python call each).
 template <typename T, class CP, int PTS>
 __global__ void __launch_bounds__(256)
 k_apply(const T *__restrict__ x, T *__restrict__ y, const uint8_t *__restrict__ code, GridGeo g, int sx, CP cp,
@@ -1750,7 +1750,7 @@ namespace pbg {
 
 // Batched mixed-precision solve through the continuous-batching engine: every
 // system takes a slot of one launch table, whose PCG iterations run as
-// replays of one captured graph, and each system's FP64 refinement steps are
+// replays of a graph, and each system's FP64 refinement steps are
 // decided on the device (k_ir_step) as soon as its own inner solve ends, so
 // no system waits for another's.  The host only watches the pinned state
 // mirror.  A system's arithmetic is the same as in pb_solve with the same

@@ -231,7 +231,7 @@ __device__ __forceinline__ void warp_nsum(float &s, float &c) {
 // MODE_P / MODE_U on the compressed FP32 operator, over every
 // system of tab (item_base ascending; total_items = sum of nitems).  With
 // nsys < 0 the table size and item total are read from queue[2] and
-// queue[3], so a captured launch follows a table that changes between
+// queue[3], so a launch of a graph follows a table that changes between
 // replays.
 // SINGLE: a launch over one system whose table entry (tensor maps,
 // geometry, coefficients) is the kernel parameter e0, so that its values are
@@ -309,8 +309,8 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
                 // direction kernel before it wrote p in item order, so the p
                 // of its last items is still in L2 when the update kernel
                 // starts there, and the next direction kernel starts on the
-                // z the update kernel wrote last.  Each item keeps its own
-                // partial slot, so the sums do not depend on the order.
+                // z the update kernel wrote last.  Each group of planes keeps
+                // its own partial slot, so the sums do not depend on the order.
                 const int it = MODE == MODE_U && !end ? total_items - 1 - item : item;
                 int sys = 0, li = 0, i0 = 0, j0 = 0, kfirst = 0, len = -1, cur = 0, tw = TWDEF;
                 const SysEntry *e = tab;
@@ -782,7 +782,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
             gt = gt0 + len + 2;
         }
     }
-    // this thread's item partials are visible device-wide before the block
+    // this thread's partials are visible device-wide before the block
     // counts itself done
     __threadfence();
     __syncthreads();
@@ -803,12 +803,12 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
     __syncthreads();
     if (!s_lastblk) return;
     __threadfence();
-    // Each system's item partials are summed in an order fixed by its
-    // item count only: systems of more than BIGSYS items by the whole
-    // block (thread t takes items t, t+NTHREADS, ...), smaller ones by
-    // one warp each.  The sums are compensated FP32 up to the warps'
-    // totals (this block runs alone at the end of the launch, on the
-    // critical path, and FP64 is a narrow pipe of GB300) and FP64 after.
+    // Each system's partials are summed in an order fixed by their number
+    // only: of systems with more than BIGSYS by the whole block (thread t
+    // takes partials t, t+NTHREADS, ...), of smaller ones by one warp each.
+    // The sums are compensated FP32 up to the warps' totals (this block runs
+    // alone at the end of the launch, on the critical path, and FP64 is a
+    // narrow pipe of GB300) and FP64 after.
     constexpr int BIGSYS = 512;
     __shared__ double s_red[2][NTHREADS / 32];
     auto finish = [&](CgState *st, double t0, double t1) {
@@ -854,8 +854,8 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
             }
         }
     };
-    // the warp's items summed; the totals are valid in lane 0
-    auto item_sums = [&](const SysEntry *e, int first, int stride, double &t0, double &t1) {
+    // the warp's partials summed; the totals are valid in lane 0
+    auto partial_sums = [&](const SysEntry *e, int first, int stride, double &t0, double &t1) {
         const int nit = e->npart;
         float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
 #pragma unroll 4
@@ -878,7 +878,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
         const int nit = e->npart;
         if (nit <= BIGSYS || *(volatile int *)&e->st->done) continue;
         double t0, t1;
-        item_sums(e, threadIdx.x, NTHREADS, t0, t1);
+        partial_sums(e, threadIdx.x, NTHREADS, t0, t1);
         if (lane == 0) {
             s_red[0][w] = t0;
             s_red[1][w] = t1;
@@ -902,7 +902,7 @@ k_stencil_tma(const tma::SysEntry *__restrict__ tab, int nsys, int total_items,
         // systems that were done at launch (or stopped by an abort) have no partials
         if (nit == 0 || nit > BIGSYS || *(volatile int *)&st->done) continue;
         double t0, t1;
-        item_sums(e, lane, 32, t0, t1);
+        partial_sums(e, lane, 32, t0, t1);
         if (lane == 0) finish(st, t0, t1);
     }
     __syncthreads();
