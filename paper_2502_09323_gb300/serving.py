@@ -27,9 +27,10 @@ from . import (CT_PAIRS, CT_SURFACE, Engine, GridSpec, OctreeSpec, Params, Solve
 GRID_SIZES = tuple(range(65, 2049, 32))
 
 # device bytes per padded node of one solve (FP64 faces, diagonal, rhs,
-# boundary values, iterate; FP32 weights, code bytes and four FP32 solver
-# vectors; grid classification), plus a fixed allowance for the crossing-edge
-# list, per-block partial sums and the launch-table entry
+# boundary values, iterate: 56; FP32 weights, code bytes and four FP32 solver
+# vectors: 29; grid classification: 1; multigrid hierarchy: 8), with a margin,
+# plus a fixed allowance for the crossing-edge list, per-block partial sums and
+# the launch-table entry
 BYTES_PER_NODE = 112
 FIXED_BYTES = 16 << 20
 
@@ -56,9 +57,9 @@ def octree_spec(atoms: np.ndarray, h_fine: float = 0.25, h_bulk: float = 1.0,
     return OctreeSpec(h_fine=h_fine, h_bulk=h_bulk, refine_dist=refine_dist, fill=fill)
 
 
-# octree: device bytes per node slot (the uniform set plus node kinds, inside
-# flags and the transition-row map), bytes per listed edge, and listed edges
-# per atom at 0.25 A (they scale with 1/h^2)
+# octree: device bytes per node slot (the uniform set's arrays plus node kinds,
+# the transition rows and their map, and the preconditioner's vectors), bytes
+# per listed edge, and listed edges per atom at 0.25 A (they scale with 1/h^2)
 OCT_BYTES_PER_SLOT = 112
 OCT_BYTES_PER_EDGE = 64
 OCT_EDGES_PER_ATOM = 400
